@@ -103,8 +103,8 @@ def _laplace(shape, g, scale):
     return -scale * torch.sign(d) * torch.log1p(-2.0 * d.abs())
 
 
-def _packed(g, N, K, B, G):
-    """A matrix in the device layout: bell-shaped signed codes as a fit leaves them, shape parameters of monotone cubics."""
+def _matrix(g, N, K, B, G):
+    """A stored matrix: bell-shaped signed codes as a fit leaves them, shape parameters of monotone cubics."""
     top = 1 if B == 1 else (1 << (B - 1)) - 1
     codes = torch.empty((N, K), dtype=torch.int8, device="cuda")
     rows = max(1, (1 << 26) // K)
@@ -118,6 +118,11 @@ def _packed(g, N, K, B, G):
     s = 0.03 + 0.06 * torch.rand(shape, generator=g, device="cuda")
     a = (0.5 + 0.5 * torch.rand(shape, generator=g, device="cuda")).half()
     b = (-0.3 * torch.rand(shape, generator=g, device="cuda")).half()
+    return codes, s, a, b
+
+
+def _packed(g, N, K, B, G):
+    codes, s, a, b = _matrix(g, N, K, B, G)
     return cq.cq_repack(cq.cq_pack_codes(codes, B), s, a, b, B, G, N, K)
 
 
@@ -135,6 +140,12 @@ def _product(g, c, N, K, B=None, G=None):
     x = _activations(g, M, K, c["dtype"])
     ws = torch.zeros(cq.cq_workspace_bytes(B, G, M, N, K, mode), dtype=torch.uint8, device="cuda")
     return pw, x, mode, ws, torch.empty((M, N), dtype=x.dtype, device="cuda")
+
+
+def _routes(g, c):
+    load = torch.rand((c["T"], c["E"]), generator=g, device="cuda") + 0.5 * torch.rand(c["E"], generator=g, device="cuda")   # some matrices are preferred
+    chosen = load.topk(c["top"], dim=1).indices
+    return chosen, chosen.flatten().argsort(stable=True)
 
 
 def _layer_sizes(c):
@@ -161,9 +172,7 @@ def prepare(case, seed):
         E, T = c["E"], c["T"]
         experts = [_packed(g, c["N"], c["K"], c["B"], c["G"]) for _ in range(E)]
         x = _activations(g, T, c["K"], c["dtype"])
-        load = torch.rand((T, E), generator=g, device="cuda") + 0.5 * torch.rand(E, generator=g, device="cuda")   # some matrices are preferred
-        chosen = load.topk(c["top"], dim=1).indices
-        order = chosen.flatten().argsort(stable=True)
+        chosen, order = _routes(g, c)
         counts = torch.bincount(chosen.flatten(), minlength=E).cumsum(0).tolist()
         return {"kind": kind, "experts": experts, "x": x, "route_token": (order // c["top"]).to(torch.int32), "offset": [0] + counts, "mode": MODE[c["mode"]]}
     W = torch.randn((c["N"], c["K"]), generator=g, device="cuda") * 0.02
@@ -221,3 +230,76 @@ def tolerance(case):
         # differences of 1e-3 in the first product move activations across INT8 rounding boundaries: whole steps of max|act| / 127
         return {"rel": 2e-2, "max": 0.2}
     return {"rel": 1e-2, "max": 0.05}   # bf16 outputs and temporary operands: 2^-9 each
+
+
+# ------------------------------------------------------------------ the same results in 64 bits
+def _levels(codes, a, b, B, G):
+    """sign(k) q(|k| / M) of rows of codes, q(t) = t (a + t (b + c t)) with c = 1 - a - b; two bits and fewer have no shape."""
+    k = codes.double()
+    if B <= 2:
+        return k
+    t = k.abs() / ((1 << (B - 1)) - 1)
+    a, b = (v.double().repeat_interleave(G, dim=1) for v in (a, b))
+    return k.sign() * t * (a + t * (b + t * (1.0 - a - b)))
+
+
+def _carriers(codes, a, b, B, G):
+    """sign(k) RNE(127 q), q by the 32-bit sequence that the format prescribes (a fused product and sum rounds once)."""
+    k = codes.double()
+    if B <= 2:
+        return 127.0 * k
+    a, b = (v.float().repeat_interleave(G, dim=1) for v in (a, b))
+    c = ((1.0 - a) - b).double()
+    t = (codes.float().abs() / float((1 << (B - 1)) - 1))
+    t64 = t.double()
+    q = t * (t64 * (t64 * c + b.double()).float().double() + a.double()).float()
+    return k.sign() * (127.0 * q).round().clamp(0, 127).double()
+
+
+def _exact_product(matrix, x, B, G, mode):
+    """x W^T in 64 bits; for Dynamic A8 from the INT8 activations and carriers, which the format defines in 32 bits."""
+    codes, s, a, b = matrix
+    out = torch.empty((x.shape[0], codes.shape[0]), dtype=torch.float64, device="cuda")
+    if mode == "a8":
+        f = x.float()
+        d = f.abs().amax(dim=1, keepdim=True).clamp_min(1e-10) / 127.0
+        v = f / d
+        x64 = (v.sign() * (v.double().abs() + 0.5).floor()).clamp(-127, 127).double()
+        decode, last = _carriers, d.double() / 127.0
+    else:
+        x64, decode, last = x.double(), _levels, 1.0
+    rows = max(1, (1 << 25) // codes.shape[1])
+    for r in range(0, codes.shape[0], rows):
+        part = slice(r, r + rows)
+        w = decode(codes[part], a[part], b[part], B, G) * s[part].double().repeat_interleave(G, dim=1)
+        out[:, part] = x64 @ w.T * last
+    return out
+
+
+def exact(case, seed):
+    c, g, kind = case, _generator(seed), case["kind"]
+    if kind in ("linear", "layer", "sweep"):
+        sizes = {"linear": lambda: [(c["N"], c["K"])], "layer": lambda: _layer_sizes(c), "sweep": lambda: [(c["N"], c["K"])] * len(SWEEP)}[kind]()
+        out = []
+        for (N, K), (B, G) in zip(sizes, SWEEP if kind == "sweep" else [(c["B"], c["G"])] * len(sizes)):
+            m = _matrix(g, N, K, B, G)
+            out.append(_exact_product(m, _activations(g, c["M"], K, c["dtype"]), B, G, c["mode"]))
+        return out
+    if kind == "mlp":
+        H, I = c["hidden"], c["inter"]
+        up, down = _matrix(g, 2 * I, H, c["B"], c["G"]), _matrix(g, H, I, c["B"], c["G"])
+        # both operators in front return the model dtype, and the last one quantises what it is given
+        h = _exact_product(up, _activations(g, c["M"], H, c["dtype"]), c["B"], c["G"], c["mode"]).to(DTYPE[c["dtype"]]).double()
+        act = (torch.nn.functional.silu(h[:, :I]) * h[:, I:]).to(DTYPE[c["dtype"]])
+        return _exact_product(down, act, c["B"], c["G"], "a8")
+    if kind == "routed":
+        experts = [_matrix(g, c["N"], c["K"], c["B"], c["G"]) for _ in range(c["E"])]
+        x = _activations(g, c["T"], c["K"], c["dtype"])
+        chosen, order = _routes(g, c)
+        expert, token = chosen.flatten()[order], order // c["top"]
+        out = torch.empty((order.numel(), c["N"]), dtype=torch.float64, device="cuda")
+        for e in range(c["E"]):
+            mine = expert == e
+            out[mine] = _exact_product(experts[e], x[token[mine]], c["B"], c["G"], c["mode"])
+        return out
+    return None   # codes and bytes: compared as they are
