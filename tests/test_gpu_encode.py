@@ -99,3 +99,22 @@ def test_encoded_on_the_gpu_runs_through_the_hot_path():
             x8, dx = oracle.quantize_a8(x)
             ref = oracle.gemm_a8(codes, sr, ar, br, B, G, K, x8, dx)
         assert np.linalg.norm(y - ref) <= 5e-3 * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("objective", ["continuous", "joint"])
+@pytest.mark.parametrize("B,G,effort", [(3, 32, "fast"), (4, 128, "fast"), (5, 512, "fast"), (7, 256, "fast"), (8, 512, "reference")])
+def test_search_where_weights_sit_on_the_thresholds(B, G, effort, objective):
+    # weights on a coarse lattice, so that many lie exactly half way between two levels of a uniform candidate; a number of
+    # groups that no block count divides; a group with one weight far outside; a group of one magnitude
+    N, K = (7, 3 * G) if effort == "fast" else (1, 2 * G)   # the dense search takes the oracle seconds a group
+    rng = np.random.default_rng(B * 1000 + G)
+    W = (rng.integers(-4 * (1 << (B - 1)), 4 * (1 << (B - 1)) + 1, size=(N, K)) * (0.25 / (1 << (B - 1)))).astype(np.float32)
+    W[0, 3] = 1e4
+    W[0, G:2 * G] = 0.5
+    W[-1, G:2 * G] *= np.float32(1e-20)
+    kr, sr, ar, br = oracle.encode(W, B, G, effort, objective=objective)
+    kg, sg, ag, bg = cq.cq_encode(dev(W), B, G, OBJ[objective], effort)
+    assert np.array_equal(kg.cpu().numpy(), kr)
+    assert np.array_equal(sg.cpu().numpy(), sr)
+    assert np.array_equal(ag.cpu().numpy().view(np.uint16), ar.view(np.uint16))
+    assert np.array_equal(bg.cpu().numpy().view(np.uint16), br.view(np.uint16))
