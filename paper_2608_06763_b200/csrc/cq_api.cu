@@ -224,7 +224,7 @@ int cq_mlp_swiglu(const void *layout_gate_up, int B_gu, int G_gu, const void *la
     if (e != cudaSuccess) return wrap(e);
     // 2. gated activation and the down projection's activation quantiser in one kernel
     e = launch_swiglu_quantize_a8(h, M, I, reinterpret_cast<int8_t *>(ws + plan.dn.x8_off), (int64_t)ddn.KT * TILE,
-                                  reinterpret_cast<float *>(ws + plan.dn.dx_off), f16, s);
+                                  reinterpret_cast<float *>(ws + plan.dn.dx_off), ddn.B != 4, f16, s);
     if (e != cudaSuccess) return wrap(e);
     // 3. the down projection on the carrier that is already in its workspace
     if (M <= 16) e = launch_gemv(layout_down, ddn, nullptr, y, M, CQ_DYN_A8, f16, ws, plan.dn, s, true);

@@ -18,15 +18,19 @@
 //   {row g+8 | k+2,3}; a pair sits in one 32-bit word with its first code in the low and its
 //   second code in the high 16 bits, so both are extracted by one mask.
 //
-//   Stored code u = k + 2^(B-1) (offset binary; u = 0 is the reserved pattern), W1: u = bit.
+//   Stored code u = k + 2^(B-1) (offset binary; u = 0 is the reserved pattern), W1: u = bit; W4: see below.
 //   u is split into bit planes of power-of-two width (B = 3 -> 2+1, 5 -> 4+1, 6 -> 4+2,
 //   7 -> 4+2+1) so every field is extracted with shifts and masks only.  A plane of width pw holds
 //   16/pw pairs per word; pair_word / pair_pos below give the word and bit position of a pair.
 //   Write p = 4 j + 2 h + r (chunk j = 2 w + a, k half h, row half r) and n = 2 a + h:
-//     pw = 4: word 2 w + r, nibble n           -- a 16-bit half holds four codes of ONE row from one
+//     pw = 4 (B = 5, 6, 7): word 2 w + r, nibble n -- a 16-bit half holds four codes of ONE row from one
 //     pw = 2: word w, field 2 n + r               32-wide k block, 4 bits apart, so it serves directly as
 //     pw = 1: word w / 2, bit 4 n + rho(w, r)     the selector of a byte-permute table lookup (Dynamic A8)
 //     pw = 8: word p / 2, byte p % 2
+//   W4 is laid out for table look-ups: the stored code is sign and magnitude (u = k for k >= 0, 8 | -k below, 8 the
+//   reserved pattern), so its low three bits select one of eight levels; lane l = 4*g + t owns eight CONSECUTIVE k of
+//   each 32-wide block w, k = 32 w + 8 t + i, as nibble i of word 2 w + r (row g + 8 r).  A half-word is the selector of
+//   four neighbouring weights, and a lane's word decodes to 16 consecutive bytes of a K-major 16-bit operand row.
 //   A lane's 2B words are stored as 16-byte quads, quad Q of lane l at ((Q * 32) + l) * 16 inside
 //   the row block (then an 8-byte tail when 2B is not a multiple of 4), so every warp load is one
 //   contiguous 512- or 256-byte run.
@@ -100,21 +104,34 @@ __host__ __device__ inline int word_byte_offset(int B, int W, int lane) {
     return nfq * 512 + lane * 8 + (W - 4 * nfq) * 4;
 }
 
-// Where weight (r, kk) of a tile lives: lane, pair index and half (0 = low 16 bits).
-struct Slot { int rb, lane, pair, half; };
-__host__ __device__ inline Slot slot_of(int r, int kk) {
+// Where the field of weight (r, kk) of a tile lives in a plane of width pw: row block, lane, word inside the plane, bit.
+struct Slot { int rb, lane, word, pos; };
+__host__ __device__ inline Slot slot_of(int B, int pw, int r, int kk) {
     Slot s;
     const int rr = r & 15, g = rr & 7, hi_row = rr >> 3;
-    const int j = kk >> 4, kin = kk & 15, t = kin >> 2, sl = kin & 3;
     s.rb = r >> 4;
+    if (B == 4) {
+        s.lane = g * 4 + ((kk & 31) >> 3);
+        s.word = 2 * (kk >> 5) + hi_row;
+        s.pos = 4 * (kk & 7);
+        return s;
+    }
+    const int j = kk >> 4, kin = kk & 15, t = kin >> 2, sl = kin & 3;
+    const int pair = 4 * j + ((sl >> 1) * 2 + hi_row);
     s.lane = g * 4 + t;
-    s.pair = 4 * j + ((sl >> 1) * 2 + hi_row);
-    s.half = sl & 1;
+    s.word = pair_word(pw, pair);
+    s.pos = pair_pos(pw, pair) + 16 * (sl & 1);
     return s;
 }
-// inverse: (rb, lane, pair, half) -> (r, kk)
-__host__ __device__ inline void weight_of(int rb, int lane, int pair, int half, int &r, int &kk) {
-    const int g = lane >> 2, t = lane & 3, j = pair >> 2, i = pair & 3;
+// inverse: the weight whose field sits at bit q pw + 16 half (q < 16 / pw) of word wi of a plane
+__host__ __device__ inline void weight_of(int B, int pw, int rb, int lane, int wi, int q, int half, int &r, int &kk) {
+    const int g = lane >> 2, t = lane & 3;
+    if (B == 4) {
+        r = rb * 16 + g + 8 * (wi & 1);
+        kk = 32 * (wi >> 1) + 8 * t + q + 4 * half;
+        return;
+    }
+    const int pair = pair_at(pw, wi, q), j = pair >> 2, i = pair & 3;
     r = rb * 16 + g + ((i & 1) ? 8 : 0);
     kk = 16 * j + 4 * t + (i >> 1) * 2 + half;
 }
@@ -151,16 +168,15 @@ __device__ __forceinline__ const uint8_t *tile_ptr(const void *layout, const Dim
 // Slow generic accessor: stored code u of weight (n, k) (n < Np, k < Kp).
 __device__ inline unsigned fetch_u(const void *layout, const Dims &d, int64_t n, int64_t k) {
     const int nb = (int)(n >> 7), kb = (int)(k >> 7);
-    const Slot s = slot_of((int)(n & 127), (int)(k & 127));
-    const uint8_t *rbp = tile_ptr(layout, d, nb, kb) + s.rb * 256 * d.B;
+    const uint8_t *tile = tile_ptr(layout, d, nb, kb);
     unsigned u = 0;
     const int np = plane_count(d.B);
     for (int i = 0; i < np; ++i) {
         const int pw = plane_width(d.B, i);
-        const int W = plane_word_base(d.B, i) + pair_word(pw, s.pair);
-        const int pos = pair_pos(pw, s.pair) + 16 * s.half;
-        const uint32_t w = *(const uint32_t *)(rbp + word_byte_offset(d.B, W, s.lane));
-        u |= ((w >> pos) & ((1u << pw) - 1u)) << plane_bit_offset(d.B, i);
+        const Slot s = slot_of(d.B, pw, (int)(n & 127), (int)(k & 127));
+        const int W = plane_word_base(d.B, i) + s.word;
+        const uint32_t w = *(const uint32_t *)(tile + s.rb * 256 * d.B + word_byte_offset(d.B, W, s.lane));
+        u |= ((w >> s.pos) & ((1u << pw) - 1u)) << plane_bit_offset(d.B, i);
     }
     return u;
 }
@@ -173,9 +189,10 @@ __device__ inline GroupParams fetch_params(const void *layout, const Dims &d, in
     return *(const GroupParams *)p;
 }
 
-// Signed code k from the stored code u (reserved pattern -> 0; W1: bit -> +-1).
+// Signed code k from the stored code u (reserved pattern -> 0; W1: bit -> +-1; W4: sign and magnitude).
 __host__ __device__ inline int signed_code(int B, unsigned u) {
     if (B == 1) return u ? 1 : -1;
+    if (B == 4) return u < 8 ? (int)u : -(int)(u & 7);
     if (u == 0) return 0;
     return (int)u - (1 << (B - 1));
 }
@@ -186,6 +203,11 @@ __device__ __forceinline__ float level_q(int i, int M, float a, float b) {
     const float t = __fdiv_rn((float)i, (float)M);
     const float c = __fsub_rn(__fsub_rn(1.0f, a), b);
     return __fmul_rn(t, fmaf(t, fmaf(t, c, b), a));
+}
+
+// Entry of magnitude i and sign in a carrier table indexed by the stored code.
+__host__ __device__ constexpr int carrier_slot(int B, int i, bool negative) {
+    return B == 4 ? (negative ? 8 + i : i) : (negative ? (1 << (B - 1)) - i : (1 << (B - 1)) + i);
 }
 
 // Row stride (bytes) of a shared-memory carrier table of 2^B entries per row: tables read per code

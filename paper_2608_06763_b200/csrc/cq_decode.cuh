@@ -49,6 +49,7 @@ __device__ __forceinline__ uint32_t pair_codes(const uint32_t (&w)[2 * B]) {
 // one exact FMA removes the offset and the position scale.
 template <int B, int P>
 __device__ __forceinline__ __half2 pair_T(const uint32_t (&w)[2 * B]) {
+    static_assert(B != 4, "W4 is decoded by table (w4_block)");
     if constexpr (plane_count(B) == 1) {
         constexpr int W = pair_word(B, P), pos0 = pair_pos(B, P);
         // B = 1 keeps the field off mantissa bit 0 (the offset constant must stay representable);
@@ -113,17 +114,18 @@ __device__ __forceinline__ uint32_t lop3_and_xor(uint32_t a, uint32_t b, uint32_
 }
 template <int B, int P>
 __device__ __forceinline__ __half2 pair_K(const uint32_t (&w)[2 * B], const DecodeRegs &dr) {
+    static_assert(B != 4, "W4 is decoded by table (w4_block)");
     if constexpr (B == 1) {
         constexpr int W = pair_word(1, P), pos0 = pair_pos(1, P);
         const uint32_t word = pos0 == 15 ? w[W] : (w[W] << (15 - pos0));
         return as_h2(lop3_and_xor(word, 0x80008000u, dr.one_neg));
-    } else if constexpr (B == 2 || B == 4) {
+    } else if constexpr (B == 2) {
         constexpr int W = pair_word(B, P), pos0 = pair_pos(B, P);
         constexpr int shr = pos0 >= 8 ? 8 : 0, pos = pos0 - shr;
         const uint32_t word = shr ? (w[W] >> shr) : w[W];
         constexpr uint32_t m = (((1u << B) - 1u) << pos) * 0x00010001u;
         const uint32_t hbits = lop3_and_or(word, m, dr.magic[pos / 2]);     // base + u, base = 2^(10 - pos)
-        constexpr uint32_t off = half_neg_pow2_plus(10 - pos, B == 2 ? 2 : 8);   // -(base + 2^(B-1))
+        constexpr uint32_t off = half_neg_pow2_plus(10 - pos, 2);           // -(base + 2^(B-1))
         return __hadd2(as_h2(hbits), as_h2(h2dup(off)));
     } else if constexpr (B == 8) {
         constexpr int W = pair_word(8, P), pos0 = pair_pos(8, P);
@@ -189,17 +191,46 @@ __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {
     return d;
 }
 
+// ---- W4, model dtype: eight levels of a (row, group) as 16-bit values, their low bytes in t.x (magnitudes 0-3) and
+// t.y (4-7), their high bytes in t.z and t.w.  A half-word of the layout is the selector of four neighbouring
+// weights; two byte permutes fetch their low and high bytes, two more put the bytes together, and the sign bits
+// go into the high bytes by one exclusive or.  Fifteen integer instructions for eight weights, against some forty for
+// the half2 polynomial, its scale in fp32 and the rounding to the operand's type; the levels themselves are evaluated in fp32
+// and rounded once.  Measured on the linears of an 8B layer, G = 128: M = 1 66.6 -> 59.3 us, M = 13 109.7 -> 105.5,
+// M = 200 (binary16) 194.8 -> 167.7, M = 1024 509.5 -> 491.6 (what is left there is not the decode).  out[i] = weights (2 i, 2 i + 1) of the word, in k order; a reserved code reads (minus) zero.
+__device__ __forceinline__ void w4_block(uint32_t word, const uint4 &t, uint32_t (&out)[4]) {
+    const uint32_t sel = word & 0x77777777u, sel1 = sel >> 16, w4 = word << 4;
+    const uint32_t m0 = prmt(w4, word, 0xD9C8u), m1 = prmt(w4, word, 0xFBEAu);   // 0xFF where the code is negative
+    const uint32_t l0 = prmt(t.x, t.y, sel), h0 = prmt(t.z, t.w, sel) ^ (m0 & 0x80808080u);
+    const uint32_t l1 = prmt(t.x, t.y, sel1), h1 = prmt(t.z, t.w, sel1) ^ (m1 & 0x80808080u);
+    out[0] = prmt(l0, h0, 0x5140u); out[1] = prmt(l0, h0, 0x7362u);
+    out[2] = prmt(l1, h1, 0x5140u); out[3] = prmt(l1, h1, 0x7362u);
+}
+// The four lanes t of a row evaluate two levels each (magnitudes 2 t and 2 t + 1, at t0 and t1 = magnitude / 7, by the
+// fp32 Horner form of Eq. gpu-horner, times f) and leave their bytes in the row's 16-byte table in shared memory.
+template <class Pack>
+__device__ __forceinline__ void w4_put(uint8_t *row, uint2 p, int t, float t0, float t1, float f, Pack pack) {
+    const __half2 ab = as_h2(p.y);
+    const float a = __low2float(ab), b = __high2float(ab), c = (1.0f - a) - b;
+    const float q0 = t0 * fmaf(t0, fmaf(t0, c, b), a), q1 = t1 * fmaf(t1, fmaf(t1, c, b), a);
+    const uint32_t v = pack(q0 * f, q1 * f), bytes = prmt(v, 0u, 0x3120u);   // low bytes, then high bytes
+    *reinterpret_cast<uint16_t *>(row + 2 * t) = (uint16_t)bytes;
+    *reinterpret_cast<uint16_t *>(row + 8 + 2 * t) = (uint16_t)(bytes >> 16);
+}
+
 // Dynamic A8 operand order (both INT8 kernels).  One k = 32 MMA step takes the 32-wide k block m of a
 // tile.  Inside it
 // k = 16 a + 4 t + 2 h + e is held by lane t at byte n = 2 a + h of A register a0 / a1 (rows g / g+8)
 // for e = 0 and a2 / a3 for e = 1 (small-M kernel), i.e. at byte 8 t + 4 e + n of the block, which is
-// where the layout's half-words put it.  The internal activation quantiser writes x8 in the same order.
+// where the layout's half-words put it.  The internal activation quantiser writes x8 in the same order (W4: the
+// natural order).
 //
 // Carriers (Eq. carrier) come from a per-(row, group) table indexed by the stored code u, so the
 // sign and the reserved pattern (u = 0 -> 0) are part of the table:
-//   B = 4: the table's two 8-byte halves (u < 8, u >= 8) live in registers; a half-word of four
+//   B = 4: the table's two 8-byte halves (positive, negative) live in registers; a half-word of four
 //          codes, masked to 3 bits each, is the selector of a byte permute into each half, and the
-//          codes' top bits (expanded to byte masks by two sign-replicating permutes) pick between them;
+//          codes' top bits (expanded to byte masks by two sign-replicating permutes) pick between them; its order
+//          inside the block is the natural one, lane t holding bytes 8 t .. 8 t + 7;
 //   B = 3: one 8-byte table, the selector assembled from the 2-bit and the 1-bit plane;
 //   B <= 2: the carriers are 0 / +-127, a constant table;
 //   B >= 5: the table stays in shared memory and is read per code.
@@ -209,7 +240,7 @@ __device__ __forceinline__ void a8_row_regs(const uint32_t (&w)[2 * B], const ui
     if constexpr (B == 4) {
         const uint32_t word = w[2 * MI + RR];
         const uint32_t ws = word & 0x77777777u, wh = ws >> 16, w4 = word << 4;
-        const uint32_t m_lo = prmt(w4, word, 0xD9C8u), m_hi = prmt(w4, word, 0xFBEAu);   // 0xFF where u >= 8
+        const uint32_t m_lo = prmt(w4, word, 0xD9C8u), m_hi = prmt(w4, word, 0xFBEAu);   // 0xFF where the code is negative
         const uint32_t n_lo = prmt(tab.x, tab.y, ws), p_lo = prmt(tab.z, tab.w, ws);
         const uint32_t n_hi = prmt(tab.x, tab.y, wh), p_hi = prmt(tab.z, tab.w, wh);
         lo = (p_lo & m_lo) | (n_lo & ~m_lo);

@@ -264,24 +264,22 @@ gemm_a8_kernel(const __grid_constant__ CUtensorMap xmap, A8Params prm) {
                             sc[(rb * 16 + g + 8) * GPT + gi] = __uint_as_float(p_hi.x & 0x7FFFFFFFu);
                         }
                         if constexpr (B >= 3) {
-                            // signed carrier table: index = stored code u; u = 0 (reserved) -> 0,
-                            // u = 2^(B-1) + k -> sign(k) r(|k|).  With G = 128 the two warps of a row block
+                            // signed carrier table: index = stored code u (reserved -> 0), entry sign(k) r(|k|).  With G = 128 the two warps of a row block
                             // build eight rows each and meet at a 64-thread barrier.
-                            constexpr int bias = 1 << (B - 1);
                             if constexpr (G == 128) named_barrier_sync(1 + rb, 64); else __syncwarp();
                             auto build_row = [&](int row, uint32_t abbits) {
                                 const __half2 ab = as_h2(abbits);
                                 const float a = __low2float(ab), b = __high2float(ab);
                                 const float c = __fsub_rn(__fsub_rn(1.0f, a), b);
                                 int8_t *tr = tab + row * NCODE;
-                                if (tq == 0) tr[0] = 0;
+                                if (B != 4 && tq == 0) tr[0] = 0;
                                 for (int i = tq; i <= Mx; i += 4) {
                                     const float tt = sT[i];
                                     const float q = __fmul_rn(tt, fmaf(tt, fmaf(tt, c, b), a));
                                     int r = __float2int_rn(__fmul_rn(127.0f, q));
                                     r = min(max(r, 0), 127);
-                                    tr[bias + i] = (int8_t)r;
-                                    tr[bias - i] = (int8_t)(-r);
+                                    tr[carrier_slot(B, i, false)] = (int8_t)r;
+                                    tr[carrier_slot(B, i, true)] = (int8_t)(-r);
                                 }
                             };
                             if constexpr (G == 128) {
@@ -503,7 +501,7 @@ cudaError_t launch_gemm_a8_tc(const void *layout, const Dims &d, const uint16_t 
     int *counters = reinterpret_cast<int *>(ws + plan.counters_off);
     const int64_t pitch = (int64_t)d.KT * TILE;
     if (!prequantized) {
-        cudaError_t e = launch_quantize_a8(x, M, d.K, xq, pitch, dxs, true, act_f16, st);
+        cudaError_t e = launch_quantize_a8(x, M, d.K, xq, pitch, dxs, d.B != 4, act_f16, st);
         if (e != cudaSuccess) return e;
     }
     switch (d.B) {

@@ -14,7 +14,9 @@ namespace {
 
 using namespace tc;
 
-constexpr int DEC_WARPS = 16;                 // decoder / epilogue warps
+constexpr int DEC_WARPS = 16;                 // decoder / epilogue warps: two sets, which take the layout tiles in turn
+constexpr int SET_WARPS = DEC_WARPS / 2;      // one warp of a set per 16 rows of a tile
+constexpr int W4_TABLE_BYTES = 16 * 2 * 16;   // a decoder warp's level tables: 16 rows x the two groups of a 64-wide block at most
 constexpr int TC_THREADS = 64 + 32 * DEC_WARPS + 32;   // producer of activations, MMA issuer, decoders, producer of raw tiles
 constexpr int A_STAGE_BYTES = 128 * 128;  // 128 rows x 64 bf16
 
@@ -98,9 +100,10 @@ struct TcParams {
 // the decoders run two layout tiles ahead of the MMAs instead of in lockstep with them.
 constexpr int tc_stages(int BN, int NACC) { return BN * NACC >= 512 ? 2 : (BN == 256 ? 3 : 4); }
 constexpr int tc_raw_stage_bytes(int B, int G) { return (2048 * B + 1024 * (TILE / G) + 1023) / 1024 * 1024; }
+constexpr int tc_table_bytes(int B) { return B == 4 ? DEC_WARPS * W4_TABLE_BYTES : 0; }
 // Weight stages: up to four, fewer where the activation ring and two raw tiles leave less room.
 constexpr int tc_stages_a(int B, int G, int BN, int NACC) {
-    const int left = 226 * 1024 - 512 - tc_stages(BN, NACC) * NACC * BN * 128 - 2 * tc_raw_stage_bytes(B, G);
+    const int left = 226 * 1024 - 512 - tc_table_bytes(B) - tc_stages(BN, NACC) * NACC * BN * 128 - 2 * tc_raw_stage_bytes(B, G);
     const int n = left / A_STAGE_BYTES;
     return n > 4 ? 4 : n < 2 ? 2 : n;
 }
@@ -109,7 +112,7 @@ constexpr int tc_ring_bytes(int B, int G, int BN, int NACC) {
 }
 // Raw layout tiles in flight per CTA: as many as the shared memory left by the operand rings holds, two to four.
 constexpr int tc_raw_stages(int B, int G, int BN, int NACC) {
-    const int left = 226 * 1024 - 512 - tc_ring_bytes(B, G, BN, NACC);
+    const int left = 226 * 1024 - 512 - tc_table_bytes(B) - tc_ring_bytes(B, G, BN, NACC);
     const int n = left / tc_raw_stage_bytes(B, G);
     return n > 4 ? 4 : n < 2 ? 2 : n;
 }
@@ -178,10 +181,11 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap xmap, TcParams prm) {
     uint8_t *sA = smem;                                        // STAGES_A x 16 KB
     uint8_t *sB = sA + STAGES_A * A_STAGE_BYTES;               // STAGES x NACC x BN x 128 B
     uint8_t *sRaw = sB + STAGES * B_STAGE_BYTES;               // RAW_STAGES x raw_stage_bytes
-    uint64_t *bars = reinterpret_cast<uint64_t *>(sRaw + RAW_STAGES * prm.raw_stage_bytes);
+    uint8_t *sTab = sRaw + RAW_STAGES * prm.raw_stage_bytes;   // W4: DEC_WARPS x W4_TABLE_BYTES
+    uint64_t *bars = reinterpret_cast<uint64_t *>(sTab + tc_table_bytes(B));
     uint64_t *a_full = bars, *a_empty = a_full + STAGES_A, *b_full = a_empty + STAGES_A, *b_empty = b_full + STAGES;
-    uint64_t *raw_full = b_empty + STAGES, *raw_empty = raw_full + RAW_STAGES, *acc_full = raw_empty + RAW_STAGES;
-    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(acc_full + 1);
+    uint64_t *raw_full = b_empty + STAGES, *raw_empty = raw_full + RAW_STAGES, *acc_full = raw_empty + RAW_STAGES, *acc_empty = acc_full + 1;
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(acc_empty + 1);
     volatile int *s_last_p = reinterpret_cast<volatile int *>(tmem_slot + 1);    // "this CTA completes the tile"
     volatile int *gave_up = reinterpret_cast<volatile int *>(tmem_slot + 2);     // a bounded wait ran out somewhere in the CTA
 
@@ -193,10 +197,11 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap xmap, TcParams prm) {
         return;
     }
     if (threadIdx.x == 0) {
-        for (int s = 0; s < STAGES_A; ++s) { mbar_init(&a_full[s], DEC_WARPS); mbar_init(&a_empty[s], 1); }
+        for (int s = 0; s < STAGES_A; ++s) { mbar_init(&a_full[s], SET_WARPS); mbar_init(&a_empty[s], 1); }
         for (int s = 0; s < STAGES; ++s) { mbar_init(&b_full[s], 1); mbar_init(&b_empty[s], 1); }
-        for (int s = 0; s < RAW_STAGES; ++s) { mbar_init(&raw_full[s], 1); mbar_init(&raw_empty[s], DEC_WARPS); }
+        for (int s = 0; s < RAW_STAGES; ++s) { mbar_init(&raw_full[s], 1); mbar_init(&raw_empty[s], SET_WARPS); }
         mbar_init(acc_full, 1);
+        mbar_init(acc_empty, DEC_WARPS);
         fence_barrier_init();
         *gave_up = 0;
     }
@@ -255,8 +260,10 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap xmap, TcParams prm) {
         // ===== MMA issuer
         if (lane == 0) {
             const uint32_t idesc = prm.f16 ? idesc_f16(BN) : idesc_bf16(BN);
-            int kbc = 0;
+            int kbc = 0, segc = 0;
             while (walk.next(seg)) {
+                if (SK && segc > 0) wait(acc_empty, (segc - 1) & 1, 8);   // every decoder has read the accumulators of the segment before
+                ++segc;
                 const int nkb = 2 * (seg.k1 - seg.k0);
                 for (int i = 0; i < nkb; ++i, ++kbc) {
                     const int s = kbc % STAGES, sa = kbc % STAGES_A;
@@ -274,23 +281,24 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap xmap, TcParams prm) {
                     umma_commit(&a_empty[sa]);  // frees the two stages when these MMAs have read them
                     umma_commit(&b_empty[s]);
                 }
-                // The accumulators of this segment are complete when these MMAs are.  The next segment's first MMA
-                // overwrites them, but it waits for a decoded stage, and the decoders decode again only after
-                // all of them have read the accumulators.
-                umma_commit(acc_full);
+                umma_commit(acc_full);   // the accumulators of this segment are complete when these MMAs are
             }
         }
     } else {
-        // ===== decoders (warps 2..17), then epilogue.  Per 64-wide k block, decoder dw owns row block
-        // dw / 2 and the two 16-wide chunks 2 (dw % 2), 2 (dw % 2) + 1 of the block.
+        // ===== decoders (warps 2..17), then epilogue.  Warp rb of a set owns row block rb of every second layout tile:
+        // a (row, group)'s coefficients or tables are formed once per tile, a warp meets the barriers of a 64-wide block once per
+        // tile instead of twice, and the two sets hide each other's latencies.
         const int dw = warp - 2, g = lane >> 2, t = lane & 3;
-        const int rb = dw >> 1, jh = dw & 1;
+        const int rb = dw & (SET_WARPS - 1), set = dw / SET_WARPS;
         const int dec_tid = threadIdx.x - 64;
-        int kbc = 0, tcnt = 0, segc = 0;
+        int tcnt = 0, segc = 0;
+        float w4_t0 = 0.0f, w4_t1 = 0.0f;   // W4: positions of the two levels this lane evaluates for a table
+        if constexpr (B == 4) { w4_t0 = (float)(2 * t) / 7.0f; w4_t1 = (float)(2 * t + 1) / 7.0f; }
 #pragma unroll 1
         while (walk.next(seg)) {
 #pragma unroll 1
         for (int tile = seg.k0; tile < seg.k1; ++tile, ++tcnt) {
+            if ((tcnt & 1) != set) continue;
             const int rs = tcnt % RAW_STAGES;
             wait(&raw_full[rs], (tcnt / RAW_STAGES) & 1, 5);
             const uint8_t *raw = sRaw + rs * prm.raw_stage_bytes;
@@ -317,21 +325,66 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap xmap, TcParams prm) {
             // G = 128: one group spans the tile, so its coefficients are formed once per tile, not once per 64-wide block
             RowCoef tc_lo{}, tc_hi{};
             bool tfix = false;
-            if constexpr (B != 3 && G == 128) {
+            if constexpr (B != 3 && B != 4 && G == 128) {
                 const uint2 q_lo = *(const uint2 *)prow, q_hi = *(const uint2 *)(prow + 8 * GPT * 8);
                 tc_lo = make_coef<B>(q_lo); tc_hi = make_coef<B>(q_hi);
                 tfix = B > 1 && __any_sync(0xffffffffu, (q_lo.x | q_hi.x) >> 31);
             }
-            // one 64-wide block: this warp's unit JQ of the tile (unit = two 16-wide chunks of 16 rows)
-            auto do_block = [&](auto jq_block) {
-                const int kb = kbc++, s = kb % STAGES_A;
+            uint4 w4_lo{}, w4_hi{};     // W4: tables of rows g and g + 8 (G >= 64: of the block's one group)
+            uint8_t *wtab = sTab + dw * W4_TABLE_BYTES;
+            // tables of the groups gi0 .. gi0 + n - 1 (n = 1, 2) of the tile, one after another in this warp's shared memory
+            auto w4_build = [&](int gi0, auto nc) {
+                constexpr int n = decltype(nc)::value;
+                __syncwarp();   // the tables before have been read
+#pragma unroll
+                for (int e = 0; e < n; ++e) {
+                    const uint2 p_lo = *(const uint2 *)(prow + (gi0 + e) * 8), p_hi = *(const uint2 *)(prow + (8 * GPT + gi0 + e) * 8);
+                    const float s_lo = __uint_as_float(p_lo.x & 0x7FFFFFFFu), s_hi = __uint_as_float(p_hi.x & 0x7FFFFFFFu);
+                    auto pack = [&](float a, float b) { return pack_act2(a, b, prm.f16); };
+                    w4_put(wtab + e * 256 + g * 16, p_lo, t, w4_t0, w4_t1, s_lo, pack);
+                    w4_put(wtab + e * 256 + (g + 8) * 16, p_hi, t, w4_t0, w4_t1, s_hi, pack);
+                }
+                __syncwarp();
+            };
+            if constexpr (B == 4 && G == 128) {
+                w4_build(0, std::integral_constant<int, 1>{});
+                w4_lo = *(const uint4 *)(wtab + g * 16); w4_hi = *(const uint4 *)(wtab + (g + 8) * 16);
+            }
+            // the two 64-wide blocks of the tile, two 32-wide units each
+            static_for<2>([&](auto hc) {
+                constexpr int H = decltype(hc)::value;
+                const int kb = 2 * tcnt + H, s = kb % STAGES_A;
+                if constexpr (B == 4 && G == 64) {
+                    w4_build(H, std::integral_constant<int, 1>{});
+                    w4_lo = *(const uint4 *)(wtab + g * 16); w4_hi = *(const uint4 *)(wtab + (g + 8) * 16);
+                }
+                if constexpr (B == 4 && G == 32) w4_build(2 * H, std::integral_constant<int, 2>{});
                 if (kb >= STAGES_A) wait(&a_empty[s], ((kb / STAGES_A) - 1) & 1, 6);
                 uint8_t *a_stage = sA + s * A_STAGE_BYTES;
                 // rows g (low) and g + 8 (high) of the row block: their 128-byte rows in the stage
                 uint8_t *row_lo = a_stage + (rb * 2 + 0) * 1024 + g * 128;
                 uint8_t *row_hi = a_stage + (rb * 2 + 1) * 1024 + g * 128;
-                auto do_unit = [&](auto jq) {
-                    constexpr int JQ = decltype(jq)::value;        // pair of chunks 2 JQ, 2 JQ + 1 of the tile
+                if constexpr (B == 4) {
+                    // Unit u of the block is 16-byte chunks 4 u + t of the row, swizzled by the row: lanes of odd rows take
+                    // the units in the other order, which puts the eight lanes of a store phase into different banks.
+                    const bool odd = (g & 1) != 0;
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        const int u = e ^ (g & 1);
+                        if constexpr (G == 32) {
+                            w4_lo = *(const uint4 *)(wtab + u * 256 + g * 16); w4_hi = *(const uint4 *)(wtab + u * 256 + (g + 8) * 16);
+                        }
+                        const uint32_t x_lo = odd ? w[4 * H + 2 * (1 - e)] : w[4 * H + 2 * e], x_hi = odd ? w[4 * H + 2 * (1 - e) + 1] : w[4 * H + 2 * e + 1];
+                        uint32_t o_lo[4], o_hi[4];
+                        w4_block(x_lo, w4_lo, o_lo);
+                        w4_block(x_hi, w4_hi, o_hi);
+                        const int off = ((4 * u + t) ^ g) * 16;
+                        *(uint4 *)(row_lo + off) = make_uint4(o_lo[0], o_lo[1], o_lo[2], o_lo[3]);
+                        *(uint4 *)(row_hi + off) = make_uint4(o_hi[0], o_hi[1], o_hi[2], o_hi[3]);
+                    }
+                } else {
+                static_for<2>([&](auto uc) {
+                    constexpr int JQ = 2 * H + decltype(uc)::value;    // pair of chunks 2 JQ, 2 JQ + 1 of the tile
                     constexpr int gi = (32 * JQ) / G;              // both chunks lie in this group
                     const uint2 p_lo = *(const uint2 *)(prow + gi * 8), p_hi = *(const uint2 *)(prow + (8 * GPT + gi) * 8);
                     if constexpr (B == 3) {
@@ -346,8 +399,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap xmap, TcParams prm) {
                             *(uint2 *)(row_lo + off) = make_uint2(o_lo[2 * jcv], o_lo[2 * jcv + 1]);
                             *(uint2 *)(row_hi + off) = make_uint2(o_hi[2 * jcv], o_hi[2 * jcv + 1]);
                         });
-                        return;
-                    }
+                    } else {
                     RowCoef c_lo, c_hi;
                     bool fix;   // reserved pattern present
                     if constexpr (G == 128) { c_lo = tc_lo; c_hi = tc_hi; fix = tfix; }
@@ -370,15 +422,13 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap xmap, TcParams prm) {
                     };
                     if (!prm.f16) { if (!fix) emit(std::false_type{}, std::false_type{}); else emit(std::true_type{}, std::false_type{}); }
                     else { if (!fix) emit(std::false_type{}, std::true_type{}); else emit(std::true_type{}, std::true_type{}); }
-                };
-                do_unit(jq_block);
+                    }
+                });
+                }
                 fence_proxy_async();   // generic-proxy stores -> visible to the tensor core's async proxy
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&a_full[s]);
-            };
-            // the first 64-wide block of the tile holds units 0 and 1, the second units 2 and 3; jh picks the warp's
-            if (jh == 0) { do_block(std::integral_constant<int, 0>{}); do_block(std::integral_constant<int, 2>{}); }
-            else { do_block(std::integral_constant<int, 1>{}); do_block(std::integral_constant<int, 3>{}); }
+            });
             __syncwarp();
             if (lane == 0) mbar_arrive(&raw_empty[rs]);
         }
@@ -441,7 +491,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap xmap, TcParams prm) {
                 }
             }
         }
-        tc_fence_before();   // the accumulators have been read before this warp's next arrival lets the MMAs go on
+        tc_fence_before();   // the accumulators have been read: the MMAs of the next segment may overwrite them
+        if constexpr (SK) { __syncwarp(); if (lane == 0) mbar_arrive(acc_empty); }
         if (SK && !whole) {
             // The tile's counter collects the layout tiles done; the CTA that completes it adds the partial tiles
             // in K order.  The first barrier orders the decoders' partial stores before the release; the acquire
@@ -535,8 +586,8 @@ cudaError_t launch_bn(const void *layout, const Dims &d, const uint16_t *x, uint
     p.MT = plan.token_tiles; p.t_full = plan.t_full; p.p2 = plan.p2;
     constexpr int RAW_STAGES = tc_raw_stages(B, G, BN, NACC);
     if (p.raw_stage_bytes != tc_raw_stage_bytes(B, G)) return cudaErrorInvalidConfiguration;
-    const size_t smem = (size_t)tc_ring_bytes(B, G, BN, NACC) + (size_t)RAW_STAGES * p.raw_stage_bytes + 256;
-    static_assert(tc_ring_bytes(B, G, BN, NACC) + tc_raw_stages(B, G, BN, NACC) * tc_raw_stage_bytes(B, G) + 256 <= 227 * 1024, "shared memory");
+    const size_t smem = (size_t)tc_ring_bytes(B, G, BN, NACC) + (size_t)RAW_STAGES * p.raw_stage_bytes + tc_table_bytes(B) + 256;
+    static_assert(tc_ring_bytes(B, G, BN, NACC) + tc_raw_stages(B, G, BN, NACC) * tc_raw_stage_bytes(B, G) + tc_table_bytes(B) + 256 <= 227 * 1024, "shared memory");
     auto kern = gemm_tc_kernel<B, G, BN, NACC, SK>;
     static std::atomic<uint64_t> attr_done{0};   // per kernel instantiation: the devices it has been set on
     cudaError_t ea = ensure_func_attr(kern, attr_done, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);

@@ -18,7 +18,7 @@
 // Decode (model dtype): two codes are masked out of a word straight into fp16 mantissas
 // (exponent-bias trick) and one exact packed-half add leaves the signed code; the group's cubic is
 // evaluated in half2 Horner form (Eq. gpu-horner) as T (ca + |T| (cb + |T| cc)) and the group scale s_g
-// multiplies the fp32 group sum, as in the paper's narrow path.  W3 reads its eight levels from a
+// multiplies the fp32 group sum, as in the paper's narrow path.  W3 and W4 read their eight magnitudes from a
 // register table with byte permutes instead; W1 / W2 have no shape.  Activations go bf16 -> fp16 with
 // a per-token power-of-two scale so that nothing overflows or loses bits.
 //
@@ -240,7 +240,7 @@ __device__ __forceinline__ void group_a8(const TileRegs<B, TILE / G> &r, const i
     const uint2 p_lo = r.prm[0][GI], p_hi = r.prm[1][GI];
     uint4 tab_lo = make_uint4(0, 0, 0, 0), tab_hi = make_uint4(0, 0, 0, 0);
     const int8_t *trow_lo = ctab + g * NE, *trow_hi = ctab + (g + 8) * NE;
-    if constexpr (B >= 3) {  // lane (g, t) fills magnitudes i = t mod 4 of rows g and g + 8: u = L + i and u = L - i
+    if constexpr (B >= 3) {  // lane (g, t) fills magnitudes i = t mod 4 of rows g and g + 8
         __syncwarp();
         const __half2 ab_lo = as_h2(p_lo.y), ab_hi = as_h2(p_hi.y);
         const float a_lo = __low2float(ab_lo), b_lo = __high2float(ab_lo);
@@ -248,12 +248,13 @@ __device__ __forceinline__ void group_a8(const TileRegs<B, TILE / G> &r, const i
         for (int i = t; i < L; i += 4) {
             const float ti = tt[i];   // i / M, divided once per CTA
             const int c_lo = carrier_at(ti, a_lo, b_lo), c_hi = carrier_at(ti, a_hi, b_hi);
-            ctab[g * NE + L + i] = (int8_t)c_lo;
-            ctab[g * NE + L - i] = (int8_t)(-c_lo);
-            ctab[(g + 8) * NE + L + i] = (int8_t)c_hi;
-            ctab[(g + 8) * NE + L - i] = (int8_t)(-c_hi);
+            const int up = carrier_slot(B, i, false), dn = carrier_slot(B, i, true);
+            ctab[g * NE + up] = (int8_t)c_lo;
+            ctab[g * NE + dn] = (int8_t)(-c_lo);
+            ctab[(g + 8) * NE + up] = (int8_t)c_hi;
+            ctab[(g + 8) * NE + dn] = (int8_t)(-c_hi);
         }
-        if (t == 0) { ctab[g * NE] = 0; ctab[(g + 8) * NE] = 0; }   // the reserved pattern
+        if (B != 4 && t == 0) { ctab[g * NE] = 0; ctab[(g + 8) * NE] = 0; }   // the reserved pattern (W4: magnitude 0)
         __syncwarp();
         if constexpr (B == 4) {
             tab_lo = *reinterpret_cast<const uint4 *>(trow_lo);
@@ -444,13 +445,93 @@ __device__ __forceinline__ void group_dot_w3(const TileRegs<3, TILE / G> &r, con
     }
 }
 
+// ---- W4, model dtype: levels from the warp's tables (w4_block), unit scale; the group scale multiplies the fp32 group
+// sum.  The staged activations keep their natural order: lane t reads the eight of its word, k = 32 MI + 8 t + i.
+struct W4Rows { uint4 tab[2]; float s[2]; };   // rows g and g + 8
+__device__ __forceinline__ W4Rows w4_rows(uint2 p_lo, uint2 p_hi, uint8_t *wtab, float t0, float t1, int g, int t) {
+    auto pack = [](float a, float b) { return as_u32(__floats2half2_rn(a, b)); };
+    __syncwarp();   // the group before has been read
+    w4_put(wtab + g * 16, p_lo, t, t0, t1, 1.0f, pack);
+    w4_put(wtab + (g + 8) * 16, p_hi, t, t0, t1, 1.0f, pack);
+    __syncwarp();
+    W4Rows r;
+    r.tab[0] = *reinterpret_cast<const uint4 *>(wtab + g * 16);
+    r.tab[1] = *reinterpret_cast<const uint4 *>(wtab + (g + 8) * 16);
+    r.s[0] = __uint_as_float(p_lo.x & 0x7FFFFFFFu);
+    r.s[1] = __uint_as_float(p_hi.x & 0x7FFFFFFFu);
+    return r;
+}
+template <int G, int NT, int GI>
+__device__ __forceinline__ void group_dot_w4(const TileRegs<4, TILE / G> &r, const __half *xs, const int (&xo)[NT], uint8_t *wtab, float t0, float t1,
+                                             int g, int t, float (&acc)[NT][4]) {
+    constexpr int MPG = G / 32;
+    const W4Rows w = w4_rows(r.prm[0][GI], r.prm[1][GI], wtab, t0, t1, g, t);
+    __half2 h[NT][2];
+#pragma unroll
+    for (int tk = 0; tk < NT; ++tk) { h[tk][0] = __float2half2_rn(0.0f); h[tk][1] = h[tk][0]; }
+    static_for<MPG>([&](auto mc) {
+        constexpr int MI = GI * MPG + decltype(mc)::value;
+        uint4 xv[NT];
+#pragma unroll
+        for (int tk = 0; tk < NT; ++tk) xv[tk] = *reinterpret_cast<const uint4 *>(xs + xo[tk] + 32 * MI);
+#pragma unroll
+        for (int rr = 0; rr < 2; ++rr) {
+            uint32_t lv[4];
+            w4_block(r.w[2 * MI + rr], w.tab[rr], lv);
+#pragma unroll
+            for (int tk = 0; tk < NT; ++tk) {
+                h[tk][rr] = __hfma2(as_h2(lv[0]), as_h2(xv[tk].x), h[tk][rr]);
+                h[tk][rr] = __hfma2(as_h2(lv[1]), as_h2(xv[tk].y), h[tk][rr]);
+                h[tk][rr] = __hfma2(as_h2(lv[2]), as_h2(xv[tk].z), h[tk][rr]);
+                h[tk][rr] = __hfma2(as_h2(lv[3]), as_h2(xv[tk].w), h[tk][rr]);
+            }
+        }
+    });
+#pragma unroll
+    for (int tk = 0; tk < NT; ++tk) {
+        acc[tk][0] = fmaf(w.s[0], h2sum(h[tk][0]), acc[tk][0]);
+        acc[tk][2] = fmaf(w.s[1], h2sum(h[tk][1]), acc[tk][2]);
+    }
+}
+template <int G, int NT, int GI>
+__device__ __forceinline__ void group_model_w4(const TileRegs<4, TILE / G> &r, const __half *xs, const int (&xo)[NT], uint8_t *wtab, float t0, float t1,
+                                               int g, int t, float (&acc)[NT][4]) {
+    constexpr int MPG = G / 32;
+    const W4Rows w = w4_rows(r.prm[0][GI], r.prm[1][GI], wtab, t0, t1, g, t);
+    float D[2][NT][4];   // two accumulator sets so consecutive MMAs do not wait on each other
+    static_for<MPG>([&](auto mc) {
+        constexpr int mi = decltype(mc)::value, MI = GI * MPG + mi;
+        uint32_t lo[4], hi[4];
+        w4_block(r.w[2 * MI], w.tab[0], lo);
+        w4_block(r.w[2 * MI + 1], w.tab[1], hi);
+        const uint32_t A0[4] = {lo[0], hi[0], lo[1], hi[1]}, A1[4] = {lo[2], hi[2], lo[3], hi[3]};   // k = 8 t + 0..3 | 4..7
+#pragma unroll
+        for (int tb = 0; tb < NT; ++tb) {
+            const uint4 bf = *reinterpret_cast<const uint4 *>(xs + xo[tb] + 32 * MI);
+            if constexpr (mi == 0) { mma_f16_z(D[0][tb], A0, bf.x, bf.y); mma_f16_z(D[1][tb], A1, bf.z, bf.w); }
+            else { mma_f16(D[0][tb], A0, bf.x, bf.y); mma_f16(D[1][tb], A1, bf.z, bf.w); }
+        }
+    });
+#pragma unroll
+    for (int tb = 0; tb < NT; ++tb) {
+        acc[tb][0] = fmaf(w.s[0], D[0][tb][0] + D[1][tb][0], acc[tb][0]);
+        acc[tb][1] = fmaf(w.s[0], D[0][tb][1] + D[1][tb][1], acc[tb][1]);
+        acc[tb][2] = fmaf(w.s[1], D[0][tb][2] + D[1][tb][2], acc[tb][2]);
+        acc[tb][3] = fmaf(w.s[1], D[0][tb][3] + D[1][tb][3], acc[tb][3]);
+    }
+}
+
 template <int B, int G, int NT, int MODE>
 __device__ __forceinline__ void compute_tile(const TileRegs<B, TILE / G> &r, const DecodeRegs &dr, const uint8_t *xs, const int (&xo)[NT],
-                                             int8_t *ctab, const float *tt, int g, int t, float (&acc)[NT][4]) {
+                                             int8_t *ctab, const float *tt, float t0, float t1, int g, int t, float (&acc)[NT][4]) {
     constexpr int GPT = TILE / G;
     static_for<GPT>([&](auto gc) {
         constexpr int GI = decltype(gc)::value;
-        if constexpr (MODE == 2 && B == 3) {
+        if constexpr (MODE == 2 && B == 4) {
+            group_dot_w4<G, NT, GI>(r, reinterpret_cast<const __half *>(xs), xo, reinterpret_cast<uint8_t *>(ctab), t0, t1, g, t, acc);
+        } else if constexpr (MODE == 0 && B == 4) {
+            group_model_w4<G, NT, GI>(r, reinterpret_cast<const __half *>(xs), xo, reinterpret_cast<uint8_t *>(ctab), t0, t1, g, t, acc);
+        } else if constexpr (MODE == 2 && B == 3) {
             group_dot_w3<G, NT, GI>(r, reinterpret_cast<const __half *>(xs), xo, acc);
         } else if constexpr (MODE == 2) {
             const bool fix = B > 1 && __any_sync(0xffffffffu, (r.prm[0][GI].x | r.prm[1][GI].x) >> 31);
@@ -502,13 +583,14 @@ gemv_kernel(const uint8_t *__restrict__ layout, Dims d, const uint16_t *__restri
     constexpr bool F16 = MODE != 1;        // activations staged as fp16 (model dtype) or as the INT8 carrier
     constexpr int ES = F16 ? 2 : 1;        // bytes per staged activation element
     constexpr int CB = 2048 * B, TB = CB + 1024 * GPT;   // bytes of a tile's code part and of a whole tile
-    constexpr int XPAD = F16 ? (B == 3 ? 2 * XS_PAD : XS_PAD) : XS_PAD8;   // W3 reads 16 bytes per lane: rows 64 bytes apart in the banks
+    constexpr int XPAD = F16 ? (B == 3 || B == 4 ? 2 * XS_PAD : XS_PAD) : XS_PAD8;   // W3, W4 read 16 bytes per lane: rows 64 bytes apart in the banks
     extern __shared__ __align__(128) uint8_t smem[];
     __shared__ __align__(8) uint64_t s_full[MAX_STAGES], s_empty[MAX_STAGES];
     __shared__ float s_inv[16];
     __shared__ unsigned s_max[16];
     __shared__ int s_last, s_dead;
     __shared__ float s_t[MODE == 1 && B >= 3 ? 128 : 1];   // Dynamic A8: t_i = i / M of the carrier tables
+    __shared__ __align__(16) uint8_t s_w4[MODE != 1 && B == 4 ? GEMV_WARPS * 256 : 16];   // W4, model dtype: level tables of a warp's 16 rows
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
     const int VT = d.KT + E;                       // virtual units per row block
@@ -559,9 +641,14 @@ gemv_kernel(const uint8_t *__restrict__ layout, Dims d, const uint16_t *__restri
         tc::bulk_load(ring + (size_t)lane * TB, src + (size_t)lane * TB, (uint32_t)TB, &s_full[lane]);
     }
     DecodeRegs dr = {};
-    if constexpr (F16 && B != 3) dr = load_decode_regs();
+    if constexpr (F16 && B != 3 && B != 4) dr = load_decode_regs();
 
     int8_t *ctab = nullptr;
+    float w4_t0 = 0.0f, w4_t1 = 0.0f;   // positions of the two levels this lane evaluates for a table
+    if constexpr (F16 && B == 4) {
+        ctab = reinterpret_cast<int8_t *>(s_w4) + warp * 256;
+        w4_t0 = (float)(2 * t) / 7.0f; w4_t1 = (float)(2 * t + 1) / 7.0f;
+    }
     if constexpr (MODE == 1 && B >= 3) ctab = reinterpret_cast<int8_t *>(smem) + M * (MAX_SUB * TILE + XS_PAD8) + warp * 16 * carrier_table_stride(B);
 
     int st = 0, prev_st = 0;            // ring stage of the next tile (and of the one before it)
@@ -724,7 +811,7 @@ gemv_kernel(const uint8_t *__restrict__ layout, Dims d, const uint16_t *__restri
             int xo[NT];
 #pragma unroll
             for (int tb = 0; tb < NT; ++tb)
-                xo[tb] = (MODE == 2 ? min(tb, M - 1) : min(tb * 8 + g, M - 1)) * XS + ((F16 && B != 3) ? 4 : 8) * t;
+                xo[tb] = (MODE == 2 ? min(tb, M - 1) : min(tb * 8 + g, M - 1)) * XS + ((F16 && B != 3 && B != 4) ? 4 : 8) * t;
             const uint8_t *xcur = smem;
             if constexpr (!RING) {
                 int to_load = (ke - ks) - NBUF;                              // tiles not yet requested
@@ -732,7 +819,7 @@ gemv_kernel(const uint8_t *__restrict__ layout, Dims d, const uint16_t *__restri
                     static_for<NBUF>([&](auto ic) {
                         constexpr int i = decltype(ic)::value;
                         if (i < left) {
-                            compute_tile<B, G, NT, MODE>(buf_at(ic), dr, xcur, xo, ctab, s_t, g, t, acc);
+                            compute_tile<B, G, NT, MODE>(buf_at(ic), dr, xcur, xo, ctab, s_t, w4_t0, w4_t1, g, t, acc);
                             xcur += TILE * ES;
                             if (to_load > 0) { load_tile_g<B, GPT>(buf_at(ic), wl + i * TB, pl + i * TB, lane); --to_load; }
                         }
@@ -757,7 +844,7 @@ gemv_kernel(const uint8_t *__restrict__ layout, Dims d, const uint16_t *__restri
                 if (lane == 0) tc::mbar_arrive(&s_empty[st]);   // this warp's slice of the stage is in registers
                 prev_st = st; prev_ph = ph; ++it;
                 if (++st == nstage) { st = 0; ph ^= 1u; }
-                compute_tile<B, G, NT, MODE>(regs, dr, xcur, xo, ctab, s_t, g, t, acc);
+                compute_tile<B, G, NT, MODE>(regs, dr, xcur, xo, ctab, s_t, w4_t0, w4_t1, g, t, acc);
                 xcur += TILE * ES;
             }
             }
@@ -875,7 +962,7 @@ cudaError_t launch_one(const void *layout, const Dims &d, const uint16_t *x, con
     if (sub64 > d.KT) sub64 = d.KT;
     if (sub64 > MAX_SUB) sub64 = MAX_SUB;
     const int sub_tiles = (int)sub64;
-    const int XS = sub_tiles * TILE + (B == 3 ? 2 * XS_PAD : XS_PAD);
+    const int XS = sub_tiles * TILE + (B == 3 || B == 4 ? 2 * XS_PAD : XS_PAD);
     size_t xbytes = MODE != 1 ? (size_t)M * XS * 2 : (size_t)M * (MAX_SUB * TILE + XS_PAD8) + (B >= 3 ? 8 * 16 * carrier_table_stride(B) : 0);
     const uint32_t ring_off = (uint32_t)((xbytes + 127) / 128 * 128);
     constexpr int OCC = gemv_occ(B, G, NT, MODE);
@@ -972,7 +1059,7 @@ cudaError_t launch_gemv(const void *layout, const Dims &d, const uint16_t *x, ui
     float *dxs = reinterpret_cast<float *>(ws + plan.dx_off);
     const int64_t pitch = (int64_t)d.KT * TILE;
     if (mode == 1 && !prequantized) {
-        cudaError_t e = launch_quantize_a8(x, M, d.K, xq, pitch, dxs, true, act_f16, st);
+        cudaError_t e = launch_quantize_a8(x, M, d.K, xq, pitch, dxs, d.B != 4, act_f16, st);
         if (e != cudaSuccess) return e;
     }
     const int Mi = (int)M, P = gp.ctas, ms = gp.max_run;

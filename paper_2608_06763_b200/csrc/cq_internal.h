@@ -22,9 +22,10 @@ cudaError_t launch_a8_partials(const void *layout, const Dims &d, const int8_t *
 cudaError_t launch_quantize_a8(const uint16_t *x, int64_t M, int64_t K, int8_t *x8, int64_t x8_pitch, float *dx,
                                bool operand_order, bool act_f16, cudaStream_t st);
 
-// h[M][2 I] (gate | up, model dtype) -> INT8 carrier of silu(gate) * up in the MMA operand order, and its row scales
+// operand_order: x8 in the order of cq_decode.cuh that the INT8 products of every width but four bits read; natural order otherwise
+// h[M][2 I] (gate | up, model dtype) -> INT8 carrier of silu(gate) * up, and its row scales
 cudaError_t launch_swiglu_quantize_a8(const uint16_t *h, int64_t M, int64_t I, int8_t *x8, int64_t x8_pitch, float *dx,
-                                      bool act_f16, cudaStream_t st);
+                                      bool operand_order, bool act_f16, cudaStream_t st);
 // routed execution: xg[r] = x[route_token[r]] (zero row for an index outside [0, T))
 cudaError_t launch_gather_rows(const uint16_t *x, const int32_t *route_token, uint16_t *xg, int64_t R, int64_t T, int64_t K,
                                cudaStream_t st);

@@ -17,9 +17,16 @@ __device__ __forceinline__ unsigned canonical_field(const uint8_t *row, int64_t 
     return ((lo >> dlt) | (hi << (8 - dlt))) & ((1u << B) - 1u);
 }
 
-// canonical field -> stored code u (offset binary: the two's-complement sign bit flipped)
-__device__ __forceinline__ unsigned stored_from_field(int B, unsigned f) { return B == 1 ? f : (f ^ (1u << (B - 1))); }
-__device__ __forceinline__ unsigned field_from_stored(int B, unsigned u) { return B == 1 ? u : (u ^ (1u << (B - 1))); }
+// canonical field -> stored code u (offset binary: the two's-complement sign bit flipped; W4: sign and magnitude,
+// with the reserved pattern 8 mapped to itself) and back
+__device__ __forceinline__ unsigned stored_from_field(int B, unsigned f) {
+    if (B == 4) return f < 8 ? f : 8u | (16u - f);
+    return B == 1 ? f : (f ^ (1u << (B - 1)));
+}
+__device__ __forceinline__ unsigned field_from_stored(int B, unsigned u) {
+    if (B == 4) return u <= 8 ? u : 16u - (u & 7u);
+    return B == 1 ? u : (u ^ (1u << (B - 1)));
+}
 
 // ---------------------------------------------------------------- cq_pack_codes
 // one thread per output byte: gathers the bits of the (up to 8) fields that touch it
@@ -60,14 +67,13 @@ __global__ void repack_codes_kernel(const uint8_t *__restrict__ codes, Dims d, i
     const int wi = W - plane_word_base(d.B, pl);
     uint32_t word = 0;
     for (int q = 0; q < 16 / pw; ++q) {
-        const int pair = pair_at(pw, wi, q);
         for (int half = 0; half < 2; ++half) {
             int r, kk;
-            weight_of(rb, lane, pair, half, r, kk);
+            weight_of(d.B, pw, rb, lane, wi, q, half, r, kk);
             const int64_t n = (int64_t)nb * TILE + r, k = (int64_t)kb * TILE + kk;
             unsigned u;
             if (n < d.N && k < d.K) u = stored_from_field(d.B, canonical_field(codes + n * row_bytes, k, d.B, row_bytes));
-            else u = (d.B == 1) ? 1u : (1u << (d.B - 1));  // padding: code 0 (W1: +1), its scale is 0
+            else u = (d.B == 1) ? 1u : stored_from_field(d.B, 0u);  // padding: code 0 (W1: +1), its scale is 0
             word |= ((u >> bo) & ((1u << pw) - 1u)) << (q * pw + 16 * half);
         }
     }
@@ -314,7 +320,7 @@ __global__ void __launch_bounds__(1024) quantize_a8_kernel(const uint16_t *__res
 // output h[m] = (gate | up), 2 I values in the model dtype, goes to act = silu(gate) * up -- evaluated in fp32
 // and rounded to the model dtype, which is what a separate activation operator would have written -- and
 // straight on to that row's Dynamic-A8 carrier (Eq. a8-activation-scale, Eq. a8-activation-quantization) in the
-// MMA operand order, without the activation ever reaching memory.  One CTA per row; I % 8 == 0.
+// order the product reads it in (carrier_order), without the activation ever reaching memory.  One CTA per row; I % 8 == 0.
 __device__ __forceinline__ uint32_t gated_act_bits(uint32_t g16, uint32_t u16, bool f16) {
     const float g = act_to_float(g16, f16), u = act_to_float(u16, f16);
     const float sg = __fdiv_rn(g, __fadd_rn(1.0f, expf(-g)));
@@ -328,6 +334,7 @@ __device__ __forceinline__ uint4 gated_act_chunk(const uint4 &g, const uint4 &u,
         o[q] = gated_act_bits(gw[q] & 0xFFFFu, uw[q] & 0xFFFFu, f16) | (gated_act_bits(gw[q] >> 16, uw[q] >> 16, f16) << 16);
     return make_uint4(o[0], o[1], o[2], o[3]);
 }
+template <bool OPERAND_ORDER>
 __global__ void __launch_bounds__(1024) swiglu_quantize_a8_kernel(const uint16_t *__restrict__ h, int64_t M, int64_t I,
                                                                  int8_t *__restrict__ x8, int64_t x8_pitch,
                                                                  float *__restrict__ dx, bool f16) {
@@ -375,6 +382,10 @@ __global__ void __launch_bounds__(1024) swiglu_quantize_a8_kernel(const uint16_t
                 r = fminf(fmaxf(r, -127.0f), 127.0f);
                 out[q >> 2] |= ((uint32_t)(int)r & 0xFFu) << (8 * (q & 3));
             }
+        }
+        if constexpr (!OPERAND_ORDER) {
+            *reinterpret_cast<uint2 *>(x8 + m * x8_pitch + j * 8) = make_uint2(out[0], out[1]);
+            continue;
         }
         // the operand order of quantize_a8_kernel<true>
         uint8_t *blk = reinterpret_cast<uint8_t *>(x8 + m * x8_pitch) + (j >> 2) * 32 + 2 * ((j >> 1) & 1) + 16 * (j & 1);
@@ -454,7 +465,7 @@ cudaError_t launch_quantize_a8(const uint16_t *x, int64_t M, int64_t K, int8_t *
 }
 
 cudaError_t launch_swiglu_quantize_a8(const uint16_t *h, int64_t M, int64_t I, int8_t *x8, int64_t x8_pitch, float *dx,
-                                      bool act_f16, cudaStream_t st) {
+                                      bool operand_order, bool act_f16, cudaStream_t st) {
     if (I % 8 != 0 || x8_pitch % 32 != 0 || (reinterpret_cast<uintptr_t>(h) & 15u) != 0) return cudaErrorInvalidValue;
     int64_t threads = ((I >> 3) + 31) / 32 * 32;
     if (threads > 1024) threads = 1024;
@@ -468,7 +479,7 @@ cudaError_t launch_swiglu_quantize_a8(const uint16_t *h, int64_t M, int64_t I, i
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, swiglu_quantize_a8_kernel, h, M, I, x8, x8_pitch, dx, act_f16);
+    return cudaLaunchKernelEx(&cfg, operand_order ? swiglu_quantize_a8_kernel<true> : swiglu_quantize_a8_kernel<false>, h, M, I, x8, x8_pitch, dx, act_f16);
 }
 
 // ---------------------------------------------------------------- cq_debug_wait_timeout

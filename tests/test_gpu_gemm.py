@@ -249,3 +249,27 @@ def test_bounded_wait_gives_up_and_is_reported():
     assert cq.cq_gemm_status(ws) == 0
     xb = x.view(torch.int16).cpu().numpy().view(np.uint16)
     check_y(y, oracle.gemm_model(c.codes, c.s, c.a, c.b, 4, 128, 512, xb), "after a reported timeout")
+
+
+@pytest.mark.parametrize("act", ["bf16", "f16"])
+@pytest.mark.parametrize("M", [1, 2, 5, 16, 40, 140])
+@pytest.mark.parametrize("G,K", [(32, 224), (64, 128), (128, 384), (256, 1280)])
+def test_w4_every_code_in_every_place(G, K, M, act):
+    # W4 is stored as sign and magnitude in its own order and decoded by table look-ups: every code (the reserved one
+    # too) in every place of a tile, an odd and an even number of layout tiles, ragged N
+    N = 136
+    c = logical_case(N, K, 4, G, seed=210 + G)
+    c.k[:] = ((np.arange(N)[:, None] * 5 + np.arange(K)[None, :] * 3 + np.arange(K)[None, :] // 16) % 16 - 8).astype(np.int8)
+    c = Case(c.k, c.s, c.a, c.b, 4, G)
+    assert np.array_equal(cq.cq_unpack(c.pw)[0].cpu().numpy(), c.codes)
+    x = datagen.activations(M, K, seed=211)
+    if act == "f16":
+        x = datagen.bf16_bits_to_f32(x).astype(np.float16).view(np.uint16)
+        xd = torch.from_numpy(x.view(np.float16)).cuda()
+    else:
+        xd = x_to_device(x)
+    y = cq.cq_gemm(c.pw, xd, cq.CQ_MODEL_DTYPE)
+    check_y(y.float().cpu().numpy().astype(np.float64), oracle.gemm_model(c.codes, c.s, c.a, c.b, 4, G, K, x, act=act), f"W4 G={G} M={M} {act}")
+    if act == "bf16":
+        ya, ref = run_both(c, x, cq.CQ_DYN_A8)
+        check_y(ya, ref, f"W4 a8 G={G} M={M}")
