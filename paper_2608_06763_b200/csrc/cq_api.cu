@@ -34,7 +34,7 @@ Workspace plan_workspace(const Dims &d, int64_t M, int mode) {
     }
     if (M > 16 && mode == CQ_MODEL_DTYPE) {   // stream-K: two partial tiles per run
         const TcPlan tp = gemm_tc_plan(d, M);
-        const size_t p2 = (size_t)tp.p2 * 2 * tp.bnt * TILE * 4;
+        const size_t p2 = (size_t)tp.p2 * tp.cw * 2 * tp.bnt * TILE * 4;
         if (p2 > part) part = p2;
     }
     w.partial_off = off; w.partial_bytes = align_up(part, 256); off += w.partial_bytes;
@@ -395,7 +395,9 @@ int cq_debug_gemm_plan(int B, int G, int64_t M, int64_t N, int64_t K, int mode, 
     const Dims d = make_dims(B, G, N, K);
     if (mode == CQ_MODEL_DTYPE) {
         const TcPlan tp = gemm_tc_plan(d, M);
-        plan[0] = tp.bnt; plan[1] = tp.t_full; plan[2] = tp.p2; plan[3] = (int64_t)d.NB * tp.token_tiles - tp.t_full;
+        // tiles of 128 channels; the last pair of an odd number of row blocks holds one
+        const int64_t nbu = (d.NB + tp.cw - 1) / tp.cw, whole = tp.t_full * tp.cw - (d.NB % tp.cw ? tp.t_full / nbu : 0);
+        plan[0] = tp.bnt; plan[1] = whole; plan[2] = (int64_t)tp.p2 * tp.cw; plan[3] = (int64_t)d.NB * tp.token_tiles - whole;
         plan[4] = tp.crossing;
     } else {
         const A8Plan ap = gemm_a8_plan(d, M);

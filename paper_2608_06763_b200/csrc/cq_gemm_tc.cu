@@ -2,7 +2,8 @@
 // sm_100a): weights stay packed in HBM and are decoded into bf16 shared-memory operand tiles
 // right before tcgen05.mma consumes them; accumulators live in TMEM.
 //
-// Roles inside a CTA (output tiles of 128 channels x BN or 2 BN tokens):
+// Roles inside a CTA (output tiles of 128 channels x BN tokens; above 128 tokens two CTAs share one stream of MMAs over 256
+// channels x 256 or 512 tokens):
 //   warp 0      TMA-loads activation tiles x[BN x 64] (128-byte swizzle) into a ring of stages; nothing but the wait
 //               for a stage stands between the MMAs that free it and the copy that refills it
 //   warp 18     bulk-copies raw layout tiles (codes + co-located group parameters) into their own ring (2-4 deep)
@@ -44,7 +45,8 @@ TcPlan gemm_tc_plan(const Dims &d, int64_t M) {
     TcPlan p;
     p.bnt = gemm_tc_token_tile(M);
     p.token_tiles = (int)((M + p.bnt - 1) / p.bnt);
-    const int64_t T = (int64_t)d.NB * p.token_tiles, sms = sm_count();
+    p.cw = p.bnt >= 256 ? 2 : 1;                    // wide token tiles are computed by CTA pairs
+    const int64_t NBU = (d.NB + p.cw - 1) / p.cw, T = NBU * p.token_tiles, sms = sm_count() / p.cw;   // tiles and places for them
     const int64_t r = T % sms;                      // tiles of the last, partial round
     p.t_full = T; p.p2 = 0; p.crossing = 0;
     if (r != 0) {
@@ -66,7 +68,7 @@ TcPlan gemm_tc_plan(const Dims &d, int64_t M) {
         }
         if (best_p2 > 0 && (whole - best) / all > 0.06) { p.p2 = (int)best_p2; p.crossing = best_crossing; p.t_full = T - r; }
     }
-    p.ctas = (int)(p.t_full + p.p2);
+    p.ctas = (int)(p.t_full + p.p2) * p.cw;
     p.stream_k = p.p2 > 0;
     return p;
 }

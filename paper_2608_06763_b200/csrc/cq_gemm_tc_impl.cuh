@@ -89,67 +89,76 @@ struct TcParams {
     float *partial;       // stream-K: fp32 partial tiles [CTA][2][BNT][128]
     int *counters;        // stream-K: layout tiles done, one per output tile
     int MT;               // token tiles
-    int64_t t_full;       // tiles computed whole, one CTA each
-    int p2;               // CTAs that share the units of the remaining tiles (stream-K)
+    int64_t t_full;       // tiles (of a CTA or a CTA pair) computed whole
+    int p2;               // CTAs or pairs that share the units of the remaining tiles (stream-K)
     bool f16;             // activations and output are binary16 instead of bfloat16 (the weights are decoded to match)
 };
 
 // ---------------------------------------------------------------- the kernel (model dtype)
-// Depth of the ring of activation tiles (64-wide k blocks) and of the ring of decoded weight tiles.  The 512-token
-// tile has room for two activation stages only (64 KB each); its weight stages are 16 KB, so four of them let
-// the decoders run two layout tiles ahead of the MMAs instead of in lockstep with them.
-constexpr int tc_stages(int BN, int NACC) { return BN * NACC >= 512 ? 2 : (BN == 256 ? 3 : 4); }
+// PAIR: two CTAs of a cluster compute 256 channels x BN NACC tokens with one stream of MMAs (cta_group::2).  Each decodes
+// its own 128 channels and loads HALF of the tokens, which the other half of the instruction reads from the partner's
+// shared memory.  Without that every SM reads all BN NACC tokens: 64 KB per 64-wide block at 512 tokens, against
+// 1048 cycles of MMA -- the 64 bytes a cycle that an SM can take from L2.  Measured (W4 G128, before -> now, with the
+// one-barrier ring below): a 64-wide block of a 128 x 512 tile 1580 -> 1060 cycles; linears of an 8B layer at M = 1024
+// 492 -> 423 us, at M = 200 168 -> 158 us; 70B gate_up, W3, M = 4096 3290 -> 2758 us (1395 TFLOP/s).
+//
+// The operand ring: a stage is one 64-wide k block, the decoded weights (16 KB) and the activations, filled behind one
+// barrier and freed by one commit (the issuing thread is on the critical path at small token tiles: with a barrier
+// and a commit for each operand it spent 560 cycles on a block of 256 cycles of MMA).  As deep as shared memory
+// allows beside two or three raw tiles, which take what is left, up to six.
+constexpr bool tc_pair(int BN) { return BN == 256; }
+constexpr int tc_b_stage_bytes(int BN, int NACC) { return NACC * (tc_pair(BN) ? BN / 2 : BN) * 128; }
 constexpr int tc_raw_stage_bytes(int B, int G) { return (2048 * B + 1024 * (TILE / G) + 1023) / 1024 * 1024; }
 constexpr int tc_table_bytes(int B) { return B == 4 ? DEC_WARPS * W4_TABLE_BYTES : 0; }
-// Weight stages: up to four, fewer where the activation ring and two raw tiles leave less room.
-constexpr int tc_stages_a(int B, int G, int BN, int NACC) {
-    const int left = 226 * 1024 - 512 - tc_table_bytes(B) - tc_stages(BN, NACC) * NACC * BN * 128 - 2 * tc_raw_stage_bytes(B, G);
-    const int n = left / A_STAGE_BYTES;
-    return n > 4 ? 4 : n < 2 ? 2 : n;
+constexpr int TC_SMEM = 226 * 1024 - 512;
+constexpr int tc_stages(int B, int G, int BN, int NACC) {
+    const int st = A_STAGE_BYTES + tc_b_stage_bytes(BN, NACC), room = TC_SMEM - tc_table_bytes(B);
+    int n = (room - 3 * tc_raw_stage_bytes(B, G)) / st;
+    if (n < 4) n = (room - 2 * tc_raw_stage_bytes(B, G)) / st;
+    return n > 8 ? 8 : n;
 }
-constexpr int tc_ring_bytes(int B, int G, int BN, int NACC) {
-    return tc_stages_a(B, G, BN, NACC) * A_STAGE_BYTES + tc_stages(BN, NACC) * NACC * BN * 128;
-}
-// Raw layout tiles in flight per CTA: as many as the shared memory left by the operand rings holds, two to four.
+constexpr int tc_ring_bytes(int B, int G, int BN, int NACC) { return tc_stages(B, G, BN, NACC) * (A_STAGE_BYTES + tc_b_stage_bytes(BN, NACC)); }
 constexpr int tc_raw_stages(int B, int G, int BN, int NACC) {
-    const int left = 226 * 1024 - 512 - tc_table_bytes(B) - tc_ring_bytes(B, G, BN, NACC);
-    const int n = left / tc_raw_stage_bytes(B, G);
-    return n > 4 ? 4 : n < 2 ? 2 : n;
+    const int n = (TC_SMEM - tc_table_bytes(B) - tc_ring_bytes(B, G, BN, NACC)) / tc_raw_stage_bytes(B, G);
+    return n > 6 ? 6 : n < 2 ? 2 : n;
 }
 
 __device__ __forceinline__ void named_barrier_sync(int id, int threads) {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
 
-// The work of one CTA.  The output is cut into tiles of 128 channels x BNT tokens (tile = mt * NB + nb, so
-// that CTAs running side by side read the same activations), each tile into its KT layout tiles along K.
-// CTAs 0 .. t_full - 1 compute one whole tile each; the hardware hands them to the SMs as these become free,
-// and CTAs that start together sweep K in step, so the activations they share stay in L2.
-// Stream-K: the units (tile, k) of the remaining tiles are dealt out as p2 contiguous runs, CTA t_full + c
+// The work of one CTA or CTA pair ("unit").  The output is cut into tiles of 128 (256) channels x BNT tokens (tile =
+// mt * NBU + nb, so that units running side by side read the same activations), each tile into its KT layout tiles
+// along K.  Units 0 .. t_full - 1 compute one whole tile each; the hardware hands them to the SMs as these become free,
+// and units that start together sweep K in step, so the activations they share stay in L2.
+// Stream-K: the steps (tile, k) of the remaining tiles are dealt out as p2 contiguous runs, unit t_full + c
 // owning [floor(V2 c / p2), floor(V2 (c + 1) / p2)), never more than one tile long; a run may begin and end
-// inside a tile, and a tile shared by several CTAs is finished by the last of them to arrive.
-struct Seg { int nb, mt, k0, k1; int64_t tile; };
-template <bool SK>
+// inside a tile, and a tile shared by several units is finished by the last of them to arrive.
+struct Seg { int nb, mt, k0, k1; int64_t tile; };   // nb: row block of this CTA; tile: of the unit
+template <bool SK, bool PAIR>
 struct SegWalk {
     int64_t t_full, v, v_end, V2;
-    int KT, NB, p2, c2;
+    int KT, NBU, p2, c2, unit, rank;
     bool whole_left;
-    __device__ SegWalk(const TcParams &prm) {
-        if constexpr (!SK) {   // one whole tile per CTA, nothing else
-            KT = prm.d.KT; NB = prm.d.NB; p2 = 0; c2 = 0; t_full = 0; v = v_end = V2 = 0; whole_left = true;
+    __device__ SegWalk(const TcParams &prm, int rank_) {
+        rank = rank_;
+        unit = PAIR ? (int)blockIdx.x >> 1 : (int)blockIdx.x;
+        KT = prm.d.KT; NBU = PAIR ? (prm.d.NB + 1) / 2 : prm.d.NB;
+        if constexpr (!SK) {   // one whole tile per unit, nothing else
+            p2 = 0; c2 = 0; t_full = 0; v = v_end = V2 = 0; whole_left = true;
             return;
         }
-        KT = prm.d.KT; NB = prm.d.NB; p2 = prm.p2; t_full = prm.t_full;
-        whole_left = (int64_t)blockIdx.x < t_full;
-        c2 = (int)((int64_t)blockIdx.x - t_full);   // index of the run
-        V2 = ((int64_t)NB * prm.MT - t_full) * KT;
+        p2 = prm.p2; t_full = prm.t_full;
+        whole_left = unit < t_full;
+        c2 = (int)(unit - t_full);   // index of the run
+        V2 = ((int64_t)NBU * prm.MT - t_full) * KT;
         if (!whole_left) { v = (V2 * c2) / p2; v_end = (V2 * (c2 + 1)) / p2; }
         else { v = 0; v_end = 0; }
     }
     __device__ bool next(Seg &s) {
         if (whole_left) {
             whole_left = false;
-            s.tile = blockIdx.x; s.k0 = 0; s.k1 = KT;
+            s.tile = unit; s.k0 = 0; s.k1 = KT;
         } else {
             if (v >= v_end) return false;
             const int64_t tl = v / KT;
@@ -159,7 +168,9 @@ struct SegWalk {
             s.k1 = s.k0 + (int)(ve - v);
             v = ve;
         }
-        s.mt = (int)(s.tile / NB); s.nb = (int)(s.tile - (int64_t)s.mt * NB);
+        s.mt = (int)(s.tile / NBU);
+        const int nbu = (int)(s.tile - (int64_t)s.mt * NBU);
+        s.nb = PAIR ? 2 * nbu + rank : nbu;
         return true;
     }
 };
@@ -170,47 +181,50 @@ template <int B, int G, int BN, int NACC, bool SK>
 __global__ void __launch_bounds__(TC_THREADS, 1)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap xmap, TcParams prm) {
     constexpr int GPT = TILE / G;
-    constexpr int STAGES = tc_stages(BN, NACC);        // ring of activation tiles (64-wide k blocks)
-    constexpr int STAGES_A = tc_stages_a(B, G, BN, NACC);   // ring of decoded weight tiles
+    constexpr int STAGES = tc_stages(B, G, BN, NACC);  // ring of 64-wide k blocks
     constexpr int RAW_STAGES = tc_raw_stages(B, G, BN, NACC);
-    constexpr int B_TILE_BYTES = BN * 128;             // one TMA box: BN tokens x 64 k
-    constexpr int B_STAGE_BYTES = NACC * B_TILE_BYTES;
+    constexpr bool PAIR = tc_pair(BN);
+    constexpr int BROWS = PAIR ? BN / 2 : BN;          // tokens of one TMA box and CTA
+    constexpr int B_TILE_BYTES = BROWS * 128;          // one TMA box: BROWS tokens x 64 k
+    constexpr int B_STAGE_BYTES = tc_b_stage_bytes(BN, NACC);
     constexpr int BNT = BN * NACC;                     // tokens per tile
     constexpr uint32_t TMEM_COLS = BNT < 32 ? 32 : BNT;
     extern __shared__ __align__(1024) uint8_t smem[];  // 1024-byte alignment is what the swizzled tiles need
-    uint8_t *sA = smem;                                        // STAGES_A x 16 KB
-    uint8_t *sB = sA + STAGES_A * A_STAGE_BYTES;               // STAGES x NACC x BN x 128 B
+    uint8_t *sA = smem;                                        // STAGES x 16 KB
+    uint8_t *sB = sA + STAGES * A_STAGE_BYTES;                 // STAGES x NACC x BROWS x 128 B
     uint8_t *sRaw = sB + STAGES * B_STAGE_BYTES;               // RAW_STAGES x raw_stage_bytes
     uint8_t *sTab = sRaw + RAW_STAGES * prm.raw_stage_bytes;   // W4: DEC_WARPS x W4_TABLE_BYTES
     uint64_t *bars = reinterpret_cast<uint64_t *>(sTab + tc_table_bytes(B));
-    uint64_t *a_full = bars, *a_empty = a_full + STAGES_A, *b_full = a_empty + STAGES_A, *b_empty = b_full + STAGES;
-    uint64_t *raw_full = b_empty + STAGES, *raw_empty = raw_full + RAW_STAGES, *acc_full = raw_empty + RAW_STAGES, *acc_empty = acc_full + 1;
+    uint64_t *full = bars, *empty = full + STAGES;
+    uint64_t *raw_full = empty + STAGES, *raw_empty = raw_full + RAW_STAGES, *acc_full = raw_empty + RAW_STAGES, *acc_empty = acc_full + 1;
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(acc_empty + 1);
     volatile int *s_last_p = reinterpret_cast<volatile int *>(tmem_slot + 1);    // "this CTA completes the tile"
     volatile int *gave_up = reinterpret_cast<volatile int *>(tmem_slot + 2);     // a bounded wait ran out somewhere in the CTA
 
     const Dims &d = prm.d;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int rank = PAIR ? (int)cluster_rank() : 0;
 
     if ((smem_u32(smem) & 1023u) != 0) {  // cannot happen with the alignment attribute; never run misaligned
         if (threadIdx.x == 0) atomicCAS(prm.status, 0, 9);
         return;
     }
     if (threadIdx.x == 0) {
-        for (int s = 0; s < STAGES_A; ++s) { mbar_init(&a_full[s], SET_WARPS); mbar_init(&a_empty[s], 1); }
-        for (int s = 0; s < STAGES; ++s) { mbar_init(&b_full[s], 1); mbar_init(&b_empty[s], 1); }
+        // full: the decoders of a set (of both CTAs of a pair) and the thread that announces the activations' bytes
+        for (int s = 0; s < STAGES; ++s) { mbar_init(&full[s], (PAIR ? 2 * SET_WARPS : SET_WARPS) + 1); mbar_init(&empty[s], 1); }
         for (int s = 0; s < RAW_STAGES; ++s) { mbar_init(&raw_full[s], 1); mbar_init(&raw_empty[s], SET_WARPS); }
         mbar_init(acc_full, 1);
-        mbar_init(acc_empty, DEC_WARPS);
+        mbar_init(acc_empty, PAIR ? 2 * DEC_WARPS : DEC_WARPS);
         fence_barrier_init();
         *gave_up = 0;
     }
     if (warp == 1) {
-        tmem_alloc(tmem_slot, TMEM_COLS);
-        tmem_relinquish();
+        if constexpr (PAIR) tmem_alloc_pair(tmem_slot, TMEM_COLS);
+        else { tmem_alloc(tmem_slot, TMEM_COLS); tmem_relinquish(); }
     }
     tc_fence_before();
     __syncthreads();
+    if constexpr (PAIR) cluster_sync();   // the partner's barriers are initialised before anything arrives on them
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
 
@@ -221,7 +235,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap xmap, TcParams prm) {
         if (!mbar_wait(bar, parity, prm.status, code, WAIT_LIMIT_CYCLES, gave_up)) *gave_up = 1;
     };
 
-    SegWalk<SK> walk(prm);
+    SegWalk<SK, PAIR> walk(prm, rank);
     Seg seg;
     if (warp == 0) {
         // ===== producer of the activation tiles.  Nothing but the wait for the stage stands between the MMAs
@@ -232,11 +246,16 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap xmap, TcParams prm) {
                 for (int t = seg.k0; t < seg.k1; ++t) {
                     for (int half_k = 0; half_k < 2; ++half_k, ++kbc) {
                         const int s = kbc % STAGES;
-                        if (kbc >= STAGES) wait(&b_empty[s], ((kbc / STAGES) - 1) & 1, 2);
-                        mbar_arrive_expect_tx(&b_full[s], B_STAGE_BYTES);
+                        if (kbc >= STAGES) wait(&empty[s], ((kbc / STAGES) - 1) & 1, 2);
+                        // a pair's stage is announced once, on the barrier of the CTA that issues the MMAs
+                        if (rank == 0) mbar_arrive_expect_tx(&full[s], (PAIR ? 2 : 1) * B_STAGE_BYTES);
 #pragma unroll
-                        for (int a = 0; a < NACC; ++a)
-                            tma_load_2d(sB + s * B_STAGE_BYTES + a * B_TILE_BYTES, &xmap, &b_full[s], (2 * t + half_k) * 64, seg.mt * BNT + a * BN);
+                        for (int a = 0; a < NACC; ++a) {
+                            uint8_t *dst = sB + s * B_STAGE_BYTES + a * B_TILE_BYTES;
+                            const int tok = seg.mt * BNT + a * BN + rank * BROWS;
+                            if constexpr (PAIR) tma_load_2d_pair(dst, &xmap, map_to_rank(&full[s], 0), (2 * t + half_k) * 64, tok);
+                            else tma_load_2d(dst, &xmap, &full[s], (2 * t + half_k) * 64, tok);
+                        }
                     }
                 }
             }
@@ -247,7 +266,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap xmap, TcParams prm) {
         if (lane == 0) {
             int tcnt = 0;    // layout tiles issued so far
             while (walk.next(seg)) {
-                const uint8_t *tiles = prm.layout + (size_t)seg.nb * d.KT * (size_t)d.tile_bytes;
+                const int nb = min(seg.nb, d.NB - 1);   // the second CTA of a last, half pair decodes what nobody stores
+                const uint8_t *tiles = prm.layout + (size_t)nb * d.KT * (size_t)d.tile_bytes;
                 for (int t = seg.k0; t < seg.k1; ++t, ++tcnt) {
                     const int rs = tcnt % RAW_STAGES;
                     if (tcnt >= RAW_STAGES) wait(&raw_empty[rs], ((tcnt / RAW_STAGES) - 1) & 1, 1);
@@ -257,31 +277,41 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap xmap, TcParams prm) {
             }
         }
     } else if (warp == 1) {
-        // ===== MMA issuer
-        if (lane == 0) {
-            const uint32_t idesc = prm.f16 ? idesc_f16(BN) : idesc_bf16(BN);
-            int kbc = 0, segc = 0;
+        // ===== MMA issuer (of a pair: rank 0).  The whole warp walks the loop, so that descriptors and addresses stay
+        // uniform; one elected lane issues.
+        if (rank == 0) {
+            constexpr int MM = PAIR ? 256 : 128;
+            const uint32_t idesc = prm.f16 ? idesc_f16(BN, MM) : idesc_bf16(BN, MM);
+            auto commit = [&](uint64_t *bar) { if constexpr (PAIR) umma_commit_pair(bar); else umma_commit(bar); };
+            const bool issuer = elect_one();
+            int s = 0, segc = 0;
+            uint32_t phase = 0;
             while (walk.next(seg)) {
                 if (SK && segc > 0) wait(acc_empty, (segc - 1) & 1, 8);   // every decoder has read the accumulators of the segment before
                 ++segc;
                 const int nkb = 2 * (seg.k1 - seg.k0);
-                for (int i = 0; i < nkb; ++i, ++kbc) {
-                    const int s = kbc % STAGES, sa = kbc % STAGES_A;
-                    wait(&a_full[sa], (kbc / STAGES_A) & 1, 3);
-                    wait(&b_full[s], (kbc / STAGES) & 1, 4);
+                for (int i = 0; i < nkb; ++i) {
+                    wait(&full[s], phase, 3);
                     tc_fence_after();
-                    const uint64_t adesc = smem_desc_sw128(smem_u32(sA + sa * A_STAGE_BYTES));
+                    const uint64_t adesc = smem_desc_sw128(smem_u32(sA) + s * A_STAGE_BYTES);
+                    const uint64_t bdesc0 = smem_desc_sw128(smem_u32(sB) + s * B_STAGE_BYTES);
+                    if (issuer) {
 #pragma unroll
-                    for (int a = 0; a < NACC; ++a) {
-                        const uint64_t bdesc = smem_desc_sw128(smem_u32(sB + s * B_STAGE_BYTES + a * B_TILE_BYTES));
+                        for (int a = 0; a < NACC; ++a) {
+                            const uint64_t bdesc = bdesc0 + (uint64_t)(a * (B_TILE_BYTES >> 4));
 #pragma unroll
-                        for (int k = 0; k < 4; ++k)  // four K = 16 steps, 32 bytes apart inside the swizzle atom
-                            umma_bf16(tmem_base + a * BN, adesc + 2 * k, bdesc + 2 * k, idesc, (i | k) != 0);
+                            for (int k = 0; k < 4; ++k) {  // four K = 16 steps, 32 bytes apart inside the swizzle atom
+                                if constexpr (PAIR) umma_bf16_pair(tmem_base + a * BN, adesc + 2 * k, bdesc + 2 * k, idesc, (i | k) != 0);
+                                else umma_bf16(tmem_base + a * BN, adesc + 2 * k, bdesc + 2 * k, idesc, (i | k) != 0);
+                            }
+                        }
+                        commit(&empty[s]);  // frees the stage when these MMAs have read it
                     }
-                    umma_commit(&a_empty[sa]);  // frees the two stages when these MMAs have read them
-                    umma_commit(&b_empty[s]);
+                    __syncwarp();
+                    if (++s == STAGES) { s = 0; phase ^= 1u; }
                 }
-                umma_commit(acc_full);   // the accumulators of this segment are complete when these MMAs are
+                if (issuer) commit(acc_full);   // the accumulators of this segment are complete when these MMAs are
+                __syncwarp();
             }
         }
     } else {
@@ -291,7 +321,11 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap xmap, TcParams prm) {
         const int dw = warp - 2, g = lane >> 2, t = lane & 3;
         const int rb = dw & (SET_WARPS - 1), set = dw / SET_WARPS;
         const int dec_tid = threadIdx.x - 64;
+        auto arrive = [&](uint64_t *bar) { if (PAIR && rank != 0) mbar_arrive_cluster(map_to_rank(bar, 0)); else mbar_arrive(bar); };
         int tcnt = 0, segc = 0;
+        // Where the MMAs of a block are short the decoders set the pace, and a fence (some 200 cycles) is shared by a tile's
+        // two blocks; a wide token tile wants its blocks as early as they are ready.
+        constexpr bool ONE_FENCE = BNT <= 128 && STAGES >= 6;
         float w4_t0 = 0.0f, w4_t1 = 0.0f;   // W4: positions of the two levels this lane evaluates for a table
         if constexpr (B == 4) { w4_t0 = (float)(2 * t) / 7.0f; w4_t1 = (float)(2 * t + 1) / 7.0f; }
 #pragma unroll 1
@@ -316,29 +350,35 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap xmap, TcParams prm) {
                     w[4 * NFQ + 0] = v.x; w[4 * NFQ + 1] = v.y;
                 }
             }
-            const uint8_t *prow = raw + d.code_bytes + ((rb * 16 + g) * GPT) * 8;
+            uint2 q_lo[GPT], q_hi[GPT];   // the parameter records of rows g and g + 8
+            {
+                const uint8_t *prow = raw + d.code_bytes + ((rb * 16 + g) * GPT) * 8;
+#pragma unroll
+                for (int i = 0; i < GPT; ++i) { q_lo[i] = *(const uint2 *)(prow + i * 8); q_hi[i] = *(const uint2 *)(prow + (8 * GPT + i) * 8); }
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&raw_empty[rs]);   // all of it is in registers
             W3Table w3_lo{}, w3_hi{};   // W3: level tables of rows g and g + 8; one per tile when the group spans it
             if constexpr (B == 3 && G == 128) {
-                w3_lo = w3_table(*(const uint2 *)prow, prm.f16);
-                w3_hi = w3_table(*(const uint2 *)(prow + 8 * GPT * 8), prm.f16);
+                w3_lo = w3_table(q_lo[0], prm.f16);
+                w3_hi = w3_table(q_hi[0], prm.f16);
             }
             // G = 128: one group spans the tile, so its coefficients are formed once per tile, not once per 64-wide block
             RowCoef tc_lo{}, tc_hi{};
             bool tfix = false;
             if constexpr (B != 3 && B != 4 && G == 128) {
-                const uint2 q_lo = *(const uint2 *)prow, q_hi = *(const uint2 *)(prow + 8 * GPT * 8);
-                tc_lo = make_coef<B>(q_lo); tc_hi = make_coef<B>(q_hi);
-                tfix = B > 1 && __any_sync(0xffffffffu, (q_lo.x | q_hi.x) >> 31);
+                tc_lo = make_coef<B>(q_lo[0]); tc_hi = make_coef<B>(q_hi[0]);
+                tfix = B > 1 && __any_sync(0xffffffffu, (q_lo[0].x | q_hi[0].x) >> 31);
             }
             uint4 w4_lo{}, w4_hi{};     // W4: tables of rows g and g + 8 (G >= 64: of the block's one group)
             uint8_t *wtab = sTab + dw * W4_TABLE_BYTES;
             // tables of the groups gi0 .. gi0 + n - 1 (n = 1, 2) of the tile, one after another in this warp's shared memory
-            auto w4_build = [&](int gi0, auto nc) {
-                constexpr int n = decltype(nc)::value;
+            auto w4_build = [&](auto g0c, auto nc) {
+                constexpr int gi0 = decltype(g0c)::value, n = decltype(nc)::value;
                 __syncwarp();   // the tables before have been read
 #pragma unroll
                 for (int e = 0; e < n; ++e) {
-                    const uint2 p_lo = *(const uint2 *)(prow + (gi0 + e) * 8), p_hi = *(const uint2 *)(prow + (8 * GPT + gi0 + e) * 8);
+                    const uint2 p_lo = q_lo[gi0 + e], p_hi = q_hi[gi0 + e];
                     const float s_lo = __uint_as_float(p_lo.x & 0x7FFFFFFFu), s_hi = __uint_as_float(p_hi.x & 0x7FFFFFFFu);
                     auto pack = [&](float a, float b) { return pack_act2(a, b, prm.f16); };
                     w4_put(wtab + e * 256 + g * 16, p_lo, t, w4_t0, w4_t1, s_lo, pack);
@@ -347,19 +387,19 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap xmap, TcParams prm) {
                 __syncwarp();
             };
             if constexpr (B == 4 && G == 128) {
-                w4_build(0, std::integral_constant<int, 1>{});
+                w4_build(std::integral_constant<int, 0>{}, std::integral_constant<int, 1>{});
                 w4_lo = *(const uint4 *)(wtab + g * 16); w4_hi = *(const uint4 *)(wtab + (g + 8) * 16);
             }
             // the two 64-wide blocks of the tile, two 32-wide units each
             static_for<2>([&](auto hc) {
                 constexpr int H = decltype(hc)::value;
-                const int kb = 2 * tcnt + H, s = kb % STAGES_A;
+                const int kb = 2 * tcnt + H, s = kb % STAGES;
                 if constexpr (B == 4 && G == 64) {
-                    w4_build(H, std::integral_constant<int, 1>{});
+                    w4_build(hc, std::integral_constant<int, 1>{});
                     w4_lo = *(const uint4 *)(wtab + g * 16); w4_hi = *(const uint4 *)(wtab + (g + 8) * 16);
                 }
-                if constexpr (B == 4 && G == 32) w4_build(2 * H, std::integral_constant<int, 2>{});
-                if (kb >= STAGES_A) wait(&a_empty[s], ((kb / STAGES_A) - 1) & 1, 6);
+                if constexpr (B == 4 && G == 32) w4_build(std::integral_constant<int, 2 * H>{}, std::integral_constant<int, 2>{});
+                if (kb >= STAGES) wait(&empty[s], ((kb / STAGES) - 1) & 1, 6);
                 uint8_t *a_stage = sA + s * A_STAGE_BYTES;
                 // rows g (low) and g + 8 (high) of the row block: their 128-byte rows in the stage
                 uint8_t *row_lo = a_stage + (rb * 2 + 0) * 1024 + g * 128;
@@ -386,7 +426,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap xmap, TcParams prm) {
                 static_for<2>([&](auto uc) {
                     constexpr int JQ = 2 * H + decltype(uc)::value;    // pair of chunks 2 JQ, 2 JQ + 1 of the tile
                     constexpr int gi = (32 * JQ) / G;              // both chunks lie in this group
-                    const uint2 p_lo = *(const uint2 *)(prow + gi * 8), p_hi = *(const uint2 *)(prow + (8 * GPT + gi) * 8);
+                    const uint2 p_lo = q_lo[gi], p_hi = q_hi[gi];
                     if constexpr (B == 3) {
                         // table decode (w3_block): no per-weight arithmetic, the reserved pattern reads zero
                         if constexpr (G < 128) { w3_lo = w3_table(p_lo, prm.f16); w3_hi = w3_table(p_hi, prm.f16); }
@@ -425,12 +465,17 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap xmap, TcParams prm) {
                     }
                 });
                 }
-                fence_proxy_async();   // generic-proxy stores -> visible to the tensor core's async proxy
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&a_full[s]);
+                if constexpr (!ONE_FENCE) {
+                    fence_proxy_async();   // generic-proxy stores -> visible to the tensor core's async proxy
+                    __syncwarp();
+                    if (lane == 0) arrive(&full[s]);
+                }
             });
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&raw_empty[rs]);
+            if constexpr (ONE_FENCE) {
+                fence_proxy_async();
+                __syncwarp();
+                if (lane == 0) { arrive(&full[(2 * tcnt) % STAGES]); arrive(&full[(2 * tcnt + 1) % STAGES]); }
+            }
         }
         // ----- epilogue of the segment: TMEM lane = output channel, column = token
         wait(acc_full, segc & 1, 7);
@@ -441,13 +486,14 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap xmap, TcParams prm) {
             const int q4 = warp & 3;                       // TMEM lane quarter this warp may access
             const int cp = dw >> 2;                        // which of four column parts
             const int64_t n = (int64_t)seg.nb * TILE + q4 * 32 + lane;
-            if ((d.N & 7) == 0 && (!SK || (int64_t)blockIdx.x < prm.t_full)) {
+            if ((d.N & 7) == 0 && (!SK || walk.unit < prm.t_full)) {
                 // A CTA whose only work is this whole tile, and rows of y that start on 16-byte boundaries: the tile goes
-                // through shared memory (the activation ring is idle by now: every MMA has completed and nothing more is
+                // through shared memory (the operand ring is idle by now: every MMA has completed and nothing more is
                 // loaded; a CTA with a run of several segments may already be loading the next one) as
                 // [token][128 channels] in the output dtype, and leaves it in 16-byte pieces, eight channels of one
                 // token per thread, instead of one 2-byte store per output.
-                uint16_t *stage = reinterpret_cast<uint16_t *>(sB);
+                static_assert(BNT * TILE * 2 <= tc_ring_bytes(B, G, BN, NACC), "the tile is staged in the operand ring");
+                uint16_t *stage = reinterpret_cast<uint16_t *>(smem);
 #pragma unroll 1
                 for (int c0 = cp * 32; c0 < BNT; c0 += 128) {
                     uint32_t r[32];
@@ -480,7 +526,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap xmap, TcParams prm) {
             } else {
                 // A run has at most two partial segments: its first (which begins inside a tile) and its last
                 // (which begins a tile without finishing it); each run owns two partial slots [BNT][128].
-                float *slot = prm.partial + ((size_t)walk.c2 * 2 + (seg.k0 > 0 ? 1 : 0)) * (size_t)(BNT * TILE) + q4 * 32 + lane;
+                constexpr int CW = PAIR ? 2 : 1;
+                float *slot = prm.partial + (((size_t)walk.c2 * CW + rank) * 2 + (seg.k0 > 0 ? 1 : 0)) * (size_t)(BNT * TILE) + q4 * 32 + lane;
 #pragma unroll 1
                 for (int c0 = cp * 32; c0 < BNT; c0 += 128) {
                     uint32_t r[32];
@@ -492,15 +539,15 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap xmap, TcParams prm) {
             }
         }
         tc_fence_before();   // the accumulators have been read: the MMAs of the next segment may overwrite them
-        if constexpr (SK) { __syncwarp(); if (lane == 0) mbar_arrive(acc_empty); }
-        if (SK && !whole) {
+        if constexpr (SK) { __syncwarp(); if (lane == 0) arrive(acc_empty); }
+        if (SK && !whole && seg.nb < d.NB) {
             // The tile's counter collects the layout tiles done; the CTA that completes it adds the partial tiles
             // in K order.  The first barrier orders the decoders' partial stores before the release; the acquire
             // plus the second barrier make the other CTAs' partials visible to every decoder.
             named_barrier_sync(1, 32 * DEC_WARPS);
             if (dec_tid == 0) {
                 int old;
-                asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], %2;" : "=r"(old) : "l"(prm.counters + seg.tile), "r"(seg.k1 - seg.k0) : "memory");
+                asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], %2;" : "=r"(old) : "l"(prm.counters + (int64_t)seg.mt * d.NB + seg.nb), "r"(seg.k1 - seg.k0) : "memory");
                 *s_last_p = (old + (seg.k1 - seg.k0) == d.KT);
             }
             named_barrier_sync(1, 32 * DEC_WARPS);
@@ -512,6 +559,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap xmap, TcParams prm) {
                 // contributors in flight (the partial tiles come from L2: it is the loads in flight that set the pace),
                 // and adds the contributors in K order.
                 constexpr int QUADS = BNT * TILE / 4, NTHR = 32 * DEC_WARPS;
+                constexpr int CW = PAIR ? 2 : 1;
                 const size_t slot_elems = (size_t)(BNT * TILE);
                 for (int base = dec_tid; base < QUADS; base += 4 * NTHR) {
                     float4 sum[4];
@@ -526,7 +574,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap xmap, TcParams prm) {
                             for (int w = 0; w < 4; ++w) {
                                 const int q = q0 + w;
                                 v[u][w] = (qd < QUADS && q < n_contrib)
-                                              ? __ldcg(reinterpret_cast<const float4 *>(prm.partial + ((size_t)(c_first + q) * 2 + (q == 0 ? 0 : 1)) * slot_elems) + qd)
+                                              ? __ldcg(reinterpret_cast<const float4 *>(prm.partial + (((size_t)(c_first + q) * CW + rank) * 2 + (q == 0 ? 0 : 1)) * slot_elems) + qd)
                                               : make_float4(0.f, 0.f, 0.f, 0.f);
                             }
                         }
@@ -548,7 +596,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap xmap, TcParams prm) {
                             if (n + e < d.N) prm.y[m * d.N + n + e] = float_to_act(o[e], prm.f16);
                     }
                 }
-                if (dec_tid == 0) prm.counters[seg.tile] = 0;  // leave the workspace ready for the next call
+                if (dec_tid == 0) prm.counters[(int64_t)seg.mt * d.NB + seg.nb] = 0;  // leave the workspace ready for the next call
             }
         }
         }
@@ -560,7 +608,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap xmap, TcParams prm) {
     }
     tc_fence_before();
     __syncthreads();
-    if (warp == 1) tmem_dealloc(tmem_base, TMEM_COLS);
+    if constexpr (PAIR) cluster_sync();   // the partner is done with this CTA's shared memory, and this one with the partner's
+    if (warp == 1) { if constexpr (PAIR) tmem_dealloc_pair(tmem_base, TMEM_COLS); else tmem_dealloc(tmem_base, TMEM_COLS); }
 }
 
 // ---------------------------------------------------------------- host side
@@ -572,29 +621,38 @@ cudaError_t launch_bn(const void *layout, const Dims &d, const uint16_t *x, uint
     CUtensorMap xmap;
     const cuuint64_t dims[2] = {(cuuint64_t)d.K, (cuuint64_t)M};
     const cuuint64_t strides[1] = {(cuuint64_t)d.K * 2};
-    const cuuint32_t box[2] = {64, (cuuint32_t)BN};
+    const cuuint32_t box[2] = {64, (cuuint32_t)(tc_pair(BN) ? BN / 2 : BN)};
     const cuuint32_t estr[2] = {1, 1};
     if (enc(&xmap, act_f16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<uint16_t *>(x), dims, strides, box, estr,
             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return cudaErrorInvalidValue;
     const TcPlan plan = gemm_tc_plan(d, M);
-    if (plan.bnt != BN * NACC || (plan.p2 > 0) != SK) return cudaErrorInvalidConfiguration;
+    if (plan.bnt != BN * NACC || (plan.p2 > 0) != SK || (plan.cw == 2) != tc_pair(BN)) return cudaErrorInvalidConfiguration;
     TcParams p;
     p.layout = (const uint8_t *)layout; p.y = y; p.status = status; p.d = d; p.M = (int)M;
     p.raw_stage_bytes = (d.tile_bytes + 1023) / 1024 * 1024;
     p.MT = plan.token_tiles; p.t_full = plan.t_full; p.p2 = plan.p2;
     constexpr int RAW_STAGES = tc_raw_stages(B, G, BN, NACC);
     if (p.raw_stage_bytes != tc_raw_stage_bytes(B, G)) return cudaErrorInvalidConfiguration;
-    const size_t smem = (size_t)tc_ring_bytes(B, G, BN, NACC) + (size_t)RAW_STAGES * p.raw_stage_bytes + tc_table_bytes(B) + 256;
-    static_assert(tc_ring_bytes(B, G, BN, NACC) + tc_raw_stages(B, G, BN, NACC) * tc_raw_stage_bytes(B, G) + tc_table_bytes(B) + 256 <= 227 * 1024, "shared memory");
+    const size_t smem = (size_t)tc_ring_bytes(B, G, BN, NACC) + (size_t)RAW_STAGES * p.raw_stage_bytes + tc_table_bytes(B) + 512;
+    static_assert(tc_ring_bytes(B, G, BN, NACC) + tc_raw_stages(B, G, BN, NACC) * tc_raw_stage_bytes(B, G) + tc_table_bytes(B) + 512 <= 227 * 1024 && tc_stages(B, G, BN, NACC) >= 3, "shared memory");
     auto kern = gemm_tc_kernel<B, G, BN, NACC, SK>;
     static std::atomic<uint64_t> attr_done{0};   // per kernel instantiation: the devices it has been set on
     cudaError_t ea = ensure_func_attr(kern, attr_done, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
     if (ea != cudaSuccess) return ea;
     p.partial = partial; p.counters = counters; p.f16 = act_f16;
-    kern<<<dim3((unsigned)plan.ctas), TC_THREADS, smem, st>>>(xmap, p);
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)plan.ctas);
+    cfg.blockDim = dim3(TC_THREADS);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = tc_pair(BN) ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kern, xmap, p);
 }
 
 template <int B, int G, bool SK>

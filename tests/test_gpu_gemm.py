@@ -273,3 +273,17 @@ def test_w4_every_code_in_every_place(G, K, M, act):
     if act == "bf16":
         ya, ref = run_both(c, x, cq.CQ_DYN_A8)
         check_y(ya, ref, f"W4 a8 G={G} M={M}")
+
+
+@pytest.mark.parametrize("B,G", [(4, 128), (8, 32), (2, 64)])
+@pytest.mark.parametrize("N,K,M", [(128, 256, 129), (136, 128, 256), (384, 640, 257), (300, 2048, 512), (520, 1024, 513)])
+def test_pairs_of_ctas(N, K, M, B, G):
+    # token tiles of 256 and 512 are computed by two CTAs together, 128 channels each: an odd number of row blocks leaves
+    # the last pair half empty; ragged channels and tokens on both sides of the halves that the CTAs load
+    c = logical_case(N, K, B, G, seed=220 + M)
+    x = datagen.activations(M, K, seed=221, outlier_cols=0.01)
+    ws = torch.zeros(cq.cq_workspace_bytes(B, G, M, N, K, 0), dtype=torch.uint8, device="cuda")
+    y = torch.full((M + 1, N), 7.0, dtype=torch.bfloat16, device="cuda")      # nothing is written beyond the last token
+    cq.cq_gemm(c.pw, x_to_device(x), cq.CQ_MODEL_DTYPE, ws, y[:M])
+    assert cq.cq_gemm_status(ws) == 0 and bool((y[M] == 7.0).all())
+    check_y(y_to_numpy(y[:M]), oracle.gemm_model(c.codes, c.s, c.a, c.b, B, G, K, x), f"pairs N={N} K={K} M={M}")
