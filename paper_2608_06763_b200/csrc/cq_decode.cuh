@@ -233,10 +233,10 @@ __device__ __forceinline__ void w4_put(uint8_t *row, uint2 p, int t, float t0, f
 //          inside the block is the natural one, lane t holding bytes 8 t .. 8 t + 7;
 //   B = 3: one 8-byte table, the selector assembled from the 2-bit and the 1-bit plane;
 //   B <= 2: the carriers are 0 / +-127, a constant table;
-//   B >= 5: the table stays in shared memory and is read per code.
+//   B >= 5: no table (a8_row_eval).
 template <int B, int RR, int MI>
-__device__ __forceinline__ void a8_row_regs(const uint32_t (&w)[2 * B], const uint4 &tab, const int8_t *trow,
-                                            uint32_t &lo, uint32_t &hi) {
+__device__ __forceinline__ void a8_row_regs(const uint32_t (&w)[2 * B], const uint4 &tab, uint32_t &lo, uint32_t &hi) {
+    static_assert(B <= 4, "wider codes are evaluated one by one (a8_row_eval)");
     if constexpr (B == 4) {
         const uint32_t word = w[2 * MI + RR];
         const uint32_t ws = word & 0x77777777u, wh = ws >> 16, w4 = word << 4;
@@ -257,20 +257,77 @@ __device__ __forceinline__ void a8_row_regs(const uint32_t (&w)[2 * B], const ui
         const uint32_t sel = (RR ? (w[MI] >> 2) : w[MI]) & 0x33333333u;
         lo = prmt(0x7F008100u, 0u, sel);          // u = 0 reserved -> 0, 1 -> -127, 2 -> 0, 3 -> +127
         hi = prmt(0x7F008100u, 0u, sel >> 16);
-    } else if constexpr (B == 1) {
+    } else {
         constexpr int rho = (2 + 2 * (MI & 1) + RR) & 3;
         const uint32_t sel = (w[MI >> 1] >> rho) & 0x11111111u;
         lo = prmt(0x00007F81u, 0u, sel);          // bit 0 -> -127, bit 1 -> +127
         hi = prmt(0x00007F81u, 0u, sel >> 16);
-    } else {
-        lo = 0; hi = 0;
-        static_for<4>([&](auto nc) {
-            constexpr int n = decltype(nc)::value, p = 4 * (2 * MI + (n >> 1)) + 2 * (n & 1) + RR;
-            const uint32_t u2 = pair_codes<B, p>(w);
-            lo |= (uint32_t)(uint8_t)trow[u2 & 0xFFFFu] << (8 * n);
-            hi |= (uint32_t)(uint8_t)trow[u2 >> 16] << (8 * n);
-        });
     }
+}
+
+// ---- B >= 5: the carrier of each code evaluated where it is needed, two at a time in packed fp32, by the pinned
+// sequence of carrier_at.  A table per (row, group) would have as many entries as the group has weights (W8, G = 128), and
+// reading it costs a shared-memory access per weight with the lanes in random banks: linears of an 8B layer, W8 G128,
+// M = 64: 400 us with tables, 204 us so.
+__device__ __forceinline__ uint64_t f2_pack(uint32_t lo, uint32_t hi) { uint64_t d; asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "r"(lo), "r"(hi)); return d; }
+__device__ __forceinline__ void f2_split(uint64_t v, uint32_t &lo, uint32_t &hi) { asm("mov.b64 {%0, %1}, %2;" : "=r"(lo), "=r"(hi) : "l"(v)); }
+__device__ __forceinline__ uint64_t f2_dup(float v) { return f2_pack(__float_as_uint(v), __float_as_uint(v)); }
+__device__ __forceinline__ uint64_t f2_add(uint64_t a, uint64_t b) { uint64_t d; asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b)); return d; }
+__device__ __forceinline__ uint64_t f2_mul(uint64_t a, uint64_t b) { uint64_t d; asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b)); return d; }
+__device__ __forceinline__ uint64_t f2_fma(uint64_t a, uint64_t b, uint64_t c) { uint64_t d; asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c)); return d; }
+__device__ __forceinline__ uint32_t mul_sat(uint32_t a, uint32_t b) {
+    float d;
+    asm("mul.rn.sat.f32 %0, %1, %2;" : "=f"(d) : "f"(__uint_as_float(a)), "f"(__uint_as_float(b)));
+    return __float_as_uint(d);
+}
+struct CarrierPoly { uint64_t a, b, c; };
+__device__ __forceinline__ CarrierPoly carrier_poly(uint32_t ab16) {
+    const __half2 ab = as_h2(ab16);
+    const float a = __low2float(ab), b = __high2float(ab);
+    return {f2_dup(a), f2_dup(b), f2_dup(__fsub_rn(__fsub_rn(1.0f, a), b))};
+}
+// Two codes, given as fp32 2^23 + u; the signed carriers come out in the low bytes.
+//   i = |u - 2^(B-1)|, exact; t = i / M as i r + i r', r + r' = 1/M to 48 bits: equal to the correctly rounded quotient for every
+//   i and M of B = 5 .. 8 (checked one by one); q as carrier_at has it; clamping q to [0, 1] before RNE(127 q) is clamping
+//   the carrier to [0, 127]; adding 1.5 2^23 rounds to nearest even, leaving the integer in the low bits.
+template <int B, bool FIX>
+__device__ __forceinline__ void carrier_pair(uint32_t f0, uint32_t f1, const CarrierPoly &p, uint32_t &r0, uint32_t &r1) {
+    constexpr int L = 1 << (B - 1), M = L - 1;
+    constexpr float r_hi = 1.0f / (float)M;
+    constexpr float r_lo = (float)(1.0 / (double)M - (double)r_hi);
+    uint32_t k0, k1, t0, t1, h0, h1, v0, v1;
+    f2_split(f2_add(f2_pack(f0, f1), f2_dup(-(8388608.0f + (float)L))), k0, k1);
+    const uint64_t i2 = f2_pack(k0 & 0x7FFFFFFFu, k1 & 0x7FFFFFFFu);
+    const uint64_t t = f2_fma(i2, f2_dup(r_hi), f2_mul(i2, f2_dup(r_lo)));
+    f2_split(f2_fma(t, f2_fma(t, p.c, p.b), p.a), h0, h1);
+    f2_split(t, t0, t1);
+    uint32_t q0 = mul_sat(t0, h0), q1 = mul_sat(t1, h1);
+    if constexpr (FIX) {   // the reserved pattern: the one code whose magnitude is beyond M
+        if (__uint_as_float(t0) > 1.0f) q0 = 0u;
+        if (__uint_as_float(t1) > 1.0f) q1 = 0u;
+    }
+    f2_split(f2_mul(f2_pack(q0, q1), f2_dup(127.0f)), v0, v1);
+    f2_split(f2_add(f2_pack(v0 | (k0 & 0x80000000u), v1 | (k1 & 0x80000000u)), f2_dup(12582912.0f)), r0, r1);
+}
+template <int B, int RR, int MI, bool FIX>
+__device__ __forceinline__ void a8_row_eval(const uint32_t (&w)[2 * B], const CarrierPoly &poly, uint32_t &lo, uint32_t &hi) {
+    uint32_t e0[4], e1[4];   // the carriers of k + 0 and k + 1 (bytes n of lo and hi)
+    static_for<4>([&](auto nc) {
+        constexpr int n = decltype(nc)::value, p = 4 * (2 * MI + (n >> 1)) + 2 * (n & 1) + RR;
+        uint32_t f0, f1;
+        if constexpr (B == 8) {
+            constexpr int W = pair_word(8, p), byte = pair_pos(8, p) / 8;
+            f0 = prmt(w[W], 0x4B000000u, 0x7440u + byte);
+            f1 = prmt(w[W], 0x4B000000u, 0x7440u + byte + 2);
+        } else {
+            const uint32_t u2 = pair_codes<B, p>(w);
+            f0 = prmt(u2, 0x4B000000u, 0x7440u);
+            f1 = prmt(u2, 0x4B000000u, 0x7442u);
+        }
+        carrier_pair<B, FIX>(f0, f1, poly, e0[n], e1[n]);
+    });
+    lo = prmt(prmt(e0[0], e0[1], 0x0040u), prmt(e0[2], e0[3], 0x0040u), 0x5410u);
+    hi = prmt(prmt(e1[0], e1[1], 0x0040u), prmt(e1[2], e1[3], 0x0040u), 0x5410u);
 }
 
 }  // namespace cq

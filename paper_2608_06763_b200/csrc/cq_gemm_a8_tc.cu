@@ -9,8 +9,8 @@
 //                the block accumulates into its own BN columns of one of two TMEM buffers
 //   warps 2..17  work warps, two jobs per K block, interleaved so the tensor core never waits on both:
 //                (a) decode block t: a signed carrier table r(k) per (row, group) (Eq. carrier, the
-//                    fp32 sequence of cq_common.cuh), then the carriers of the block (byte-permute look-ups
-//                    in register tables for B <= 4, one shared-memory look-up per weight otherwise) go
+//                    fp32 sequence of cq_common.cuh), then the carriers of the block by byte-permute look-ups
+//                    in it (B <= 4; wider codes are evaluated one by one) go
 //                    into the K-major swizzled INT8 operand tile in the operand order of cq_decode.cuh;
 //                (b) drain block t-1: tcgen05.ld of its int32 partials P_g, acc += s_g * P_g in fp32
 //                    registers (Eq. a8-output), which frees that TMEM buffer for block t+1.
@@ -263,55 +263,71 @@ gemm_a8_kernel(const __grid_constant__ CUtensorMap xmap, A8Params prm) {
                             sc[(rb * 16 + g) * GPT + gi] = __uint_as_float(p_lo.x & 0x7FFFFFFFu);
                             sc[(rb * 16 + g + 8) * GPT + gi] = __uint_as_float(p_hi.x & 0x7FFFFFFFu);
                         }
-                        if constexpr (B >= 3) {
-                            // signed carrier table: index = stored code u (reserved -> 0), entry sign(k) r(|k|).  With G = 128 the two warps of a row block
-                            // build eight rows each and meet at a 64-thread barrier.
-                            if constexpr (G == 128) named_barrier_sync(1 + rb, 64); else __syncwarp();
-                            auto build_row = [&](int row, uint32_t abbits) {
-                                const __half2 ab = as_h2(abbits);
-                                const float a = __low2float(ab), b = __high2float(ab);
-                                const float c = __fsub_rn(__fsub_rn(1.0f, a), b);
-                                int8_t *tr = tab + row * NCODE;
-                                if (B != 4 && tq == 0) tr[0] = 0;
-                                for (int i = tq; i <= Mx; i += 4) {
-                                    const float tt = sT[i];
-                                    const float q = __fmul_rn(tt, fmaf(tt, fmaf(tt, c, b), a));
-                                    int r = __float2int_rn(__fmul_rn(127.0f, q));
-                                    r = min(max(r, 0), 127);
-                                    tr[carrier_slot(B, i, false)] = (int8_t)r;
-                                    tr[carrier_slot(B, i, true)] = (int8_t)(-r);
-                                }
+                        // bytes 32 MI + 8 tq of the row: 16-byte chunk 2 MI + tq / 2, swizzled by the row
+                        auto place = [&](int MI) { return (((2 * MI + (tq >> 1)) ^ g) * 16) + (tq & 1) * 8; };
+                        if constexpr (B >= 5) {
+                            // wider codes: carriers evaluated one by one, row after row
+                            const bool fix = __any_sync(0xffffffffu, (p_lo.x | p_hi.x) >> 31);   // reserved pattern present
+                            auto eval = [&](auto fx) {
+                                constexpr bool FIX = decltype(fx)::value;
+                                static_for<2>([&](auto rc) {
+                                    constexpr int RR = decltype(rc)::value;
+                                    const CarrierPoly poly = carrier_poly(RR ? p_hi.y : p_lo.y);
+                                    static_for<CPGH / 2>([&](auto mc) {
+                                        constexpr int MI = 2 * JH + decltype(gc)::value * (CPGH / 2) + decltype(mc)::value;
+                                        uint2 v;
+                                        a8_row_eval<B, RR, MI, FIX>(w, poly, v.x, v.y);
+                                        *(uint2 *)((RR ? row_hi : row_lo) + place(MI)) = v;
+                                    });
+                                });
                             };
-                            if constexpr (G == 128) {
-                                if (JH == 0) build_row(g, p_lo.y); else build_row(g + 8, p_hi.y);
-                                named_barrier_sync(1 + rb, 64);
-                            } else {
-                                build_row(g, p_lo.y);
-                                build_row(g + 8, p_hi.y);
-                                __syncwarp();
+                            if (!fix) eval(std::false_type{}); else eval(std::true_type{});
+                        } else {
+                            if constexpr (B >= 3) {
+                                // signed carrier table: index = stored code u (reserved -> 0), entry sign(k) r(|k|).
+                                // With G = 128 the two warps of a row block build eight rows each and meet at a
+                                // 64-thread barrier.
+                                if constexpr (G == 128) named_barrier_sync(1 + rb, 64); else __syncwarp();
+                                auto build_row = [&](int row, uint32_t abbits) {
+                                    const __half2 ab = as_h2(abbits);
+                                    const float a = __low2float(ab), b = __high2float(ab);
+                                    int8_t *tr = tab + row * NCODE;
+                                    if (B != 4 && tq == 0) tr[0] = 0;
+                                    for (int i = tq; i <= Mx; i += 4) {
+                                        const int r = carrier_at(sT[i], a, b);
+                                        tr[carrier_slot(B, i, false)] = (int8_t)r;
+                                        tr[carrier_slot(B, i, true)] = (int8_t)(-r);
+                                    }
+                                };
+                                if constexpr (G == 128) {
+                                    if (JH == 0) build_row(g, p_lo.y); else build_row(g + 8, p_hi.y);
+                                    named_barrier_sync(1 + rb, 64);
+                                } else {
+                                    build_row(g, p_lo.y);
+                                    build_row(g + 8, p_hi.y);
+                                    __syncwarp();
+                                }
                             }
+                            // carriers of the group's 32-wide k blocks, straight into the MMA operand order
+                            // (a8_row_regs): lane tq holds bytes 8 tq .. 8 tq + 7 of block m for rows g and g + 8
+                            const int8_t *t_lo = tab + g * NCODE, *t_hi = tab + (g + 8) * NCODE;
+                            uint4 tab_lo = make_uint4(0, 0, 0, 0), tab_hi = make_uint4(0, 0, 0, 0);
+                            if constexpr (B == 4) {
+                                tab_lo = *reinterpret_cast<const uint4 *>(t_lo);
+                                tab_hi = *reinterpret_cast<const uint4 *>(t_hi);
+                            } else if constexpr (B == 3) {
+                                const uint2 v0 = *reinterpret_cast<const uint2 *>(t_lo), v1 = *reinterpret_cast<const uint2 *>(t_hi);
+                                tab_lo.x = v0.x; tab_lo.y = v0.y; tab_hi.x = v1.x; tab_hi.y = v1.y;
+                            }
+                            static_for<CPGH / 2>([&](auto mc) {
+                                constexpr int MI = 2 * JH + decltype(gc)::value * (CPGH / 2) + decltype(mc)::value;
+                                uint2 lo, hi;
+                                a8_row_regs<B, 0, MI>(w, tab_lo, lo.x, lo.y);
+                                a8_row_regs<B, 1, MI>(w, tab_hi, hi.x, hi.y);
+                                *(uint2 *)(row_lo + place(MI)) = lo;
+                                *(uint2 *)(row_hi + place(MI)) = hi;
+                            });
                         }
-                        // carriers of the group's 32-wide k blocks, straight into the MMA operand order
-                        // (a8_row_regs): lane tq holds bytes 8 tq .. 8 tq + 7 of block m for rows g and g + 8
-                        const int8_t *t_lo = tab + g * NCODE, *t_hi = tab + (g + 8) * NCODE;
-                        uint4 tab_lo = make_uint4(0, 0, 0, 0), tab_hi = make_uint4(0, 0, 0, 0);
-                        if constexpr (B == 4) {
-                            tab_lo = *reinterpret_cast<const uint4 *>(t_lo);
-                            tab_hi = *reinterpret_cast<const uint4 *>(t_hi);
-                        } else if constexpr (B == 3) {
-                            const uint2 v0 = *reinterpret_cast<const uint2 *>(t_lo), v1 = *reinterpret_cast<const uint2 *>(t_hi);
-                            tab_lo.x = v0.x; tab_lo.y = v0.y; tab_hi.x = v1.x; tab_hi.y = v1.y;
-                        }
-                        static_for<CPGH / 2>([&](auto mc) {
-                            constexpr int MI = 2 * JH + decltype(gc)::value * (CPGH / 2) + decltype(mc)::value;
-                            uint2 lo, hi;
-                            a8_row_regs<B, 0, MI>(w, tab_lo, t_lo, lo.x, lo.y);
-                            a8_row_regs<B, 1, MI>(w, tab_hi, t_hi, hi.x, hi.y);
-                            // bytes 32 MI + 8 tq of the row: 16-byte chunk 2 MI + tq / 2, swizzled by the row
-                            const int off = (((2 * MI + (tq >> 1)) ^ g) * 16) + (tq & 1) * 8;
-                            *(uint2 *)(row_lo + off) = lo;
-                            *(uint2 *)(row_hi + off) = hi;
-                        });
                     });
                 };
                 if (jh == 0) do_half(std::integral_constant<int, 0>{}); else do_half(std::integral_constant<int, 1>{});

@@ -28,8 +28,8 @@
 // m16n8k16 MMA (fp16 in, fp32 accumulate), the weights' loads landing directly in its A fragment.
 //
 // Dynamic A8 uses the INT8 m16n8k32 MMA on signed carriers (Eq. carrier) taken from a per-(row, group)
-// table indexed by the stored code -- in registers and read with byte permutes for B <= 4, in shared
-// memory otherwise (a8_row_regs in cq_decode.cuh) -- int32 group partials, fp32 rescale (Eq. a8-output).
+// table indexed by the stored code, in registers and read with byte permutes (B <= 4: a8_row_regs in cq_decode.cuh), or
+// evaluated code by code (wider: a8_row_eval); int32 group partials, fp32 rescale (Eq. a8-output).
 #include <cstdlib>
 
 #include "cq_common.cuh"
@@ -54,7 +54,7 @@ constexpr int MAX_SUB = 16;    // K tiles staged at a time (bounds shared memory
 __host__ __device__ constexpr int gemv_rows(int NT, int MODE) { return MODE == 2 ? NT : 8 * NT; }
 // most shared memory the staged activations (and the Dynamic-A8 carrier tables) of a variant can take
 __host__ __device__ constexpr int gemv_x_bytes_max(int B, int NT, int MODE) {
-    return MODE == 1 ? gemv_rows(NT, MODE) * (MAX_SUB * TILE + XS_PAD8) + (B >= 3 ? 8 * 16 * carrier_table_stride(B) : 0)
+    return MODE == 1 ? gemv_rows(NT, MODE) * (MAX_SUB * TILE + XS_PAD8) + (B == 3 || B == 4 ? 8 * 16 * carrier_table_stride(B) : 0)
                      : gemv_rows(NT, MODE) * (MAX_SUB * TILE + 2 * XS_PAD) * 2;
 }
 __host__ __device__ constexpr int gemv_smem_budget(int ctas) { return (227 * 1024) / ctas - 2048; }   // dynamic shared memory of a CTA
@@ -238,9 +238,15 @@ __device__ __forceinline__ void group_a8(const TileRegs<B, TILE / G> &r, const i
     constexpr int L = B == 1 ? 1 : (1 << (B - 1));
     constexpr int NE = carrier_table_stride(B);   // bytes from one row's table to the next
     const uint2 p_lo = r.prm[0][GI], p_hi = r.prm[1][GI];
+    CarrierPoly poly_lo{}, poly_hi{};
+    bool fix = false;
+    if constexpr (B >= 5) {
+        poly_lo = carrier_poly(p_lo.y); poly_hi = carrier_poly(p_hi.y);
+        fix = __any_sync(0xffffffffu, (p_lo.x | p_hi.x) >> 31);
+    }
     uint4 tab_lo = make_uint4(0, 0, 0, 0), tab_hi = make_uint4(0, 0, 0, 0);
     const int8_t *trow_lo = ctab + g * NE, *trow_hi = ctab + (g + 8) * NE;
-    if constexpr (B >= 3) {  // lane (g, t) fills magnitudes i = t mod 4 of rows g and g + 8
+    if constexpr (B == 3 || B == 4) {  // lane (g, t) fills magnitudes i = t mod 4 of rows g and g + 8
         __syncwarp();
         const __half2 ab_lo = as_h2(p_lo.y), ab_hi = as_h2(p_hi.y);
         const float a_lo = __low2float(ab_lo), b_lo = __high2float(ab_lo);
@@ -268,8 +274,16 @@ __device__ __forceinline__ void group_a8(const TileRegs<B, TILE / G> &r, const i
     static_for<MPG>([&](auto mc) {
         constexpr int mi = decltype(mc)::value, MI = GI * MPG + mi;
         uint32_t A[4];
-        a8_row_regs<B, 0, MI>(r.w, tab_lo, trow_lo, A[0], A[2]);
-        a8_row_regs<B, 1, MI>(r.w, tab_hi, trow_hi, A[1], A[3]);
+        if constexpr (B <= 4) {
+            a8_row_regs<B, 0, MI>(r.w, tab_lo, A[0], A[2]);
+            a8_row_regs<B, 1, MI>(r.w, tab_hi, A[1], A[3]);
+        } else if (!fix) {
+            a8_row_eval<B, 0, MI, false>(r.w, poly_lo, A[0], A[2]);
+            a8_row_eval<B, 1, MI, false>(r.w, poly_hi, A[1], A[3]);
+        } else {
+            a8_row_eval<B, 0, MI, true>(r.w, poly_lo, A[0], A[2]);
+            a8_row_eval<B, 1, MI, true>(r.w, poly_hi, A[1], A[3]);
+        }
 #pragma unroll
         for (int tb = 0; tb < NT; ++tb) {
             const uint2 bf = *reinterpret_cast<const uint2 *>(xs + xo[tb] + 32 * MI);
@@ -589,7 +603,7 @@ gemv_kernel(const uint8_t *__restrict__ layout, Dims d, const uint16_t *__restri
     __shared__ float s_inv[16];
     __shared__ unsigned s_max[16];
     __shared__ int s_last, s_dead;
-    __shared__ float s_t[MODE == 1 && B >= 3 ? 128 : 1];   // Dynamic A8: t_i = i / M of the carrier tables
+    __shared__ float s_t[MODE == 1 && (B == 3 || B == 4) ? 8 : 1];   // Dynamic A8: t_i = i / M of the carrier tables
     __shared__ __align__(16) uint8_t s_w4[MODE != 1 && B == 4 ? GEMV_WARPS * 256 : 16];   // W4, model dtype: level tables of a warp's 16 rows
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
@@ -609,7 +623,7 @@ gemv_kernel(const uint8_t *__restrict__ layout, Dims d, const uint16_t *__restri
     if (threadIdx.x < 32) tc::fence_barrier_init();
     if (threadIdx.x == 0) s_dead = 0;
     if (threadIdx.x < 16) { s_max[threadIdx.x] = 0; s_inv[threadIdx.x] = 1.0f; }
-    if constexpr (MODE == 1 && B >= 3) {
+    if constexpr (MODE == 1 && (B == 3 || B == 4)) {
         if (threadIdx.x < L) s_t[threadIdx.x] = __fdiv_rn((float)threadIdx.x, (float)(L - 1));
     }
     __syncthreads();
@@ -649,7 +663,7 @@ gemv_kernel(const uint8_t *__restrict__ layout, Dims d, const uint16_t *__restri
         ctab = reinterpret_cast<int8_t *>(s_w4) + warp * 256;
         w4_t0 = (float)(2 * t) / 7.0f; w4_t1 = (float)(2 * t + 1) / 7.0f;
     }
-    if constexpr (MODE == 1 && B >= 3) ctab = reinterpret_cast<int8_t *>(smem) + M * (MAX_SUB * TILE + XS_PAD8) + warp * 16 * carrier_table_stride(B);
+    if constexpr (MODE == 1 && (B == 3 || B == 4)) ctab = reinterpret_cast<int8_t *>(smem) + M * (MAX_SUB * TILE + XS_PAD8) + warp * 16 * carrier_table_stride(B);
 
     int st = 0, prev_st = 0;            // ring stage of the next tile (and of the one before it)
     uint32_t ph = 0, prev_ph = 0;       // and the parity its "full" barrier completes with
@@ -963,7 +977,7 @@ cudaError_t launch_one(const void *layout, const Dims &d, const uint16_t *x, con
     if (sub64 > MAX_SUB) sub64 = MAX_SUB;
     const int sub_tiles = (int)sub64;
     const int XS = sub_tiles * TILE + (B == 3 || B == 4 ? 2 * XS_PAD : XS_PAD);
-    size_t xbytes = MODE != 1 ? (size_t)M * XS * 2 : (size_t)M * (MAX_SUB * TILE + XS_PAD8) + (B >= 3 ? 8 * 16 * carrier_table_stride(B) : 0);
+    size_t xbytes = MODE != 1 ? (size_t)M * XS * 2 : (size_t)M * (MAX_SUB * TILE + XS_PAD8) + (B == 3 || B == 4 ? 8 * 16 * carrier_table_stride(B) : 0);
     const uint32_t ring_off = (uint32_t)((xbytes + 127) / 128 * 128);
     constexpr int OCC = gemv_occ(B, G, NT, MODE);
     int nstage = 0;

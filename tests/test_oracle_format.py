@@ -229,3 +229,15 @@ def test_half_conversion_matches_ieee_binary16():
         ref = probes.astype(np.float16).view(np.uint16)
     mine = np.array([L.cqo_double_to_half(float(v)) for v in probes], dtype=np.uint16)
     assert np.array_equal(mine, ref), np.flatnonzero(mine != ref)[:10]
+
+
+def test_quotient_as_two_products():
+    # the INT8 kernels form t = i / M (M of five to eight bits) as fma(i, r, i r'), r + r' = 1 / M in two fp32 parts: the
+    # correctly rounded quotient for every i (the products of a 7-bit i are exact in fp64)
+    for B in (5, 6, 7, 8):
+        M = (1 << (B - 1)) - 1
+        i = np.arange(M + 1, dtype=np.float32)
+        r = np.float32(1) / np.float32(M)
+        r2 = np.float32(1.0 / M - float(r))
+        t = (i.astype(np.float64) * float(r) + (i * r2).astype(np.float64)).astype(np.float32)
+        assert np.array_equal(t, i / np.float32(M))
