@@ -214,7 +214,7 @@ def cq_gemm_routed(experts, x: torch.Tensor, route_token: torch.Tensor, expert_o
     assert route_token.numel() == R
     need = lib().cq_routed_workspace_bytes(p0.B, p0.G, E, off, p0.N, p0.K, mode)
     if workspace is None:
-        workspace = torch.zeros(max(need, 512), dtype=torch.uint8, device=x.device)
+        workspace = torch.empty(max(need, 512), dtype=torch.uint8, device=x.device)   # the call zeroes what it counts in
     y = torch.empty((R, p0.N), dtype=x.dtype, device=x.device)
     _check(lib().cq_gemm_routed(ptrs, E, p0.B, p0.G, _ptr(x), _ptr(route_token), off, _ptr(y), x.shape[0], p0.N, p0.K, mode,
                                 1 if x.dtype == torch.float16 else 0, _ptr(workspace), workspace.numel(), _stream()),

@@ -232,26 +232,69 @@ int cq_mlp_swiglu(const void *layout_gate_up, int B_gu, int G_gu, const void *la
     return wrap(e);
 }
 
-// Workspace of the routed product: [gathered rows: R x K model-dtype values][the largest per-matrix cq_gemm workspace].
+// Routed product.  The groups (matrices with routes) are sorted into classes of token tiles, and a class of several
+// groups is one launch: up to 16 rows the small-M kernel, above it the GEMM, the token tiles up to 128 together (its time is
+// the decode of the weights there, not the tokens) and 256 and 512 by themselves; Dynamic A8 keeps one class per token
+// tile, whose drain grows with the tile.  A class of one group is an ordinary product, which may share its tiles along K.
+// Sixteen matrices of 2816 x 2048 (W4 G64, 384 routes): one after another 192 us, most of it launches that leave SMs idle; 61 us so.
+// Workspace: [status][gathered rows: R x K][Dynamic A8: INT8 carrier of all rows, row scales][small-M groups: counters and
+// partial sums][the largest workspace of an ordinary product].
+struct RoutedPlan {
+    size_t xg_off, x8_off, dx_off, ctr_off, part_off, sub_off, total;
+    int P;           // CTAs of a small-M group
+    int n_small;     // groups of at most 16 rows
+};
 static bool routed_offsets_ok(const int64_t *off, int E, int64_t R) {
     if (!off || off[0] != 0 || off[E] != R) return false;
     for (int e = 0; e < E; ++e) if (off[e + 1] < off[e]) return false;
     return true;
 }
-static size_t routed_sub_bytes(const Dims &d, const int64_t *off, int E, int mode) {
-    size_t need = 0;
-    for (int e = 0; e < E; ++e) {
-        const int64_t m = off[e + 1] - off[e];
-        if (m > 0) { const size_t t = plan_workspace(d, m, mode).total; if (t > need) need = t; }
+static int routed_class(const Dims &d, int64_t m, int mode) {   // 0: small M; else a token tile
+    if (m <= 16) return 0;
+    if (mode == CQ_DYN_A8) return gemm_a8_token_tile(d, m);
+    const int t = gemm_tc_token_tile(m);
+    return t < 128 ? 128 : t;
+}
+static const int ROUTED_CLASSES[6] = {0, 32, 64, 128, 256, 512};   // every value of routed_class
+static RoutedPlan plan_routed(const Dims &d, const int64_t *off, int E, int mode) {
+    RoutedPlan p{};
+    const int64_t R = off[E];
+    size_t sub = 0, o = 256;
+    for (int cls : ROUTED_CLASSES) {
+        int n = 0;
+        int64_t last = 0;
+        for (int e = 0; e < E; ++e) {
+            const int64_t m = off[e + 1] - off[e];
+            if (m > 0 && routed_class(d, m, mode) == cls) { ++n; last = m; }
+        }
+        if (cls == 0) p.n_small = n;
+        if (n % MAX_GROUPS == 1) { const size_t t = plan_workspace(d, last, mode).total; if (t > sub) sub = t; }   // launched by itself
     }
-    return need;
+    p.xg_off = o; o += align_up((size_t)R * d.K * 2, 256);
+    if (mode == CQ_DYN_A8) {
+        p.x8_off = o; o += align_up((size_t)R * d.KT * TILE, 256);
+        p.dx_off = o; o += align_up((size_t)R * 4, 256);
+    }
+    if (p.n_small > 1) {
+        // the groups share the places of the whole GPU; a run of fewer than four tiles is mostly overhead
+        const int64_t T = (int64_t)d.NB * d.KT, places = gemv_plan(d, 16, mode).ctas;
+        int64_t P = places / p.n_small;
+        if (P > T / 4) P = T / 4;
+        p.P = (int)(P < 1 ? 1 : P);
+        const size_t n = p.n_small < MAX_GROUPS ? p.n_small : MAX_GROUPS;
+        p.ctr_off = o; o += align_up(n * d.NB * 4, 256);
+        p.part_off = o; o += align_up(n * p.P * 2 * 16 * TILE * 4, 256);
+    }
+    p.sub_off = o;
+    p.total = o + sub;
+    return p;
 }
 
 size_t cq_routed_workspace_bytes(int B, int G, int E, const int64_t *expert_offset_host, int64_t N, int64_t K, int mode) {
     if (check_format(B, G, N, K) != CQ_OK || E <= 0 || !expert_offset_host || (mode != CQ_MODEL_DTYPE && mode != CQ_DYN_A8)) return 0;
     const int64_t R = expert_offset_host[E];
     if (R <= 0 || !routed_offsets_ok(expert_offset_host, E, R)) return 0;
-    return align_up((size_t)R * K * 2, 256) + routed_sub_bytes(make_dims(B, G, N, K), expert_offset_host, E, mode);
+    return plan_routed(make_dims(B, G, N, K), expert_offset_host, E, mode).total;
 }
 
 int cq_gemm_routed(const void *const *layouts_host, int E, int B, int G, const uint16_t *x, const int32_t *route_token,
@@ -270,18 +313,59 @@ int cq_gemm_routed(const void *const *layouts_host, int E, int B, int G, const u
     }
     if (misaligned(x) || misaligned(y_routes) || misaligned(workspace) || (K * 2) % 16 != 0 || (N * 2) % 16 != 0) return CQ_ERR_ALIGNMENT;
     const Dims d = make_dims(B, G, N, K);
-    const size_t xg_bytes = align_up((size_t)R * K * 2, 256), sub = routed_sub_bytes(d, expert_offset_host, E, mode);
-    if (workspace_bytes < xg_bytes + sub) return CQ_ERR_WORKSPACE;
+    const RoutedPlan plan = plan_routed(d, expert_offset_host, E, mode);
+    if (workspace_bytes < plan.total) return CQ_ERR_WORKSPACE;
     st = check_arch();
     if (st != CQ_OK) return st;
-    uint16_t *xg = reinterpret_cast<uint16_t *>(workspace);
-    cudaError_t e0 = launch_gather_rows(x, route_token, xg, R, T, K, (cudaStream_t)stream);
-    if (e0 != cudaSuccess) return wrap(e0);
-    uint8_t *sub_ws = (uint8_t *)workspace + xg_bytes;
-    for (int e = 0; e < E; ++e) {   // one dispatch per matrix that has routes: its decoded tiles serve all of them
-        const int64_t r0 = expert_offset_host[e], m = expert_offset_host[e + 1] - r0;
-        if (m == 0) continue;
-        st = gemm_any(layouts_host[e], B, G, xg + r0 * K, y_routes + r0 * N, m, N, K, mode, act_f16 != 0, sub_ws, sub, stream);
+    cudaStream_t s = (cudaStream_t)stream;
+    uint8_t *ws = (uint8_t *)workspace;
+    int *status = reinterpret_cast<int *>(ws);
+    uint16_t *xg = reinterpret_cast<uint16_t *>(ws + plan.xg_off);
+    int8_t *xq = reinterpret_cast<int8_t *>(ws + plan.x8_off);
+    float *dxs = reinterpret_cast<float *>(ws + plan.dx_off);
+    const bool f16 = act_f16 != 0;
+    // the gather also zeroes the status word and the groups' arrival counters: which words these are changes with the routing
+    cudaError_t err = launch_gather_rows(x, route_token, xg, R, T, K, status, reinterpret_cast<int *>(ws + plan.ctr_off),
+                                         (int64_t)(plan.part_off - plan.ctr_off) / 4, s);
+    if (err != cudaSuccess) return wrap(err);
+    bool quantised = false;
+    auto flush = [&](const GroupTable &t, int cls, int64_t max_rows) -> int {   // one class, up to MAX_GROUPS groups
+        if (t.n == 0) return CQ_OK;
+        if (t.n == 1) {
+            const Group &g = t.g[0];
+            const cudaError_t e = cudaMemsetAsync(ws + plan.sub_off, 0, 256 + plan_workspace(d, g.rows, mode).counters_bytes, s);
+            if (e != cudaSuccess) return wrap(e);
+            return gemm_any(g.layout, B, G, xg + (int64_t)g.row0 * K, y_routes + (int64_t)g.row0 * N, g.rows, N, K, mode, f16,
+                            ws + plan.sub_off, plan.total - plan.sub_off, stream);
+        }
+        if (mode == CQ_DYN_A8 && !quantised) {
+            const cudaError_t e = launch_quantize_a8(xg, R, K, xq, (int64_t)d.KT * TILE, dxs, B != 4, f16, s);
+            if (e != cudaSuccess) return wrap(e);
+            quantised = true;
+        }
+        if (cls == 0) {
+            // every launch leaves the arrival counters at zero
+            return wrap(launch_gemv_groups(t, d, xg, xq, dxs, y_routes, mode, f16, plan.P, reinterpret_cast<float *>(ws + plan.part_off),
+                                           reinterpret_cast<int *>(ws + plan.ctr_off), status, s));
+        }
+        if (mode == CQ_MODEL_DTYPE) return wrap(launch_gemm_tc_groups(t, d, xg, y_routes, R, max_rows, f16, status, s));
+        return wrap(launch_gemm_a8_groups(t, d, xq, dxs, y_routes, R, max_rows, f16, status, s));
+    };
+    for (int cls : ROUTED_CLASSES) {
+        GroupTable t{};
+        int64_t max_rows = 0;
+        for (int e = 0; e < E; ++e) {
+            const int64_t r0 = expert_offset_host[e], m = expert_offset_host[e + 1] - r0;
+            if (m == 0 || routed_class(d, m, mode) != cls) continue;
+            t.g[t.n++] = {layouts_host[e], (int)r0, (int)m, 0};
+            if (m > max_rows) max_rows = m;
+            if (t.n == MAX_GROUPS) {
+                st = flush(t, cls, max_rows);
+                if (st != CQ_OK) return st;
+                t.n = 0; max_rows = 0;
+            }
+        }
+        st = flush(t, cls, max_rows);
         if (st != CQ_OK) return st;
     }
     return CQ_OK;

@@ -77,12 +77,11 @@ constexpr int A8_SRING = 8;      // ring of per-block scale snapshots for the dr
 constexpr int A8_A_STAGE_BYTES = 128 * 128;
 
 struct A8Params {
-    const uint8_t *layout;
     const float *dx;
     uint16_t *y;
     int *status;
     Dims d;
-    int M;
+    GroupTable groups;    // an ordinary product is one group; a routed one (whole tiles only) has several
     int raw_stage_bytes;
     float *partial;       // sliced tiles: fp32 partial tiles [shared tile][slice][BN][128] (before the d_x / 127 factor)
     int *counters;        // sliced tiles: arrival counters, one per output tile
@@ -97,7 +96,7 @@ __device__ __forceinline__ void named_barrier_sync(int id, int threads) {
 
 template <int B, int G, int BN>
 __global__ void __launch_bounds__(A8_THREADS, 1)
-gemm_a8_kernel(const __grid_constant__ CUtensorMap xmap, A8Params prm) {
+gemm_a8_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ A8Params prm) {
     constexpr int GPT = TILE / G;                 // groups per 128-wide block
     constexpr int MPG = 4 / GPT;                  // K = 32 MMAs per group
     constexpr int NCODE = carrier_table_stride(B);   // bytes per table row (2^B entries indexed by the stored code u, padded)
@@ -124,18 +123,20 @@ gemm_a8_kernel(const __grid_constant__ CUtensorMap xmap, A8Params prm) {
     const Dims &d = prm.d;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // This CTA's tile and, for a tile of the last round, its slice z of nz: the layout tiles [kt0, kt0 + KT)
-    int kt0, KT, p_nb, p_mt;
+    int kt0, KT, p_nb, p_mt, grp = 0;
     {
         const int bid = (int)blockIdx.x;
         const int nz = bid < prm.t_full ? 1 : prm.slices;
         const int tile_id = bid < prm.t_full ? bid : prm.t_full + (bid - prm.t_full) / prm.slices;
         const int z = bid < prm.t_full ? 0 : (bid - prm.t_full) % prm.slices;
-        p_mt = tile_id / d.NB; p_nb = tile_id - p_mt * d.NB;
+        while (grp + 1 < prm.groups.n && tile_id >= prm.groups.g[grp + 1].unit0) ++grp;
+        const int in_group = tile_id - prm.groups.g[grp].unit0;
+        p_mt = in_group / d.NB; p_nb = in_group - p_mt * d.NB;
         kt0 = (int)(((int64_t)d.KT * z) / nz);
         KT = (int)(((int64_t)d.KT * (z + 1)) / nz) - kt0;
         if (threadIdx.x == 0) {   // what only the epilogue needs is parked in shared memory (set up below, before the barrier)
             uint32_t *park = reinterpret_cast<uint32_t *>(acc_empty + 2);
-            park[4] = (uint32_t)nz; park[5] = (uint32_t)z; park[6] = (uint32_t)tile_id; park[7] = (uint32_t)p_nb; park[8] = (uint32_t)p_mt;
+            park[4] = (uint32_t)nz; park[5] = (uint32_t)z; park[6] = (uint32_t)tile_id; park[7] = (uint32_t)p_nb; park[8] = (uint32_t)p_mt; park[9] = (uint32_t)grp;
         }
     }
     const int nb = p_nb, mt = p_mt;   // the producer's coordinates
@@ -151,7 +152,7 @@ gemm_a8_kernel(const __grid_constant__ CUtensorMap xmap, A8Params prm) {
         fence_barrier_init();
         tmem_slot[2] = 0;   // the work warps' "a wait gave up" flag
         tmem_slot[3] = prm.f16 ? 1u : 0u;   // the output dtype, parked in shared memory: a register held across the main loop is one too many
-        // tmem_slot[4 .. 8]: slice count, slice, tile, row block and token tile of this CTA (written above)
+        // tmem_slot[4 .. 9]: slice count, slice, tile, row block, token tile and group of this CTA (written above)
     }
     if (threadIdx.x < 128) sT[threadIdx.x] = __fdiv_rn((float)threadIdx.x, (float)Mx);  // the pinned t = i / M
     if (warp == 1) {
@@ -173,13 +174,13 @@ gemm_a8_kernel(const __grid_constant__ CUtensorMap xmap, A8Params prm) {
                 if (t >= A8_STAGES) ok = mbar_wait(&st_empty[s], ((t / A8_STAGES) - 1) & 1, prm.status, 12);
                 if (!ok) break;
                 mbar_arrive_expect_tx(&b_full[s], B_STAGE_BYTES);
-                tma_load_2d(sB + s * B_STAGE_BYTES, &xmap, &b_full[s], (kt0 + t) * 128, mt * BN);
+                tma_load_2d(sB + s * B_STAGE_BYTES, &xmap, &b_full[s], (kt0 + t) * 128, prm.groups.g[grp].row0 + mt * BN);
             }
         }
     } else if (warp == 2 + A8_WORK_WARPS) {
         // ===== producer of the raw layout tiles (its own warp: a wait for the work warps never delays an activation tile)
         if (lane == 0) {
-            const uint8_t *tiles = prm.layout + ((size_t)nb * d.KT + kt0) * (size_t)d.tile_bytes;
+            const uint8_t *tiles = (const uint8_t *)prm.groups.g[grp].layout + ((size_t)nb * d.KT + kt0) * (size_t)d.tile_bytes;
             bool ok = true;
             for (int t = 0; t < KT && ok; ++t) {
                 const int rs = t % A8_RAW_STAGES;
@@ -363,6 +364,7 @@ gemm_a8_kernel(const __grid_constant__ CUtensorMap xmap, A8Params prm) {
             const int e_mt = (int)*reinterpret_cast<volatile uint32_t *>(tmem_slot + 8);
             const int64_t n = (int64_t)e_nb * TILE + drow;
             const int e_nz = (int)*reinterpret_cast<volatile uint32_t *>(tmem_slot + 4);
+            const Group &e_gr = prm.groups.g[*reinterpret_cast<volatile uint32_t *>(tmem_slot + 9)];
             if (n < d.N || e_nz > 1) {   // partial sums of padding channels are written too (zeros), never read back as y
                 // the output dtype is decided once, outside the loop over the 64 accumulators (a select inside it
                 // costs the registers this kernel does not have)
@@ -375,11 +377,11 @@ gemm_a8_kernel(const __grid_constant__ CUtensorMap xmap, A8Params prm) {
 #pragma unroll
                     for (int i = 0; i < QCOLS; ++i) {
                         const int64_t m = (int64_t)e_mt * BN + cq4 * QCOLS + i;
-                        if (m < prm.M) {
+                        if (m < e_gr.rows) {
                             if (e_nz == 1) {
-                                const float v = acc[i] * (prm.dx[m] * (1.0f / 127.0f));
+                                const float v = acc[i] * (prm.dx[e_gr.row0 + m] * (1.0f / 127.0f));
                                 if constexpr (STAGED) reinterpret_cast<uint16_t *>(sB)[(cq4 * QCOLS + i) * TILE + drow] = float_to_act(v, F16);
-                                else prm.y[m * d.N + n] = float_to_act(v, F16);
+                                else prm.y[(e_gr.row0 + m) * d.N + n] = float_to_act(v, F16);
                             } else {
                                 pslot[(size_t)(cq4 * QCOLS + i) * TILE] = acc[i];
                             }
@@ -406,10 +408,11 @@ gemm_a8_kernel(const __grid_constant__ CUtensorMap xmap, A8Params prm) {
         const int64_t m0 = (int64_t)*reinterpret_cast<volatile uint32_t *>(tmem_slot + 8) * BN;
         const int64_t n0 = (int64_t)*reinterpret_cast<volatile uint32_t *>(tmem_slot + 7) * TILE;
         const uint16_t *stage = reinterpret_cast<const uint16_t *>(sB);
+        const Group &gr = prm.groups.g[*reinterpret_cast<volatile uint32_t *>(tmem_slot + 9)];
         for (int c = threadIdx.x; c < BN * (TILE / 8); c += A8_THREADS) {
             const int tok = c / (TILE / 8), part = c % (TILE / 8);
-            if (m0 + tok < prm.M && n0 + part * 8 < d.N)
-                *reinterpret_cast<uint4 *>(prm.y + (m0 + tok) * d.N + n0 + part * 8) = *reinterpret_cast<const uint4 *>(stage + tok * TILE + part * 8);
+            if (m0 + tok < gr.rows && n0 + part * 8 < d.N)
+                *reinterpret_cast<uint4 *>(prm.y + (gr.row0 + m0 + tok) * d.N + n0 + part * 8) = *reinterpret_cast<const uint4 *>(stage + tok * TILE + part * 8);
         }
     }
     if (*reinterpret_cast<volatile uint32_t *>(tmem_slot + 4) > 1) {
@@ -432,7 +435,7 @@ gemm_a8_kernel(const __grid_constant__ CUtensorMap xmap, A8Params prm) {
             const float4 *src = reinterpret_cast<const float4 *>(prm.partial + (size_t)(tile_id - prm.t_full) * prm.slices * (size_t)(BN * TILE));
             for (int qd = threadIdx.x; qd < QUADS; qd += A8_THREADS) {
                 const int64_t m = (int64_t)mt * BN + qd / (TILE / 4), n = (int64_t)nb * TILE + (qd % (TILE / 4)) * 4;
-                if (m >= prm.M) continue;
+                if (m >= prm.groups.g[0].rows) continue;   // slices: one group
                 float4 v[8];
 #pragma unroll
                 for (int q = 0; q < 8; ++q)
@@ -452,9 +455,8 @@ gemm_a8_kernel(const __grid_constant__ CUtensorMap xmap, A8Params prm) {
 }
 
 template <int B, int G, int BN>
-cudaError_t launch_a8(const void *layout, const Dims &d, const int8_t *x8, int64_t pitch, const float *dx, uint16_t *y,
+cudaError_t launch_a8(const GroupTable &groups, const Dims &d, const int8_t *x8, int64_t pitch, const float *dx, uint16_t *y,
                       int64_t M, int *status, float *partial, int *counters, bool act_f16, cudaStream_t st) {
-    constexpr int GPT = TILE / G;
     EncodeTiledFn enc = encode_tiled();
     if (!enc) return cudaErrorNotSupported;
     CUtensorMap xmap;
@@ -467,7 +469,7 @@ cudaError_t launch_a8(const void *layout, const Dims &d, const int8_t *x8, int64
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return cudaErrorInvalidValue;
     A8Params p;
-    p.layout = (const uint8_t *)layout; p.dx = dx; p.y = y; p.status = status; p.d = d; p.M = (int)M;
+    p.groups = groups; p.dx = dx; p.y = y; p.status = status; p.d = d;
     p.partial = partial; p.counters = counters; p.f16 = act_f16;
     p.raw_stage_bytes = (d.tile_bytes + 1023) / 1024 * 1024;
     static_assert(A8_STAGES == 2 && A8_A_STAGE_BYTES == 128 * 128 && A8_SRING == 8, "a8_fixed_smem spells these out");
@@ -477,31 +479,53 @@ cudaError_t launch_a8(const void *layout, const Dims &d, const int8_t *x8, int64
     static std::atomic<uint64_t> attr_done{0};   // per kernel instantiation: the devices it has been set on
     cudaError_t ea = ensure_func_attr(kern, attr_done, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
     if (ea != cudaSuccess) return ea;
-    const A8Plan plan = gemm_a8_plan(d, M);
+    A8Plan plan;
+    if (counters) {   // an ordinary product; the groups of a routed one are computed in whole tiles and bring no workspace
+        plan = gemm_a8_plan(d, M);
+    } else {
+        int units = 0;
+        for (int i = 0; i < groups.n; ++i) { p.groups.g[i].unit0 = units; units += d.NB * ((groups.g[i].rows + BN - 1) / BN); }
+        plan = {BN, 0, 1, units, units};
+    }
     if (plan.bn != BN) return cudaErrorInvalidConfiguration;
     p.t_full = (int)plan.t_full; p.slices = plan.slices;
     kern<<<dim3((unsigned)plan.ctas), A8_THREADS, smem, st>>>(xmap, p);
     return cudaGetLastError();
 }
 
+// M: rows of x8; tile_m: the rows whose token tile is taken (of an ordinary product, M)
 // token tile: two accumulator buffers of GPT x BN columns must fit the 512 TMEM columns
 template <int B, int G>
-cudaError_t launch_a8_bn(const void *layout, const Dims &d, const int8_t *x8, int64_t pitch, const float *dx, uint16_t *y,
-                         int64_t M, int *status, float *partial, int *counters, bool act_f16, cudaStream_t st) {
+cudaError_t launch_a8_bn(const GroupTable &groups, const Dims &d, const int8_t *x8, int64_t pitch, const float *dx, uint16_t *y,
+                         int64_t M, int64_t tile_m, int *status, float *partial, int *counters, bool act_f16, cudaStream_t st) {
     constexpr int BMAX = 256 / (TILE / G);
-    const int bn = gemm_a8_token_tile(d, M);
-    if constexpr (BMAX >= 256) if (bn == 256) return launch_a8<B, G, 256>(layout, d, x8, pitch, dx, y, M, status, partial, counters, act_f16, st);
-    if constexpr (BMAX >= 128) if (bn == 128) return launch_a8<B, G, 128>(layout, d, x8, pitch, dx, y, M, status, partial, counters, act_f16, st);
-    return launch_a8<B, G, 64>(layout, d, x8, pitch, dx, y, M, status, partial, counters, act_f16, st);
+    const int bn = gemm_a8_token_tile(d, tile_m);
+    if constexpr (BMAX >= 256) if (bn == 256) return launch_a8<B, G, 256>(groups, d, x8, pitch, dx, y, M, status, partial, counters, act_f16, st);
+    if constexpr (BMAX >= 128) if (bn == 128) return launch_a8<B, G, 128>(groups, d, x8, pitch, dx, y, M, status, partial, counters, act_f16, st);
+    return launch_a8<B, G, 64>(groups, d, x8, pitch, dx, y, M, status, partial, counters, act_f16, st);
 }
 
 template <int B>
-cudaError_t launch_a8_b(const void *layout, const Dims &d, const int8_t *x8, int64_t pitch, const float *dx, uint16_t *y,
-                        int64_t M, int *status, float *partial, int *counters, bool act_f16, cudaStream_t st) {
+cudaError_t launch_a8_b(const GroupTable &groups, const Dims &d, const int8_t *x8, int64_t pitch, const float *dx, uint16_t *y,
+                        int64_t M, int64_t tile_m, int *status, float *partial, int *counters, bool act_f16, cudaStream_t st) {
     switch (d.G) {
-        case 32: return launch_a8_bn<B, 32>(layout, d, x8, pitch, dx, y, M, status, partial, counters, act_f16, st);
-        case 64: return launch_a8_bn<B, 64>(layout, d, x8, pitch, dx, y, M, status, partial, counters, act_f16, st);
-        default: return launch_a8_bn<B, 128>(layout, d, x8, pitch, dx, y, M, status, partial, counters, act_f16, st);
+        case 32: return launch_a8_bn<B, 32>(groups, d, x8, pitch, dx, y, M, tile_m, status, partial, counters, act_f16, st);
+        case 64: return launch_a8_bn<B, 64>(groups, d, x8, pitch, dx, y, M, tile_m, status, partial, counters, act_f16, st);
+        default: return launch_a8_bn<B, 128>(groups, d, x8, pitch, dx, y, M, tile_m, status, partial, counters, act_f16, st);
+    }
+}
+
+cudaError_t launch_a8_any(const GroupTable &groups, const Dims &d, const int8_t *x8, int64_t pitch, const float *dx, uint16_t *y,
+                          int64_t M, int64_t tile_m, int *status, float *partial, int *counters, bool act_f16, cudaStream_t st) {
+    switch (d.B) {
+        case 1: return launch_a8_b<1>(groups, d, x8, pitch, dx, y, M, tile_m, status, partial, counters, act_f16, st);
+        case 2: return launch_a8_b<2>(groups, d, x8, pitch, dx, y, M, tile_m, status, partial, counters, act_f16, st);
+        case 3: return launch_a8_b<3>(groups, d, x8, pitch, dx, y, M, tile_m, status, partial, counters, act_f16, st);
+        case 4: return launch_a8_b<4>(groups, d, x8, pitch, dx, y, M, tile_m, status, partial, counters, act_f16, st);
+        case 5: return launch_a8_b<5>(groups, d, x8, pitch, dx, y, M, tile_m, status, partial, counters, act_f16, st);
+        case 6: return launch_a8_b<6>(groups, d, x8, pitch, dx, y, M, tile_m, status, partial, counters, act_f16, st);
+        case 7: return launch_a8_b<7>(groups, d, x8, pitch, dx, y, M, tile_m, status, partial, counters, act_f16, st);
+        default: return launch_a8_b<8>(groups, d, x8, pitch, dx, y, M, tile_m, status, partial, counters, act_f16, st);
     }
 }
 
@@ -520,16 +544,15 @@ cudaError_t launch_gemm_a8_tc(const void *layout, const Dims &d, const uint16_t 
         cudaError_t e = launch_quantize_a8(x, M, d.K, xq, pitch, dxs, d.B != 4, act_f16, st);
         if (e != cudaSuccess) return e;
     }
-    switch (d.B) {
-        case 1: return launch_a8_b<1>(layout, d, xq, pitch, dxs, y, M, status, partial, counters, act_f16, st);
-        case 2: return launch_a8_b<2>(layout, d, xq, pitch, dxs, y, M, status, partial, counters, act_f16, st);
-        case 3: return launch_a8_b<3>(layout, d, xq, pitch, dxs, y, M, status, partial, counters, act_f16, st);
-        case 4: return launch_a8_b<4>(layout, d, xq, pitch, dxs, y, M, status, partial, counters, act_f16, st);
-        case 5: return launch_a8_b<5>(layout, d, xq, pitch, dxs, y, M, status, partial, counters, act_f16, st);
-        case 6: return launch_a8_b<6>(layout, d, xq, pitch, dxs, y, M, status, partial, counters, act_f16, st);
-        case 7: return launch_a8_b<7>(layout, d, xq, pitch, dxs, y, M, status, partial, counters, act_f16, st);
-        default: return launch_a8_b<8>(layout, d, xq, pitch, dxs, y, M, status, partial, counters, act_f16, st);
-    }
+    GroupTable one{};
+    one.n = 1;
+    one.g[0] = {layout, 0, (int)M, 0};
+    return launch_a8_any(one, d, xq, pitch, dxs, y, M, M, status, partial, counters, act_f16, st);
+}
+
+cudaError_t launch_gemm_a8_groups(const GroupTable &groups, const Dims &d, const int8_t *xq, const float *dxs, uint16_t *y, int64_t R,
+                                  int64_t tile_m, bool act_f16, int *status, cudaStream_t st) {
+    return launch_a8_any(groups, d, xq, (int64_t)d.KT * TILE, dxs, y, R, tile_m, status, nullptr, nullptr, act_f16, st);
 }
 
 }  // namespace cq

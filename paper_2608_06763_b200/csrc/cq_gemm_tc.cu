@@ -74,7 +74,7 @@ TcPlan gemm_tc_plan(const Dims &d, int64_t M) {
 }
 
 // stream-K instantiations: cq_gemm_tc_sk.cu
-cudaError_t launch_gemm_tc_streamk(const void *layout, const Dims &d, const uint16_t *x, uint16_t *y, int64_t M, int *status,
+cudaError_t launch_gemm_tc_streamk(const GroupTable &groups, const Dims &d, const uint16_t *x, uint16_t *y, int64_t M, int *status,
                                    float *partial, int *counters, bool act_f16, cudaStream_t st);
 
 cudaError_t launch_gemm_tc(const void *layout, const Dims &d, const uint16_t *x, uint16_t *y, int64_t M, int mode,
@@ -83,8 +83,16 @@ cudaError_t launch_gemm_tc(const void *layout, const Dims &d, const uint16_t *x,
     int *status = reinterpret_cast<int *>(ws + plan.status_off);
     float *partial = reinterpret_cast<float *>(ws + plan.partial_off);
     int *counters = reinterpret_cast<int *>(ws + plan.counters_off);
-    if (gemm_tc_plan(d, M).p2 > 0) return launch_gemm_tc_streamk(layout, d, x, y, M, status, partial, counters, act_f16, st);
-    return launch_tc_variant<false>(layout, d, x, y, M, status, partial, counters, act_f16, st);
+    GroupTable one{};
+    one.n = 1;
+    one.g[0] = {layout, 0, (int)M, 0};
+    if (gemm_tc_plan(d, M).p2 > 0) return launch_gemm_tc_streamk(one, d, x, y, M, status, partial, counters, act_f16, st);
+    return launch_tc_variant<false>(one, d, x, y, M, M, status, partial, counters, act_f16, st);
+}
+
+cudaError_t launch_gemm_tc_groups(const GroupTable &groups, const Dims &d, const uint16_t *x, uint16_t *y, int64_t R, int64_t tile_m,
+                                  bool act_f16, int *status, cudaStream_t st) {
+    return launch_tc_variant<false>(groups, d, x, y, R, tile_m, status, nullptr, nullptr, act_f16, st);
 }
 
 }  // namespace cq

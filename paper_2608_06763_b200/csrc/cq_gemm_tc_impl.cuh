@@ -80,11 +80,10 @@ __device__ __forceinline__ void w3_block(const uint32_t (&w)[6], const W3Table &
 }
 
 struct TcParams {
-    const uint8_t *layout;
     uint16_t *y;
     int *status;
     Dims d;
-    int M;
+    GroupTable groups;    // an ordinary product is one group; a routed one (whole tiles only) has several
     int raw_stage_bytes;  // tile_bytes rounded up to 1024
     float *partial;       // stream-K: fp32 partial tiles [CTA][2][BNT][128]
     int *counters;        // stream-K: layout tiles done, one per output tile
@@ -139,10 +138,16 @@ template <bool SK, bool PAIR>
 struct SegWalk {
     int64_t t_full, v, v_end, V2;
     int KT, NBU, p2, c2, unit, rank;
+    int grp;              // this unit's group
     bool whole_left;
     __device__ SegWalk(const TcParams &prm, int rank_) {
         rank = rank_;
         unit = PAIR ? (int)blockIdx.x >> 1 : (int)blockIdx.x;
+        grp = 0;
+        if constexpr (!SK) {
+            while (grp + 1 < prm.groups.n && unit >= prm.groups.g[grp + 1].unit0) ++grp;
+            unit -= prm.groups.g[grp].unit0;
+        }
         KT = prm.d.KT; NBU = PAIR ? (prm.d.NB + 1) / 2 : prm.d.NB;
         if constexpr (!SK) {   // one whole tile per unit, nothing else
             p2 = 0; c2 = 0; t_full = 0; v = v_end = V2 = 0; whole_left = true;
@@ -179,7 +184,7 @@ struct SegWalk {
 // every decoded weight tile, which halves the decode work per flop at NACC = 2.
 template <int B, int G, int BN, int NACC, bool SK>
 __global__ void __launch_bounds__(TC_THREADS, 1)
-gemm_tc_kernel(const __grid_constant__ CUtensorMap xmap, TcParams prm) {
+gemm_tc_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ TcParams prm) {
     constexpr int GPT = TILE / G;
     constexpr int STAGES = tc_stages(B, G, BN, NACC);  // ring of 64-wide k blocks
     constexpr int RAW_STAGES = tc_raw_stages(B, G, BN, NACC);
@@ -236,6 +241,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap xmap, TcParams prm) {
     };
 
     SegWalk<SK, PAIR> walk(prm, rank);
+    const Group &group = prm.groups.g[SK ? 0 : walk.grp];
     Seg seg;
     if (warp == 0) {
         // ===== producer of the activation tiles.  Nothing but the wait for the stage stands between the MMAs
@@ -252,7 +258,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap xmap, TcParams prm) {
 #pragma unroll
                         for (int a = 0; a < NACC; ++a) {
                             uint8_t *dst = sB + s * B_STAGE_BYTES + a * B_TILE_BYTES;
-                            const int tok = seg.mt * BNT + a * BN + rank * BROWS;
+                            const int tok = group.row0 + seg.mt * BNT + a * BN + rank * BROWS;
                             if constexpr (PAIR) tma_load_2d_pair(dst, &xmap, map_to_rank(&full[s], 0), (2 * t + half_k) * 64, tok);
                             else tma_load_2d(dst, &xmap, &full[s], (2 * t + half_k) * 64, tok);
                         }
@@ -267,7 +273,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap xmap, TcParams prm) {
             int tcnt = 0;    // layout tiles issued so far
             while (walk.next(seg)) {
                 const int nb = min(seg.nb, d.NB - 1);   // the second CTA of a last, half pair decodes what nobody stores
-                const uint8_t *tiles = prm.layout + (size_t)nb * d.KT * (size_t)d.tile_bytes;
+                const uint8_t *tiles = (const uint8_t *)group.layout + (size_t)nb * d.KT * (size_t)d.tile_bytes;
                 for (int t = seg.k0; t < seg.k1; ++t, ++tcnt) {
                     const int rs = tcnt % RAW_STAGES;
                     if (tcnt >= RAW_STAGES) wait(&raw_empty[rs], ((tcnt / RAW_STAGES) - 1) & 1, 1);
@@ -321,6 +327,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap xmap, TcParams prm) {
         const int dw = warp - 2, g = lane >> 2, t = lane & 3;
         const int rb = dw & (SET_WARPS - 1), set = dw / SET_WARPS;
         const int dec_tid = threadIdx.x - 64;
+        const int M = group.rows;
+        uint16_t *y = prm.y + (int64_t)group.row0 * d.N;
         auto arrive = [&](uint64_t *bar) { if (PAIR && rank != 0) mbar_arrive_cluster(map_to_rank(bar, 0)); else mbar_arrive(bar); };
         int tcnt = 0, segc = 0;
         // Where the MMAs of a block are short the decoders set the pace, and a fence (some 200 cycles) is shared by a tile's
@@ -506,8 +514,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap xmap, TcParams prm) {
                 const int64_t m0 = (int64_t)seg.mt * BNT, n0 = (int64_t)seg.nb * TILE;
                 for (int c = dec_tid; c < BNT * (TILE / 8); c += 32 * DEC_WARPS) {
                     const int tok = c / (TILE / 8), part = c % (TILE / 8);
-                    if (m0 + tok < prm.M && n0 + part * 8 < d.N)   // N is a multiple of 8: a piece is inside or outside as a whole
-                        *reinterpret_cast<uint4 *>(prm.y + (m0 + tok) * d.N + n0 + part * 8) = *reinterpret_cast<const uint4 *>(stage + tok * TILE + part * 8);
+                    if (m0 + tok < M && n0 + part * 8 < d.N)   // N is a multiple of 8: a piece is inside or outside as a whole
+                        *reinterpret_cast<uint4 *>(y + (m0 + tok) * d.N + n0 + part * 8) = *reinterpret_cast<const uint4 *>(stage + tok * TILE + part * 8);
                 }
             } else if (whole) {
 #pragma unroll 1
@@ -519,7 +527,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap xmap, TcParams prm) {
 #pragma unroll
                         for (int i = 0; i < 32; ++i) {
                             const int64_t m = (int64_t)seg.mt * BNT + c0 + i;
-                            if (m < prm.M) prm.y[m * d.N + n] = float_to_act(__uint_as_float(r[i]), prm.f16);
+                            if (m < M) y[m * d.N + n] = float_to_act(__uint_as_float(r[i]), prm.f16);
                         }
                     }
                 }
@@ -589,11 +597,11 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap xmap, TcParams prm) {
                         if (qd >= QUADS) continue;
                         const int ml = qd / (TILE / 4), ch = (qd % (TILE / 4)) * 4;
                         const int64_t m = (int64_t)seg.mt * BNT + ml, n = (int64_t)seg.nb * TILE + ch;
-                        if (m >= prm.M) continue;
+                        if (m >= M) continue;
                         const float o[4] = {sum[u].x, sum[u].y, sum[u].z, sum[u].w};
 #pragma unroll
                         for (int e = 0; e < 4; ++e)
-                            if (n + e < d.N) prm.y[m * d.N + n + e] = float_to_act(o[e], prm.f16);
+                            if (n + e < d.N) y[m * d.N + n + e] = float_to_act(o[e], prm.f16);
                     }
                 }
                 if (dec_tid == 0) prm.counters[(int64_t)seg.mt * d.NB + seg.nb] = 0;  // leave the workspace ready for the next call
@@ -614,7 +622,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap xmap, TcParams prm) {
 
 // ---------------------------------------------------------------- host side
 template <int B, int G, int BN, int NACC, bool SK>
-cudaError_t launch_bn(const void *layout, const Dims &d, const uint16_t *x, uint16_t *y, int64_t M, int *status,
+cudaError_t launch_bn(const GroupTable &groups, const Dims &d, const uint16_t *x, uint16_t *y, int64_t M, int *status,
                       float *partial, int *counters, bool act_f16, cudaStream_t st) {
     EncodeTiledFn enc = encode_tiled();
     if (!enc) return cudaErrorNotSupported;
@@ -627,10 +635,20 @@ cudaError_t launch_bn(const void *layout, const Dims &d, const uint16_t *x, uint
             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return cudaErrorInvalidValue;
-    const TcPlan plan = gemm_tc_plan(d, M);
-    if (plan.bnt != BN * NACC || (plan.p2 > 0) != SK || (plan.cw == 2) != tc_pair(BN)) return cudaErrorInvalidConfiguration;
     TcParams p;
-    p.layout = (const uint8_t *)layout; p.y = y; p.status = status; p.d = d; p.M = (int)M;
+    p.groups = groups;
+    TcPlan plan;
+    if (counters) {   // an ordinary product; the groups of a routed one are computed in whole tiles and bring no workspace
+        plan = gemm_tc_plan(d, groups.g[0].rows);
+    } else {
+        constexpr int CW = tc_pair(BN) ? 2 : 1;
+        const int NBU = (d.NB + CW - 1) / CW;
+        int units = 0;
+        for (int i = 0; i < groups.n; ++i) { p.groups.g[i].unit0 = units; units += NBU * ((groups.g[i].rows + BN * NACC - 1) / (BN * NACC)); }
+        plan = {BN * NACC, 0, units * CW, 0, 0, 0, CW, units};
+    }
+    if (plan.bnt != BN * NACC || (plan.p2 > 0) != SK || (plan.cw == 2) != tc_pair(BN)) return cudaErrorInvalidConfiguration;
+    p.y = y; p.status = status; p.d = d;
     p.raw_stage_bytes = (d.tile_bytes + 1023) / 1024 * 1024;
     p.MT = plan.token_tiles; p.t_full = plan.t_full; p.p2 = plan.p2;
     constexpr int RAW_STAGES = tc_raw_stages(B, G, BN, NACC);
@@ -655,38 +673,39 @@ cudaError_t launch_bn(const void *layout, const Dims &d, const uint16_t *x, uint
     return cudaLaunchKernelEx(&cfg, kern, xmap, p);
 }
 
+// M: rows of x; tile_m: the rows whose token tile is taken (of an ordinary product, M)
 template <int B, int G, bool SK>
-cudaError_t launch_g(const void *layout, const Dims &d, const uint16_t *x, uint16_t *y, int64_t M, int *status,
+cudaError_t launch_g(const GroupTable &groups, const Dims &d, const uint16_t *x, uint16_t *y, int64_t M, int64_t tile_m, int *status,
                      float *partial, int *counters, bool act_f16, cudaStream_t st) {
-    if (M <= 32) return launch_bn<B, G, 32, 1, SK>(layout, d, x, y, M, status, partial, counters, act_f16, st);
-    if (M <= 64) return launch_bn<B, G, 64, 1, SK>(layout, d, x, y, M, status, partial, counters, act_f16, st);
-    if (M <= 128) return launch_bn<B, G, 128, 1, SK>(layout, d, x, y, M, status, partial, counters, act_f16, st);
-    if (M <= 256) return launch_bn<B, G, 256, 1, SK>(layout, d, x, y, M, status, partial, counters, act_f16, st);
-    return launch_bn<B, G, 256, 2, SK>(layout, d, x, y, M, status, partial, counters, act_f16, st);
+    if (tile_m <= 32) return launch_bn<B, G, 32, 1, SK>(groups, d, x, y, M, status, partial, counters, act_f16, st);
+    if (tile_m <= 64) return launch_bn<B, G, 64, 1, SK>(groups, d, x, y, M, status, partial, counters, act_f16, st);
+    if (tile_m <= 128) return launch_bn<B, G, 128, 1, SK>(groups, d, x, y, M, status, partial, counters, act_f16, st);
+    if (tile_m <= 256) return launch_bn<B, G, 256, 1, SK>(groups, d, x, y, M, status, partial, counters, act_f16, st);
+    return launch_bn<B, G, 256, 2, SK>(groups, d, x, y, M, status, partial, counters, act_f16, st);
 }
 
 template <int B, bool SK>
-cudaError_t launch_b(const void *layout, const Dims &d, const uint16_t *x, uint16_t *y, int64_t M, int *status,
+cudaError_t launch_b(const GroupTable &groups, const Dims &d, const uint16_t *x, uint16_t *y, int64_t M, int64_t tile_m, int *status,
                      float *partial, int *counters, bool act_f16, cudaStream_t st) {
     switch (d.G) {
-        case 32: return launch_g<B, 32, SK>(layout, d, x, y, M, status, partial, counters, act_f16, st);
-        case 64: return launch_g<B, 64, SK>(layout, d, x, y, M, status, partial, counters, act_f16, st);
-        default: return launch_g<B, 128, SK>(layout, d, x, y, M, status, partial, counters, act_f16, st);
+        case 32: return launch_g<B, 32, SK>(groups, d, x, y, M, tile_m, status, partial, counters, act_f16, st);
+        case 64: return launch_g<B, 64, SK>(groups, d, x, y, M, tile_m, status, partial, counters, act_f16, st);
+        default: return launch_g<B, 128, SK>(groups, d, x, y, M, tile_m, status, partial, counters, act_f16, st);
     }
 }
 
 template <bool SK>
-cudaError_t launch_tc_variant(const void *layout, const Dims &d, const uint16_t *x, uint16_t *y, int64_t M, int *status,
+cudaError_t launch_tc_variant(const GroupTable &groups, const Dims &d, const uint16_t *x, uint16_t *y, int64_t M, int64_t tile_m, int *status,
                               float *partial, int *counters, bool act_f16, cudaStream_t st) {
     switch (d.B) {
-        case 1: return launch_b<1, SK>(layout, d, x, y, M, status, partial, counters, act_f16, st);
-        case 2: return launch_b<2, SK>(layout, d, x, y, M, status, partial, counters, act_f16, st);
-        case 3: return launch_b<3, SK>(layout, d, x, y, M, status, partial, counters, act_f16, st);
-        case 4: return launch_b<4, SK>(layout, d, x, y, M, status, partial, counters, act_f16, st);
-        case 5: return launch_b<5, SK>(layout, d, x, y, M, status, partial, counters, act_f16, st);
-        case 6: return launch_b<6, SK>(layout, d, x, y, M, status, partial, counters, act_f16, st);
-        case 7: return launch_b<7, SK>(layout, d, x, y, M, status, partial, counters, act_f16, st);
-        default: return launch_b<8, SK>(layout, d, x, y, M, status, partial, counters, act_f16, st);
+        case 1: return launch_b<1, SK>(groups, d, x, y, M, tile_m, status, partial, counters, act_f16, st);
+        case 2: return launch_b<2, SK>(groups, d, x, y, M, tile_m, status, partial, counters, act_f16, st);
+        case 3: return launch_b<3, SK>(groups, d, x, y, M, tile_m, status, partial, counters, act_f16, st);
+        case 4: return launch_b<4, SK>(groups, d, x, y, M, tile_m, status, partial, counters, act_f16, st);
+        case 5: return launch_b<5, SK>(groups, d, x, y, M, tile_m, status, partial, counters, act_f16, st);
+        case 6: return launch_b<6, SK>(groups, d, x, y, M, tile_m, status, partial, counters, act_f16, st);
+        case 7: return launch_b<7, SK>(groups, d, x, y, M, tile_m, status, partial, counters, act_f16, st);
+        default: return launch_b<8, SK>(groups, d, x, y, M, tile_m, status, partial, counters, act_f16, st);
     }
 }
 

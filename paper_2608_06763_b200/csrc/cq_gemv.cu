@@ -586,11 +586,22 @@ __device__ __forceinline__ void ring_wait(uint64_t *bar, uint32_t parity, volati
 // ------------------------------------------------------------------------------------------
 // MODE 0: model dtype (MMA, NT blocks of 8 tokens).  MODE 1: Dynamic A8 (xq = int8 carrier [M][x8_pitch],
 // dxs = row scales).  MODE 2: model dtype without MMA for NT = M <= 2 tokens.
-template <int B, int G, int NT, int MODE>
+// GRP: blockIdx.y is a group of a routed product, with its own matrix, rows and slice of the workspace.
+template <int B, int G, int NT, int MODE, bool GRP>
 __global__ void __launch_bounds__(GEMV_THREADS, gemv_occ(B, G, NT, MODE))
 gemv_kernel(const uint8_t *__restrict__ layout, Dims d, const uint16_t *__restrict__ x, const int8_t *__restrict__ xq,
             int64_t x8_pitch, const float *__restrict__ dxs, uint16_t *__restrict__ y, int M, int E,
-            float *__restrict__ partial, int *__restrict__ counters, int nstage, uint32_t ring_off, int *__restrict__ status, bool xf16) {
+            float *__restrict__ partial, int *__restrict__ counters, int nstage, uint32_t ring_off, int *__restrict__ status, bool xf16,
+            const __grid_constant__ GroupTable groups) {
+    if constexpr (GRP) {
+        const Group &gr = groups.g[blockIdx.y];
+        layout = (const uint8_t *)gr.layout;
+        M = gr.rows;
+        if constexpr (MODE == 1) { xq += (int64_t)gr.row0 * x8_pitch; dxs += gr.row0; } else x += (int64_t)gr.row0 * d.K;
+        y += (int64_t)gr.row0 * d.N;
+        partial += (size_t)blockIdx.y * gridDim.x * 2 * (8 * NT * TILE);
+        counters += (int64_t)blockIdx.y * d.NB;
+    }
     constexpr int GPT = TILE / G;
     constexpr int L = B == 1 ? 1 : (1 << (B - 1));
     constexpr bool RING = gemv_uses_ring(B, G, NT, MODE);
@@ -966,10 +977,10 @@ gemv_kernel(const uint8_t *__restrict__ layout, Dims d, const uint16_t *__restri
     }
 }
 
-template <int B, int G, int NT, int MODE>
+template <int B, int G, int NT, int MODE, bool GRP = false>
 cudaError_t launch_one(const void *layout, const Dims &d, const uint16_t *x, const int8_t *xq, int64_t x8_pitch,
                        const float *dxs, uint16_t *y, int M, int P, int max_run, int E, float *partial, int *counters,
-                       int *status, bool act_f16, cudaStream_t st) {
+                       int *status, bool act_f16, cudaStream_t st, const GroupTable *groups = nullptr) {
     constexpr int GPT = TILE / G;
     constexpr int TB = 2048 * B + 1024 * GPT;
     int64_t sub64 = max_run;   // the longest run bounds the activation slice a CTA stages
@@ -988,7 +999,7 @@ cudaError_t launch_one(const void *layout, const Dims &d, const uint16_t *x, con
         if (nstage < 2) return cudaErrorInvalidConfiguration;
     }
     const size_t smem = ring_off + (size_t)nstage * TB;
-    auto kern = gemv_kernel<B, G, NT, MODE>;
+    auto kern = gemv_kernel<B, G, NT, MODE, GRP>;
     static std::atomic<uint64_t> attr_done{0};
     cudaError_t e = ensure_func_attr(kern, attr_done, cudaFuncAttributeMaxDynamicSharedMemorySize, gemv_smem_budget(OCC));
     if (e != cudaSuccess) return e;
@@ -996,7 +1007,7 @@ cudaError_t launch_one(const void *layout, const Dims &d, const uint16_t *x, con
     // kernel of the stream drains; it waits for that kernel before touching anything but the weights.
     static const bool use_pdl = getenv("CQ_NO_PDL") == nullptr;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)P);
+    cfg.gridDim = dim3((unsigned)P, GRP ? (unsigned)groups->n : 1u);
     cfg.blockDim = dim3(GEMV_THREADS);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
@@ -1005,8 +1016,9 @@ cudaError_t launch_one(const void *layout, const Dims &d, const uint16_t *x, con
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = use_pdl ? 1 : 0;
+    static const GroupTable none = {};
     return cudaLaunchKernelEx(&cfg, kern, (const uint8_t *)layout, d, x, xq, x8_pitch, dxs, y, M, E, partial, counters, nstage,
-                              ring_off, status, act_f16);
+                              ring_off, status, act_f16, GRP ? *groups : none);
 }
 
 template <int B, int G>
@@ -1034,7 +1046,42 @@ cudaError_t dispatch_g(const void *layout, const Dims &d, const uint16_t *x, con
     }
 }
 
+// Routed products: sixteen-row variants, all groups in one launch.
+template <int B, int G>
+cudaError_t launch_groups_g(const GroupTable &t, const Dims &d, const uint16_t *x, const int8_t *xq, const float *dxs, uint16_t *y, int mode,
+                            bool act_f16, int P, int max_run, int max_rows, float *partial, int *counters, int *status, cudaStream_t st) {
+    const int64_t pitch = (int64_t)d.KT * TILE;
+    if (mode == 0) return launch_one<B, G, 2, 0, true>(nullptr, d, x, nullptr, pitch, nullptr, y, max_rows, P, max_run, 0, partial, counters, status, act_f16, st, &t);
+    return launch_one<B, G, 2, 1, true>(nullptr, d, nullptr, xq, pitch, dxs, y, max_rows, P, max_run, 0, partial, counters, status, act_f16, st, &t);
+}
+template <int B>
+cudaError_t launch_groups_b(const GroupTable &t, const Dims &d, const uint16_t *x, const int8_t *xq, const float *dxs, uint16_t *y, int mode,
+                            bool act_f16, int P, int max_run, int max_rows, float *partial, int *counters, int *status, cudaStream_t st) {
+    switch (d.G) {
+        case 32: return launch_groups_g<B, 32>(t, d, x, xq, dxs, y, mode, act_f16, P, max_run, max_rows, partial, counters, status, st);
+        case 64: return launch_groups_g<B, 64>(t, d, x, xq, dxs, y, mode, act_f16, P, max_run, max_rows, partial, counters, status, st);
+        default: return launch_groups_g<B, 128>(t, d, x, xq, dxs, y, mode, act_f16, P, max_run, max_rows, partial, counters, status, st);
+    }
+}
+
 }  // namespace
+
+cudaError_t launch_gemv_groups(const GroupTable &t, const Dims &d, const uint16_t *x, const int8_t *xq, const float *dxs, uint16_t *y,
+                               int mode, bool act_f16, int P, float *partial, int *counters, int *status, cudaStream_t st) {
+    const int max_run = (int)(((int64_t)d.NB * d.KT) / P + 1);
+    int max_rows = 1;
+    for (int i = 0; i < t.n; ++i) if (t.g[i].rows > max_rows) max_rows = t.g[i].rows;
+    switch (d.B) {
+        case 1: return launch_groups_b<1>(t, d, x, xq, dxs, y, mode, act_f16, P, max_run, max_rows, partial, counters, status, st);
+        case 2: return launch_groups_b<2>(t, d, x, xq, dxs, y, mode, act_f16, P, max_run, max_rows, partial, counters, status, st);
+        case 3: return launch_groups_b<3>(t, d, x, xq, dxs, y, mode, act_f16, P, max_run, max_rows, partial, counters, status, st);
+        case 4: return launch_groups_b<4>(t, d, x, xq, dxs, y, mode, act_f16, P, max_run, max_rows, partial, counters, status, st);
+        case 5: return launch_groups_b<5>(t, d, x, xq, dxs, y, mode, act_f16, P, max_run, max_rows, partial, counters, status, st);
+        case 6: return launch_groups_b<6>(t, d, x, xq, dxs, y, mode, act_f16, P, max_run, max_rows, partial, counters, status, st);
+        case 7: return launch_groups_b<7>(t, d, x, xq, dxs, y, mode, act_f16, P, max_run, max_rows, partial, counters, status, st);
+        default: return launch_groups_b<8>(t, d, x, xq, dxs, y, mode, act_f16, P, max_run, max_rows, partial, counters, status, st);
+    }
+}
 
 // Streaming multiprocessors of the current device (148 on a B200; that figure also stands in when no
 // device can be asked, so that size queries work on a machine without a GPU).

@@ -26,9 +26,9 @@ cudaError_t launch_quantize_a8(const uint16_t *x, int64_t M, int64_t K, int8_t *
 // h[M][2 I] (gate | up, model dtype) -> INT8 carrier of silu(gate) * up, and its row scales
 cudaError_t launch_swiglu_quantize_a8(const uint16_t *h, int64_t M, int64_t I, int8_t *x8, int64_t x8_pitch, float *dx,
                                       bool operand_order, bool act_f16, cudaStream_t st);
-// routed execution: xg[r] = x[route_token[r]] (zero row for an index outside [0, T))
+// routed execution: xg[r] = x[route_token[r]] (zero row for an index outside [0, T)); the status word and n counters are zeroed
 cudaError_t launch_gather_rows(const uint16_t *x, const int32_t *route_token, uint16_t *xg, int64_t R, int64_t T, int64_t K,
-                               cudaStream_t st);
+                               int *status, int *counters, int64_t n, cudaStream_t st);
 cudaError_t launch_wait_timeout(int *status, long long limit_cycles, cudaStream_t st);
 
 // Workspace carving (all offsets 256-byte aligned).
@@ -63,6 +63,13 @@ cudaError_t ensure_func_attr(Kern kern, std::atomic<uint64_t> &done, cudaFuncAtt
 // the thread's record of the last failed CUDA call (what cq_last_cuda_error returns)
 void set_last_cuda_error(cudaError_t e);
 
+// Several products over one activation matrix in one launch (routed execution): rows [row0, row0 + rows) of x and y
+// belong to the matrix `layout`; all matrices share shape and format.  unit0 is filled in by the launcher: the first
+// output tile (or pair of tiles) of the group.  More groups than a table holds go out as several launches.
+constexpr int MAX_GROUPS = 32;
+struct Group { const void *layout; int row0, rows, unit0; };
+struct GroupTable { int n; Group g[MAX_GROUPS]; };
+
 // Decomposition of the small-M path: number of CTAs (one contiguous run of tiles each) and the
 // largest number of CTAs that contribute to one 128-row block.
 struct GemvPlan { int ctas, max_run, overhead; };
@@ -72,6 +79,14 @@ GemvPlan gemv_plan(const Dims &d, int64_t M, int mode);
 // prequantized (Dynamic A8 only): the workspace already holds the INT8 carrier and the row scales of x (x is not read)
 cudaError_t launch_gemv(const void *layout, const Dims &d, const uint16_t *x, uint16_t *y, int64_t M, int mode,
                         bool act_f16, uint8_t *ws, const Workspace &plan, cudaStream_t st, bool prequantized = false);
+// every group 1 .. 16 rows; x and y are those of all groups; P CTAs and a workspace slice for each group
+cudaError_t launch_gemv_groups(const GroupTable &groups, const Dims &d, const uint16_t *x, const int8_t *xq, const float *dxs, uint16_t *y,
+                               int mode, bool act_f16, int P, float *partial, int *counters, int *status, cudaStream_t st);
+// `R` rows of x in all, every group at most `tile_m` rows to a token tile of that size class
+cudaError_t launch_gemm_tc_groups(const GroupTable &groups, const Dims &d, const uint16_t *x, uint16_t *y, int64_t R, int64_t tile_m,
+                                  bool act_f16, int *status, cudaStream_t st);
+cudaError_t launch_gemm_a8_groups(const GroupTable &groups, const Dims &d, const int8_t *xq, const float *dxs, uint16_t *y, int64_t R,
+                                  int64_t tile_m, bool act_f16, int *status, cudaStream_t st);
 int gemm_tc_token_tile(int64_t M);
 // cw: CTAs that compute a tile together (2: a pair, 256 channels); t_full whole tiles and p2 runs are counted in such units
 struct TcPlan { int bnt, token_tiles, ctas, stream_k, p2, crossing, cw; int64_t t_full; };

@@ -67,3 +67,33 @@ def test_routed_argument_errors_and_bad_token():
     assert L.cq_gemm_routed(None, 2, 4, 128, one, one, off, one, 4, 128, 256, 0, 0, one, 1 << 30, None) == -1
     assert L.cq_routed_workspace_bytes(4, 128, 2, off, 128, 256, 0) > 0
     assert L.cq_routed_workspace_bytes(4, 128, 2, bad, 128, 256, 0) == 0
+
+
+@pytest.mark.parametrize("mode", [cq.CQ_MODEL_DTYPE, cq.CQ_DYN_A8])
+@pytest.mark.parametrize("B,G", [(4, 64), (8, 128), (2, 32)])
+def test_routed_classes_share_launches(B, G, mode):
+    # every class of row counts with none, one, several and more groups than one launch holds; one workspace for routings
+    # of different sizes, never cleared in between
+    N, K, T = 136, 384, 300
+    rng = np.random.default_rng(900 + B)
+    routings = [[1, 3, 16, 7, 0, 17, 40, 128, 129, 256, 300, 5], [9], [2] * 35, [20, 0, 90, 33], [300, 280, 16, 260], [16] * 33 + [18]]
+    E = 36
+    parts = [datagen.logical_quantized(N, K, B, G, 901 + e) for e in range(3)]
+    cases = [Case(*parts[e % 3], B, G) for e in range(3)]
+    dicts = [dict(codes=c.codes, s=c.s, a=c.a, b=c.b, B=B, G=G, K=K) for c in cases]
+    x = datagen.activations(T, K, seed=902)
+    xd = torch.from_numpy(x.view(np.int16)).cuda().view(torch.bfloat16)
+    ws = torch.full((64 << 20,), 0x5A, dtype=torch.uint8, device="cuda")
+    for counts in routings:
+        n = len(counts)
+        assert n <= E
+        offset = np.concatenate([[0], np.cumsum(counts)])
+        tokens = rng.integers(0, T, offset[-1]).astype(np.int32)
+        which = [e % 3 for e in range(n)]
+        y = cq.cq_gemm_routed([cases[w].pw for w in which], xd, torch.from_numpy(tokens).cuda(), offset, mode, ws)
+        assert cq.cq_gemm_status(ws) == 0
+        ref = oracle.gemm_routed([dicts[w] for w in which], x, tokens, offset, "model" if mode == cq.CQ_MODEL_DTYPE else "a8")
+        yn = y_to_numpy(y)
+        for e in range(n):
+            if counts[e]:
+                check_y(yn[offset[e]:offset[e + 1]], ref[offset[e]:offset[e + 1]], f"{counts[e]} routes, matrix {e} of {n}")
