@@ -210,8 +210,9 @@ __host__ __device__ constexpr int carrier_slot(int B, int i, bool negative) {
     return B == 4 ? (negative ? 8 + i : i) : (negative ? (1 << (B - 1)) - i : (1 << (B - 1)) + i);
 }
 
-// Row stride (bytes) of a shared-memory carrier table of 2^B entries per row (B = 3, 4: wider codes have none).
-__host__ __device__ constexpr int carrier_table_stride(int B) { return B <= 4 ? (1 << B) : 0; }
+// Row stride (bytes) of a shared-memory carrier table of 2^B entries per row (B = 3, 4, 5: wider codes have none).
+__host__ __device__ constexpr bool carrier_by_table(int B) { return B >= 3 && B <= 5; }
+__host__ __device__ constexpr int carrier_table_stride(int B) { return B <= 5 ? (1 << B) : 0; }
 
 // INT8 carrier (Eq. carrier) at the normalised position t = i / M: RNE(127 q(t)), clamped to [0, 127],
 // by the fp32 sequence c = (1 - a) - b, q = t fma(t, fma(t, c, b), a).

@@ -233,11 +233,33 @@ __device__ __forceinline__ void w4_put(uint8_t *row, uint2 p, int t, float t0, f
 //          inside the block is the natural one, lane t holding bytes 8 t .. 8 t + 7;
 //   B = 3: one 8-byte table, the selector assembled from the 2-bit and the 1-bit plane;
 //   B <= 2: the carriers are 0 / +-127, a constant table;
-//   B >= 5: no table (a8_row_eval).
+//   B = 5: four 8-byte quarters, the low three bits select in each, the upper two (one of them from the 1-bit
+//          plane) pick between them;
+//   B >= 6: no table (a8_row_eval).
+struct CarrierTab { uint4 v[2]; };   // entries 0 .. 15 and (B = 5) 16 .. 31
+template <int B>
+__device__ __forceinline__ CarrierTab load_carrier_tab(const int8_t *row) {
+    CarrierTab t{};
+    if constexpr (B == 3) { const uint2 v = *reinterpret_cast<const uint2 *>(row); t.v[0].x = v.x; t.v[0].y = v.y; }
+    if constexpr (B >= 4) t.v[0] = *reinterpret_cast<const uint4 *>(row);
+    if constexpr (B == 5) t.v[1] = *reinterpret_cast<const uint4 *>(row + 16);
+    return t;
+}
+__device__ __forceinline__ uint32_t pick(uint32_t mask, uint32_t a, uint32_t b) { return (a & mask) | (b & ~mask); }
 template <int B, int RR, int MI>
-__device__ __forceinline__ void a8_row_regs(const uint32_t (&w)[2 * B], const uint4 &tab, uint32_t &lo, uint32_t &hi) {
-    static_assert(B <= 4, "wider codes are evaluated one by one (a8_row_eval)");
-    if constexpr (B == 4) {
+__device__ __forceinline__ void a8_row_regs(const uint32_t (&w)[2 * B], const CarrierTab &ct, uint32_t &lo, uint32_t &hi) {
+    static_assert(B <= 5, "wider codes are evaluated one by one (a8_row_eval)");
+    const uint4 &tab = ct.v[0];
+    if constexpr (B == 5) {
+        constexpr int rho = (2 + 2 * (MI & 1) + RR) & 3;   // where the 1-bit plane keeps the top bits: bit 4 n + rho
+        const uint32_t word = w[2 * MI + RR], z = w[plane_word_base(5, 1) + (MI >> 1)] << (3 - rho);
+        const uint32_t ws = word & 0x77777777u, wh = ws >> 16, w4 = word << 4, z4 = z << 4;
+        const uint32_t m_lo = prmt(w4, word, 0xD9C8u), m_hi = prmt(w4, word, 0xFBEAu);   // 0xFF where bit 3 is set
+        const uint32_t k_lo = prmt(z4, z, 0xD9C8u), k_hi = prmt(z4, z, 0xFBEAu);         // 0xFF where bit 4 is set
+        const uint4 &t2 = ct.v[1];
+        lo = pick(k_lo, pick(m_lo, prmt(t2.z, t2.w, ws), prmt(t2.x, t2.y, ws)), pick(m_lo, prmt(tab.z, tab.w, ws), prmt(tab.x, tab.y, ws)));
+        hi = pick(k_hi, pick(m_hi, prmt(t2.z, t2.w, wh), prmt(t2.x, t2.y, wh)), pick(m_hi, prmt(tab.z, tab.w, wh), prmt(tab.x, tab.y, wh)));
+    } else if constexpr (B == 4) {
         const uint32_t word = w[2 * MI + RR];
         const uint32_t ws = word & 0x77777777u, wh = ws >> 16, w4 = word << 4;
         const uint32_t m_lo = prmt(w4, word, 0xD9C8u), m_hi = prmt(w4, word, 0xFBEAu);   // 0xFF where the code is negative
@@ -265,7 +287,7 @@ __device__ __forceinline__ void a8_row_regs(const uint32_t (&w)[2 * B], const ui
     }
 }
 
-// ---- B >= 5: the carrier of each code evaluated where it is needed, two at a time in packed fp32, by the pinned
+// ---- B >= 6: the carrier of each code evaluated where it is needed, two at a time in packed fp32, by the pinned
 // sequence of carrier_at.  A table per (row, group) would have as many entries as the group has weights (W8, G = 128), and
 // reading it costs a shared-memory access per weight with the lanes in random banks: linears of an 8B layer, W8 G128,
 // M = 64: 400 us with tables, 204 us so.

@@ -3,16 +3,17 @@
 //
 // CTA = 128 output channels x BN tokens, K (or one slice of it, for a tile of the last round) walked in 128-wide
 // blocks (one layout tile).
-//   warp 0       TMA of the x8 tiles [BN x 128] (swizzled) into a ring of two stages
-//   warp 18      bulk copies of the raw layout tiles into their own ring (2-4 deep)
+//   warp 0       TMA of the x8 tiles [BN x 128] (swizzled) into the operand ring (2-4 stages)
+//   warp 18      bulk copies of the raw layout tiles into their own ring (2-6 deep)
 //   warp 1       TMEM allocation, tcgen05.mma kind::i8 (K = 32 per instruction); every group of
 //                the block accumulates into its own BN columns of one of two TMEM buffers
-//   warps 2..17  work warps, two jobs per K block, interleaved so the tensor core never waits on both:
-//                (a) decode block t: a signed carrier table r(k) per (row, group) (Eq. carrier, the
-//                    fp32 sequence of cq_common.cuh), then the carriers of the block by byte-permute look-ups
-//                    in it (B <= 4; wider codes are evaluated one by one) go
-//                    into the K-major swizzled INT8 operand tile in the operand order of cq_decode.cuh;
-//                (b) drain block t-1: tcgen05.ld of its int32 partials P_g, acc += s_g * P_g in fp32
+//   warps 2..17  work warps, two jobs, interleaved so the tensor core never waits on both:
+//                (a) decode: two sets of eight warps take the blocks in turn, a warp 16 rows of one.  A signed carrier
+//                    table r(k) per (row, group) (Eq. carrier, the fp32 sequence of cq_common.cuh; the warp's own, so no
+//                    other warp is waited for), then the carriers of the block by byte-permute look-ups in it (B <= 5;
+//                    wider codes are evaluated one by one) go into the K-major swizzled INT8 operand tile in the
+//                    operand order of cq_decode.cuh;
+//                (b) drain block t-1, all sixteen: tcgen05.ld of its int32 partials P_g, acc += s_g * P_g in fp32
 //                    registers (Eq. a8-output), which frees that TMEM buffer for block t+1.
 //                At the end y = (d_x / 127) * acc, rounded to bf16.
 // All mbarrier waits are bounded and report through the workspace status word.
@@ -63,15 +64,19 @@ using namespace tc;
 
 constexpr int A8_WORK_WARPS = 16;
 constexpr int A8_THREADS = 32 * (3 + A8_WORK_WARPS);   // producer of activations, MMA issuer, work warps, producer of raw tiles
-constexpr int A8_STAGES = 2;     // operand stages (one 128-wide k block each)
-// Raw layout tiles in flight per CTA: as many as the shared memory left by the rest holds, two to four.
+constexpr int A8_SET_WARPS = A8_WORK_WARPS / 2;   // warps that decode a block, one per 16 rows
 constexpr int a8_raw_stage_bytes(int B, int G) { return (2048 * B + 1024 * (TILE / G) + 1023) / 1024 * 1024; }
-constexpr int a8_fixed_smem(int B, int G, int BN) {
-    return 2 * (128 * 128 + BN * 128) + 8 * 2 * 16 * carrier_table_stride(B) + 8 * 128 * (TILE / G) * 4 + 512 + 256;
+constexpr int a8_fixed_smem(int B, int G) {   // tables, scale snapshots, t_i, barriers
+    return A8_WORK_WARPS * 16 * (B >= 3 ? carrier_table_stride(B) : 0) + 8 * 128 * (TILE / G) * 4 + 512 + 512;
+}
+// Operand stages (one 128-wide k block each): up to four beside two raw tiles; raw tiles: what is left, two to six.
+constexpr int a8_stages(int B, int G, int BN) {
+    const int n = (226 * 1024 - a8_fixed_smem(B, G) - 2 * a8_raw_stage_bytes(B, G)) / (128 * 128 + BN * 128);
+    return n > 4 ? 4 : n;
 }
 constexpr int a8_raw_stages(int B, int G, int BN) {
-    const int n = (226 * 1024 - a8_fixed_smem(B, G, BN)) / a8_raw_stage_bytes(B, G);
-    return n > 4 ? 4 : n < 2 ? 2 : n;
+    const int n = (226 * 1024 - a8_fixed_smem(B, G) - a8_stages(B, G, BN) * (128 * 128 + BN * 128)) / a8_raw_stage_bytes(B, G);
+    return n > 6 ? 6 : n;
 }
 constexpr int A8_SRING = 8;      // ring of per-block scale snapshots for the drain warps
 constexpr int A8_A_STAGE_BYTES = 128 * 128;
@@ -90,10 +95,6 @@ struct A8Params {
     bool f16;             // y is written as binary16 instead of bfloat16
 };
 
-__device__ __forceinline__ void named_barrier_sync(int id, int threads) {
-    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
-}
-
 template <int B, int G, int BN>
 __global__ void __launch_bounds__(A8_THREADS, 1)
 gemm_a8_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ A8Params prm) {
@@ -105,17 +106,18 @@ gemm_a8_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
     constexpr uint32_t ACC_COLS = GPT * BN;       // columns of one accumulator buffer
     constexpr uint32_t TMEM_COLS = 2 * ACC_COLS;  // 512
     constexpr int QCOLS = BN / 4;                 // columns per work thread in the drain
-    constexpr int A8_RAW_STAGES = a8_raw_stages(B, G, BN);
+    constexpr int A8_STAGES = a8_stages(B, G, BN), A8_RAW_STAGES = a8_raw_stages(B, G, BN);
+    static_assert(A8_STAGES >= 2 && A8_RAW_STAGES >= 2, "shared memory");
     static_assert(TMEM_COLS <= 512 && (TMEM_COLS & (TMEM_COLS - 1)) == 0, "TMEM columns");
     extern __shared__ __align__(1024) uint8_t smem[];
     uint8_t *sA = smem;
     uint8_t *sB = sA + A8_STAGES * A8_A_STAGE_BYTES;
     uint8_t *sRaw = sB + A8_STAGES * B_STAGE_BYTES;
-    int8_t *sTab = reinterpret_cast<int8_t *>(sRaw + A8_RAW_STAGES * prm.raw_stage_bytes);   // [8 row blocks][2][16 rows][NCODE]
-    float *sScale = reinterpret_cast<float *>(sTab + 8 * 2 * 16 * NCODE);                      // [SRING][128][GPT]
+    int8_t *sTab = reinterpret_cast<int8_t *>(sRaw + A8_RAW_STAGES * prm.raw_stage_bytes);   // [work warp][16 rows][NCODE]
+    float *sScale = reinterpret_cast<float *>(sTab + (B >= 3 ? A8_WORK_WARPS * 16 * NCODE : 0));                      // [SRING][128][GPT]
     float *sT = sScale + A8_SRING * 128 * GPT;                                                 // t_i = i / M, i = 0..127
     uint64_t *bars = reinterpret_cast<uint64_t *>(sT + 128);
-    uint64_t *a_full = bars, *b_full = a_full + A8_STAGES, *st_empty = b_full + A8_STAGES;
+    uint64_t *st_full = bars, *st_empty = st_full + A8_STAGES;
     uint64_t *raw_full = st_empty + A8_STAGES, *raw_empty = raw_full + A8_RAW_STAGES;
     uint64_t *acc_full = raw_empty + A8_RAW_STAGES, *acc_empty = acc_full + 2;
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(acc_empty + 2);
@@ -146,8 +148,8 @@ gemm_a8_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
         return;
     }
     if (threadIdx.x == 0) {
-        for (int s = 0; s < A8_STAGES; ++s) { mbar_init(&a_full[s], A8_WORK_WARPS); mbar_init(&b_full[s], 1); mbar_init(&st_empty[s], 1); }
-        for (int s = 0; s < A8_RAW_STAGES; ++s) { mbar_init(&raw_full[s], 1); mbar_init(&raw_empty[s], A8_WORK_WARPS); }
+        for (int s = 0; s < A8_STAGES; ++s) { mbar_init(&st_full[s], A8_SET_WARPS + 1); mbar_init(&st_empty[s], 1); }   // full: a set's warps and the announced bytes
+        for (int s = 0; s < A8_RAW_STAGES; ++s) { mbar_init(&raw_full[s], 1); mbar_init(&raw_empty[s], A8_SET_WARPS); }
         for (int s = 0; s < 2; ++s) { mbar_init(&acc_full[s], 1); mbar_init(&acc_empty[s], A8_WORK_WARPS); }
         fence_barrier_init();
         tmem_slot[2] = 0;   // the work warps' "a wait gave up" flag
@@ -173,8 +175,8 @@ gemm_a8_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
                 const int s = t % A8_STAGES;
                 if (t >= A8_STAGES) ok = mbar_wait(&st_empty[s], ((t / A8_STAGES) - 1) & 1, prm.status, 12);
                 if (!ok) break;
-                mbar_arrive_expect_tx(&b_full[s], B_STAGE_BYTES);
-                tma_load_2d(sB + s * B_STAGE_BYTES, &xmap, &b_full[s], (kt0 + t) * 128, prm.groups.g[grp].row0 + mt * BN);
+                mbar_arrive_expect_tx(&st_full[s], B_STAGE_BYTES);
+                tma_load_2d(sB + s * B_STAGE_BYTES, &xmap, &st_full[s], (kt0 + t) * 128, prm.groups.g[grp].row0 + mt * BN);
             }
         }
     } else if (warp == 2 + A8_WORK_WARPS) {
@@ -191,44 +193,48 @@ gemm_a8_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
             }
         }
     } else if (warp == 1) {
-        // ===== MMA issuer
-        if (lane == 0) {
-            constexpr uint32_t idesc = idesc_i8(BN);
-            bool ok = true;
-            for (int t = 0; t < KT && ok; ++t) {
-                const int s = t % A8_STAGES, ab = t & 1;
-                ok = mbar_wait(&a_full[s], (t / A8_STAGES) & 1, prm.status, 13) &&
-                     mbar_wait(&b_full[s], (t / A8_STAGES) & 1, prm.status, 14);
-                if (ok && t >= 2) ok = mbar_wait(&acc_empty[ab], ((t >> 1) - 1) & 1, prm.status, 15);
-                if (!ok) break;
-                tc_fence_after();
-                const uint64_t adesc = smem_desc_sw128(smem_u32(sA + s * A8_A_STAGE_BYTES));
-                const uint64_t bdesc = smem_desc_sw128(smem_u32(sB + s * B_STAGE_BYTES));
+        // ===== MMA issuer: the whole warp walks the loop (descriptors and addresses stay uniform), one elected lane issues
+        constexpr uint32_t idesc = idesc_i8(BN);
+        const bool issuer = elect_one();
+        bool ok = true;
+        int s = 0;
+        uint32_t phase = 0;
+        for (int t = 0; t < KT && ok; ++t) {
+            const int ab = t & 1;
+            ok = mbar_wait(&st_full[s], phase, prm.status, 13);
+            if (ok && t >= 2) ok = mbar_wait(&acc_empty[ab], ((t >> 1) - 1) & 1, prm.status, 15);
+            ok = __all_sync(0xffffffffu, ok);
+            if (!ok) break;
+            tc_fence_after();
+            const uint64_t adesc = smem_desc_sw128(smem_u32(sA) + s * A8_A_STAGE_BYTES);
+            const uint64_t bdesc = smem_desc_sw128(smem_u32(sB) + s * B_STAGE_BYTES);
+            if (issuer) {
 #pragma unroll
                 for (int mi = 0; mi < 4; ++mi)   // four K = 32 steps, 32 bytes apart; a new group restarts the sum
                     umma_i8(tmem_base + ab * ACC_COLS + (mi / MPG) * BN, adesc + 2 * mi, bdesc + 2 * mi, idesc, (mi % MPG) != 0);
                 umma_commit(&st_empty[s]);
                 umma_commit(&acc_full[ab]);
             }
+            __syncwarp();
+            if (++s == A8_STAGES) { s = 0; phase ^= 1u; }
         }
     } else {
-        // ===== work warps.  Decode: warp dw owns row block dw / 2 and the 64-wide half dw % 2 of every
-        // block.  Drain: TMEM lane quarter warp % 4, column quarter dw / 4.
+        // ===== work warps.  Decode: warp rb of a set owns row block rb of every second block.  Drain: TMEM lane quarter
+        // warp % 4, column quarter dw / 4.
         const int dw = warp - 2, g = lane >> 2, tq = lane & 3;
-        const int rb = dw >> 1, jh = dw & 1;
+        const int rb = dw & (A8_SET_WARPS - 1), set = dw / A8_SET_WARPS;
         const int q4 = warp & 3, cq4 = dw >> 2;
         const int drow = q4 * 32 + lane;
-        int8_t *tab = sTab + (rb * 2 + (G == 128 ? 0 : jh)) * 16 * NCODE;   // G = 128: the two halves share one table
+        int8_t *tab = sTab + dw * 16 * NCODE;
         float acc[QCOLS];
 #pragma unroll
         for (int i = 0; i < QCOLS; ++i) acc[i] = 0.0f;
-        // A wait that gives up (bounded, see mbar_wait) must not make this warp leave the loop: with G = 128
-        // its partner of the row block would then wait for it at the 64-thread barrier for ever.  The warp
-        // keeps walking the blocks instead, without waiting any more, so every barrier still sees both
-        // warps; what it computes from then on is discarded (the status word is set, nothing is stored).
+        // A wait that gives up (bounded, see mbar_wait) does not make this warp leave the loop: it keeps walking the
+        // blocks without waiting any more; what it computes from then on is discarded (the status word is set, nothing
+        // is stored).
         volatile int *gave_up = reinterpret_cast<volatile int *>(tmem_slot + 2);   // CTA-wide flag, cleared at start
         for (int t = 0; t <= KT; ++t) {
-            if (t < KT) {
+            if (t < KT && (t & 1) == set) {
                 // ---------------- (a) decode block t
                 const int rs = t % A8_RAW_STAGES, s = t % A8_STAGES;
                 if (!*gave_up && !mbar_wait(&raw_full[rs], (t / A8_RAW_STAGES) & 1, prm.status, 16)) *gave_up = 1;
@@ -253,20 +259,16 @@ gemm_a8_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
                 uint8_t *row_lo = a_stage + (rb * 2 + 0) * 1024 + g * 128;
                 uint8_t *row_hi = a_stage + (rb * 2 + 1) * 1024 + g * 128;
                 float *sc = sScale + (size_t)(t % A8_SRING) * 128 * GPT;
-                constexpr int GH = GPT >= 2 ? GPT / 2 : 1;   // groups this warp's 64-wide half touches
-                constexpr int CPGH = 4 / GH;                 // 16-wide chunks of the half per such group
-                auto do_half = [&](auto jhc) {
-                    constexpr int JH = decltype(jhc)::value;
-                    static_for<GH>([&](auto gc) {
-                        constexpr int gi = (GPT >= 2) ? JH * GH + decltype(gc)::value : 0;
+                static_for<GPT>([&](auto gc) {
+                        constexpr int gi = decltype(gc)::value;
                         const uint2 p_lo = *(const uint2 *)(prow + gi * 8), p_hi = *(const uint2 *)(prow + (8 * GPT + gi) * 8);
-                        if (tq == 0 && (G != 128 || JH == 0)) {
+                        if (tq == 0) {
                             sc[(rb * 16 + g) * GPT + gi] = __uint_as_float(p_lo.x & 0x7FFFFFFFu);
                             sc[(rb * 16 + g + 8) * GPT + gi] = __uint_as_float(p_hi.x & 0x7FFFFFFFu);
                         }
                         // bytes 32 MI + 8 tq of the row: 16-byte chunk 2 MI + tq / 2, swizzled by the row
                         auto place = [&](int MI) { return (((2 * MI + (tq >> 1)) ^ g) * 16) + (tq & 1) * 8; };
-                        if constexpr (B >= 5) {
+                        if constexpr (B >= 6) {
                             // wider codes: carriers evaluated one by one, row after row
                             const bool fix = __any_sync(0xffffffffu, (p_lo.x | p_hi.x) >> 31);   // reserved pattern present
                             auto eval = [&](auto fx) {
@@ -274,8 +276,8 @@ gemm_a8_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
                                 static_for<2>([&](auto rc) {
                                     constexpr int RR = decltype(rc)::value;
                                     const CarrierPoly poly = carrier_poly(RR ? p_hi.y : p_lo.y);
-                                    static_for<CPGH / 2>([&](auto mc) {
-                                        constexpr int MI = 2 * JH + decltype(gc)::value * (CPGH / 2) + decltype(mc)::value;
+                                    static_for<MPG>([&](auto mc) {
+                                        constexpr int MI = gi * MPG + decltype(mc)::value;
                                         uint2 v;
                                         a8_row_eval<B, RR, MI, FIX>(w, poly, v.x, v.y);
                                         *(uint2 *)((RR ? row_hi : row_lo) + place(MI)) = v;
@@ -285,43 +287,31 @@ gemm_a8_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
                             if (!fix) eval(std::false_type{}); else eval(std::true_type{});
                         } else {
                             if constexpr (B >= 3) {
-                                // signed carrier table: index = stored code u (reserved -> 0), entry sign(k) r(|k|).
-                                // With G = 128 the two warps of a row block build eight rows each and meet at a
-                                // 64-thread barrier.
-                                if constexpr (G == 128) named_barrier_sync(1 + rb, 64); else __syncwarp();
+                                // signed carrier table: index = stored code u (reserved -> 0), entry sign(k) r(|k|)
+                                __syncwarp();
                                 auto build_row = [&](int row, uint32_t abbits) {
                                     const __half2 ab = as_h2(abbits);
                                     const float a = __low2float(ab), b = __high2float(ab);
                                     int8_t *tr = tab + row * NCODE;
                                     if (B != 4 && tq == 0) tr[0] = 0;
-                                    for (int i = tq; i <= Mx; i += 4) {
+#pragma unroll
+                                    for (int i0 = 0; i0 <= Mx; i0 += 4) {
+                                        const int i = i0 + tq;
                                         const int r = carrier_at(sT[i], a, b);
                                         tr[carrier_slot(B, i, false)] = (int8_t)r;
-                                        tr[carrier_slot(B, i, true)] = (int8_t)(-r);
+                                        if (B == 4 || i > 0) tr[carrier_slot(B, i, true)] = (int8_t)(-r);
                                     }
                                 };
-                                if constexpr (G == 128) {
-                                    if (JH == 0) build_row(g, p_lo.y); else build_row(g + 8, p_hi.y);
-                                    named_barrier_sync(1 + rb, 64);
-                                } else {
-                                    build_row(g, p_lo.y);
-                                    build_row(g + 8, p_hi.y);
-                                    __syncwarp();
-                                }
+                                build_row(g, p_lo.y);
+                                build_row(g + 8, p_hi.y);
+                                __syncwarp();
                             }
                             // carriers of the group's 32-wide k blocks, straight into the MMA operand order
                             // (a8_row_regs): lane tq holds bytes 8 tq .. 8 tq + 7 of block m for rows g and g + 8
-                            const int8_t *t_lo = tab + g * NCODE, *t_hi = tab + (g + 8) * NCODE;
-                            uint4 tab_lo = make_uint4(0, 0, 0, 0), tab_hi = make_uint4(0, 0, 0, 0);
-                            if constexpr (B == 4) {
-                                tab_lo = *reinterpret_cast<const uint4 *>(t_lo);
-                                tab_hi = *reinterpret_cast<const uint4 *>(t_hi);
-                            } else if constexpr (B == 3) {
-                                const uint2 v0 = *reinterpret_cast<const uint2 *>(t_lo), v1 = *reinterpret_cast<const uint2 *>(t_hi);
-                                tab_lo.x = v0.x; tab_lo.y = v0.y; tab_hi.x = v1.x; tab_hi.y = v1.y;
-                            }
-                            static_for<CPGH / 2>([&](auto mc) {
-                                constexpr int MI = 2 * JH + decltype(gc)::value * (CPGH / 2) + decltype(mc)::value;
+                            CarrierTab tab_lo{}, tab_hi{};
+                            if constexpr (carrier_by_table(B)) { tab_lo = load_carrier_tab<B>(tab + g * NCODE); tab_hi = load_carrier_tab<B>(tab + (g + 8) * NCODE); }
+                            static_for<MPG>([&](auto mc) {
+                                constexpr int MI = gi * MPG + decltype(mc)::value;
                                 uint2 lo, hi;
                                 a8_row_regs<B, 0, MI>(w, tab_lo, lo.x, lo.y);
                                 a8_row_regs<B, 1, MI>(w, tab_hi, hi.x, hi.y);
@@ -329,12 +319,10 @@ gemm_a8_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
                                 *(uint2 *)(row_hi + place(MI)) = hi;
                             });
                         }
-                    });
-                };
-                if (jh == 0) do_half(std::integral_constant<int, 0>{}); else do_half(std::integral_constant<int, 1>{});
+                });
                 fence_proxy_async();
                 __syncwarp();
-                if (lane == 0) { mbar_arrive(&a_full[s]); mbar_arrive(&raw_empty[rs]); }
+                if (lane == 0) { mbar_arrive(&st_full[s]); mbar_arrive(&raw_empty[rs]); }
             }
             if (t >= 1) {
                 // ---------------- (b) drain block t - 1
@@ -472,9 +460,9 @@ cudaError_t launch_a8(const GroupTable &groups, const Dims &d, const int8_t *x8,
     p.groups = groups; p.dx = dx; p.y = y; p.status = status; p.d = d;
     p.partial = partial; p.counters = counters; p.f16 = act_f16;
     p.raw_stage_bytes = (d.tile_bytes + 1023) / 1024 * 1024;
-    static_assert(A8_STAGES == 2 && A8_A_STAGE_BYTES == 128 * 128 && A8_SRING == 8, "a8_fixed_smem spells these out");
+    static_assert(A8_A_STAGE_BYTES == 128 * 128 && A8_SRING == 8, "a8_fixed_smem and a8_stages spell these out");
     if (p.raw_stage_bytes != a8_raw_stage_bytes(B, G)) return cudaErrorInvalidConfiguration;
-    const size_t smem = (size_t)a8_fixed_smem(B, G, BN) + (size_t)a8_raw_stages(B, G, BN) * p.raw_stage_bytes;
+    const size_t smem = (size_t)a8_fixed_smem(B, G) + (size_t)a8_stages(B, G, BN) * (A8_A_STAGE_BYTES + BN * 128) + (size_t)a8_raw_stages(B, G, BN) * p.raw_stage_bytes;
     auto kern = gemm_a8_kernel<B, G, BN>;
     static std::atomic<uint64_t> attr_done{0};   // per kernel instantiation: the devices it has been set on
     cudaError_t ea = ensure_func_attr(kern, attr_done, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);

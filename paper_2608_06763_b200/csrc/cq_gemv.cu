@@ -28,7 +28,7 @@
 // m16n8k16 MMA (fp16 in, fp32 accumulate), the weights' loads landing directly in its A fragment.
 //
 // Dynamic A8 uses the INT8 m16n8k32 MMA on signed carriers (Eq. carrier) taken from a per-(row, group)
-// table indexed by the stored code, in registers and read with byte permutes (B <= 4: a8_row_regs in cq_decode.cuh), or
+// table indexed by the stored code, in registers and read with byte permutes (B <= 5: a8_row_regs in cq_decode.cuh), or
 // evaluated code by code (wider: a8_row_eval); int32 group partials, fp32 rescale (Eq. a8-output).
 #include <cstdlib>
 
@@ -54,7 +54,7 @@ constexpr int MAX_SUB = 16;    // K tiles staged at a time (bounds shared memory
 __host__ __device__ constexpr int gemv_rows(int NT, int MODE) { return MODE == 2 ? NT : 8 * NT; }
 // most shared memory the staged activations (and the Dynamic-A8 carrier tables) of a variant can take
 __host__ __device__ constexpr int gemv_x_bytes_max(int B, int NT, int MODE) {
-    return MODE == 1 ? gemv_rows(NT, MODE) * (MAX_SUB * TILE + XS_PAD8) + (B == 3 || B == 4 ? 8 * 16 * carrier_table_stride(B) : 0)
+    return MODE == 1 ? gemv_rows(NT, MODE) * (MAX_SUB * TILE + XS_PAD8) + (carrier_by_table(B) ? 8 * 16 * carrier_table_stride(B) : 0)
                      : gemv_rows(NT, MODE) * (MAX_SUB * TILE + 2 * XS_PAD) * 2;
 }
 __host__ __device__ constexpr int gemv_smem_budget(int ctas) { return (227 * 1024) / ctas - 2048; }   // dynamic shared memory of a CTA
@@ -240,13 +240,13 @@ __device__ __forceinline__ void group_a8(const TileRegs<B, TILE / G> &r, const i
     const uint2 p_lo = r.prm[0][GI], p_hi = r.prm[1][GI];
     CarrierPoly poly_lo{}, poly_hi{};
     bool fix = false;
-    if constexpr (B >= 5) {
+    if constexpr (B >= 6) {
         poly_lo = carrier_poly(p_lo.y); poly_hi = carrier_poly(p_hi.y);
         fix = __any_sync(0xffffffffu, (p_lo.x | p_hi.x) >> 31);
     }
-    uint4 tab_lo = make_uint4(0, 0, 0, 0), tab_hi = make_uint4(0, 0, 0, 0);
+    CarrierTab tab_lo{}, tab_hi{};
     const int8_t *trow_lo = ctab + g * NE, *trow_hi = ctab + (g + 8) * NE;
-    if constexpr (B == 3 || B == 4) {  // lane (g, t) fills magnitudes i = t mod 4 of rows g and g + 8
+    if constexpr (carrier_by_table(B)) {  // lane (g, t) fills magnitudes i = t mod 4 of rows g and g + 8
         __syncwarp();
         const __half2 ab_lo = as_h2(p_lo.y), ab_hi = as_h2(p_hi.y);
         const float a_lo = __low2float(ab_lo), b_lo = __high2float(ab_lo);
@@ -262,19 +262,14 @@ __device__ __forceinline__ void group_a8(const TileRegs<B, TILE / G> &r, const i
         }
         if (B != 4 && t == 0) { ctab[g * NE] = 0; ctab[(g + 8) * NE] = 0; }   // the reserved pattern (W4: magnitude 0)
         __syncwarp();
-        if constexpr (B == 4) {
-            tab_lo = *reinterpret_cast<const uint4 *>(trow_lo);
-            tab_hi = *reinterpret_cast<const uint4 *>(trow_hi);
-        } else if constexpr (B == 3) {
-            const uint2 v0 = *reinterpret_cast<const uint2 *>(trow_lo), v1 = *reinterpret_cast<const uint2 *>(trow_hi);
-            tab_lo.x = v0.x; tab_lo.y = v0.y; tab_hi.x = v1.x; tab_hi.y = v1.y;
-        }
+        tab_lo = load_carrier_tab<B>(trow_lo);
+        tab_hi = load_carrier_tab<B>(trow_hi);
     }
     int D[NT][4];
     static_for<MPG>([&](auto mc) {
         constexpr int mi = decltype(mc)::value, MI = GI * MPG + mi;
         uint32_t A[4];
-        if constexpr (B <= 4) {
+        if constexpr (B <= 5) {
             a8_row_regs<B, 0, MI>(r.w, tab_lo, A[0], A[2]);
             a8_row_regs<B, 1, MI>(r.w, tab_hi, A[1], A[3]);
         } else if (!fix) {
@@ -614,7 +609,7 @@ gemv_kernel(const uint8_t *__restrict__ layout, Dims d, const uint16_t *__restri
     __shared__ float s_inv[16];
     __shared__ unsigned s_max[16];
     __shared__ int s_last, s_dead;
-    __shared__ float s_t[MODE == 1 && (B == 3 || B == 4) ? 8 : 1];   // Dynamic A8: t_i = i / M of the carrier tables
+    __shared__ float s_t[MODE == 1 && carrier_by_table(B) ? 16 : 1];   // Dynamic A8: t_i = i / M of the carrier tables
     __shared__ __align__(16) uint8_t s_w4[MODE != 1 && B == 4 ? GEMV_WARPS * 256 : 16];   // W4, model dtype: level tables of a warp's 16 rows
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
@@ -634,7 +629,7 @@ gemv_kernel(const uint8_t *__restrict__ layout, Dims d, const uint16_t *__restri
     if (threadIdx.x < 32) tc::fence_barrier_init();
     if (threadIdx.x == 0) s_dead = 0;
     if (threadIdx.x < 16) { s_max[threadIdx.x] = 0; s_inv[threadIdx.x] = 1.0f; }
-    if constexpr (MODE == 1 && (B == 3 || B == 4)) {
+    if constexpr (MODE == 1 && carrier_by_table(B)) {
         if (threadIdx.x < L) s_t[threadIdx.x] = __fdiv_rn((float)threadIdx.x, (float)(L - 1));
     }
     __syncthreads();
@@ -674,7 +669,7 @@ gemv_kernel(const uint8_t *__restrict__ layout, Dims d, const uint16_t *__restri
         ctab = reinterpret_cast<int8_t *>(s_w4) + warp * 256;
         w4_t0 = (float)(2 * t) / 7.0f; w4_t1 = (float)(2 * t + 1) / 7.0f;
     }
-    if constexpr (MODE == 1 && (B == 3 || B == 4)) ctab = reinterpret_cast<int8_t *>(smem) + M * (MAX_SUB * TILE + XS_PAD8) + warp * 16 * carrier_table_stride(B);
+    if constexpr (MODE == 1 && carrier_by_table(B)) ctab = reinterpret_cast<int8_t *>(smem) + M * (MAX_SUB * TILE + XS_PAD8) + warp * 16 * carrier_table_stride(B);
 
     int st = 0, prev_st = 0;            // ring stage of the next tile (and of the one before it)
     uint32_t ph = 0, prev_ph = 0;       // and the parity its "full" barrier completes with
@@ -988,7 +983,7 @@ cudaError_t launch_one(const void *layout, const Dims &d, const uint16_t *x, con
     if (sub64 > MAX_SUB) sub64 = MAX_SUB;
     const int sub_tiles = (int)sub64;
     const int XS = sub_tiles * TILE + (B == 3 || B == 4 ? 2 * XS_PAD : XS_PAD);
-    size_t xbytes = MODE != 1 ? (size_t)M * XS * 2 : (size_t)M * (MAX_SUB * TILE + XS_PAD8) + (B == 3 || B == 4 ? 8 * 16 * carrier_table_stride(B) : 0);
+    size_t xbytes = MODE != 1 ? (size_t)M * XS * 2 : (size_t)M * (MAX_SUB * TILE + XS_PAD8) + (carrier_by_table(B) ? 8 * 16 * carrier_table_stride(B) : 0);
     const uint32_t ring_off = (uint32_t)((xbytes + 127) / 128 * 128);
     constexpr int OCC = gemv_occ(B, G, NT, MODE);
     int nstage = 0;
