@@ -364,8 +364,6 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
 #pragma unroll
                 for (int i = 0; i < GPT; ++i) { q_lo[i] = *(const uint2 *)(prow + i * 8); q_hi[i] = *(const uint2 *)(prow + (8 * GPT + i) * 8); }
             }
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&raw_empty[rs]);   // all of it is in registers
             W3Table w3_lo{}, w3_hi{};   // W3: level tables of rows g and g + 8; one per tile when the group spans it
             if constexpr (B == 3 && G == 128) {
                 w3_lo = w3_table(q_lo[0], prm.f16);
@@ -484,6 +482,10 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
                 __syncwarp();
                 if (lane == 0) { arrive(&full[(2 * tcnt) % STAGES]); arrive(&full[(2 * tcnt + 1) % STAGES]); }
             }
+            // The raw tile goes back when the whole of it has been used, not when it is in registers: where registers are short
+            // (W8) the compiler may read parts of it again.
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&raw_empty[rs]);
         }
         // ----- epilogue of the segment: TMEM lane = output channel, column = token
         wait(acc_full, segc & 1, 7);
