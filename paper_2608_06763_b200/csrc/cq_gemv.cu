@@ -581,22 +581,11 @@ __device__ __forceinline__ void ring_wait(uint64_t *bar, uint32_t parity, volati
 // ------------------------------------------------------------------------------------------
 // MODE 0: model dtype (MMA, NT blocks of 8 tokens).  MODE 1: Dynamic A8 (xq = int8 carrier [M][x8_pitch],
 // dxs = row scales).  MODE 2: model dtype without MMA for NT = M <= 2 tokens.
-// GRP: blockIdx.y is a group of a routed product, with its own matrix, rows and slice of the workspace.
-template <int B, int G, int NT, int MODE, bool GRP>
-__global__ void __launch_bounds__(GEMV_THREADS, gemv_occ(B, G, NT, MODE))
-gemv_kernel(const uint8_t *__restrict__ layout, Dims d, const uint16_t *__restrict__ x, const int8_t *__restrict__ xq,
-            int64_t x8_pitch, const float *__restrict__ dxs, uint16_t *__restrict__ y, int M, int E,
-            float *__restrict__ partial, int *__restrict__ counters, int nstage, uint32_t ring_off, int *__restrict__ status, bool xf16,
-            const __grid_constant__ GroupTable groups) {
-    if constexpr (GRP) {
-        const Group &gr = groups.g[blockIdx.y];
-        layout = (const uint8_t *)gr.layout;
-        M = gr.rows;
-        if constexpr (MODE == 1) { xq += (int64_t)gr.row0 * x8_pitch; dxs += gr.row0; } else x += (int64_t)gr.row0 * d.K;
-        y += (int64_t)gr.row0 * d.N;
-        partial += (size_t)blockIdx.y * gridDim.x * 2 * (8 * NT * TILE);
-        counters += (int64_t)blockIdx.y * d.NB;
-    }
+template <int B, int G, int NT, int MODE>
+__device__ __forceinline__ void
+gemv_body(const uint8_t *__restrict__ layout, const Dims &d, const uint16_t *__restrict__ x, const int8_t *__restrict__ xq,
+          int64_t x8_pitch, const float *__restrict__ dxs, uint16_t *__restrict__ y, int M, int E,
+          float *__restrict__ partial, int *__restrict__ counters, int nstage, uint32_t ring_off, int *__restrict__ status, bool xf16) {
     constexpr int GPT = TILE / G;
     constexpr int L = B == 1 ? 1 : (1 << (B - 1));
     constexpr bool RING = gemv_uses_ring(B, G, NT, MODE);
@@ -972,6 +961,28 @@ gemv_kernel(const uint8_t *__restrict__ layout, Dims d, const uint16_t *__restri
     }
 }
 
+template <int B, int G, int NT, int MODE>
+__global__ void __launch_bounds__(GEMV_THREADS, gemv_occ(B, G, NT, MODE))
+gemv_kernel(const uint8_t *__restrict__ layout, Dims d, const uint16_t *__restrict__ x, const int8_t *__restrict__ xq,
+            int64_t x8_pitch, const float *__restrict__ dxs, uint16_t *__restrict__ y, int M, int E,
+            float *__restrict__ partial, int *__restrict__ counters, int nstage, uint32_t ring_off, int *__restrict__ status, bool xf16) {
+    gemv_body<B, G, NT, MODE>(layout, d, x, xq, x8_pitch, dxs, y, M, E, partial, counters, nstage, ring_off, status, xf16);
+}
+
+// Routed products: blockIdx.y is a group, with its own matrix, rows and slice of the workspace.  (A kernel of its own:
+// the table among the parameters of every small product cost the sweep over formats at M = 1 four per cent.)
+template <int B, int G, int NT, int MODE>
+__global__ void __launch_bounds__(GEMV_THREADS, gemv_occ(B, G, NT, MODE))
+gemv_groups_kernel(Dims d, const uint16_t *__restrict__ x, const int8_t *__restrict__ xq, int64_t x8_pitch, const float *__restrict__ dxs,
+                   uint16_t *__restrict__ y, int E, float *__restrict__ partial, int *__restrict__ counters, int nstage, uint32_t ring_off,
+                   int *__restrict__ status, bool xf16, const __grid_constant__ GroupTable groups) {
+    const Group &gr = groups.g[blockIdx.y];
+    if constexpr (MODE == 1) { xq += (int64_t)gr.row0 * x8_pitch; dxs += gr.row0; } else x += (int64_t)gr.row0 * d.K;
+    gemv_body<B, G, NT, MODE>((const uint8_t *)gr.layout, d, x, xq, x8_pitch, dxs, y + (int64_t)gr.row0 * d.N, gr.rows, E,
+                              partial + (size_t)blockIdx.y * gridDim.x * 2 * (8 * NT * TILE), counters + (int64_t)blockIdx.y * d.NB,
+                              nstage, ring_off, status, xf16);
+}
+
 template <int B, int G, int NT, int MODE, bool GRP = false>
 cudaError_t launch_one(const void *layout, const Dims &d, const uint16_t *x, const int8_t *xq, int64_t x8_pitch,
                        const float *dxs, uint16_t *y, int M, int P, int max_run, int E, float *partial, int *counters,
@@ -994,9 +1005,10 @@ cudaError_t launch_one(const void *layout, const Dims &d, const uint16_t *x, con
         if (nstage < 2) return cudaErrorInvalidConfiguration;
     }
     const size_t smem = ring_off + (size_t)nstage * TB;
-    auto kern = gemv_kernel<B, G, NT, MODE, GRP>;
     static std::atomic<uint64_t> attr_done{0};
-    cudaError_t e = ensure_func_attr(kern, attr_done, cudaFuncAttributeMaxDynamicSharedMemorySize, gemv_smem_budget(OCC));
+    cudaError_t e;
+    if constexpr (GRP) e = ensure_func_attr(gemv_groups_kernel<B, G, NT, MODE>, attr_done, cudaFuncAttributeMaxDynamicSharedMemorySize, gemv_smem_budget(OCC));
+    else e = ensure_func_attr(gemv_kernel<B, G, NT, MODE>, attr_done, cudaFuncAttributeMaxDynamicSharedMemorySize, gemv_smem_budget(OCC));
     if (e != cudaSuccess) return e;
     // Programmatic dependent launch: this kernel may begin (and prefetch weights) while the previous
     // kernel of the stream drains; it waits for that kernel before touching anything but the weights.
@@ -1011,9 +1023,12 @@ cudaError_t launch_one(const void *layout, const Dims &d, const uint16_t *x, con
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = use_pdl ? 1 : 0;
-    static const GroupTable none = {};
-    return cudaLaunchKernelEx(&cfg, kern, (const uint8_t *)layout, d, x, xq, x8_pitch, dxs, y, M, E, partial, counters, nstage,
-                              ring_off, status, act_f16, GRP ? *groups : none);
+    if constexpr (GRP)
+        return cudaLaunchKernelEx(&cfg, gemv_groups_kernel<B, G, NT, MODE>, d, x, xq, x8_pitch, dxs, y, E, partial, counters, nstage, ring_off, status,
+                                  act_f16, *groups);
+    else
+        return cudaLaunchKernelEx(&cfg, gemv_kernel<B, G, NT, MODE>, (const uint8_t *)layout, d, x, xq, x8_pitch, dxs, y, M, E, partial, counters, nstage,
+                                  ring_off, status, act_f16);
 }
 
 template <int B, int G>
