@@ -29,8 +29,10 @@
 //     pw = 8: word p / 2, byte p % 2
 //   W4 is laid out for table look-ups: the stored code is sign and magnitude (u = k for k >= 0, 8 | -k below, 8 the
 //   reserved pattern), so its low three bits select one of eight levels; lane l = 4*g + t owns eight CONSECUTIVE k of
-//   each 32-wide block w, k = 32 w + 8 t + i, as nibble i of word 2 w + r (row g + 8 r).  A half-word is the selector of
-//   four neighbouring weights, and a lane's word decodes to 16 consecutive bytes of a K-major 16-bit operand row.
+//   each 32-wide block w, k = 32 w + 8 t + i, in word 2 w + r (row g + 8 r): the magnitude in the low three bits of nibble
+//   i, so that a half-word is the selector of four neighbouring weights; the sign in the fourth bit of some nibble, where it
+//   falls on the top bit of the byte its weight is looked up into (w4_sign_bit).  A lane's word decodes to 16
+//   consecutive bytes of a K-major 16-bit operand row.
 //   A lane's 2B words are stored as 16-byte quads, quad Q of lane l at ((Q * 32) + l) * 16 inside
 //   the row block (then an 8-byte tail when 2B is not a multiple of 4), so every warp load is one
 //   contiguous 512- or 256-byte run.
@@ -104,7 +106,10 @@ __host__ __device__ inline int word_byte_offset(int B, int W, int lane) {
     return nfq * 512 + lane * 8 + (W - 4 * nfq) * 4;
 }
 
-// Where the field of weight (r, kk) of a tile lives in a plane of width pw: row block, lane, word inside the plane, bit.
+// W4: bit of the sign of weight i of a word: the top bit of byte i for the first half-word, one nibble lower for the second.
+__host__ __device__ constexpr int w4_sign_bit(int i) { return i < 4 ? 8 * i + 7 : 8 * (i - 4) + 3; }
+
+// Where the field (W4: the magnitude) of weight (r, kk) of a tile lives in a plane of width pw: row block, lane, word inside the plane, bit.
 struct Slot { int rb, lane, word, pos; };
 __host__ __device__ inline Slot slot_of(int B, int pw, int r, int kk) {
     Slot s;
@@ -176,6 +181,7 @@ __device__ inline unsigned fetch_u(const void *layout, const Dims &d, int64_t n,
         const Slot s = slot_of(d.B, pw, (int)(n & 127), (int)(k & 127));
         const int W = plane_word_base(d.B, i) + s.word;
         const uint32_t w = *(const uint32_t *)(tile + s.rb * 256 * d.B + word_byte_offset(d.B, W, s.lane));
+        if (d.B == 4) return ((w >> s.pos) & 7u) | (((w >> w4_sign_bit((int)(k & 7))) & 1u) << 3);
         u |= ((w >> s.pos) & ((1u << pw) - 1u)) << plane_bit_offset(d.B, i);
     }
     return u;

@@ -194,15 +194,14 @@ __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {
 // ---- W4, model dtype: eight levels of a (row, group) as 16-bit values, their low bytes in t.x (magnitudes 0-3) and
 // t.y (4-7), their high bytes in t.z and t.w.  A half-word of the layout is the selector of four neighbouring
 // weights; two byte permutes fetch their low and high bytes, two more put the bytes together, and the sign bits
-// go into the high bytes by one exclusive or.  Fifteen integer instructions for eight weights, against some forty for
+// go into the high bytes by one exclusive or.  Thirteen integer instructions for eight weights, against some forty for
 // the half2 polynomial, its scale in fp32 and the rounding to the operand's type; the levels themselves are evaluated in fp32
 // and rounded once.  Measured on the linears of an 8B layer, G = 128: M = 1 66.6 -> 59.3 us, M = 13 109.7 -> 105.5,
 // M = 200 (binary16) 194.8 -> 167.7, M = 1024 509.5 -> 491.6 (what is left there is not the decode).  out[i] = weights (2 i, 2 i + 1) of the word, in k order; a reserved code reads (minus) zero.
 __device__ __forceinline__ void w4_block(uint32_t word, const uint4 &t, uint32_t (&out)[4]) {
     const uint32_t sel = word & 0x77777777u, sel1 = sel >> 16, w4 = word << 4;
-    const uint32_t m0 = prmt(w4, word, 0xD9C8u), m1 = prmt(w4, word, 0xFBEAu);   // 0xFF where the code is negative
-    const uint32_t l0 = prmt(t.x, t.y, sel), h0 = prmt(t.z, t.w, sel) ^ (m0 & 0x80808080u);
-    const uint32_t l1 = prmt(t.x, t.y, sel1), h1 = prmt(t.z, t.w, sel1) ^ (m1 & 0x80808080u);
+    const uint32_t l0 = prmt(t.x, t.y, sel), h0 = prmt(t.z, t.w, sel) ^ (word & 0x80808080u);
+    const uint32_t l1 = prmt(t.x, t.y, sel1), h1 = prmt(t.z, t.w, sel1) ^ (w4 & 0x80808080u);
     out[0] = prmt(l0, h0, 0x5140u); out[1] = prmt(l0, h0, 0x7362u);
     out[2] = prmt(l1, h1, 0x5140u); out[3] = prmt(l1, h1, 0x7362u);
 }
@@ -229,7 +228,7 @@ __device__ __forceinline__ void w4_put(uint8_t *row, uint2 p, int t, float t0, f
 // sign and the reserved pattern (u = 0 -> 0) are part of the table:
 //   B = 4: the table's two 8-byte halves (positive, negative) live in registers; a half-word of four
 //          codes, masked to 3 bits each, is the selector of a byte permute into each half, and the
-//          codes' top bits (expanded to byte masks by two sign-replicating permutes) pick between them; its order
+//          sign bits (expanded to byte masks by two sign-replicating permutes) pick between them; its order
 //          inside the block is the natural one, lane t holding bytes 8 t .. 8 t + 7;
 //   B = 3: one 8-byte table, the selector assembled from the 2-bit and the 1-bit plane;
 //   B <= 2: the carriers are 0 / +-127, a constant table;
@@ -262,7 +261,7 @@ __device__ __forceinline__ void a8_row_regs(const uint32_t (&w)[2 * B], const Ca
     } else if constexpr (B == 4) {
         const uint32_t word = w[2 * MI + RR];
         const uint32_t ws = word & 0x77777777u, wh = ws >> 16, w4 = word << 4;
-        const uint32_t m_lo = prmt(w4, word, 0xD9C8u), m_hi = prmt(w4, word, 0xFBEAu);   // 0xFF where the code is negative
+        const uint32_t m_lo = prmt(word, word, 0xBA98u), m_hi = prmt(w4, w4, 0xBA98u);   // 0xFF where the code is negative
         const uint32_t n_lo = prmt(tab.x, tab.y, ws), p_lo = prmt(tab.z, tab.w, ws);
         const uint32_t n_hi = prmt(tab.x, tab.y, wh), p_hi = prmt(tab.z, tab.w, wh);
         lo = (p_lo & m_lo) | (n_lo & ~m_lo);

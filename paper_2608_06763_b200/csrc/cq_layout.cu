@@ -1,5 +1,7 @@
 // Format kernels: canonical <-> device layout, debug decoders, and the Dynamic-A8 activation
 // quantiser.  All of them are one-time or test-side operations except cq::launch_quantize_a8.
+#include <type_traits>
+
 #include "cq_common.cuh"
 #include "cq_internal.h"
 #include "cq_tc_ptx.cuh"
@@ -30,7 +32,8 @@ __device__ __forceinline__ unsigned field_from_stored(int B, unsigned u) {
 
 // ---------------------------------------------------------------- cq_pack_codes
 // one thread per output byte: gathers the bits of the (up to 8) fields that touch it
-__global__ void pack_codes_kernel(const int8_t *__restrict__ k, int B, int64_t N, int64_t K, int64_t row_bytes,
+template <int B>
+__global__ void pack_codes_kernel(const int8_t *__restrict__ k, int64_t N, int64_t K, int64_t row_bytes,
                                   uint8_t *__restrict__ codes) {
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= N * row_bytes) return;
@@ -49,7 +52,9 @@ __global__ void pack_codes_kernel(const int8_t *__restrict__ k, int B, int64_t N
 
 // ---------------------------------------------------------------- cq_repack
 // one thread per 32-bit code word of the layout
+template <int B>
 __global__ void repack_codes_kernel(const uint8_t *__restrict__ codes, Dims d, int64_t row_bytes, uint8_t *__restrict__ layout) {
+    d.B = B; d.code_bytes = 2048 * B;   // known here: field positions are then constants
     const int words_per_rb = 64 * d.B;   // 32 lanes * 2B words
     const int words_per_tile = 8 * words_per_rb;
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -74,7 +79,8 @@ __global__ void repack_codes_kernel(const uint8_t *__restrict__ codes, Dims d, i
             unsigned u;
             if (n < d.N && k < d.K) u = stored_from_field(d.B, canonical_field(codes + n * row_bytes, k, d.B, row_bytes));
             else u = (d.B == 1) ? 1u : stored_from_field(d.B, 0u);  // padding: code 0 (W1: +1), its scale is 0
-            word |= ((u >> bo) & ((1u << pw) - 1u)) << (q * pw + 16 * half);
+            if (d.B == 4) word |= ((u & 7u) << (4 * (q + 4 * half))) | ((u >> 3) << w4_sign_bit(q + 4 * half));
+            else word |= ((u >> bo) & ((1u << pw) - 1u)) << (q * pw + 16 * half);
         }
     }
     uint8_t *dst = layout + (size_t)tile * d.tile_bytes + rb * 256 * d.B + word_byte_offset(d.B, W, lane);
@@ -113,7 +119,9 @@ __global__ void repack_params_kernel(const uint8_t *__restrict__ codes, const fl
 
 // ---------------------------------------------------------------- cq_unpack
 // one thread per canonical byte
+template <int B>
 __global__ void unpack_codes_kernel(const void *__restrict__ layout, Dims d, int64_t row_bytes, uint8_t *__restrict__ codes) {
+    d.B = B;
     const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= d.N * row_bytes) return;
     const int64_t n = idx / row_bytes, byte = idx % row_bytes;
@@ -401,9 +409,24 @@ __global__ void __launch_bounds__(1024) swiglu_quantize_a8_kernel(const uint16_t
 // ---------------------------------------------------------------- launchers
 static inline unsigned blocks_for(int64_t n, int t) { return (unsigned)((n + t - 1) / t); }
 
+// f(std::integral_constant<int, B>) for the width at hand
+template <class F>
+static void with_width(int B, F &&f) {
+    switch (B) {
+        case 1: f(std::integral_constant<int, 1>{}); break;
+        case 2: f(std::integral_constant<int, 2>{}); break;
+        case 3: f(std::integral_constant<int, 3>{}); break;
+        case 4: f(std::integral_constant<int, 4>{}); break;
+        case 5: f(std::integral_constant<int, 5>{}); break;
+        case 6: f(std::integral_constant<int, 6>{}); break;
+        case 7: f(std::integral_constant<int, 7>{}); break;
+        default: f(std::integral_constant<int, 8>{}); break;
+    }
+}
+
 cudaError_t launch_pack_codes(const int8_t *k, int B, int64_t N, int64_t K, uint8_t *codes, cudaStream_t st) {
     const int64_t rbts = (K * B + 7) / 8;
-    pack_codes_kernel<<<blocks_for(N * rbts, 256), 256, 0, st>>>(k, B, N, K, rbts, codes);
+    with_width(B, [&](auto w) { pack_codes_kernel<decltype(w)::value><<<blocks_for(N * rbts, 256), 256, 0, st>>>(k, N, K, rbts, codes); });
     return cudaGetLastError();
 }
 
@@ -411,7 +434,7 @@ cudaError_t launch_repack(const uint8_t *codes, const float *scale, const uint16
                           void *layout, cudaStream_t st) {
     const int64_t rbts = (d.K * d.B + 7) / 8;
     const int64_t words = (int64_t)d.NB * d.KT * 8 * 64 * d.B;
-    repack_codes_kernel<<<blocks_for(words, 256), 256, 0, st>>>(codes, d, rbts, (uint8_t *)layout);
+    with_width(d.B, [&](auto w) { repack_codes_kernel<decltype(w)::value><<<blocks_for(words, 256), 256, 0, st>>>(codes, d, rbts, (uint8_t *)layout); });
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const int64_t recs = (int64_t)d.NB * d.KT * TILE * d.gpt;
@@ -422,7 +445,7 @@ cudaError_t launch_repack(const uint8_t *codes, const float *scale, const uint16
 cudaError_t launch_unpack(const void *layout, const Dims &d, uint8_t *codes, float *scale, uint16_t *a, uint16_t *b,
                           cudaStream_t st) {
     const int64_t rbts = (d.K * d.B + 7) / 8;
-    unpack_codes_kernel<<<blocks_for(d.N * rbts, 256), 256, 0, st>>>(layout, d, rbts, codes);
+    with_width(d.B, [&](auto w) { unpack_codes_kernel<decltype(w)::value><<<blocks_for(d.N * rbts, 256), 256, 0, st>>>(layout, d, rbts, codes); });
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     unpack_params_kernel<<<blocks_for(d.N * (d.K / d.G), 256), 256, 0, st>>>(layout, d, scale, a, b);
