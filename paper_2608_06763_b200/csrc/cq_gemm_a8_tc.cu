@@ -76,7 +76,7 @@ constexpr int a8_stages(int B, int G, int BN) {
 }
 constexpr int a8_raw_stages(int B, int G, int BN) {
     const int n = (226 * 1024 - a8_fixed_smem(B, G) - a8_stages(B, G, BN) * (128 * 128 + BN * 128)) / a8_raw_stage_bytes(B, G);
-    return n > 6 ? 6 : n;
+    return n > 6 ? 6 : n & ~1;   // even: a stage belongs to one set of decoders, which sees every phase of its barrier
 }
 constexpr int A8_SRING = 8;      // ring of per-block scale snapshots for the drain warps
 constexpr int A8_A_STAGE_BYTES = 128 * 128;

@@ -119,7 +119,9 @@ constexpr int tc_stages(int B, int G, int BN, int NACC) {
 constexpr int tc_ring_bytes(int B, int G, int BN, int NACC) { return tc_stages(B, G, BN, NACC) * (A_STAGE_BYTES + tc_b_stage_bytes(BN, NACC)); }
 constexpr int tc_raw_stages(int B, int G, int BN, int NACC) {
     const int n = (TC_SMEM - tc_table_bytes(B) - tc_ring_bytes(B, G, BN, NACC)) / tc_raw_stage_bytes(B, G);
-    return n > 6 ? 6 : n < 2 ? 2 : n;
+    // an even number: a stage then belongs to one decoder set, which sees every phase of its barrier (a wait tells two phases
+    // apart, so a set that skipped one could take a tile that is still being copied for its own)
+    return n > 6 ? 6 : n < 2 ? 2 : n & ~1;
 }
 
 __device__ __forceinline__ void named_barrier_sync(int id, int threads) {
