@@ -320,7 +320,7 @@ gemm_a8_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
                             });
                         }
                 });
-                fence_proxy_async();
+                fence_proxy_async();   // the operand's stores for the MMAs, and the loads of the raw tile for the copy that refills it
                 __syncwarp();
                 if (lane == 0) { mbar_arrive(&st_full[s]); mbar_arrive(&raw_empty[rs]); }
             }

@@ -484,8 +484,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
                 __syncwarp();
                 if (lane == 0) { arrive(&full[(2 * tcnt) % STAGES]); arrive(&full[(2 * tcnt + 1) % STAGES]); }
             }
-            // The raw tile goes back when the whole of it has been used, not when it is in registers: where registers are short
-            // (W8) the compiler may read parts of it again.
+            // The raw tile goes back behind the proxy fence that the operand's stores need: it orders the loads above before
+            // the copy that refills the tile (release_read_stage).  Handed back right after those loads, without a fence,
+            // a block of sixteen channels was wrong in one run of three at W8, 6144 x 4096, 1024 tokens.
             __syncwarp();
             if (lane == 0) mbar_arrive(&raw_empty[rs]);
         }

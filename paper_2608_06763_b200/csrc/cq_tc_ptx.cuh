@@ -53,6 +53,15 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, int *s
 }
 __device__ __forceinline__ void fence_barrier_init() { asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory"); }
 __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+// Hands a shared-memory stage that the lanes of this warp have read with ordinary loads back to the thread that refills it
+// with a bulk copy.  The loads go through the generic proxy, the copy writes through the async proxy, and only a proxy
+// fence on the way from the one to the other orders them; the arrival and the warp barrier do not.  Each lane fences its
+// own loads.
+__device__ __forceinline__ void release_read_stage(uint64_t *bar, int lane) {
+    fence_proxy_async();
+    __syncwarp();
+    if (lane == 0) mbar_arrive(bar);
+}
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 

@@ -291,8 +291,8 @@ def test_pairs_of_ctas(N, K, M, B, G):
 
 @pytest.mark.parametrize("B,N,M", [(8, 6144, 1024), (7, 4096, 512), (8, 6144, 200)])
 def test_repeated_calls_agree_bit_for_bit(B, N, M):
-    # whole tiles of a wide code, whose decoders are short of registers: nothing may be read again from a raw tile that has
-    # been handed back (one run in three differed in a block of sixteen channels when the tile went back early)
+    # a raw tile is refilled by a bulk copy as soon as it is handed back: what its readers had loaded must be ordered before
+    # that (one run in three of the first shape differed in a block of sixteen channels when no proxy fence stood between)
     c = logical_case(N, 4096, B, 128, seed=230)
     x = x_to_device(datagen.activations(M, 4096, seed=231, outlier_cols=0.01))
     ws = torch.zeros(cq.cq_workspace_bytes(B, 128, M, N, 4096, 0), dtype=torch.uint8, device="cuda")
@@ -300,3 +300,27 @@ def test_repeated_calls_agree_bit_for_bit(B, N, M):
     for _ in range(40):
         assert torch.equal(cq.cq_gemm(c.pw, x, 0, ws).view(torch.int16), y0.view(torch.int16))
     assert cq.cq_gemm_status(ws) == 0
+
+
+@pytest.mark.parametrize("mode", [cq.CQ_MODEL_DTYPE, cq.CQ_DYN_A8])
+@pytest.mark.parametrize("M", [1, 2, 8, 16])
+@pytest.mark.parametrize("B,G", [(5, 128), (6, 64), (7, 128), (1, 32), (3, 32), (4, 32), (8, 32)])
+def test_small_m_ring_repeats_bit_for_bit(B, G, M, mode):
+    # the variants whose tiles come through a shared-memory ring (G = 32, widths of several planes): more tiles to a CTA than
+    # the ring has stages, so that stages are refilled while other warps still read theirs
+    N, K = 8192, 4096
+    c = logical_case(256, K, B, G, seed=240 + B)
+    rep = lambda t: t.repeat((N // 256,) + (1,) * (t.dim() - 1)).contiguous()
+    pw = cq.cq_repack(rep(c.d_codes), rep(c.d_s), rep(c.d_a), rep(c.d_b), B, G, N, K)
+    xb = datagen.activations(M, K, seed=241, outlier_cols=0.01)
+    x = x_to_device(xb)
+    ws = torch.zeros(cq.cq_workspace_bytes(B, G, M, N, K, mode), dtype=torch.uint8, device="cuda")
+    y0 = cq.cq_gemm(pw, x, mode, ws).clone()
+    for _ in range(30):
+        assert torch.equal(cq.cq_gemm(pw, x, mode, ws).view(torch.int16), y0.view(torch.int16))
+    assert cq.cq_gemm_status(ws) == 0
+    if mode == cq.CQ_MODEL_DTYPE:
+        ref = oracle.gemm_model(c.codes, c.s, c.a, c.b, B, G, K, xb)
+    else:
+        ref = oracle.gemm_a8(c.codes, c.s, c.a, c.b, B, G, K, *oracle.quantize_a8(xb))
+    check_y(y_to_numpy(y0), np.tile(ref, (1, N // 256)), f"ring B={B} G={G} M={M} mode={mode}")   # every block of 256 channels is the same matrix
