@@ -103,18 +103,25 @@ struct TcParams {
 //
 // The operand ring: a stage is one 64-wide k block, the decoded weights (16 KB) and the activations, filled behind one
 // barrier and freed by one commit (the issuing thread is on the critical path at small token tiles: with a barrier
-// and a commit for each operand it spent 560 cycles on a block of 256 cycles of MMA).  As deep as shared memory
-// allows beside two or three raw tiles, which take what is left, up to six.
+// and a commit for each operand it spent 560 cycles on a block of 256 cycles of MMA).  Up to eight stages beside four raw
+// tiles (two where a stage holds 512 tokens); raw tiles take what is left, up to six.
 constexpr bool tc_pair(int BN) { return BN == 256; }
 constexpr int tc_b_stage_bytes(int BN, int NACC) { return NACC * (tc_pair(BN) ? BN / 2 : BN) * 128; }
 constexpr int tc_raw_stage_bytes(int B, int G) { return (2048 * B + 1024 * (TILE / G) + 1023) / 1024 * 1024; }
 constexpr int tc_table_bytes(int B) { return B == 4 ? DEC_WARPS * W4_TABLE_BYTES : 0; }
 constexpr int TC_SMEM = 226 * 1024 - 512;
-constexpr int tc_stages(int B, int G, int BN, int NACC) {
-    const int st = A_STAGE_BYTES + tc_b_stage_bytes(BN, NACC), room = TC_SMEM - tc_table_bytes(B);
-    int n = (room - 3 * tc_raw_stage_bytes(B, G)) / st;
-    if (n < 4) n = (room - 2 * tc_raw_stage_bytes(B, G)) / st;
+// Stages that fit beside `raw` raw tiles.
+constexpr int tc_stages_beside(int B, int G, int BN, int NACC, int raw) {
+    const int n = (TC_SMEM - tc_table_bytes(B) - raw * tc_raw_stage_bytes(B, G)) / (A_STAGE_BYTES + tc_b_stage_bytes(BN, NACC));
     return n > 8 ? 8 : n;
+}
+// Two raw tiles for each of the two decoder sets wherever four operand stages remain beside them: with one, a set that has
+// used its tile waits a whole copy for the next.  (Spending that memory on a fifth to eighth operand stage instead had made
+// wide codes slower than before the rings were joined.  W8 G128, before / one raw tile / two: 28672 x 4096, 64 tokens 69.3 /
+// 74.7 / 60.3 us, 256 tokens 81.3 / 91.0 / 68.5; 4096 x 14336, 64 tokens 39.3 / 42.7 / 34.4, 256 tokens 50.2 / 53.7 / 45.2.)
+constexpr int tc_stages(int B, int G, int BN, int NACC) {
+    const int n = tc_stages_beside(B, G, BN, NACC, 4);
+    return n >= 4 ? n : tc_stages_beside(B, G, BN, NACC, 2);
 }
 constexpr int tc_ring_bytes(int B, int G, int BN, int NACC) { return tc_stages(B, G, BN, NACC) * (A_STAGE_BYTES + tc_b_stage_bytes(BN, NACC)); }
 constexpr int tc_raw_stages(int B, int G, int BN, int NACC) {
@@ -122,6 +129,14 @@ constexpr int tc_raw_stages(int B, int G, int BN, int NACC) {
     // an even number: a stage then belongs to one decoder set, which sees every phase of its barrier (a wait tells two phases
     // apart, so a set that skipped one could take a tile that is still being copied for its own)
     return n > 6 ? 6 : n < 2 ? 2 : n & ~1;
+}
+// The rings a kernel is compiled with.  Four raw tiles, or else fewer than four stages would be left (stages of 48 KB, nowhere else).
+// Operand stages: at least three, because a set waits for every second pair of blocks only, and its last wait has to tell it
+// that the stage's phase before the one it waits for is over.
+constexpr bool tc_rings_ok(int B, int G, int BN, int NACC) {
+    const int st = tc_stages(B, G, BN, NACC), raw = tc_raw_stages(B, G, BN, NACC);
+    return st >= 3 && raw % 2 == 0 && (raw >= 4 ? true : st >= 4 && A_STAGE_BYTES + tc_b_stage_bytes(BN, NACC) >= 48 * 1024)
+        && tc_ring_bytes(B, G, BN, NACC) + raw * tc_raw_stage_bytes(B, G) + tc_table_bytes(B) + 512 <= 227 * 1024;
 }
 
 __device__ __forceinline__ void named_barrier_sync(int id, int threads) {
@@ -659,7 +674,7 @@ cudaError_t launch_bn(const GroupTable &groups, const Dims &d, const uint16_t *x
     constexpr int RAW_STAGES = tc_raw_stages(B, G, BN, NACC);
     if (p.raw_stage_bytes != tc_raw_stage_bytes(B, G)) return cudaErrorInvalidConfiguration;
     const size_t smem = (size_t)tc_ring_bytes(B, G, BN, NACC) + (size_t)RAW_STAGES * p.raw_stage_bytes + tc_table_bytes(B) + 512;
-    static_assert(tc_ring_bytes(B, G, BN, NACC) + tc_raw_stages(B, G, BN, NACC) * tc_raw_stage_bytes(B, G) + tc_table_bytes(B) + 512 <= 227 * 1024 && tc_stages(B, G, BN, NACC) >= 3, "shared memory");
+    static_assert(tc_rings_ok(B, G, BN, NACC), "rings");
     auto kern = gemm_tc_kernel<B, G, BN, NACC, SK>;
     static std::atomic<uint64_t> attr_done{0};   // per kernel instantiation: the devices it has been set on
     cudaError_t ea = ensure_func_attr(kern, attr_done, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);

@@ -302,6 +302,24 @@ def test_repeated_calls_agree_bit_for_bit(B, N, M):
     assert cq.cq_gemm_status(ws) == 0
 
 
+# one shape for every depth of the rings that the kernel is compiled with (operand stages / raw tiles)
+@pytest.mark.parametrize("B,G,M", [(1, 128, 20), (8, 128, 20), (1, 32, 40), (8, 64, 40), (3, 32, 100), (8, 128, 100), (2, 128, 200), (4, 128, 200), (7, 32, 200),
+                                   (2, 64, 500), (4, 128, 500), (7, 32, 500)])
+def test_rings_of_every_depth_repeat_bit_for_bit(B, G, M):
+    N, K = 2048, 4096
+    c = logical_case(256, K, B, G, seed=250 + B)
+    rep = lambda t: t.repeat((N // 256,) + (1,) * (t.dim() - 1)).contiguous()
+    pw = cq.cq_repack(rep(c.d_codes), rep(c.d_s), rep(c.d_a), rep(c.d_b), B, G, N, K)
+    xb = datagen.activations(M, K, seed=251, outlier_cols=0.01)
+    x = x_to_device(xb)
+    ws = torch.zeros(cq.cq_workspace_bytes(B, G, M, N, K, 0), dtype=torch.uint8, device="cuda")
+    y0 = cq.cq_gemm(pw, x, 0, ws).clone()
+    for _ in range(30):
+        assert torch.equal(cq.cq_gemm(pw, x, 0, ws).view(torch.int16), y0.view(torch.int16))
+    assert cq.cq_gemm_status(ws) == 0
+    check_y(y_to_numpy(y0), np.tile(oracle.gemm_model(c.codes, c.s, c.a, c.b, B, G, K, xb), (1, N // 256)), f"rings B={B} G={G} M={M}")
+
+
 @pytest.mark.parametrize("mode", [cq.CQ_MODEL_DTYPE, cq.CQ_DYN_A8])
 @pytest.mark.parametrize("M", [1, 2, 8, 16])
 @pytest.mark.parametrize("B,G", [(5, 128), (6, 64), (7, 128), (1, 32), (3, 32), (4, 32), (8, 32)])
