@@ -24,7 +24,8 @@
  *       a, b   fp16   [N][K/G]         shape coefficients as IEEE binary16 bit patterns
  *   - Device layout: private, tiled and interleaved for 128-bit coalesced loads with the
  *     group parameters stored beside the codes of their tile; produced by cq_repack and
- *     inverted bit-exactly by cq_unpack.
+ *     inverted bit-exactly by cq_unpack.  It changes between versions of the library: store the
+ *     canonical form and repack it when a model is loaded.
  *   - Supported: B in 1..8; G in {32, 64, 128, 256, 512}; K % G == 0; M, N, K >= 1.  K and N need
  *     not be multiples of the 128 x 128 tile (the layout pads).  For G = 256 / 512 the device layout
  *     repeats a group's parameter record in each of its 128-wide tiles, so it is 8 (G/128 - 1) bytes
@@ -130,8 +131,11 @@ int cq_mlp_swiglu(const void *layout_gate_up, int B_gate_up, int G_gate_up, cons
  *                         [expert_offset[e], expert_offset[e+1])
  *     expert_offset_host  HOST int64 [E + 1], non-decreasing, [0] = 0, [E] = R
  *     x [T][K], y_routes [R][N] (route-major output, model dtype); act_f16 as for cq_mlp_swiglu
- * One gather kernel, then one ordinary cq_gemm dispatch per matrix that has routes, on `stream`.  A token index outside
- * [0, T) yields a zero input row.  workspace: cq_routed_workspace_bytes() bytes, zeroed once with cq_workspace_init.
+ * On `stream`: one gather kernel, then the matrices that have routes, sorted by their row counts into classes; the
+ * matrices of a class (up to 32) share a launch, one by itself is an ordinary cq_gemm dispatch.  A token index outside
+ * [0, T) yields a zero input row.  workspace: cq_routed_workspace_bytes() bytes for these offsets; it need not be
+ * initialised, each call zeroes what it counts in and the status word: cq_gemm_status(workspace) reports the bounded waits
+ * of the LAST routed call on it, whichever launch gave up, so ask after each call whose result matters.
  * Errors as cq_gemm; CQ_ERR_INVALID_ARG for an inconsistent offset array; N and K must be multiples of 8. */
 size_t cq_routed_workspace_bytes(int B, int G, int E, const int64_t *expert_offset_host, int64_t N, int64_t K, int mode);
 int cq_gemm_routed(const void *const *layouts_host, int E, int B, int G, const uint16_t *x, const int32_t *route_token,
@@ -212,6 +216,14 @@ int cq_debug_wait_timeout(void *workspace, size_t workspace_bytes, int64_t limit
  * tiles, plan[4] = 1 when a run may cross from one tile into the next, 0 when every shared tile is cut into the same
  * number of runs (always 0 in CQ_DYN_A8).  CQ_ERR_INVALID_ARG for M <= 16, an unknown mode or a null pointer. */
 int cq_debug_gemm_plan(int B, int G, int64_t M, int64_t N, int64_t K, int mode, int64_t *plan);
+
+/* The launches that cq_gemm_routed makes after its gather for this routing on the current device (host-side query, launches
+ * nothing; the paper has no counterpart).  Returns their number, or a negative CQ_ERR_* code; for each of the first
+ * max_launches five values go to `launches`: the class of row counts (0: at most 16 rows; else tokens per output tile),
+ * the matrices that share the launch, the largest row count among them, the CTAs of each matrix (class 0 with several
+ * matrices, else 0), and the byte offset in the workspace of the status word that the launch reports into. */
+int cq_debug_routed_plan(int B, int G, int E, const int64_t *expert_offset_host, int64_t N, int64_t K, int mode, int64_t *launches,
+                         int max_launches);
 
 /* ---- Offline encoder (the step before the hot path; Sections 4.1 and 4.3) --------------------------
  * W[N][K] float, logical signed codes k[N][K] int8 (what cq_pack_codes takes), scale[N][K/G] float,

@@ -71,6 +71,8 @@ def lib():
         L.cq_debug_a8_partials.argtypes = [vp, i, i, vp, i64, i64, i64, vp, vp]
         L.cq_debug_gemm_plan.argtypes = [i, i, i64, i64, i64, i, vp]
         L.cq_debug_gemm_plan.restype = i
+        L.cq_debug_routed_plan.argtypes = [i, i, i, vp, i64, i64, i, vp, i]
+        L.cq_debug_routed_plan.restype = i
         L.cq_debug_wait_timeout.argtypes = [vp, sz, i64, vp]
         L.cq_debug_wait_timeout.restype = i
         L.cq_encode_assign.argtypes = [vp, i, i, i64, i64, vp, vp, vp, i, vp, vp]
@@ -296,6 +298,17 @@ def cq_debug_gemm_plan(B: int, G: int, M: int, N: int, K: int, mode: int = CQ_MO
     _check(lib().cq_debug_gemm_plan(B, G, M, N, K, mode, out), "cq_debug_gemm_plan")
     return {"token_tile": out[0], "whole_tile_ctas": out[1], "stream_k_ctas": out[2], "stream_k_tiles": out[3],
             "runs_cross_tiles": bool(out[4])}
+
+
+def cq_debug_routed_plan(B: int, G: int, expert_offset, N: int, K: int, mode: int = CQ_MODEL_DTYPE) -> list:
+    """The launches of cq_gemm_routed after its gather, for this routing on the current device."""
+    E = len(expert_offset) - 1
+    off = (C.c_int64 * (E + 1))(*[int(v) for v in expert_offset])
+    out = (C.c_int64 * (5 * E))()
+    n = lib().cq_debug_routed_plan(B, G, E, off, N, K, mode, out, E)
+    _check(min(n, 0), "cq_debug_routed_plan")
+    names = ("row_class", "matrices", "max_rows", "ctas_per_matrix", "status_offset")
+    return [dict(zip(names, out[5 * j:5 * j + 5])) for j in range(n)]
 
 
 def cq_debug_wait_timeout(workspace: torch.Tensor, limit_cycles: int = 2_000_000):

@@ -145,6 +145,14 @@ int cq_unpack(const void *layout, int B, int G, int64_t N, int64_t K, uint8_t *c
     return wrap(launch_unpack(layout, make_dims(B, G, N, K), codes, scale, a, b, (cudaStream_t)stream));
 }
 
+// One product in the workspace that `plan` lays out from ws.
+static cudaError_t launch_product(const void *layout, const Dims &d, const uint16_t *x, uint16_t *y, int64_t M, int mode, bool act_f16,
+                                  uint8_t *ws, const Workspace &plan, cudaStream_t s) {
+    if (M <= 16) return launch_gemv(layout, d, x, y, M, mode, act_f16, ws, plan, s);
+    if (mode == CQ_MODEL_DTYPE) return launch_gemm_tc(layout, d, x, y, M, mode, act_f16, ws, plan, s);
+    return launch_gemm_a8_tc(layout, d, x, y, M, act_f16, ws, plan, s);
+}
+
 static int gemm_any(const void *layout, int B, int G, const uint16_t *x, uint16_t *y, int64_t M, int64_t N, int64_t K,
                     int mode, bool act_f16, void *workspace, size_t workspace_bytes, void *stream) {
     if (!layout || !x || !y || !workspace || M <= 0) return CQ_ERR_INVALID_ARG;
@@ -157,11 +165,7 @@ static int gemm_any(const void *layout, int B, int G, const uint16_t *x, uint16_
     if (workspace_bytes < plan.total) return CQ_ERR_WORKSPACE;
     st = check_arch();
     if (st != CQ_OK) return st;
-    cudaStream_t s = (cudaStream_t)stream;
-    uint8_t *ws = (uint8_t *)workspace;
-    if (M <= 16) return wrap(launch_gemv(layout, d, x, y, M, mode, act_f16, ws, plan, s));
-    if (mode == CQ_MODEL_DTYPE) return wrap(launch_gemm_tc(layout, d, x, y, M, mode, act_f16, ws, plan, s));
-    return wrap(launch_gemm_a8_tc(layout, d, x, y, M, act_f16, ws, plan, s));
+    return wrap(launch_product(layout, d, x, y, M, mode, act_f16, (uint8_t *)workspace, plan, (cudaStream_t)stream));
 }
 
 int cq_gemm(const void *layout, int B, int G, const uint16_t *x, uint16_t *y, int64_t M, int64_t N, int64_t K,
@@ -217,10 +221,7 @@ int cq_mlp_swiglu(const void *layout_gate_up, int B_gu, int G_gu, const void *la
     uint16_t *h = reinterpret_cast<uint16_t *>(ws + plan.h_off);
     const bool f16 = act_f16 != 0;
     // 1. gate_up, an ordinary operator: model-dtype output
-    cudaError_t e;
-    if (M <= 16) e = launch_gemv(layout_gate_up, dgu, x, h, M, mode_gate_up, f16, ws, plan.gu, s);
-    else if (mode_gate_up == CQ_MODEL_DTYPE) e = launch_gemm_tc(layout_gate_up, dgu, x, h, M, mode_gate_up, f16, ws, plan.gu, s);
-    else e = launch_gemm_a8_tc(layout_gate_up, dgu, x, h, M, f16, ws, plan.gu, s);
+    cudaError_t e = launch_product(layout_gate_up, dgu, x, h, M, mode_gate_up, f16, ws, plan.gu, s);
     if (e != cudaSuccess) return wrap(e);
     // 2. gated activation and the down projection's activation quantiser in one kernel
     e = launch_swiglu_quantize_a8(h, M, I, reinterpret_cast<int8_t *>(ws + plan.dn.x8_off), (int64_t)ddn.KT * TILE,
@@ -235,15 +236,12 @@ int cq_mlp_swiglu(const void *layout_gate_up, int B_gu, int G_gu, const void *la
 // Routed product.  The groups (matrices with routes) are sorted into classes of token tiles, and a class of several
 // groups is one launch: up to 16 rows the small-M kernel, above it the GEMM, the token tiles up to 128 together (its time is
 // the decode of the weights there, not the tokens) and 256 and 512 by themselves; Dynamic A8 keeps one class per token
-// tile, whose drain grows with the tile.  A class of one group is an ordinary product, which may share its tiles along K.
-// Sixteen matrices of 2816 x 2048 (W4 G64, 384 routes): one after another 192 us, most of it launches that leave SMs idle; 61 us so.
-// Workspace: [status][gathered rows: R x K][Dynamic A8: INT8 carrier of all rows, row scales][small-M groups: counters and
-// partial sums][the largest workspace of an ordinary product].
-struct RoutedPlan {
-    size_t xg_off, x8_off, dx_off, ctr_off, part_off, sub_off, total;
-    int P;           // CTAs of a small-M group
-    int n_small;     // groups of at most 16 rows
-};
+// tile, whose drain grows with the tile.  A group by itself is an ordinary product, which may share its tiles along K.
+// Sixteen matrices of 2816 x 2048 (W4 G64, 384 routes): one after another 203 us, most of it launches that leave SMs idle; 61 us so.
+// Workspace: [status][gathered rows: R x K][Dynamic A8: INT8 carrier of all rows, row scales][arrival counters][partial sums
+// of the small-M groups][what else an ordinary product needs].  Every launch reports into the one status word at the
+// front, and every launch leaves the arrival counters at zero for the next one; the gather zeroes both.
+struct RoutedPlan { size_t xg_off, x8_off, dx_off, ctr_off, ctr_bytes, part_off, sub_off, total; };
 static bool routed_offsets_ok(const int64_t *off, int E, int64_t R) {
     if (!off || off[0] != 0 || off[E] != R) return false;
     for (int e = 0; e < E; ++e) if (off[e + 1] < off[e]) return false;
@@ -255,39 +253,78 @@ static int routed_class(const Dims &d, int64_t m, int mode) {   // 0: small M; e
     const int t = gemm_tc_token_tile(m);
     return t < 128 ? 128 : t;
 }
-static const int ROUTED_CLASSES[6] = {0, 32, 64, 128, 256, 512};   // every value of routed_class
+static const int ROUTED_CLASSES[5] = {0, 64, 128, 256, 512};   // every value of routed_class
+// The launches that follow the gather, in order: f(groups, class, largest row count, CTAs of a small-M group).  A table of one
+// group is an ordinary product.  The sizes, the launches themselves and cq_debug_routed_plan all walk this.
+extern "C++" {
+template <class F>
+static int for_routed_launches(const Dims &d, const void *const *layouts, const int64_t *off, int E, int mode, F &&f) {
+    int in_class = 0;   // matrices of the class at hand
+    auto emit = [&](const GroupTable &t, int cls, int64_t max_rows) -> int {
+        if (t.n == 0) return CQ_OK;
+        // small-M groups share the places of the whole GPU; a run of fewer than four tiles is mostly overhead
+        const int64_t T = (int64_t)d.NB * d.KT, places = cls == 0 ? gemv_plan(d, 16, mode).ctas : 0;
+        int64_t P = places / in_class;
+        if (P > T / 4) P = T / 4;
+        return f(t, cls, max_rows, (int)(P < 1 ? 1 : P));
+    };
+    for (int cls : ROUTED_CLASSES) {
+        GroupTable t{};
+        int64_t max_rows = 0;
+        in_class = 0;
+        for (int e = 0; e < E; ++e) if (off[e + 1] > off[e] && routed_class(d, off[e + 1] - off[e], mode) == cls) ++in_class;
+        for (int e = 0; e < E; ++e) {
+            const int64_t r0 = off[e], m = off[e + 1] - r0;
+            if (m == 0 || routed_class(d, m, mode) != cls) continue;
+            t.g[t.n++] = {layouts ? layouts[e] : nullptr, (int)r0, (int)m, 0};
+            if (m > max_rows) max_rows = m;
+            if (t.n == MAX_GROUPS) {
+                const int st = emit(t, cls, max_rows);
+                if (st != CQ_OK) return st;
+                t.n = 0; max_rows = 0;
+            }
+        }
+        const int st = emit(t, cls, max_rows);
+        if (st != CQ_OK) return st;
+    }
+    return CQ_OK;
+}
+}  // extern "C++"
 static RoutedPlan plan_routed(const Dims &d, const int64_t *off, int E, int mode) {
     RoutedPlan p{};
     const int64_t R = off[E];
-    size_t sub = 0, o = 256;
-    for (int cls : ROUTED_CLASSES) {
-        int n = 0;
-        int64_t last = 0;
-        for (int e = 0; e < E; ++e) {
-            const int64_t m = off[e + 1] - off[e];
-            if (m > 0 && routed_class(d, m, mode) == cls) { ++n; last = m; }
+    size_t ctr = 0, part = 0, sub = 0;
+    bool together = false;
+    auto most = [](size_t &v, size_t x) { if (x > v) v = x; };
+    for_routed_launches(d, nullptr, off, E, mode, [&](const GroupTable &t, int cls, int64_t max_rows, int P) -> int {
+        if (t.n == 1) {
+            const Workspace w = plan_workspace(d, max_rows, mode);
+            most(ctr, w.counters_bytes);
+            most(sub, w.total - w.partial_off);
+        } else {
+            together = true;
+            if (cls == 0) { most(ctr, (size_t)t.n * d.NB * 4); most(part, (size_t)t.n * P * 2 * 16 * TILE * 4); }
         }
-        if (cls == 0) p.n_small = n;
-        if (n % MAX_GROUPS == 1) { const size_t t = plan_workspace(d, last, mode).total; if (t > sub) sub = t; }   // launched by itself
-    }
+        return CQ_OK;
+    });
+    size_t o = 256;
     p.xg_off = o; o += align_up((size_t)R * d.K * 2, 256);
-    if (mode == CQ_DYN_A8) {
+    if (mode == CQ_DYN_A8 && together) {
         p.x8_off = o; o += align_up((size_t)R * d.KT * TILE, 256);
         p.dx_off = o; o += align_up((size_t)R * 4, 256);
     }
-    if (p.n_small > 1) {
-        // the groups share the places of the whole GPU; a run of fewer than four tiles is mostly overhead
-        const int64_t T = (int64_t)d.NB * d.KT, places = gemv_plan(d, 16, mode).ctas;
-        int64_t P = places / p.n_small;
-        if (P > T / 4) P = T / 4;
-        p.P = (int)(P < 1 ? 1 : P);
-        const size_t n = p.n_small < MAX_GROUPS ? p.n_small : MAX_GROUPS;
-        p.ctr_off = o; o += align_up(n * d.NB * 4, 256);
-        p.part_off = o; o += align_up(n * p.P * 2 * 16 * TILE * 4, 256);
-    }
-    p.sub_off = o;
-    p.total = o + sub;
+    p.ctr_off = o; p.ctr_bytes = align_up(ctr, 256); o += p.ctr_bytes;
+    p.part_off = o; o += align_up(part, 256);
+    p.sub_off = o; o += align_up(sub, 256);
+    p.total = o;
     return p;
+}
+// the workspace of an ordinary product of m rows inside that of the routed call
+static Workspace routed_product_workspace(const RoutedPlan &p, const Dims &d, int64_t m, int mode) {
+    Workspace w = plan_workspace(d, m, mode);
+    w.x8_off += p.sub_off - w.partial_off; w.dx_off += p.sub_off - w.partial_off;
+    w.partial_off = p.sub_off; w.counters_off = p.ctr_off; w.status_off = 0;
+    return w;
 }
 
 size_t cq_routed_workspace_bytes(int B, int G, int E, const int64_t *expert_offset_host, int64_t N, int64_t K, int mode) {
@@ -319,56 +356,30 @@ int cq_gemm_routed(const void *const *layouts_host, int E, int B, int G, const u
     if (st != CQ_OK) return st;
     cudaStream_t s = (cudaStream_t)stream;
     uint8_t *ws = (uint8_t *)workspace;
-    int *status = reinterpret_cast<int *>(ws);
+    int *status = reinterpret_cast<int *>(ws), *counters = reinterpret_cast<int *>(ws + plan.ctr_off);
     uint16_t *xg = reinterpret_cast<uint16_t *>(ws + plan.xg_off);
     int8_t *xq = reinterpret_cast<int8_t *>(ws + plan.x8_off);
     float *dxs = reinterpret_cast<float *>(ws + plan.dx_off);
     const bool f16 = act_f16 != 0;
-    // the gather also zeroes the status word and the groups' arrival counters: which words these are changes with the routing
-    cudaError_t err = launch_gather_rows(x, route_token, xg, R, T, K, status, reinterpret_cast<int *>(ws + plan.ctr_off),
-                                         (int64_t)(plan.part_off - plan.ctr_off) / 4, s);
+    // the gather also zeroes the status word and the arrival counters: which words these are changes with the routing
+    const cudaError_t err = launch_gather_rows(x, route_token, xg, R, T, K, status, counters, (int64_t)plan.ctr_bytes / 4, s);
     if (err != cudaSuccess) return wrap(err);
     bool quantised = false;
-    auto flush = [&](const GroupTable &t, int cls, int64_t max_rows) -> int {   // one class, up to MAX_GROUPS groups
-        if (t.n == 0) return CQ_OK;
+    return for_routed_launches(d, layouts_host, expert_offset_host, E, mode, [&](const GroupTable &t, int cls, int64_t max_rows, int P) -> int {
         if (t.n == 1) {
             const Group &g = t.g[0];
-            const cudaError_t e = cudaMemsetAsync(ws + plan.sub_off, 0, 256 + plan_workspace(d, g.rows, mode).counters_bytes, s);
-            if (e != cudaSuccess) return wrap(e);
-            return gemm_any(g.layout, B, G, xg + (int64_t)g.row0 * K, y_routes + (int64_t)g.row0 * N, g.rows, N, K, mode, f16,
-                            ws + plan.sub_off, plan.total - plan.sub_off, stream);
+            return wrap(launch_product(g.layout, d, xg + (int64_t)g.row0 * K, y_routes + (int64_t)g.row0 * N, g.rows, mode, f16, ws,
+                                       routed_product_workspace(plan, d, g.rows, mode), s));
         }
         if (mode == CQ_DYN_A8 && !quantised) {
             const cudaError_t e = launch_quantize_a8(xg, R, K, xq, (int64_t)d.KT * TILE, dxs, B != 4, f16, s);
             if (e != cudaSuccess) return wrap(e);
             quantised = true;
         }
-        if (cls == 0) {
-            // every launch leaves the arrival counters at zero
-            return wrap(launch_gemv_groups(t, d, xg, xq, dxs, y_routes, mode, f16, plan.P, reinterpret_cast<float *>(ws + plan.part_off),
-                                           reinterpret_cast<int *>(ws + plan.ctr_off), status, s));
-        }
+        if (cls == 0) return wrap(launch_gemv_groups(t, d, xg, xq, dxs, y_routes, mode, f16, P, reinterpret_cast<float *>(ws + plan.part_off), counters, status, s));
         if (mode == CQ_MODEL_DTYPE) return wrap(launch_gemm_tc_groups(t, d, xg, y_routes, R, max_rows, f16, status, s));
         return wrap(launch_gemm_a8_groups(t, d, xq, dxs, y_routes, R, max_rows, f16, status, s));
-    };
-    for (int cls : ROUTED_CLASSES) {
-        GroupTable t{};
-        int64_t max_rows = 0;
-        for (int e = 0; e < E; ++e) {
-            const int64_t r0 = expert_offset_host[e], m = expert_offset_host[e + 1] - r0;
-            if (m == 0 || routed_class(d, m, mode) != cls) continue;
-            t.g[t.n++] = {layouts_host[e], (int)r0, (int)m, 0};
-            if (m > max_rows) max_rows = m;
-            if (t.n == MAX_GROUPS) {
-                st = flush(t, cls, max_rows);
-                if (st != CQ_OK) return st;
-                t.n = 0; max_rows = 0;
-            }
-        }
-        st = flush(t, cls, max_rows);
-        if (st != CQ_OK) return st;
-    }
-    return CQ_OK;
+    });
 }
 
 int cq_gemm_status(const void *workspace, size_t workspace_bytes, void *stream) {
@@ -489,6 +500,26 @@ int cq_debug_gemm_plan(int B, int G, int64_t M, int64_t N, int64_t K, int mode, 
         plan[0] = ap.bn; plan[1] = ap.t_full; plan[2] = shared * ap.slices; plan[3] = shared; plan[4] = 0;
     }
     return CQ_OK;
+}
+
+int cq_debug_routed_plan(int B, int G, int E, const int64_t *expert_offset_host, int64_t N, int64_t K, int mode, int64_t *launches, int max_launches) {
+    if (E <= 0 || !expert_offset_host || (mode != CQ_MODEL_DTYPE && mode != CQ_DYN_A8) || max_launches < 0 || (max_launches > 0 && !launches)) return CQ_ERR_INVALID_ARG;
+    const int st = check_format(B, G, N, K);
+    if (st != CQ_OK) return st;
+    if (expert_offset_host[E] <= 0 || !routed_offsets_ok(expert_offset_host, E, expert_offset_host[E])) return CQ_ERR_INVALID_ARG;
+    const Dims d = make_dims(B, G, N, K);
+    const RoutedPlan plan = plan_routed(d, expert_offset_host, E, mode);
+    int n = 0;
+    for_routed_launches(d, nullptr, expert_offset_host, E, mode, [&](const GroupTable &t, int cls, int64_t max_rows, int P) -> int {
+        if (n < max_launches) {
+            int64_t *v = launches + 5 * n;
+            v[0] = cls; v[1] = t.n; v[2] = max_rows; v[3] = cls == 0 && t.n > 1 ? P : 0;
+            v[4] = t.n == 1 ? (int64_t)routed_product_workspace(plan, d, max_rows, mode).status_off : 0;   // the launches together report into the front word
+        }
+        ++n;
+        return CQ_OK;
+    });
+    return n;
 }
 
 int cq_debug_wait_timeout(void *workspace, size_t workspace_bytes, int64_t limit_cycles, void *stream) {

@@ -96,3 +96,21 @@ def test_gemm_plan_shares_the_last_round_only_when_it_pays():
     assert ask(4, 128, 300, 200, 512, 1)[2] == 0                      # four blocks of K: nothing to cut
     bn, whole, runs, shared, crossing = ask(4, 128, 100, 200, 2048, 1)
     assert (bn, whole, shared, crossing) == (128, 0, 2, 0) and runs in (4, 6, 8)
+
+
+@pytest.mark.parametrize("mode", [0, 1])
+def test_routed_launches_report_into_the_front_word(mode):
+    """Every launch of a routed call, those of a single matrix too, reports into the word that cq_gemm_status reads."""
+    for counts in ([5], [90], [1, 2, 3], [16] * 33 + [18], [3, 17, 40, 128, 129, 300, 8, 600], [0, 20, 0, 500]):
+        off = [0]
+        for c in counts:
+            off.append(off[-1] + c)
+        launches = cq.cq_debug_routed_plan(4, 128, off, 4096, 4096, mode)
+        assert [v["status_offset"] for v in launches] == [0] * len(launches)
+        assert sum(v["matrices"] for v in launches) == sum(c > 0 for c in counts) and all(v["matrices"] <= 32 for v in launches)
+        assert max(v["max_rows"] for v in launches) == max(counts)
+    L = cq.lib()
+    bad = (ctypes.c_int64 * 3)(0, 3, 2)
+    assert L.cq_debug_routed_plan(4, 128, 2, bad, 128, 256, 0, None, 0) == -1
+    assert L.cq_debug_routed_plan(4, 96, 2, bad, 128, 256, 0, None, 0) == -2
+    assert L.cq_debug_routed_plan(4, 128, 2, (ctypes.c_int64 * 3)(0, 2, 3), 128, 256, 0, None, 0) == 1

@@ -97,3 +97,26 @@ def test_routed_classes_share_launches(B, G, mode):
         for e in range(n):
             if counts[e]:
                 check_y(yn[offset[e]:offset[e + 1]], ref[offset[e]:offset[e + 1]], f"{counts[e]} routes, matrix {e} of {n}")
+
+
+@pytest.mark.parametrize("mode", [cq.CQ_MODEL_DTYPE, cq.CQ_DYN_A8])
+@pytest.mark.parametrize("rows", [5, 90])
+def test_routed_single_matrix_adds_nothing_but_the_gather(rows, mode):
+    # one matrix with routes: the gather, in Dynamic A8 the quantiser, and the product; its counters and its status word are
+    # cleared by the gather and not by operations of their own
+    from cuda.bindings import runtime as rt
+    N, K, T, B, G = 256, 512, 16, 4, 64
+    c = Case(*datagen.logical_quantized(N, K, B, G, 940), B, G)
+    x = torch.from_numpy(datagen.activations(T, K, seed=941).view(np.int16)).cuda().view(torch.bfloat16)
+    tok = torch.arange(rows, dtype=torch.int32, device="cuda") % T
+    ws = torch.full((8 << 20,), 0x5A, dtype=torch.uint8, device="cuda")
+    eager = cq.cq_gemm_routed([c.pw], x, tok, [0, rows], mode, ws).clone()
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        y = cq.cq_gemm_routed([c.pw], x, tok, [0, rows], mode, ws)
+    err, _, n = rt.cudaGraphGetNodes(graph.raw_cuda_graph(), 0)
+    assert int(err) == 0 and n == (2 if mode == cq.CQ_MODEL_DTYPE else 3), n
+    graph.instantiate()
+    ws.fill_(0x5A)
+    graph.replay()
+    assert torch.equal(y.view(torch.int16), eager.view(torch.int16)) and cq.cq_gemm_status(ws) == 0
