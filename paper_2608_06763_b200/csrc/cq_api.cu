@@ -259,20 +259,17 @@ static const int ROUTED_CLASSES[5] = {0, 64, 128, 256, 512};   // every value of
 extern "C++" {
 template <class F>
 static int for_routed_launches(const Dims &d, const void *const *layouts, const int64_t *off, int E, int mode, F &&f) {
-    int in_class = 0;   // matrices of the class at hand
     auto emit = [&](const GroupTable &t, int cls, int64_t max_rows) -> int {
         if (t.n == 0) return CQ_OK;
         // small-M groups share the places of the whole GPU; a run of fewer than four tiles is mostly overhead
         const int64_t T = (int64_t)d.NB * d.KT, places = cls == 0 ? gemv_plan(d, 16, mode).ctas : 0;
-        int64_t P = places / in_class;
+        int64_t P = places / t.n;
         if (P > T / 4) P = T / 4;
         return f(t, cls, max_rows, (int)(P < 1 ? 1 : P));
     };
     for (int cls : ROUTED_CLASSES) {
         GroupTable t{};
         int64_t max_rows = 0;
-        in_class = 0;
-        for (int e = 0; e < E; ++e) if (off[e + 1] > off[e] && routed_class(d, off[e + 1] - off[e], mode) == cls) ++in_class;
         for (int e = 0; e < E; ++e) {
             const int64_t r0 = off[e], m = off[e + 1] - r0;
             if (m == 0 || routed_class(d, m, mode) != cls) continue;

@@ -114,3 +114,15 @@ def test_routed_launches_report_into_the_front_word(mode):
     assert L.cq_debug_routed_plan(4, 128, 2, bad, 128, 256, 0, None, 0) == -1
     assert L.cq_debug_routed_plan(4, 96, 2, bad, 128, 256, 0, None, 0) == -2
     assert L.cq_debug_routed_plan(4, 128, 2, (ctypes.c_int64 * 3)(0, 2, 3), 128, 256, 0, None, 0) == 1
+
+
+@pytest.mark.parametrize("mode", [0, 1])
+def test_routed_small_groups_share_the_places_of_their_own_launch(mode):
+    """Sixty-four or thirty-five small matrices go out as two launches; each launch has the whole GPU to itself."""
+    def places(n):
+        return [v["ctas_per_matrix"] * v["matrices"] for v in cq.cq_debug_routed_plan(4, 128, list(range(0, 6 * n + 1, 6)), 4096, 4096, mode)]
+
+    full = places(32)[0]
+    assert full > 148                                       # thirty-two matrices fill the places once
+    assert places(64) == [full, full]
+    assert places(35)[0] == full and places(35)[1] >= 0.9 * full   # three matrices: a third of the places each
