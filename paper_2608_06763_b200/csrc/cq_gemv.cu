@@ -57,7 +57,11 @@ __host__ __device__ constexpr int gemv_x_bytes_max(int B, int NT, int MODE) {
     return MODE == 1 ? gemv_rows(NT, MODE) * (MAX_SUB * TILE + XS_PAD8) + (carrier_by_table(B) ? 8 * 16 * carrier_table_stride(B) : 0)
                      : gemv_rows(NT, MODE) * (MAX_SUB * TILE + 2 * XS_PAD) * 2;
 }
-__host__ __device__ constexpr int gemv_smem_budget(int ctas) { return (227 * 1024) / ctas - 2048; }   // dynamic shared memory of a CTA
+// shared memory of fixed size in the kernel: barriers, scales and flags; W4 in the model dtype: the warps' level tables
+__host__ __device__ constexpr int gemv_static_bytes(int B, int MODE) { return 512 + (MODE != 1 && B == 4 ? GEMV_WARPS * 256 : 0); }
+// Dynamic shared memory of a CTA when `ctas` share an SM's 228 KB, of which each takes 1 KB for the system.  (With the W4
+// tables left out of the count a ring filled to its limit cost a CTA per SM: 11008 x 4096, W4 G64, two tokens 18.5 -> 20.7 us.)
+__host__ __device__ constexpr int gemv_smem_budget(int B, int MODE, int ctas) { return (227 * 1024) / ctas - 1536 - gemv_static_bytes(B, MODE); }
 // How a CTA's tiles reach the registers.  Straight from global memory into a two- or three-deep register
 // prefetch where that fits the registers (it measured a little faster there); through a shared-memory ring
 // filled by bulk copies where it does not: G = 32 (four parameter records per tile row), the widths made of
@@ -71,7 +75,7 @@ __host__ __device__ constexpr int gemv_occ(int B, int G, int NT, int MODE) {
     if (MODE != 2 && NT == 2) return 2;
     if (!gemv_uses_ring(B, G, NT, MODE)) return CQ_GEMV_CTAS_PER_SM;
     const int tb = 2048 * B + 1024 * (TILE / G);
-    return (gemv_smem_budget(CQ_GEMV_CTAS_PER_SM) - (gemv_x_bytes_max(B, NT, MODE) + 127) / 128 * 128) / tb >= 4 ? CQ_GEMV_CTAS_PER_SM : 2;
+    return (gemv_smem_budget(B, MODE, CQ_GEMV_CTAS_PER_SM) - (gemv_x_bytes_max(B, NT, MODE) + 127) / 128 * 128) / tb >= 4 ? CQ_GEMV_CTAS_PER_SM : 2;
 }
 // the variant that serves M rows in an activation mode
 __host__ __device__ constexpr int gemv_variant_mode(int64_t M, int mode) { return mode == 1 ? 1 : (M <= 2 ? 2 : 0); }
@@ -601,6 +605,8 @@ gemv_body(const uint8_t *__restrict__ layout, const Dims &d, const uint16_t *__r
     __shared__ float s_t[MODE == 1 && carrier_by_table(B) ? 16 : 1];   // Dynamic A8: t_i = i / M of the carrier tables
     __shared__ __align__(16) uint8_t s_w4[MODE != 1 && B == 4 ? GEMV_WARPS * 256 : 16];   // W4, model dtype: level tables of a warp's 16 rows
 
+    static_assert(sizeof(s_full) + sizeof(s_empty) + sizeof(s_inv) + sizeof(s_max) + sizeof(s_last) + sizeof(s_dead) + sizeof(s_t) + sizeof(s_w4) <= gemv_static_bytes(B, MODE) + 16, "gemv_static_bytes");
+    static_assert(gemv_occ(B, G, NT, MODE) * (gemv_smem_budget(B, MODE, gemv_occ(B, G, NT, MODE)) + gemv_static_bytes(B, MODE) + 1024 + 128) <= 228 * 1024, "the resident CTAs' shared memory");
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
     const int VT = d.KT + E;                       // virtual units per row block
     const int64_t V = (int64_t)d.NB * VT, P = gridDim.x;
@@ -1001,7 +1007,7 @@ cudaError_t launch_one(const void *layout, const Dims &d, const uint16_t *x, con
     constexpr int OCC = gemv_occ(B, G, NT, MODE);
     int nstage = 0;
     if (gemv_uses_ring(B, G, NT, MODE)) {
-        nstage = (int)((gemv_smem_budget(OCC) - (int64_t)ring_off) / TB);
+        nstage = (int)((gemv_smem_budget(B, MODE, OCC) - (int64_t)ring_off) / TB);
         if (nstage > MAX_STAGES) nstage = MAX_STAGES;
         if (nstage > max_run) nstage = max_run < 2 ? 2 : max_run;   // a run never holds more tiles than this
         if (nstage < 2) return cudaErrorInvalidConfiguration;
@@ -1009,8 +1015,8 @@ cudaError_t launch_one(const void *layout, const Dims &d, const uint16_t *x, con
     const size_t smem = ring_off + (size_t)nstage * TB;
     static std::atomic<uint64_t> attr_done{0};
     cudaError_t e;
-    if constexpr (GRP) e = ensure_func_attr(gemv_groups_kernel<B, G, NT, MODE>, attr_done, cudaFuncAttributeMaxDynamicSharedMemorySize, gemv_smem_budget(OCC));
-    else e = ensure_func_attr(gemv_kernel<B, G, NT, MODE>, attr_done, cudaFuncAttributeMaxDynamicSharedMemorySize, gemv_smem_budget(OCC));
+    if constexpr (GRP) e = ensure_func_attr(gemv_groups_kernel<B, G, NT, MODE>, attr_done, cudaFuncAttributeMaxDynamicSharedMemorySize, gemv_smem_budget(B, MODE, OCC));
+    else e = ensure_func_attr(gemv_kernel<B, G, NT, MODE>, attr_done, cudaFuncAttributeMaxDynamicSharedMemorySize, gemv_smem_budget(B, MODE, OCC));
     if (e != cudaSuccess) return e;
     // Programmatic dependent launch: this kernel may begin (and prefetch weights) while the previous
     // kernel of the stream drains; it waits for that kernel before touching anything but the weights.
