@@ -308,18 +308,23 @@ __device__ __forceinline__ CarrierPoly carrier_poly(uint32_t ab16) {
     return {f2_dup(a), f2_dup(b), f2_dup(__fsub_rn(__fsub_rn(1.0f, a), b))};
 }
 // Two codes, given as fp32 2^23 + u; the signed carriers come out in the low bytes.
-//   i = |u - 2^(B-1)|, exact; t = i / M as i r + i r', r + r' = 1/M to 48 bits: equal to the correctly rounded quotient for every
-//   i and M of B = 5 .. 8 (checked one by one); q as carrier_at has it; clamping q to [0, 1] before RNE(127 q) is clamping
+//   i = |u - 2^(B-1)|, exact; t = i / M, the correctly rounded quotient for every i > 0 (checked one by one): B = 7 as i r + i r',
+//   r + r' = 1/M to 48 bits; B = 6 and 8 as i r plus a constant that is below half a unit of every quotient and pushes the
+//   few products that round down over the tie (for i = 0 it leaves t = 2^-30 or less, whose carrier is 0 for every a and b in
+//   binary16).  The multiplication saved is what W6 at G = 128 had lost to the 64-entry table it used to read
+//   (4096 square, M = 8: 18.4 us with the table, 20.6 with both products); q as carrier_at has it; clamping q to [0, 1] before RNE(127 q) is clamping
 //   the carrier to [0, 127]; adding 1.5 2^23 rounds to nearest even, leaving the integer in the low bits.
 template <int B, bool FIX>
 __device__ __forceinline__ void carrier_pair(uint32_t f0, uint32_t f1, const CarrierPoly &p, uint32_t &r0, uint32_t &r1) {
     constexpr int L = 1 << (B - 1), M = L - 1;
     constexpr float r_hi = 1.0f / (float)M;
-    constexpr float r_lo = (float)(1.0 / (double)M - (double)r_hi);
+    static_assert(B >= 6 && B <= 8, "");
     uint32_t k0, k1, t0, t1, h0, h1, v0, v1;
     f2_split(f2_add(f2_pack(f0, f1), f2_dup(-(8388608.0f + (float)L))), k0, k1);
     const uint64_t i2 = f2_pack(k0 & 0x7FFFFFFFu, k1 & 0x7FFFFFFFu);
-    const uint64_t t = f2_fma(i2, f2_dup(r_hi), f2_mul(i2, f2_dup(r_lo)));
+    uint64_t t;
+    if constexpr (B == 7) t = f2_fma(i2, f2_dup(r_hi), f2_mul(i2, f2_dup((float)(1.0 / (double)M - (double)r_hi))));
+    else t = f2_fma(i2, f2_dup(r_hi), f2_dup(B == 6 ? 0x1p-30f : 0x1p-32f));
     f2_split(f2_fma(t, f2_fma(t, p.c, p.b), p.a), h0, h1);
     f2_split(t, t0, t1);
     uint32_t q0 = mul_sat(t0, h0), q1 = mul_sat(t1, h1);

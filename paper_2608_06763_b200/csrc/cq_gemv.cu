@@ -73,6 +73,7 @@ __host__ __device__ constexpr bool gemv_uses_ring(int B, int G, int NT, int MODE
 // four stages allow it, otherwise two.
 __host__ __device__ constexpr int gemv_occ(int B, int G, int NT, int MODE) {
     if (MODE != 2 && NT == 2) return 2;
+    if (MODE == 1 && B == 6) return 2;   // W6, 4096 square, Dynamic A8, G = 128, M = 1: 17.7 us with two, 19.1 with three (shorter runs, 80 registers)
     if (!gemv_uses_ring(B, G, NT, MODE)) return CQ_GEMV_CTAS_PER_SM;
     const int tb = 2048 * B + 1024 * (TILE / G);
     return (gemv_smem_budget(B, MODE, CQ_GEMV_CTAS_PER_SM) - (gemv_x_bytes_max(B, NT, MODE) + 127) / 128 * 128) / tb >= 4 ? CQ_GEMV_CTAS_PER_SM : 2;

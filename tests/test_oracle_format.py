@@ -241,3 +241,11 @@ def test_quotient_as_two_products():
         r2 = np.float32(1.0 / M - float(r))
         t = (i.astype(np.float64) * float(r) + (i * r2).astype(np.float64)).astype(np.float32)
         assert np.array_equal(t, i / np.float32(M))
+    # six and eight bits: one product and a constant; the reserved pattern (i = M + 1) stays above 1, and i = 0 gives carrier 0
+    # for the largest a and b that binary16 holds
+    for B, c in ((6, 2.0 ** -30), (8, 2.0 ** -32)):
+        M = (1 << (B - 1)) - 1
+        i = np.arange(M + 2, dtype=np.float64)
+        t = (i * float(np.float32(1) / np.float32(M)) + c).astype(np.float32)
+        assert np.array_equal(t[1:M + 1], np.arange(1, M + 1, dtype=np.float32) / np.float32(M)) and t[M + 1] > 1
+        assert 127 * c * 65504 * (1 + 3 * c * 65504) < 0.5
