@@ -698,7 +698,9 @@ gemv_body(const uint8_t *__restrict__ layout, const Dims &d, const uint16_t *__r
                 first_slice = false;
             }
             // direct variant: the first tiles of the slice are requested before the activations are staged
-            constexpr int NBUF = RING ? 1 : (B <= 4 ? 3 : 2);
+            // (W4, G = 64 with the MMA holds two: with three, 196 bytes of spills at 80 registers, and M = 3 on a 4096 square
+            // took 14.2 us)
+            constexpr int NBUF = RING ? 1 : (B <= 4 && !(B == 4 && G == 64 && MODE == 0) ? 3 : 2);
             const uint8_t *tile0 = layout + ((size_t)nb * d.KT + ks) * (size_t)TB;
             const uint8_t *wl = tile0 + warp * 256 * B + lane * 16;              // next tile to load (codes)
             const uint8_t *pl = tile0 + CB + ((warp * 16 + g) * GPT) * 8;        // next tile to load (params)
