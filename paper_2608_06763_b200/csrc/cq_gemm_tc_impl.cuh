@@ -105,38 +105,38 @@ struct TcParams {
 // barrier and freed by one commit (the issuing thread is on the critical path at small token tiles: with a barrier
 // and a commit for each operand it spent 560 cycles on a block of 256 cycles of MMA).  Up to eight stages beside four raw
 // tiles (two where a stage holds 512 tokens); raw tiles take what is left, up to six.
-constexpr bool tc_pair(int BN) { return BN == 256; }
-constexpr int tc_b_stage_bytes(int BN, int NACC) { return NACC * (tc_pair(BN) ? BN / 2 : BN) * 128; }
+constexpr int tc_b_stage_bytes(int BN, int NACC, bool PAIR) { return NACC * (PAIR ? BN / 2 : BN) * 128; }
 constexpr int tc_raw_stage_bytes(int B, int G) { return (2048 * B + 1024 * (TILE / G) + 1023) / 1024 * 1024; }
 constexpr int tc_table_bytes(int B) { return B == 4 ? DEC_WARPS * W4_TABLE_BYTES : 0; }
 constexpr int TC_SMEM = 226 * 1024 - 512;
 // Stages that fit beside `raw` raw tiles.
-constexpr int tc_stages_beside(int B, int G, int BN, int NACC, int raw) {
-    const int n = (TC_SMEM - tc_table_bytes(B) - raw * tc_raw_stage_bytes(B, G)) / (A_STAGE_BYTES + tc_b_stage_bytes(BN, NACC));
+constexpr int tc_stages_beside(int B, int G, int BN, int NACC, bool PAIR, int raw) {
+    const int n = (TC_SMEM - tc_table_bytes(B) - raw * tc_raw_stage_bytes(B, G)) / (A_STAGE_BYTES + tc_b_stage_bytes(BN, NACC, PAIR));
     return n > 8 ? 8 : n;
 }
-// Two raw tiles for each of the two decoder sets wherever four operand stages remain beside them: with one, a set that has
+// Two raw tiles for each of the two decoder sets, of W4 at 512 tokens only if four operand stages remain beside them (its decode
+// keeps up with the MMAs on one tile and three stages do not): with one, a set that has
 // used its tile waits a whole copy for the next.  (Spending that memory on a fifth to eighth operand stage instead had made
 // wide codes slower than before the rings were joined.  W8 G128, before / one raw tile / two: 28672 x 4096, 64 tokens 69.3 /
 // 74.7 / 60.3 us, 256 tokens 81.3 / 91.0 / 68.5; 4096 x 14336, 64 tokens 39.3 / 42.7 / 34.4, 256 tokens 50.2 / 53.7 / 45.2.)
-constexpr int tc_stages(int B, int G, int BN, int NACC) {
-    const int n = tc_stages_beside(B, G, BN, NACC, 4);
-    return n >= 4 ? n : tc_stages_beside(B, G, BN, NACC, 2);
+constexpr int tc_stages(int B, int G, int BN, int NACC, bool PAIR) {
+    const int n = tc_stages_beside(B, G, BN, NACC, PAIR, 4);
+    return n >= 4 || !(B == 4 && PAIR) ? n : tc_stages_beside(B, G, BN, NACC, PAIR, 2);
 }
-constexpr int tc_ring_bytes(int B, int G, int BN, int NACC) { return tc_stages(B, G, BN, NACC) * (A_STAGE_BYTES + tc_b_stage_bytes(BN, NACC)); }
-constexpr int tc_raw_stages(int B, int G, int BN, int NACC) {
-    const int n = (TC_SMEM - tc_table_bytes(B) - tc_ring_bytes(B, G, BN, NACC)) / tc_raw_stage_bytes(B, G);
+constexpr int tc_ring_bytes(int B, int G, int BN, int NACC, bool PAIR) { return tc_stages(B, G, BN, NACC, PAIR) * (A_STAGE_BYTES + tc_b_stage_bytes(BN, NACC, PAIR)); }
+constexpr int tc_raw_stages(int B, int G, int BN, int NACC, bool PAIR) {
+    const int n = (TC_SMEM - tc_table_bytes(B) - tc_ring_bytes(B, G, BN, NACC, PAIR)) / tc_raw_stage_bytes(B, G);
     // an even number: a stage then belongs to one decoder set, which sees every phase of its barrier (a wait tells two phases
     // apart, so a set that skipped one could take a tile that is still being copied for its own)
     return n > 6 ? 6 : n < 2 ? 2 : n & ~1;
 }
-// The rings a kernel is compiled with.  Four raw tiles, or else fewer than four stages would be left (stages of 48 KB, nowhere else).
+// The rings a kernel is compiled with.
 // Operand stages: at least three, because a set waits for every second pair of blocks only, and its last wait has to tell it
 // that the stage's phase before the one it waits for is over.
-constexpr bool tc_rings_ok(int B, int G, int BN, int NACC) {
-    const int st = tc_stages(B, G, BN, NACC), raw = tc_raw_stages(B, G, BN, NACC);
-    return st >= 3 && raw % 2 == 0 && (raw >= 4 ? true : st >= 4 && A_STAGE_BYTES + tc_b_stage_bytes(BN, NACC) >= 48 * 1024)
-        && tc_ring_bytes(B, G, BN, NACC) + raw * tc_raw_stage_bytes(B, G) + tc_table_bytes(B) + 512 <= 227 * 1024;
+constexpr bool tc_rings_ok(int B, int G, int BN, int NACC, bool PAIR) {
+    const int st = tc_stages(B, G, BN, NACC, PAIR), raw = tc_raw_stages(B, G, BN, NACC, PAIR);
+    return st >= 3 && raw % 2 == 0 && (raw >= 4 || (B == 4 && BN * NACC == 512 && st >= 4))
+        && tc_ring_bytes(B, G, BN, NACC, PAIR) + raw * tc_raw_stage_bytes(B, G) + tc_table_bytes(B) + 512 <= 227 * 1024;
 }
 
 __device__ __forceinline__ void named_barrier_sync(int id, int threads) {
@@ -199,16 +199,15 @@ struct SegWalk {
 
 // One CTA computes tiles of 128 output channels x (NACC * BN) tokens: NACC accumulators of BN columns share
 // every decoded weight tile, which halves the decode work per flop at NACC = 2.
-template <int B, int G, int BN, int NACC, bool SK>
+template <int B, int G, int BN, int NACC, bool PAIR, bool SK>
 __global__ void __launch_bounds__(TC_THREADS, 1)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ TcParams prm) {
     constexpr int GPT = TILE / G;
-    constexpr int STAGES = tc_stages(B, G, BN, NACC);  // ring of 64-wide k blocks
-    constexpr int RAW_STAGES = tc_raw_stages(B, G, BN, NACC);
-    constexpr bool PAIR = tc_pair(BN);
+    constexpr int STAGES = tc_stages(B, G, BN, NACC, PAIR);  // ring of 64-wide k blocks
+    constexpr int RAW_STAGES = tc_raw_stages(B, G, BN, NACC, PAIR);
     constexpr int BROWS = PAIR ? BN / 2 : BN;          // tokens of one TMA box and CTA
     constexpr int B_TILE_BYTES = BROWS * 128;          // one TMA box: BROWS tokens x 64 k
-    constexpr int B_STAGE_BYTES = tc_b_stage_bytes(BN, NACC);
+    constexpr int B_STAGE_BYTES = tc_b_stage_bytes(BN, NACC, PAIR);
     constexpr int BNT = BN * NACC;                     // tokens per tile
     constexpr uint32_t TMEM_COLS = BNT < 32 ? 32 : BNT;
     extern __shared__ __align__(1024) uint8_t smem[];  // 1024-byte alignment is what the swizzled tiles need
@@ -520,7 +519,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
                 // loaded; a CTA with a run of several segments may already be loading the next one) as
                 // [token][128 channels] in the output dtype, and leaves it in 16-byte pieces, eight channels of one
                 // token per thread, instead of one 2-byte store per output.
-                static_assert(BNT * TILE * 2 <= tc_ring_bytes(B, G, BN, NACC), "the tile is staged in the operand ring");
+                static_assert(BNT * TILE * 2 <= tc_ring_bytes(B, G, BN, NACC, PAIR), "the tile is staged in the operand ring");
                 uint16_t *stage = reinterpret_cast<uint16_t *>(smem);
 #pragma unroll 1
                 for (int c0 = cp * 32; c0 < BNT; c0 += 128) {
@@ -641,15 +640,15 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
 }
 
 // ---------------------------------------------------------------- host side
-template <int B, int G, int BN, int NACC, bool SK>
-cudaError_t launch_bn(const GroupTable &groups, const Dims &d, const uint16_t *x, uint16_t *y, int64_t M, int *status,
+template <int B, int G, int BN, int NACC, bool PAIR, bool SK>
+cudaError_t launch_bn(const GroupTable &groups, const Dims &d, const uint16_t *x, uint16_t *y, int64_t M, TcPlan plan, int *status,
                       float *partial, int *counters, bool act_f16, cudaStream_t st) {
     EncodeTiledFn enc = encode_tiled();
     if (!enc) return cudaErrorNotSupported;
     CUtensorMap xmap;
     const cuuint64_t dims[2] = {(cuuint64_t)d.K, (cuuint64_t)M};
     const cuuint64_t strides[1] = {(cuuint64_t)d.K * 2};
-    const cuuint32_t box[2] = {64, (cuuint32_t)(tc_pair(BN) ? BN / 2 : BN)};
+    const cuuint32_t box[2] = {64, (cuuint32_t)(PAIR ? BN / 2 : BN)};
     const cuuint32_t estr[2] = {1, 1};
     if (enc(&xmap, act_f16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<uint16_t *>(x), dims, strides, box, estr,
             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
@@ -657,25 +656,22 @@ cudaError_t launch_bn(const GroupTable &groups, const Dims &d, const uint16_t *x
         return cudaErrorInvalidValue;
     TcParams p;
     p.groups = groups;
-    TcPlan plan;
-    if (counters) {   // an ordinary product; the groups of a routed one are computed in whole tiles and bring no workspace
-        plan = gemm_tc_plan(d, groups.g[0].rows);
-    } else {
-        constexpr int CW = tc_pair(BN) ? 2 : 1;
+    if (!counters) {   // the groups of a routed call are computed in whole tiles and bring no workspace
+        constexpr int CW = PAIR ? 2 : 1;
         const int NBU = (d.NB + CW - 1) / CW;
         int units = 0;
         for (int i = 0; i < groups.n; ++i) { p.groups.g[i].unit0 = units; units += NBU * ((groups.g[i].rows + BN * NACC - 1) / (BN * NACC)); }
-        plan = {BN * NACC, 0, units * CW, 0, 0, 0, CW, units};
+        plan.ctas = units * CW; plan.t_full = units;
     }
-    if (plan.bnt != BN * NACC || (plan.p2 > 0) != SK || (plan.cw == 2) != tc_pair(BN)) return cudaErrorInvalidConfiguration;
+    if (plan.bnt != BN * NACC || (plan.p2 > 0) != SK || (plan.cw == 2) != PAIR) return cudaErrorInvalidConfiguration;
     p.y = y; p.status = status; p.d = d;
     p.raw_stage_bytes = (d.tile_bytes + 1023) / 1024 * 1024;
     p.MT = plan.token_tiles; p.t_full = plan.t_full; p.p2 = plan.p2;
-    constexpr int RAW_STAGES = tc_raw_stages(B, G, BN, NACC);
+    constexpr int RAW_STAGES = tc_raw_stages(B, G, BN, NACC, PAIR);
     if (p.raw_stage_bytes != tc_raw_stage_bytes(B, G)) return cudaErrorInvalidConfiguration;
-    const size_t smem = (size_t)tc_ring_bytes(B, G, BN, NACC) + (size_t)RAW_STAGES * p.raw_stage_bytes + tc_table_bytes(B) + 512;
-    static_assert(tc_rings_ok(B, G, BN, NACC), "rings");
-    auto kern = gemm_tc_kernel<B, G, BN, NACC, SK>;
+    const size_t smem = (size_t)tc_ring_bytes(B, G, BN, NACC, PAIR) + (size_t)RAW_STAGES * p.raw_stage_bytes + tc_table_bytes(B) + 512;
+    static_assert(tc_rings_ok(B, G, BN, NACC, PAIR), "rings");
+    auto kern = gemm_tc_kernel<B, G, BN, NACC, PAIR, SK>;
     static std::atomic<uint64_t> attr_done{0};   // per kernel instantiation: the devices it has been set on
     cudaError_t ea = ensure_func_attr(kern, attr_done, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
     if (ea != cudaSuccess) return ea;
@@ -689,43 +685,47 @@ cudaError_t launch_bn(const GroupTable &groups, const Dims &d, const uint16_t *x
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = tc_pair(BN) ? 1 : 0;
+    cfg.numAttrs = PAIR ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kern, xmap, p);
 }
 
-// M: rows of x; tile_m: the rows whose token tile is taken (of an ordinary product, M)
+// M: rows of x; plan: of the product, or (routed) the token tile of the class
 template <int B, int G, bool SK>
-cudaError_t launch_g(const GroupTable &groups, const Dims &d, const uint16_t *x, uint16_t *y, int64_t M, int64_t tile_m, int *status,
+cudaError_t launch_g(const GroupTable &groups, const Dims &d, const uint16_t *x, uint16_t *y, int64_t M, const TcPlan &plan, int *status,
                      float *partial, int *counters, bool act_f16, cudaStream_t st) {
-    if (tile_m <= 32) return launch_bn<B, G, 32, 1, SK>(groups, d, x, y, M, status, partial, counters, act_f16, st);
-    if (tile_m <= 64) return launch_bn<B, G, 64, 1, SK>(groups, d, x, y, M, status, partial, counters, act_f16, st);
-    if (tile_m <= 128) return launch_bn<B, G, 128, 1, SK>(groups, d, x, y, M, status, partial, counters, act_f16, st);
-    if (tile_m <= 256) return launch_bn<B, G, 256, 1, SK>(groups, d, x, y, M, status, partial, counters, act_f16, st);
-    return launch_bn<B, G, 256, 2, SK>(groups, d, x, y, M, status, partial, counters, act_f16, st);
+    switch (plan.bnt) {
+        case 32: return launch_bn<B, G, 32, 1, false, SK>(groups, d, x, y, M, plan, status, partial, counters, act_f16, st);
+        case 64: return launch_bn<B, G, 64, 1, false, SK>(groups, d, x, y, M, plan, status, partial, counters, act_f16, st);
+        case 128: return launch_bn<B, G, 128, 1, false, SK>(groups, d, x, y, M, plan, status, partial, counters, act_f16, st);
+        case 256:
+            if (plan.cw == 1) return launch_bn<B, G, 256, 1, false, SK>(groups, d, x, y, M, plan, status, partial, counters, act_f16, st);
+            return launch_bn<B, G, 256, 1, true, SK>(groups, d, x, y, M, plan, status, partial, counters, act_f16, st);
+        default: return launch_bn<B, G, 256, 2, true, SK>(groups, d, x, y, M, plan, status, partial, counters, act_f16, st);
+    }
 }
 
 template <int B, bool SK>
-cudaError_t launch_b(const GroupTable &groups, const Dims &d, const uint16_t *x, uint16_t *y, int64_t M, int64_t tile_m, int *status,
+cudaError_t launch_b(const GroupTable &groups, const Dims &d, const uint16_t *x, uint16_t *y, int64_t M, const TcPlan &plan, int *status,
                      float *partial, int *counters, bool act_f16, cudaStream_t st) {
     switch (d.G) {
-        case 32: return launch_g<B, 32, SK>(groups, d, x, y, M, tile_m, status, partial, counters, act_f16, st);
-        case 64: return launch_g<B, 64, SK>(groups, d, x, y, M, tile_m, status, partial, counters, act_f16, st);
-        default: return launch_g<B, 128, SK>(groups, d, x, y, M, tile_m, status, partial, counters, act_f16, st);
+        case 32: return launch_g<B, 32, SK>(groups, d, x, y, M, plan, status, partial, counters, act_f16, st);
+        case 64: return launch_g<B, 64, SK>(groups, d, x, y, M, plan, status, partial, counters, act_f16, st);
+        default: return launch_g<B, 128, SK>(groups, d, x, y, M, plan, status, partial, counters, act_f16, st);
     }
 }
 
 template <bool SK>
-cudaError_t launch_tc_variant(const GroupTable &groups, const Dims &d, const uint16_t *x, uint16_t *y, int64_t M, int64_t tile_m, int *status,
+cudaError_t launch_tc_variant(const GroupTable &groups, const Dims &d, const uint16_t *x, uint16_t *y, int64_t M, const TcPlan &plan, int *status,
                               float *partial, int *counters, bool act_f16, cudaStream_t st) {
     switch (d.B) {
-        case 1: return launch_b<1, SK>(groups, d, x, y, M, tile_m, status, partial, counters, act_f16, st);
-        case 2: return launch_b<2, SK>(groups, d, x, y, M, tile_m, status, partial, counters, act_f16, st);
-        case 3: return launch_b<3, SK>(groups, d, x, y, M, tile_m, status, partial, counters, act_f16, st);
-        case 4: return launch_b<4, SK>(groups, d, x, y, M, tile_m, status, partial, counters, act_f16, st);
-        case 5: return launch_b<5, SK>(groups, d, x, y, M, tile_m, status, partial, counters, act_f16, st);
-        case 6: return launch_b<6, SK>(groups, d, x, y, M, tile_m, status, partial, counters, act_f16, st);
-        case 7: return launch_b<7, SK>(groups, d, x, y, M, tile_m, status, partial, counters, act_f16, st);
-        default: return launch_b<8, SK>(groups, d, x, y, M, tile_m, status, partial, counters, act_f16, st);
+        case 1: return launch_b<1, SK>(groups, d, x, y, M, plan, status, partial, counters, act_f16, st);
+        case 2: return launch_b<2, SK>(groups, d, x, y, M, plan, status, partial, counters, act_f16, st);
+        case 3: return launch_b<3, SK>(groups, d, x, y, M, plan, status, partial, counters, act_f16, st);
+        case 4: return launch_b<4, SK>(groups, d, x, y, M, plan, status, partial, counters, act_f16, st);
+        case 5: return launch_b<5, SK>(groups, d, x, y, M, plan, status, partial, counters, act_f16, st);
+        case 6: return launch_b<6, SK>(groups, d, x, y, M, plan, status, partial, counters, act_f16, st);
+        case 7: return launch_b<7, SK>(groups, d, x, y, M, plan, status, partial, counters, act_f16, st);
+        default: return launch_b<8, SK>(groups, d, x, y, M, plan, status, partial, counters, act_f16, st);
     }
 }
 

@@ -4,9 +4,9 @@
 
 namespace cq {
 
-cudaError_t launch_gemm_tc_streamk(const GroupTable &groups, const Dims &d, const uint16_t *x, uint16_t *y, int64_t M, int *status,
+cudaError_t launch_gemm_tc_streamk(const GroupTable &groups, const Dims &d, const uint16_t *x, uint16_t *y, int64_t M, const TcPlan &plan, int *status,
                                    float *partial, int *counters, bool act_f16, cudaStream_t st) {
-    return launch_tc_variant<true>(groups, d, x, y, M, M, status, partial, counters, act_f16, st);
+    return launch_tc_variant<true>(groups, d, x, y, M, plan, status, partial, counters, act_f16, st);
 }
 
 }  // namespace cq

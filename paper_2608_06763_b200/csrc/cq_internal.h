@@ -89,7 +89,8 @@ cudaError_t launch_gemm_a8_groups(const GroupTable &groups, const Dims &d, const
                                   int64_t tile_m, bool act_f16, int *status, cudaStream_t st);
 int gemm_tc_token_tile(int64_t M);
 // cw: CTAs that compute a tile together (2: a pair, 256 channels); t_full whole tiles and p2 runs are counted in such units
-struct TcPlan { int bnt, token_tiles, ctas, stream_k, p2, crossing, cw; int64_t t_full; };
+// cost: microseconds, rough
+struct TcPlan { int bnt, token_tiles, ctas, stream_k, p2, crossing, cw; int64_t t_full; double cost; };
 TcPlan gemm_tc_plan(const Dims &d, int64_t M);
 int gemm_a8_token_tile(const Dims &d, int64_t M);
 struct A8Plan { int bn, token_tiles, slices, ctas; int64_t t_full; };

@@ -98,6 +98,18 @@ def test_gemm_plan_shares_the_last_round_only_when_it_pays():
     assert (bn, whole, shared, crossing) == (128, 0, 2, 0) and runs in (4, 6, 8)
 
 
+def test_gemm_plan_of_small_matrices_above_128_tokens():
+    """Sharing a tile costs more the finer it is cut (the partial tiles are added by one CTA), and a short K does not pay for it."""
+    for M in (160, 256, 300, 700, 1024):
+        assert cq.cq_debug_gemm_plan(4, 128, M, 2816, 2048)["stream_k_ctas"] == 0
+        for N in (1024, 4096):
+            p = cq.cq_debug_gemm_plan(4, 128, M, N, 4096)
+            assert p["stream_k_ctas"] <= 4 * p["stream_k_tiles"] + (4 * p["stream_k_tiles"] if N == 1024 and M <= 512 else 0), (M, N, p)
+            assert p["token_tile"] == 256
+    # the widest tile where 256 tokens would take another round
+    assert cq.cq_debug_gemm_plan(4, 128, 1024, 6144, 4096)["token_tile"] == 512
+
+
 @pytest.mark.parametrize("mode", [0, 1])
 def test_routed_launches_report_into_the_front_word(mode):
     """Every launch of a routed call, those of a single matrix too, reports into the word that cq_gemm_status reads."""

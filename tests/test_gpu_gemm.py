@@ -320,6 +320,30 @@ def test_rings_of_every_depth_repeat_bit_for_bit(B, G, M):
     check_y(y_to_numpy(y0), np.tile(oracle.gemm_model(c.codes, c.s, c.a, c.b, B, G, K, xb), (1, N // 256)), f"rings B={B} G={G} M={M}")
 
 
+# the kinds of output tile above 128 tokens, whole and shared between runs: 256 tokens by one CTA, by a pair (an odd number of row
+# blocks leaves its last pair half empty), 512 by a pair; ragged channels and tokens
+@pytest.mark.parametrize("B,G,N,K,M,tile,shared", [(2, 64, 136, 256, 200, 256, False), (3, 32, 300, 128, 255, 256, False), (1, 128, 4096, 4096, 257, 256, True),
+                                                   (8, 128, 136, 4224, 300, 256, True), (4, 128, 300, 1024, 129, 256, False), (8, 32, 392, 1024, 256, 256, False),
+                                                   (4, 128, 4096, 14336, 200, 256, True), (8, 128, 9816, 256, 300, 512, False), (4, 64, 9816, 256, 512, 512, False),
+                                                   (8, 128, 4096, 14336, 500, 512, True)])
+def test_kinds_of_output_tile(B, G, N, K, M, tile, shared):
+    plan = cq.cq_debug_gemm_plan(B, G, M, N, K)
+    if torch.cuda.get_device_properties(0).multi_processor_count == 148:
+        assert plan["token_tile"] == tile and (plan["stream_k_ctas"] > 0) == shared, plan
+    block = min(N, 256)   # large matrices repeat a block of channels: the reference is computed for one block
+    c = logical_case(block, K, B, G, seed=260 + M)
+    rep = lambda t: t.repeat((-(-N // block),) + (1,) * (t.dim() - 1))[:N].contiguous()
+    pw = cq.cq_repack(rep(c.d_codes), rep(c.d_s), rep(c.d_a), rep(c.d_b), B, G, N, K)
+    xb = datagen.activations(M, K, seed=261, outlier_cols=0.01)
+    ws = torch.zeros(cq.cq_workspace_bytes(B, G, M, N, K, 0), dtype=torch.uint8, device="cuda")
+    y = torch.full((M + 1, N), 7.0, dtype=torch.bfloat16, device="cuda")      # nothing is written beyond the last token
+    first = cq.cq_gemm(pw, x_to_device(xb), cq.CQ_MODEL_DTYPE, ws, y[:M]).clone()
+    again = cq.cq_gemm(pw, x_to_device(xb), cq.CQ_MODEL_DTYPE, ws, y[:M])
+    assert cq.cq_gemm_status(ws) == 0 and bool((y[M] == 7.0).all()) and torch.equal(first.view(torch.int16), again.view(torch.int16))
+    ref = oracle.gemm_model(c.codes, c.s, c.a, c.b, B, G, K, xb)
+    check_y(y_to_numpy(first), np.tile(ref, (1, -(-N // block)))[:, :N], f"tile B={B} G={G} N={N} K={K} M={M}")
+
+
 @pytest.mark.parametrize("mode", [cq.CQ_MODEL_DTYPE, cq.CQ_DYN_A8])
 @pytest.mark.parametrize("M", [1, 2, 8, 16])
 @pytest.mark.parametrize("B,G", [(5, 128), (6, 64), (7, 128), (1, 32), (3, 32), (4, 32), (8, 32)])
