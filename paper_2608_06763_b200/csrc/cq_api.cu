@@ -236,7 +236,8 @@ int cq_mlp_swiglu(const void *layout_gate_up, int B_gu, int G_gu, const void *la
 // Routed product.  The groups (matrices with routes) are sorted into classes of token tiles, and a class of several
 // groups is one launch: up to 16 rows the small-M kernel, above it the GEMM, the token tiles up to 128 together (its time is
 // the decode of the weights there, not the tokens) and 256 and 512 by themselves; Dynamic A8 keeps one class per token
-// tile, whose drain grows with the tile.  A group by itself is an ordinary product, which may share its tiles along K.
+// tile, whose drain grows with the tile.  A group by itself is an ordinary product, which may share its tiles along K, and so
+// are the groups of a GEMM class that would leave most of the GPU idle in whole tiles (together_pays).
 // Sixteen matrices of 2816 x 2048 (W4 G64, 384 routes): one after another 203 us, most of it launches that leave SMs idle; 61 us so.
 // Workspace: [status][gathered rows: R x K][Dynamic A8: INT8 carrier of all rows, row scales][arrival counters][partial sums
 // of the small-M groups][what else an ordinary product needs].  Every launch reports into the one status word at the
@@ -254,6 +255,19 @@ static int routed_class(const Dims &d, int64_t m, int mode) {   // 0: small M; e
     return t < 128 ? 128 : t;
 }
 static const int ROUTED_CLASSES[5] = {0, 64, 128, 256, 512};   // every value of routed_class
+// Whether the groups of a GEMM class are faster in one launch of whole tiles than one after another.  A few matrices of
+// few row blocks leave most SMs idle in whole tiles, while each of them by itself shares its tiles along K among all SMs.
+// Two matrices of 1024 x 4096, W8 G128, model dtype, 20 rows each: 30.7 us together, 25.5 one after another; W3 G32, Dynamic A8:
+// 45.2 and 31.6; but 2816 x 2048, W4 G64, 64 rows each: together 20 % faster.  An ordinary product of Dynamic A8 adds a launch and
+// a quantiser of its own, some five blocks of main loop.
+static bool together_pays(const Dims &d, const GroupTable &t, int64_t max_rows, int mode) {
+    const bool tc = mode == CQ_MODEL_DTYPE;
+    const double together = tc ? gemm_tc_groups_cost(t, d, max_rows) : gemm_a8_groups_cost(t, d, max_rows) + 5.0;
+    const double least = tc ? 4.6 : 9.0;   // no ordinary product costs less
+    double one_by_one = least * t.n;
+    for (int i = 0; i < t.n && one_by_one < together; ++i) one_by_one += (tc ? gemm_tc_plan(d, t.g[i].rows).cost : gemm_a8_plan(d, t.g[i].rows).cost + 5.0) - least;
+    return together <= one_by_one;
+}
 // The launches that follow the gather, in order: f(groups, class, largest row count, CTAs of a small-M group).  A table of one
 // group is an ordinary product.  The sizes, the launches themselves and cq_debug_routed_plan all walk this.
 extern "C++" {
@@ -261,6 +275,16 @@ template <class F>
 static int for_routed_launches(const Dims &d, const void *const *layouts, const int64_t *off, int E, int mode, F &&f) {
     auto emit = [&](const GroupTable &t, int cls, int64_t max_rows) -> int {
         if (t.n == 0) return CQ_OK;
+        if (t.n > 1 && cls != 0 && !together_pays(d, t, max_rows, mode)) {
+            for (int i = 0; i < t.n; ++i) {
+                GroupTable one{};
+                one.n = 1;
+                one.g[0] = t.g[i];
+                const int st = f(one, cls, (int64_t)t.g[i].rows, 1);
+                if (st != CQ_OK) return st;
+            }
+            return CQ_OK;
+        }
         // small-M groups share the places of the whole GPU; a run of fewer than four tiles is mostly overhead
         const int64_t T = (int64_t)d.NB * d.KT, places = cls == 0 ? gemv_plan(d, 16, mode).ctas : 0;
         int64_t P = places / t.n;

@@ -44,6 +44,7 @@ A8Plan gemm_a8_plan(const Dims &d, int64_t M) {
     const int64_t T = (int64_t)d.NB * p.token_tiles, sms = sm_count();
     const int64_t r = T % sms;
     p.t_full = T; p.slices = 1;
+    p.cost = (double)(T / sms) * (double)(d.KT + 3);
     if (r != 0) {
         const double wide = (double)p.bn / 256.0;
         const double whole = (double)(d.KT + 3), all = (double)(T / sms + 1) * whole;
@@ -52,10 +53,17 @@ A8Plan gemm_a8_plan(const Dims &d, int64_t M) {
             const double c = (double)((r * s + sms - 1) / sms) * ((double)d.KT / (double)s + 3.0 + 4.0 * wide);
             if (c < best) { best = c; p.slices = (int)s; }
         }
-        if ((whole - best) / all > 0.03) p.t_full = T - r; else p.slices = 1;
+        if ((whole - best) / all > 0.03) p.t_full = T - r; else { p.slices = 1; best = whole; }
+        p.cost += best;
     }
     p.ctas = (int)(p.t_full + (T - p.t_full) * p.slices);
     return p;
+}
+double gemm_a8_groups_cost(const GroupTable &groups, const Dims &d, int64_t tile_m) {
+    const int bn = gemm_a8_token_tile(d, tile_m);
+    int64_t units = 0;
+    for (int i = 0; i < groups.n; ++i) units += (int64_t)d.NB * ((groups.g[i].rows + bn - 1) / bn);
+    return (double)((units + sm_count() - 1) / sm_count()) * (double)(d.KT + 3);
 }
 
 namespace {

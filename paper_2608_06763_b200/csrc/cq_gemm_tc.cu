@@ -123,6 +123,15 @@ TcPlan gemm_tc_plan(const Dims &d, int64_t M) {
     return best;
 }
 
+double gemm_tc_groups_cost(const GroupTable &groups, const Dims &d, int64_t tile_m) {
+    const int bnt = gemm_tc_token_tile(tile_m), cw = bnt >= 256 ? 2 : 1;
+    const TileKind k = tile_kind(d, bnt, cw);
+    int64_t units = 0;
+    for (int i = 0; i < groups.n; ++i) units += (int64_t)((d.NB + cw - 1) / cw) * ((groups.g[i].rows + bnt - 1) / bnt);
+    const int64_t places = sm_count() / cw;
+    return (double)((units + places - 1) / places) * (k.fixed + k.tile * (double)d.KT);
+}
+
 // stream-K instantiations: cq_gemm_tc_sk.cu
 cudaError_t launch_gemm_tc_streamk(const GroupTable &groups, const Dims &d, const uint16_t *x, uint16_t *y, int64_t M, const TcPlan &plan, int *status,
                                    float *partial, int *counters, bool act_f16, cudaStream_t st);

@@ -93,8 +93,12 @@ int gemm_tc_token_tile(int64_t M);
 struct TcPlan { int bnt, token_tiles, ctas, stream_k, p2, crossing, cw; int64_t t_full; double cost; };
 TcPlan gemm_tc_plan(const Dims &d, int64_t M);
 int gemm_a8_token_tile(const Dims &d, int64_t M);
-struct A8Plan { int bn, token_tiles, slices, ctas; int64_t t_full; };
+// cost: blocks of 128 k in the main loop
+struct A8Plan { int bn, token_tiles, slices, ctas; int64_t t_full; double cost; };
 A8Plan gemm_a8_plan(const Dims &d, int64_t M);
+// the groups of a class in one launch of whole tiles, in the units of the plans' costs
+double gemm_tc_groups_cost(const GroupTable &groups, const Dims &d, int64_t tile_m);
+double gemm_a8_groups_cost(const GroupTable &groups, const Dims &d, int64_t tile_m);
 
 // offline encoder steps (cq_encode.cu)
 cudaError_t launch_encode_assign(const float *W, int B, int G, int64_t N, int64_t K, const float *scale, const uint16_t *a,

@@ -138,3 +138,17 @@ def test_routed_small_groups_share_the_places_of_their_own_launch(mode):
     assert full > 148                                       # thirty-two matrices fill the places once
     assert places(64) == [full, full]
     assert places(35)[0] == full and places(35)[1] >= 0.9 * full   # three matrices: a third of the places each
+
+
+def test_routed_groups_that_would_idle_the_gpu_run_one_by_one():
+    """A few matrices of few row blocks share their tiles along K as products of their own; more of them, or a short K, go together."""
+    def launches(N, K, counts, B=8, G=128, mode=0):
+        off = [0]
+        for c in counts:
+            off.append(off[-1] + c)
+        return [v["matrices"] for v in cq.cq_debug_routed_plan(B, G, off, N, K, mode)]
+
+    assert launches(1024, 4096, [20, 20]) == [1, 1] and launches(1024, 4096, [64, 64], 3, 32) == [1, 1]
+    assert launches(1024, 4096, [20, 20], 3, 32, 1) == [1, 1] and launches(1024, 4096, [128, 128], 4, 64, 1) == [1, 1]
+    assert launches(2816, 2048, [64, 64], 4, 64) == [2] and launches(1024, 4096, [64] * 8) == [8]
+    assert launches(2816, 2048, [48] * 16, 4, 64) == [16] and launches(1024, 4096, [64] * 8, 4, 64, 1) == [8]
