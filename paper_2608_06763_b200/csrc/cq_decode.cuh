@@ -196,7 +196,7 @@ __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {
 // weights; two byte permutes fetch their low and high bytes, two more put the bytes together, and the sign bits
 // go into the high bytes by one exclusive or.  Thirteen integer instructions for eight weights, against some forty for
 // the half2 polynomial, its scale in fp32 and the rounding to the operand's type; the levels themselves are evaluated in fp32
-// and rounded once.  Measured on the linears of an 8B layer, G = 128: M = 1 66.6 -> 59.3 us, M = 13 109.7 -> 105.5,
+// and rounded once.  Measured on the linears of an 8B layer, G = 128: M = 1 66.6 -> 56.8 us, M = 13 109.7 -> 105.5,
 // M = 200 (binary16) 194.8 -> 167.7, M = 1024 509.5 -> 491.6 (what is left there is not the decode).  out[i] = weights (2 i, 2 i + 1) of the word, in k order; a reserved code reads (minus) zero.
 __device__ __forceinline__ void w4_block(uint32_t word, const uint4 &t, uint32_t (&out)[4]) {
     const uint32_t sel = word & 0x77777777u, sel1 = sel >> 16, w4 = word << 4;
@@ -262,10 +262,10 @@ __device__ __forceinline__ void a8_row_regs(const uint32_t (&w)[2 * B], const Ca
         const uint32_t word = w[2 * MI + RR];
         const uint32_t ws = word & 0x77777777u, wh = ws >> 16, w4 = word << 4;
         const uint32_t m_lo = prmt(word, word, 0xBA98u), m_hi = prmt(w4, w4, 0xBA98u);   // 0xFF where the code is negative
-        const uint32_t n_lo = prmt(tab.x, tab.y, ws), p_lo = prmt(tab.z, tab.w, ws);
-        const uint32_t n_hi = prmt(tab.x, tab.y, wh), p_hi = prmt(tab.z, tab.w, wh);
-        lo = (p_lo & m_lo) | (n_lo & ~m_lo);
-        hi = (p_hi & m_hi) | (n_hi & ~m_hi);
+        const uint32_t p_lo = prmt(tab.x, tab.y, ws), n_lo = prmt(tab.z, tab.w, ws);
+        const uint32_t p_hi = prmt(tab.x, tab.y, wh), n_hi = prmt(tab.z, tab.w, wh);
+        lo = (n_lo & m_lo) | (p_lo & ~m_lo);
+        hi = (n_hi & m_hi) | (p_hi & ~m_hi);
     } else if constexpr (B == 3) {
         constexpr int rho = (2 + 2 * (MI & 1) + RR) & 3;   // where the 1-bit plane keeps this selector's bits
         const uint32_t x0 = RR ? (w[MI] >> 2) : w[MI];

@@ -192,7 +192,7 @@ __global__ void __launch_bounds__(128) losses_kernel(const float *__restrict__ W
 //   joint        the cost of level i, (u - s z_i)^2 + (u - s zt_i)^2, is 2 u^2 plus a line in u whose slope falls
 //                with i, so the best level changes at u = s beta_i, beta_i = (dz mz + dzt mzt) / (dz + dzt) with d the
 //                step and m the midpoint between neighbours.  Thresholds are formed in fp32; a weight within
-//                GUARD s of one (a relative 1e-5, above every rounding error of beta and of the fp64 costs), and any lane
+//                GUARD s = 4e-6 s of one (beta s <= s carries a few rounding errors of 2^-24 s = 6e-8 s), and any lane
 //                whose levels or scale do not meet the conditions of joint_thresholds, takes the definition
 //                (joint_level), so the codes are those of the definition everywhere.
 struct SearchPlan {      // what the host fixes for a launch

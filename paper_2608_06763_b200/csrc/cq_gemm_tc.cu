@@ -70,7 +70,7 @@ TcPlan plan_with(const Dims &d, int64_t M, const TileKind &k) {
     TcPlan p;
     p.bnt = k.bnt; p.cw = k.cw;
     p.token_tiles = (int)((M + p.bnt - 1) / p.bnt);
-    const int64_t NBU = (d.NB + p.cw - 1) / p.cw, T = NBU * p.token_tiles, sms = sm_count() / p.cw;   // tiles and places for them
+    const int64_t NBU = (d.NB + p.cw - 1) / p.cw, T = NBU * p.token_tiles, sms = sm_count() > p.cw ? sm_count() / p.cw : 1;   // tiles and places for them
     const int64_t r = T % sms;                      // tiles of the last, partial round
     const double round_us = k.fixed + k.tile * (double)d.KT;
     p.t_full = T; p.p2 = 0; p.crossing = 0;
@@ -128,7 +128,7 @@ double gemm_tc_groups_cost(const GroupTable &groups, const Dims &d, int64_t tile
     const TileKind k = tile_kind(d, bnt, cw);
     int64_t units = 0;
     for (int i = 0; i < groups.n; ++i) units += (int64_t)((d.NB + cw - 1) / cw) * ((groups.g[i].rows + bnt - 1) / bnt);
-    const int64_t places = sm_count() / cw;
+    const int64_t places = sm_count() > cw ? sm_count() / cw : 1;
     return (double)((units + places - 1) / places) * (k.fixed + k.tile * (double)d.KT);
 }
 

@@ -99,7 +99,8 @@ struct TcParams {
 // shared memory.  Without that every SM reads all BN NACC tokens: 64 KB per 64-wide block at 512 tokens, against
 // 1048 cycles of MMA -- the 64 bytes a cycle that an SM can take from L2.  Measured (W4 G128, before -> now, with the
 // one-barrier ring below): a 64-wide block of a 128 x 512 tile 1580 -> 1060 cycles; linears of an 8B layer at M = 1024
-// 492 -> 423 us, at M = 200 168 -> 158 us; 70B gate_up, W3, M = 4096 3290 -> 2758 us (1395 TFLOP/s).
+// 492 -> 423 us, at M = 200 168 -> 158 us; 70B gate_up, W3, M = 4096 3290 -> 2760 .. 2840 us (some 1370
+// TFLOP/s, under the power limit).
 //
 // The operand ring: a stage is one 64-wide k block, the decoded weights (16 KB) and the activations, filled behind one
 // barrier and freed by one commit (the issuing thread is on the critical path at small token tiles: with a barrier

@@ -41,9 +41,7 @@ namespace cq {
 
 namespace {
 
-#ifndef CQ_GEMV_CTAS_PER_SM
-#define CQ_GEMV_CTAS_PER_SM 3
-#endif
+constexpr int CTAS_PER_SM = 3;                       // where registers and ring allow it (gemv_occ)
 constexpr int GEMV_WARPS = 8;                        // one warp per group of 16 rows of a tile
 constexpr int GEMV_THREADS = GEMV_WARPS * 32;
 constexpr int XS_PAD = 16;     // elements of padding per staged fp16 activation row (bank spread: 32 bytes)
@@ -74,9 +72,9 @@ __host__ __device__ constexpr bool gemv_uses_ring(int B, int G, int NT, int MODE
 __host__ __device__ constexpr int gemv_occ(int B, int G, int NT, int MODE) {
     if (MODE != 2 && NT == 2) return 2;
     if (MODE == 1 && B == 6) return 2;   // W6, 4096 square, Dynamic A8, G = 128, M = 1: 17.7 us with two, 19.1 with three (shorter runs, 80 registers)
-    if (!gemv_uses_ring(B, G, NT, MODE)) return CQ_GEMV_CTAS_PER_SM;
+    if (!gemv_uses_ring(B, G, NT, MODE)) return CTAS_PER_SM;
     const int tb = 2048 * B + 1024 * (TILE / G);
-    return (gemv_smem_budget(B, MODE, CQ_GEMV_CTAS_PER_SM) - (gemv_x_bytes_max(B, NT, MODE) + 127) / 128 * 128) / tb >= 4 ? CQ_GEMV_CTAS_PER_SM : 2;
+    return (gemv_smem_budget(B, MODE, CTAS_PER_SM) - (gemv_x_bytes_max(B, NT, MODE) + 127) / 128 * 128) / tb >= 4 ? CTAS_PER_SM : 2;
 }
 // the variant that serves M rows in an activation mode
 __host__ __device__ constexpr int gemv_variant_mode(int64_t M, int mode) { return mode == 1 ? 1 : (M <= 2 ? 2 : 0); }
@@ -234,7 +232,7 @@ __device__ __forceinline__ void group_model(const TileRegs<B, TILE / G> &r, cons
 }
 
 // One group of a tile, Dynamic A8: INT8 MMAs into int32 partials P_g, then acc += s * P_g.
-// xs = staged INT8 activations in operand order, xo[tb] = byte offset of this lane's token row plus 8 t;
+// xs = staged INT8 activations in the order of a8_row_regs (W4: natural), xo[tb] = byte offset of this lane's token row plus 8 t;
 // ctab = this warp's table space.
 template <int B, int G, int NT, int GI>
 __device__ __forceinline__ void group_a8(const TileRegs<B, TILE / G> &r, const int8_t *xs, const int (&xo)[NT], int8_t *ctab,
@@ -732,7 +730,7 @@ gemv_body(const uint8_t *__restrict__ layout, const Dims &d, const uint16_t *__r
                         const int64_t k = k_base + (int64_t)c * 8;
                         if (k < d.K) src = x + (int64_t)m * d.K + k;   // K % 8 == 0 always
                     } else {
-                        src = xq + (int64_t)m * x8_pitch + k_base + c * 16;  // already in MMA operand order; pitch multiple of 128, zero beyond K
+                        src = xq + (int64_t)m * x8_pitch + k_base + c * 16;  // in the order the product reads (a8_row_regs; W4: natural); pitch multiple of 128, zero beyond K
                     }
                     if (src) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
                     else *(uint4 *)dst = make_uint4(0, 0, 0, 0);
@@ -1146,13 +1144,6 @@ cudaError_t launch_gemv(const void *layout, const Dims &d, const uint16_t *x, ui
     }
     const int Mi = (int)M, P = gp.ctas, ms = gp.max_run;
     const int E = gp.overhead;
-#ifdef CQ_GEMV_SUBSET   // development builds: only the widths under study
-    switch (d.B) {
-        case 1: return dispatch_g<1>(layout, d, x, xq, pitch, dxs, y, Mi, mode, P, ms, E, partial, counters, status, act_f16, st);
-        case 4: return dispatch_g<4>(layout, d, x, xq, pitch, dxs, y, Mi, mode, P, ms, E, partial, counters, status, act_f16, st);
-        default: return cudaErrorNotSupported;
-    }
-#else
     switch (d.B) {
         case 1: return dispatch_g<1>(layout, d, x, xq, pitch, dxs, y, Mi, mode, P, ms, E, partial, counters, status, act_f16, st);
         case 2: return dispatch_g<2>(layout, d, x, xq, pitch, dxs, y, Mi, mode, P, ms, E, partial, counters, status, act_f16, st);
@@ -1163,7 +1154,6 @@ cudaError_t launch_gemv(const void *layout, const Dims &d, const uint16_t *x, ui
         case 7: return dispatch_g<7>(layout, d, x, xq, pitch, dxs, y, Mi, mode, P, ms, E, partial, counters, status, act_f16, st);
         default: return dispatch_g<8>(layout, d, x, xq, pitch, dxs, y, Mi, mode, P, ms, E, partial, counters, status, act_f16, st);
     }
-#endif
 }
 
 }  // namespace cq

@@ -19,10 +19,9 @@ cudaError_t launch_decode_carriers(const void *layout, const Dims &d, int8_t *ca
 cudaError_t launch_decode_weights(const void *layout, const Dims &d, float *What, cudaStream_t st);
 cudaError_t launch_a8_partials(const void *layout, const Dims &d, const int8_t *x8, int64_t M, int32_t *P, cudaStream_t st);
 // act_f16 (here and below): the 16-bit activation / output patterns are binary16 instead of bfloat16
+// operand_order: x8 in the order of cq_decode.cuh that the INT8 products of every width but four bits read; natural order otherwise
 cudaError_t launch_quantize_a8(const uint16_t *x, int64_t M, int64_t K, int8_t *x8, int64_t x8_pitch, float *dx,
                                bool operand_order, bool act_f16, cudaStream_t st);
-
-// operand_order: x8 in the order of cq_decode.cuh that the INT8 products of every width but four bits read; natural order otherwise
 // h[M][2 I] (gate | up, model dtype) -> INT8 carrier of silu(gate) * up, and its row scales
 cudaError_t launch_swiglu_quantize_a8(const uint16_t *h, int64_t M, int64_t I, int8_t *x8, int64_t x8_pitch, float *dx,
                                       bool operand_order, bool act_f16, cudaStream_t st);
@@ -34,7 +33,7 @@ cudaError_t launch_wait_timeout(int *status, long long limit_cycles, cudaStream_
 // Workspace carving (all offsets 256-byte aligned).
 struct Workspace {
     size_t counters_off, counters_bytes;   // int32 arrival counters, one per 128-row block
-    size_t partial_off, partial_bytes;     // fp32 split-K partial sums: small M [CTA][2][M][128]; model-dtype GEMM [CTA][2][BNT][128]; A8 GEMM [shared tile][slice][BN][128]
+    size_t partial_off, partial_bytes;     // fp32 split-K partial sums: small M [CTA][2][M][128]; model-dtype GEMM [run, CTA of a pair][2][tokens][128]; A8 GEMM [shared tile][slice][BN][128]
     size_t x8_off, x8_bytes;               // Dynamic A8: int8 activation carrier [M][Kp]
     size_t dx_off, dx_bytes;               // Dynamic A8: row scales [M]
     size_t status_off;                     // int32 device status word (bounded waits report here)

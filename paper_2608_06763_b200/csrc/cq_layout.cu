@@ -328,7 +328,7 @@ __global__ void __launch_bounds__(1024) quantize_a8_kernel(const uint16_t *__res
 // output h[m] = (gate | up), 2 I values in the model dtype, goes to act = silu(gate) * up -- evaluated in fp32
 // and rounded to the model dtype, which is what a separate activation operator would have written -- and
 // straight on to that row's Dynamic-A8 carrier (Eq. a8-activation-scale, Eq. a8-activation-quantization) in the
-// order the product reads it in (carrier_order), without the activation ever reaching memory.  One CTA per row; I % 8 == 0.
+// order the product reads it in (launch_quantize_a8), without the activation ever reaching memory.  One CTA per row; I % 8 == 0.
 __device__ __forceinline__ uint32_t gated_act_bits(uint32_t g16, uint32_t u16, bool f16) {
     const float g = act_to_float(g16, f16), u = act_to_float(u16, f16);
     const float sg = __fdiv_rn(g, __fadd_rn(1.0f, expf(-g)));
