@@ -155,6 +155,10 @@ gemm_a8_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
         if (threadIdx.x == 0) atomicCAS(prm.status, 0, 9);
         return;
     }
+    // as in gemm_tc_kernel: set-up and the first raw tiles on their way to L2 while the kernel before this one drains
+    if (warp == 0 && lane == 0) prefetch_tensormap(&xmap);
+    if (warp == 2 + A8_WORK_WARPS && lane == 0 && KT > 0)
+        prefetch_l2((const uint8_t *)prm.groups.g[grp].layout + ((size_t)nb * d.KT + kt0) * (size_t)d.tile_bytes, (uint32_t)(min(KT, A8_RAW_STAGES) * d.tile_bytes));
     if (threadIdx.x == 0) {
         for (int s = 0; s < A8_STAGES; ++s) { mbar_init(&st_full[s], A8_SET_WARPS + 1); mbar_init(&st_empty[s], 1); }   // full: a set's warps and the announced bytes
         for (int s = 0; s < A8_RAW_STAGES; ++s) { mbar_init(&raw_full[s], 1); mbar_init(&raw_empty[s], A8_SET_WARPS); }
@@ -173,6 +177,7 @@ gemm_a8_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
+    wait_for_previous_kernel();   // the carrier, its scales, y and the workspace
 
     if (warp == 0) {
         // ===== producer of the activation tiles: only the wait for the stage stands between the MMAs that free it
@@ -485,8 +490,7 @@ cudaError_t launch_a8(const GroupTable &groups, const Dims &d, const int8_t *x8,
     }
     if (plan.bn != BN) return cudaErrorInvalidConfiguration;
     p.t_full = (int)plan.t_full; p.slices = plan.slices;
-    kern<<<dim3((unsigned)plan.ctas), A8_THREADS, smem, st>>>(xmap, p);
-    return cudaGetLastError();
+    return launch_overlapped(kern, dim3((unsigned)plan.ctas), A8_THREADS, smem, st, 1, xmap, p);
 }
 
 // M: rows of x8; tile_m: the rows whose token tile is taken (of an ordinary product, M)

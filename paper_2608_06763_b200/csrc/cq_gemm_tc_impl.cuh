@@ -231,6 +231,16 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
         if (threadIdx.x == 0) atomicCAS(prm.status, 0, 9);
         return;
     }
+    // The kernel before this one may still be running (launch_overlapped): until its results are waited for, below, the barriers
+    // and the tensor memory are set up and the first raw tiles are brought to L2 (not further: L2 sees every write to them).
+    if (warp == 0 && lane == 0) prefetch_tensormap(&xmap);
+    if (warp == 2 + DEC_WARPS && lane == 0) {
+        SegWalk<SK, PAIR> first(prm, rank);
+        Seg s0;
+        if (first.next(s0))
+            prefetch_l2((const uint8_t *)prm.groups.g[SK ? 0 : first.grp].layout + ((size_t)min(s0.nb, d.NB - 1) * d.KT + s0.k0) * (size_t)d.tile_bytes,
+                        (uint32_t)(min(s0.k1 - s0.k0, RAW_STAGES) * d.tile_bytes));
+    }
     if (threadIdx.x == 0) {
         // full: the decoders of a set (of both CTAs of a pair) and the thread that announces the activations' bytes
         for (int s = 0; s < STAGES; ++s) { mbar_init(&full[s], (PAIR ? 2 * SET_WARPS : SET_WARPS) + 1); mbar_init(&empty[s], 1); }
@@ -249,6 +259,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
     if constexpr (PAIR) cluster_sync();   // the partner's barriers are initialised before anything arrives on them
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
+    wait_for_previous_kernel();   // x, y and the workspace belong to the kernels before until here
 
     // Every wait is bounded.  One that runs out records its code in the status word and raises the CTA's flag;
     // from then on no role waits any more, but each still walks its loops to the end (the decoders meet at
@@ -677,17 +688,7 @@ cudaError_t launch_bn(const GroupTable &groups, const Dims &d, const uint16_t *x
     cudaError_t ea = ensure_func_attr(kern, attr_done, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
     if (ea != cudaSuccess) return ea;
     p.partial = partial; p.counters = counters; p.f16 = act_f16;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)plan.ctas);
-    cfg.blockDim = dim3(TC_THREADS);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = PAIR ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, kern, xmap, p);
+    return launch_overlapped(kern, dim3((unsigned)plan.ctas), TC_THREADS, smem, st, PAIR ? 2 : 1, xmap, p);
 }
 
 // M: rows of x; plan: of the product, or (routed) the token tile of the class

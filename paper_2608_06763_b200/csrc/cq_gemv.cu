@@ -30,8 +30,6 @@
 // Dynamic A8 uses the INT8 m16n8k32 MMA on signed carriers (Eq. carrier) taken from a per-(row, group)
 // table indexed by the stored code, in registers and read with byte permutes (B <= 5: a8_row_regs in cq_decode.cuh), or
 // evaluated code by code (wider: a8_row_eval); int32 group partials, fp32 rescale (Eq. a8-output).
-#include <cstdlib>
-
 #include "cq_common.cuh"
 #include "cq_decode.cuh"
 #include "cq_internal.h"
@@ -1019,25 +1017,15 @@ cudaError_t launch_one(const void *layout, const Dims &d, const uint16_t *x, con
     if constexpr (GRP) e = ensure_func_attr(gemv_groups_kernel<B, G, NT, MODE>, attr_done, cudaFuncAttributeMaxDynamicSharedMemorySize, gemv_smem_budget(B, MODE, OCC));
     else e = ensure_func_attr(gemv_kernel<B, G, NT, MODE>, attr_done, cudaFuncAttributeMaxDynamicSharedMemorySize, gemv_smem_budget(B, MODE, OCC));
     if (e != cudaSuccess) return e;
-    // Programmatic dependent launch: this kernel may begin (and prefetch weights) while the previous
-    // kernel of the stream drains; it waits for that kernel before touching anything but the weights.
-    static const bool use_pdl = getenv("CQ_NO_PDL") == nullptr;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)P, GRP ? (unsigned)groups->n : 1u);
-    cfg.blockDim = dim3(GEMV_THREADS);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = use_pdl ? 1 : 0;
+    // Programmatic overlap: this kernel may begin (and prefetch weights) while the previous kernel of the stream drains; it
+    // waits for that kernel before touching anything but the weights.
+    const dim3 grid((unsigned)P, GRP ? (unsigned)groups->n : 1u);
     if constexpr (GRP)
-        return cudaLaunchKernelEx(&cfg, gemv_groups_kernel<B, G, NT, MODE>, d, x, xq, x8_pitch, dxs, y, E, partial, counters, nstage, ring_off, status,
-                                  act_f16, *groups);
+        return launch_overlapped(gemv_groups_kernel<B, G, NT, MODE>, grid, GEMV_THREADS, smem, st, 1, d, x, xq, x8_pitch, dxs, y, E, partial, counters, nstage,
+                                 ring_off, status, act_f16, *groups);
     else
-        return cudaLaunchKernelEx(&cfg, gemv_kernel<B, G, NT, MODE>, (const uint8_t *)layout, d, x, xq, x8_pitch, dxs, y, M, E, partial, counters, nstage,
-                                  ring_off, status, act_f16);
+        return launch_overlapped(gemv_kernel<B, G, NT, MODE>, grid, GEMV_THREADS, smem, st, 1, (const uint8_t *)layout, d, x, xq, x8_pitch, dxs, y, M, E,
+                                 partial, counters, nstage, ring_off, status, act_f16);
 }
 
 template <int B, int G>

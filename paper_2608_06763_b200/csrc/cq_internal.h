@@ -4,6 +4,7 @@
 #include <stdint.h>
 
 #include <atomic>
+#include <cstdlib>
 
 #include "cq_common.cuh"
 
@@ -58,6 +59,31 @@ cudaError_t ensure_func_attr(Kern kern, std::atomic<uint64_t> &done, cudaFuncAtt
     e = cudaFuncSetAttribute(kern, attr, value);
     if (e == cudaSuccess && tracked) done.fetch_or(bit, std::memory_order_release);
     return e;
+}
+// Launch that may begin while the kernel before it in the stream drains (programmatic dependent launch): every kernel started
+// this way runs griddepcontrol.wait before it touches anything but weights and its own on-chip state.  What is hidden is
+// the launch itself and the set-up in front of the wait.  cluster: CTAs per cluster (1: none).
+template <class... P, class... A>
+cudaError_t launch_overlapped(void (*kern)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t st, int cluster, A &&...args) {
+    static const bool use_pdl = getenv("CQ_NO_PDL") == nullptr;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    int n = 0;
+    if (use_pdl) {
+        attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[n++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (cluster > 1) {
+        attr[n].id = cudaLaunchAttributeClusterDimension;
+        attr[n].val.clusterDim.x = (unsigned)cluster; attr[n].val.clusterDim.y = 1; attr[n++].val.clusterDim.z = 1;
+    }
+    cfg.attrs = attr;
+    cfg.numAttrs = n;
+    return cudaLaunchKernelEx(&cfg, kern, static_cast<A &&>(args)...);
 }
 // the thread's record of the last failed CUDA call (what cq_last_cuda_error returns)
 void set_last_cuda_error(cudaError_t e);

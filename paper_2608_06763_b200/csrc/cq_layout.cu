@@ -258,8 +258,7 @@ template <bool OPERAND_ORDER>
 __global__ void __launch_bounds__(1024) quantize_a8_kernel(const uint16_t *__restrict__ x, int64_t M, int64_t K,
                                                           int8_t *__restrict__ x8, int64_t x8_pitch,
                                                           float *__restrict__ dx, bool f16) {
-    // the kernel launched next may start now (its first steps do not touch what this one writes)
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    tc::wait_for_previous_kernel();   // x comes from it, and it may still read the carrier that this one replaces
     __shared__ unsigned red[32];
     __shared__ float s_d;
     const int64_t m = blockIdx.x;
@@ -346,8 +345,7 @@ template <bool OPERAND_ORDER>
 __global__ void __launch_bounds__(1024) swiglu_quantize_a8_kernel(const uint16_t *__restrict__ h, int64_t M, int64_t I,
                                                                  int8_t *__restrict__ x8, int64_t x8_pitch,
                                                                  float *__restrict__ dx, bool f16) {
-    asm volatile("griddepcontrol.wait;" ::: "memory");               // h comes from the kernel launched before
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    tc::wait_for_previous_kernel();   // h comes from it
     __shared__ unsigned red[32];
     __shared__ float s_d;
     const int64_t m = blockIdx.x;
@@ -482,9 +480,8 @@ cudaError_t launch_quantize_a8(const uint16_t *x, int64_t M, int64_t K, int8_t *
     int64_t threads = ((K >> 3) + 31) / 32 * 32;   // one 8-value chunk per thread when the row is short enough
     if (threads > 1024) threads = 1024;
     if (M > 64 && threads > 256) threads = 256;    // many rows: smaller CTAs fill the SMs better
-    if (operand_order) quantize_a8_kernel<true><<<(unsigned)M, (unsigned)threads, 0, st>>>(x, M, K, x8, x8_pitch, dx, act_f16);
-    else quantize_a8_kernel<false><<<(unsigned)M, (unsigned)threads, 0, st>>>(x, M, K, x8, x8_pitch, dx, act_f16);
-    return cudaGetLastError();
+    return launch_overlapped(operand_order ? quantize_a8_kernel<true> : quantize_a8_kernel<false>, dim3((unsigned)M), (unsigned)threads, 0, st, 1, x, M, K,
+                             x8, x8_pitch, dx, act_f16);
 }
 
 cudaError_t launch_swiglu_quantize_a8(const uint16_t *h, int64_t M, int64_t I, int8_t *x8, int64_t x8_pitch, float *dx,
@@ -493,16 +490,8 @@ cudaError_t launch_swiglu_quantize_a8(const uint16_t *h, int64_t M, int64_t I, i
     int64_t threads = ((I >> 3) + 31) / 32 * 32;
     if (threads > 1024) threads = 1024;
     if (M > 64 && threads > 256) threads = 256;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)M);
-    cfg.blockDim = dim3((unsigned)threads);
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, operand_order ? swiglu_quantize_a8_kernel<true> : swiglu_quantize_a8_kernel<false>, h, M, I, x8, x8_pitch, dx, act_f16);
+    return launch_overlapped(operand_order ? swiglu_quantize_a8_kernel<true> : swiglu_quantize_a8_kernel<false>, dim3((unsigned)M), (unsigned)threads, 0, st, 1,
+                             h, M, I, x8, x8_pitch, dx, act_f16);
 }
 
 // ---------------------------------------------------------------- cq_debug_wait_timeout

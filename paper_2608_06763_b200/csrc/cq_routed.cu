@@ -4,6 +4,7 @@
 // all matrices of a class of row counts (cq_gemm_routed in cq_api.cu).
 #include "cq_common.cuh"
 #include "cq_internal.h"
+#include "cq_tc_ptx.cuh"
 
 namespace cq {
 
@@ -12,6 +13,7 @@ namespace cq {
 __global__ void __launch_bounds__(256) gather_rows_kernel(const uint16_t *__restrict__ x, const int32_t *__restrict__ route_token,
                                                          uint16_t *__restrict__ xg, int64_t R, int64_t T, int64_t K, bool wide,
                                                          int *__restrict__ status, int *__restrict__ counters, int64_t n) {
+    tc::wait_for_previous_kernel();
     const int64_t r = blockIdx.x;
     for (int64_t i = r * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) counters[i] = 0;
     if (r == 0 && threadIdx.x == 0) *status = 0;
@@ -30,8 +32,7 @@ __global__ void __launch_bounds__(256) gather_rows_kernel(const uint16_t *__rest
 cudaError_t launch_gather_rows(const uint16_t *x, const int32_t *route_token, uint16_t *xg, int64_t R, int64_t T, int64_t K,
                                int *status, int *counters, int64_t n, cudaStream_t st) {
     const bool wide = K % 8 == 0 && ((reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(xg)) & 15u) == 0;
-    gather_rows_kernel<<<(unsigned)R, 256, 0, st>>>(x, route_token, xg, R, T, K, wide, status, counters, n);
-    return cudaGetLastError();
+    return launch_overlapped(gather_rows_kernel, dim3((unsigned)R), 256, 0, st, 1, x, route_token, xg, R, T, K, wide, status, counters, n);
 }
 
 }  // namespace cq
