@@ -104,6 +104,10 @@ GemvPlan gemv_plan(const Dims &d, int64_t M, int mode);
 // prequantized (Dynamic A8 only): the workspace already holds the INT8 carrier and the row scales of x (x is not read)
 cudaError_t launch_gemv(const void *layout, const Dims &d, const uint16_t *x, uint16_t *y, int64_t M, int mode,
                         bool act_f16, uint8_t *ws, const Workspace &plan, cudaStream_t st, bool prequantized = false);
+// One and two tokens in the model dtype, strips of sixteen channels, where K and the workspace allow it (cq_gemv_strip.cu).
+bool gemv_strip_ok(const Dims &d, int64_t M, const Workspace &plan);
+cudaError_t launch_gemv_strip(const void *layout, const Dims &d, const uint16_t *x, uint16_t *y, int64_t M, bool act_f16,
+                              float *partial, int *counters, cudaStream_t st);
 // every group 1 .. 16 rows; x and y are those of all groups; P CTAs and a workspace slice for each group
 cudaError_t launch_gemv_groups(const GroupTable &groups, const Dims &d, const uint16_t *x, const int8_t *xq, const float *dxs, uint16_t *y,
                                int mode, bool act_f16, int P, float *partial, int *counters, int *status, cudaStream_t st);
