@@ -3,6 +3,8 @@
 
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 #include "cq_common.cuh"
 #include "cq_internal.h"
 
@@ -19,7 +21,7 @@ Workspace plan_workspace(const Dims &d, int64_t M, int mode) {
     Workspace w{};
     const int64_t Kp = (int64_t)d.KT * TILE;
     const int64_t Mc = M < 16 ? M : 16;  // rows handled by one small-M launch
-    const GemvPlan gp = gemv_plan(d, Mc, mode);
+    const GemvPlan gp = gemv_plan(d);
     size_t off = 0;
     w.status_off = off; off += 256;  // first, so cq_gemm_status finds it without knowing the problem
     // arrival counters: one per 128-row block (small M) or per output tile (split-K GEMM)
@@ -286,7 +288,7 @@ static int for_routed_launches(const Dims &d, const void *const *layouts, const 
             return CQ_OK;
         }
         // small-M groups share the places of the whole GPU; a run of fewer than four tiles is mostly overhead
-        const int64_t T = (int64_t)d.NB * d.KT, places = cls == 0 ? gemv_plan(d, 16, mode).ctas : 0;
+        const int64_t T = (int64_t)d.NB * d.KT, places = cls == 0 ? std::min<int64_t>(2 * (int64_t)sm_count(), T) : 0;
         int64_t P = places / t.n;
         if (P > T / 4) P = T / 4;
         return f(t, cls, max_rows, (int)(P < 1 ? 1 : P));
@@ -397,7 +399,7 @@ int cq_gemm_routed(const void *const *layouts_host, int E, int B, int G, const u
             if (e != cudaSuccess) return wrap(e);
             quantised = true;
         }
-        if (cls == 0) return wrap(launch_gemv_groups(t, d, xg, xq, dxs, y_routes, mode, f16, P, reinterpret_cast<float *>(ws + plan.part_off), counters, status, s));
+        if (cls == 0) return wrap(launch_gemv_groups(t, d, xg, xq, dxs, y_routes, mode, f16, P, reinterpret_cast<float *>(ws + plan.part_off), counters, s));
         if (mode == CQ_MODEL_DTYPE) return wrap(launch_gemm_tc_groups(t, d, xg, y_routes, R, max_rows, f16, status, s));
         return wrap(launch_gemm_a8_groups(t, d, xq, dxs, y_routes, R, max_rows, f16, status, s));
     });

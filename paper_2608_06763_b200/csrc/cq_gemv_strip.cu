@@ -45,13 +45,6 @@ __host__ __device__ constexpr int64_t strip_smem_bytes(int B, int G, int NT, int
 __host__ __device__ inline int64_t run_start(int64_t c, int64_t U, int64_t P) { return U * c / P; }
 __host__ __device__ inline int64_t run_of(int64_t u, int64_t U, int64_t P) { return ((u + 1) * P - 1) / U; }
 
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void *src) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async8(uint32_t dst, const void *src) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst), "l"(src) : "memory");
-}
-
 struct StripParams {
     const uint8_t *layout;
     const uint16_t *x;
@@ -163,32 +156,10 @@ gemv_strip_kernel(const __grid_constant__ StripParams p) {
             uint4 v4 = make_uint4(0u, 0u, 0u, 0u);
             if ((int64_t)c * 8 < p.K) v4 = *reinterpret_cast<const uint4 *>(p.x + m * p.K + (int64_t)c * 8);   // K % 8 == 0 always
             uint32_t ws[4] = {v4.x, v4.y, v4.z, v4.w};
-            unsigned mx = 0;
-#pragma unroll
-            for (int q = 0; q < 4; ++q) mx = __vmaxu2(mx, ws[q] & 0x7FFF7FFFu);
-            const unsigned half_warp = (lane & 16) ? 0xFFFF0000u : 0x0000FFFFu;   // chunks and threads are multiples of sixteen
-#pragma unroll
-            for (int o = 1; o < 16; o <<= 1) mx = __vmaxu2(mx, __shfl_xor_sync(half_warp, mx, o));
-            bool usable;
-            const int e_max = act_max_exponent(max(mx & 0xFFFFu, mx >> 16), p.xf16, usable);   // |x| of the tile below 2^(e_max + 1)
-            int sh = usable ? 10 - e_max : 0;   // the largest in [2^10, 2^11): sixteen products of a normalised level stay in fp16
-            sh = max(min(sh, 100), -100);
-            const float sc = __uint_as_float((uint32_t)(127 + sh) << 23);
-            if ((lane & 15) == 0) s_inv[(c >> 4) * NT + m] = __uint_as_float((uint32_t)(127 - sh) << 23);
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-                ws[q] = as_u32(__floats2half2_rn(act_to_float(ws[q] & 0xFFFFu, p.xf16) * sc, act_to_float(ws[q] >> 16, p.xf16) * sc));
-            __half *row = xs + (size_t)m * KT * TILE;
-            if constexpr (B != 3) {
-                *reinterpret_cast<uint4 *>(row + c * 8) = make_uint4(ws[0], ws[1], ws[2], ws[3]);
-            } else {   // W3 reads its activations in the operand order of cq_decode.cuh
-                __half *blk = row + (c >> 2) * 32 + 16 * (c & 1) + 2 * ((c >> 1) & 1);   // t = 2 (c & 1), a = (c >> 1) & 1
-#pragma unroll
-                for (int tt = 0; tt < 2; ++tt) {   // values k+0, k+2 (e = 0) | k+1, k+3 (e = 1) of t = 2 (c & 1) + tt
-                    *reinterpret_cast<uint32_t *>(blk + 8 * tt) = prmt(ws[2 * tt], ws[2 * tt + 1], 0x5410u);
-                    *reinterpret_cast<uint32_t *>(blk + 8 * tt + 4) = prmt(ws[2 * tt], ws[2 * tt + 1], 0x7632u);
-                }
-            }
+            // the largest in [2^10, 2^11): sixteen products of a normalised level stay in fp16
+            const float back = scale_to_half(ws, p.xf16, 10, lane);   // chunks and threads are multiples of sixteen
+            if ((lane & 15) == 0) s_inv[(c >> 4) * NT + m] = back;
+            store_half_chunk<B>(xs + (size_t)m * KT * TILE + (c & ~15) * 8, c & 15, ws);
         }
     }
     __syncthreads();

@@ -34,6 +34,46 @@ __device__ __forceinline__ void mma_s8_z(int (&d)[4], const uint32_t (&a)[4], ui
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "r"(0));
 }
 
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void *src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async8(uint32_t dst, const void *src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst), "l"(src) : "memory");
+}
+
+// Activations for the fp16 products.  Sixteen lanes hold the 128 k of a token and tile, eight values each (v, in the model
+// dtype); they agree on the power of two that puts the largest into [2^top, 2^(top + 1)) and leave with fp16 values.  Returns
+// what takes the scale back.  Both halves of a warp need not hold work, but a half that does holds it in all its lanes.
+__device__ __forceinline__ float scale_to_half(uint32_t (&v)[4], bool xf16, int top, int lane) {
+    unsigned mx = 0;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) mx = __vmaxu2(mx, v[q] & 0x7FFF7FFFu);
+    const unsigned half_warp = (lane & 16) ? 0xFFFF0000u : 0x0000FFFFu;
+#pragma unroll
+    for (int o = 1; o < 16; o <<= 1) mx = __vmaxu2(mx, __shfl_xor_sync(half_warp, mx, o));
+    bool usable;
+    const int e_max = act_max_exponent(max(mx & 0xFFFFu, mx >> 16), xf16, usable);   // the largest lies in [2^e_max, 2^(e_max + 1))
+    const int sh = max(min(usable ? top - e_max : 0, 100), -100);
+    const float sc = __uint_as_float((uint32_t)(127 + sh) << 23);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) v[q] = as_u32(__floats2half2_rn(act_to_float(v[q] & 0xFFFFu, xf16) * sc, act_to_float(v[q] >> 16, xf16) * sc));
+    return __uint_as_float((uint32_t)(127 - sh) << 23);
+}
+// Chunk c (eight values) of a tile's 128 staged activations; W3 reads them in the operand order of cq_decode.cuh.
+template <int B>
+__device__ __forceinline__ void store_half_chunk(__half *tile, int c, const uint32_t (&v)[4]) {
+    if constexpr (B != 3) {
+        *reinterpret_cast<uint4 *>(tile + c * 8) = make_uint4(v[0], v[1], v[2], v[3]);
+    } else {
+        __half *blk = tile + (c >> 2) * 32 + 16 * (c & 1) + 2 * ((c >> 1) & 1);   // t = 2 (c & 1), a = (c >> 1) & 1
+#pragma unroll
+        for (int tt = 0; tt < 2; ++tt) {   // values k+0, k+2 (e = 0) | k+1, k+3 (e = 1) of t = 2 (c & 1) + tt
+            *reinterpret_cast<uint32_t *>(blk + 8 * tt) = prmt(v[2 * tt], v[2 * tt + 1], 0x5410u);
+            *reinterpret_cast<uint32_t *>(blk + 8 * tt + 4) = prmt(v[2 * tt], v[2 * tt + 1], 0x7632u);
+        }
+    }
+}
+
 template <int B, int GPT>
 struct TileRegs {
     uint32_t w[2 * B];

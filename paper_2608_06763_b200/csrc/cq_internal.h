@@ -95,10 +95,9 @@ constexpr int MAX_GROUPS = 32;
 struct Group { const void *layout; int row0, rows, unit0; };
 struct GroupTable { int n; Group g[MAX_GROUPS]; };
 
-// Decomposition of the small-M path: number of CTAs (one contiguous run of tiles each) and the
-// largest number of CTAs that contribute to one 128-row block.
-struct GemvPlan { int ctas, max_run, overhead; };
-GemvPlan gemv_plan(const Dims &d, int64_t M, int mode);
+// Decomposition of the small-M path: number of CTAs (one contiguous run of tiles each).
+struct GemvPlan { int ctas; };
+GemvPlan gemv_plan(const Dims &d);
 
 // Small-M (M <= 16) split-K tensor-core GEMV, both activation modes.
 // prequantized (Dynamic A8 only): the workspace already holds the INT8 carrier and the row scales of x (x is not read)
@@ -110,7 +109,7 @@ cudaError_t launch_gemv_strip(const void *layout, const Dims &d, const uint16_t 
                               float *partial, int *counters, cudaStream_t st);
 // every group 1 .. 16 rows; x and y are those of all groups; P CTAs and a workspace slice for each group
 cudaError_t launch_gemv_groups(const GroupTable &groups, const Dims &d, const uint16_t *x, const int8_t *xq, const float *dxs, uint16_t *y,
-                               int mode, bool act_f16, int P, float *partial, int *counters, int *status, cudaStream_t st);
+                               int mode, bool act_f16, int P, float *partial, int *counters, cudaStream_t st);
 // `R` rows of x in all, every group at most `tile_m` rows to a token tile of that size class
 cudaError_t launch_gemm_tc_groups(const GroupTable &groups, const Dims &d, const uint16_t *x, uint16_t *y, int64_t R, int64_t tile_m,
                                   bool act_f16, int *status, cudaStream_t st);

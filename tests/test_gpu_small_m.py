@@ -69,3 +69,16 @@ def check(N, K, B, G, M, mode, dtype=torch.bfloat16):
 ])
 def test_strips(N, K, B, G, M):
     check(N, K, B, G, M, cq.CQ_MODEL_DTYPE, torch.float16 if N == 2000 else torch.bfloat16)
+
+
+@pytest.mark.parametrize("mode", [cq.CQ_MODEL_DTYPE, cq.CQ_DYN_A8])
+@pytest.mark.parametrize("M", [3, 8, 9, 16])
+@pytest.mark.parametrize("N,K,B,G", [
+    (100, 128, 4, 128),       # one tile
+    (2816, 2048, 4, 64),      # runs that cross into the next row block
+    (57344, 128, 5, 64),      # a row block is a single tile
+    (8192, 8192, 8, 128),     # long runs; sixteen rows of a run do not fit shared memory at a time
+    (24576, 1056, 6, 32),     # K ends inside a tile, several row blocks to a run
+])
+def test_row_blocks(N, K, B, G, M, mode):
+    check(N, K, B, G, M, mode, torch.float16 if N == 2816 else torch.bfloat16)
