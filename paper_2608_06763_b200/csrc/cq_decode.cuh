@@ -191,30 +191,82 @@ __device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t sel) {
     return d;
 }
 
-// ---- W4, model dtype: eight levels of a (row, group) as 16-bit values, their low bytes in t.x (magnitudes 0-3) and
-// t.y (4-7), their high bytes in t.z and t.w.  A half-word of the layout is the selector of four neighbouring
-// weights; two byte permutes fetch their low and high bytes, two more put the bytes together, and the sign bits
-// go into the high bytes by one exclusive or.  Thirteen integer instructions for eight weights, against some forty for
+// packed pairs of fp32
+__device__ __forceinline__ uint64_t f2_pack(uint32_t lo, uint32_t hi) { uint64_t d; asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "r"(lo), "r"(hi)); return d; }
+__device__ __forceinline__ void f2_split(uint64_t v, uint32_t &lo, uint32_t &hi) { asm("mov.b64 {%0, %1}, %2;" : "=r"(lo), "=r"(hi) : "l"(v)); }
+__device__ __forceinline__ uint64_t f2_dup(float v) { return f2_pack(__float_as_uint(v), __float_as_uint(v)); }
+__device__ __forceinline__ uint64_t f2_add(uint64_t a, uint64_t b) { uint64_t d; asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b)); return d; }
+__device__ __forceinline__ uint64_t f2_mul(uint64_t a, uint64_t b) { uint64_t d; asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b)); return d; }
+__device__ __forceinline__ uint64_t f2_fma(uint64_t a, uint64_t b, uint64_t c) { uint64_t d; asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c)); return d; }
+__device__ __forceinline__ uint32_t mul_sat(uint32_t a, uint32_t b) {
+    float d;
+    asm("mul.rn.sat.f32 %0, %1, %2;" : "=f"(d) : "f"(__uint_as_float(a)), "f"(__uint_as_float(b)));
+    return __float_as_uint(d);
+}
+
+// ---- W4: eight magnitudes of a (row, group) by table.  In the model dtype the levels are 16-bit values, kept as
+// {low bytes of magnitudes 0-3, high bytes of 0-3, low bytes of 4-7, high bytes of 4-7}.  A half-word of the layout is the selector
+// of four neighbouring weights; two byte permutes fetch their low and high bytes, two more put the bytes together, and the
+// sign bits go into the high bytes by one exclusive or.  Thirteen integer instructions for eight weights, against some forty for
 // the half2 polynomial, its scale in fp32 and the rounding to the operand's type; the levels themselves are evaluated in fp32
 // and rounded once.  Measured on the linears of an 8B layer, G = 128: M = 1 66.6 -> 56.8 us, M = 13 109.7 -> 105.5,
-// M = 200 (binary16) 194.8 -> 167.7, M = 1024 509.5 -> 491.6 (what is left there is not the decode).  out[i] = weights (2 i, 2 i + 1) of the word, in k order; a reserved code reads (minus) zero.
-__device__ __forceinline__ void w4_block(uint32_t word, const uint4 &t, uint32_t (&out)[4]) {
-    const uint32_t sel = word & 0x77777777u, sel1 = sel >> 16, w4 = word << 4;
-    const uint32_t l0 = prmt(t.x, t.y, sel), h0 = prmt(t.z, t.w, sel) ^ (word & 0x80808080u);
-    const uint32_t l1 = prmt(t.x, t.y, sel1), h1 = prmt(t.z, t.w, sel1) ^ (w4 & 0x80808080u);
+// M = 200 (binary16) 194.8 -> 167.7, M = 1024 509.5 -> 491.6 (what is left there is not the decode).  The integer pipe takes one
+// of these instructions every other cycle and bounds the small products, so the shift by four is a multiplication, which
+// goes to another pipe: x16 is 16, read from memory so that it stays one.  out[i] = weights (2 i, 2 i + 1) of the word, in k
+// order; a reserved code reads (minus) zero.
+__constant__ uint32_t c_w4_x16 = 16u;
+__device__ __forceinline__ void w4_block(uint32_t word, const uint4 &t, uint32_t x16, uint32_t (&out)[4]) {
+    const uint32_t sel = word & 0x77777777u, sel1 = sel >> 16, w4 = word * x16;
+    const uint32_t l0 = prmt(t.x, t.z, sel), h0 = prmt(t.y, t.w, sel) ^ (word & 0x80808080u);
+    const uint32_t l1 = prmt(t.x, t.z, sel1), h1 = prmt(t.y, t.w, sel1) ^ (w4 & 0x80808080u);
     out[0] = prmt(l0, h0, 0x5140u); out[1] = prmt(l0, h0, 0x7362u);
     out[2] = prmt(l1, h1, 0x5140u); out[3] = prmt(l1, h1, 0x7362u);
 }
-// The four lanes t of a row evaluate two levels each (magnitudes 2 t and 2 t + 1, at t0 and t1 = magnitude / 7, by the
-// fp32 Horner form of Eq. gpu-horner, times f) and leave their bytes in the row's 16-byte table in shared memory.
+// The tables of a warp's sixteen rows: lane l evaluates the four magnitudes 4 (l & 1) .. + 3 of row l >> 1, two at a time in
+// packed fp32, by the Horner form of Eq. gpu-horner.
+struct W4Lane { uint64_t t01, t23; };   // their positions, magnitude / 7
+__device__ __forceinline__ W4Lane w4_lane(int lane) {
+    const int i = 4 * (lane & 1);
+    auto at = [](int k) { return __float_as_uint((float)k / 7.0f); };
+    return {f2_pack(at(i), at(i + 1)), f2_pack(at(i + 2), at(i + 3))};
+}
+// q at the four positions; rec: the record of the lane's row
+__device__ __forceinline__ void w4_curve(const W4Lane &w, uint2 rec, uint64_t &q01, uint64_t &q23) {
+    const __half2 ab = as_h2(rec.y);
+    const float a = __low2float(ab), b = __high2float(ab);
+    const uint64_t a2 = f2_dup(a), b2 = f2_dup(b), c2 = f2_dup(__fsub_rn(__fsub_rn(1.0f, a), b));
+    q01 = f2_mul(w.t01, f2_fma(w.t01, f2_fma(w.t01, c2, b2), a2));
+    q23 = f2_mul(w.t23, f2_fma(w.t23, f2_fma(w.t23, c2, b2), a2));
+}
+// levels times f into the warp's tables, [row][16 bytes]; pack: two fp32 values to the operand's type
 template <class Pack>
-__device__ __forceinline__ void w4_put(uint8_t *row, uint2 p, int t, float t0, float t1, float f, Pack pack) {
-    const __half2 ab = as_h2(p.y);
-    const float a = __low2float(ab), b = __high2float(ab), c = (1.0f - a) - b;
-    const float q0 = t0 * fmaf(t0, fmaf(t0, c, b), a), q1 = t1 * fmaf(t1, fmaf(t1, c, b), a);
-    const uint32_t v = pack(q0 * f, q1 * f), bytes = prmt(v, 0u, 0x3120u);   // low bytes, then high bytes
-    *reinterpret_cast<uint16_t *>(row + 2 * t) = (uint16_t)bytes;
-    *reinterpret_cast<uint16_t *>(row + 8 + 2 * t) = (uint16_t)(bytes >> 16);
+__device__ __forceinline__ void w4_put(uint8_t *tables, int lane, const W4Lane &w, uint2 rec, float f, Pack pack) {
+    uint64_t q01, q23;
+    uint32_t q[4];
+    w4_curve(w, rec, q01, q23);
+    f2_split(q01, q[0], q[1]); f2_split(q23, q[2], q[3]);
+    const uint32_t v0 = pack(__uint_as_float(q[0]) * f, __uint_as_float(q[1]) * f), v1 = pack(__uint_as_float(q[2]) * f, __uint_as_float(q[3]) * f);
+    *reinterpret_cast<uint2 *>(tables + lane * 8) = make_uint2(prmt(v0, v1, 0x6420u), prmt(v0, v1, 0x7531u));
+}
+// Dynamic A8: carriers (carrier_at: clamping q to [0, 1] clamps them, adding 1.5 2^23 rounds to nearest even and leaves the
+// integer in the low bits), positive ones at 0 .. 7 of the row's table, negative ones at 8 .. 15
+__device__ __forceinline__ void w4_put_carriers(int8_t *tables, int lane, const W4Lane &w, uint2 rec) {
+    const __half2 ab = as_h2(rec.y);
+    const float a = __low2float(ab), b = __high2float(ab);
+    const uint64_t a2 = f2_dup(a), b2 = f2_dup(b), c2 = f2_dup(__fsub_rn(__fsub_rn(1.0f, a), b));
+    auto pair = [&](uint64_t t, uint32_t &r0, uint32_t &r1) {
+        uint32_t t0, t1, h0, h1;
+        f2_split(t, t0, t1);
+        f2_split(f2_fma(t, f2_fma(t, c2, b2), a2), h0, h1);
+        f2_split(f2_add(f2_mul(f2_pack(mul_sat(t0, h0), mul_sat(t1, h1)), f2_dup(127.0f)), f2_dup(12582912.0f)), r0, r1);
+    };
+    uint32_t r[4];
+    pair(w.t01, r[0], r[1]);
+    pair(w.t23, r[2], r[3]);
+    const uint32_t up = prmt(prmt(r[0], r[1], 0x0040u), prmt(r[2], r[3], 0x0040u), 0x5410u);   // four bytes of 0 .. 127
+    uint32_t *row = reinterpret_cast<uint32_t *>(tables + (lane >> 1) * 16) + (lane & 1);
+    row[0] = up;
+    row[2] = (0x80808080u - up) ^ 0x80808080u;   // their negatives: no byte borrows, and zero stays zero
 }
 
 // Dynamic A8 operand order (both INT8 kernels).  One k = 32 MMA step takes the 32-wide k block m of a
@@ -246,7 +298,7 @@ __device__ __forceinline__ CarrierTab load_carrier_tab(const int8_t *row) {
 }
 __device__ __forceinline__ uint32_t pick(uint32_t mask, uint32_t a, uint32_t b) { return (a & mask) | (b & ~mask); }
 template <int B, int RR, int MI>
-__device__ __forceinline__ void a8_row_regs(const uint32_t (&w)[2 * B], const CarrierTab &ct, uint32_t &lo, uint32_t &hi) {
+__device__ __forceinline__ void a8_row_regs(const uint32_t (&w)[2 * B], const CarrierTab &ct, uint32_t x16, uint32_t &lo, uint32_t &hi) {
     static_assert(B <= 5, "wider codes are evaluated one by one (a8_row_eval)");
     const uint4 &tab = ct.v[0];
     if constexpr (B == 5) {
@@ -260,7 +312,7 @@ __device__ __forceinline__ void a8_row_regs(const uint32_t (&w)[2 * B], const Ca
         hi = pick(k_hi, pick(m_hi, prmt(t2.z, t2.w, wh), prmt(t2.x, t2.y, wh)), pick(m_hi, prmt(tab.z, tab.w, wh), prmt(tab.x, tab.y, wh)));
     } else if constexpr (B == 4) {
         const uint32_t word = w[2 * MI + RR];
-        const uint32_t ws = word & 0x77777777u, wh = ws >> 16, w4 = word << 4;
+        const uint32_t ws = word & 0x77777777u, wh = ws >> 16, w4 = word * x16;   // x16 = 16 (w4_block)
         const uint32_t m_lo = prmt(word, word, 0xBA98u), m_hi = prmt(w4, w4, 0xBA98u);   // 0xFF where the code is negative
         const uint32_t p_lo = prmt(tab.x, tab.y, ws), n_lo = prmt(tab.z, tab.w, ws);
         const uint32_t p_hi = prmt(tab.x, tab.y, wh), n_hi = prmt(tab.z, tab.w, wh);
@@ -290,17 +342,6 @@ __device__ __forceinline__ void a8_row_regs(const uint32_t (&w)[2 * B], const Ca
 // sequence of carrier_at.  A table per (row, group) would have as many entries as the group has weights (W8, G = 128), and
 // reading it costs a shared-memory access per weight with the lanes in random banks: linears of an 8B layer, W8 G128,
 // M = 64: 400 us with tables, 204 us so.
-__device__ __forceinline__ uint64_t f2_pack(uint32_t lo, uint32_t hi) { uint64_t d; asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "r"(lo), "r"(hi)); return d; }
-__device__ __forceinline__ void f2_split(uint64_t v, uint32_t &lo, uint32_t &hi) { asm("mov.b64 {%0, %1}, %2;" : "=r"(lo), "=r"(hi) : "l"(v)); }
-__device__ __forceinline__ uint64_t f2_dup(float v) { return f2_pack(__float_as_uint(v), __float_as_uint(v)); }
-__device__ __forceinline__ uint64_t f2_add(uint64_t a, uint64_t b) { uint64_t d; asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b)); return d; }
-__device__ __forceinline__ uint64_t f2_mul(uint64_t a, uint64_t b) { uint64_t d; asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b)); return d; }
-__device__ __forceinline__ uint64_t f2_fma(uint64_t a, uint64_t b, uint64_t c) { uint64_t d; asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c)); return d; }
-__device__ __forceinline__ uint32_t mul_sat(uint32_t a, uint32_t b) {
-    float d;
-    asm("mul.rn.sat.f32 %0, %1, %2;" : "=f"(d) : "f"(__uint_as_float(a)), "f"(__uint_as_float(b)));
-    return __float_as_uint(d);
-}
 struct CarrierPoly { uint64_t a, b, c; };
 __device__ __forceinline__ CarrierPoly carrier_poly(uint32_t ab16) {
     const __half2 ab = as_h2(ab16);

@@ -239,6 +239,9 @@ gemm_a8_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
         const int q4 = warp & 3, cq4 = dw >> 2;
         const int drow = q4 * 32 + lane;
         int8_t *tab = sTab + dw * 16 * NCODE;
+        W4Lane w4{};
+        uint32_t x16 = 16u;
+        if constexpr (B == 4) { w4 = w4_lane(lane); x16 = c_w4_x16; }
         float acc[QCOLS];
 #pragma unroll
         for (int i = 0; i < QCOLS; ++i) acc[i] = 0.0f;
@@ -299,20 +302,24 @@ gemm_a8_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
                             };
                             if (!fix) eval(std::false_type{}); else eval(std::true_type{});
                         } else {
-                            if constexpr (B >= 3) {
+                            if constexpr (B == 4) {
+                                __syncwarp();
+                                w4_put_carriers(tab, lane, w4, *(const uint2 *)(raw + d.code_bytes + ((rb * 16 + (lane >> 1)) * GPT + gi) * 8));
+                                __syncwarp();
+                            } else if constexpr (B >= 3) {
                                 // signed carrier table: index = stored code u (reserved -> 0), entry sign(k) r(|k|)
                                 __syncwarp();
                                 auto build_row = [&](int row, uint32_t abbits) {
                                     const __half2 ab = as_h2(abbits);
                                     const float a = __low2float(ab), b = __high2float(ab);
                                     int8_t *tr = tab + row * NCODE;
-                                    if (B != 4 && tq == 0) tr[0] = 0;
+                                    if (tq == 0) tr[0] = 0;
 #pragma unroll
                                     for (int i0 = 0; i0 <= Mx; i0 += 4) {
                                         const int i = i0 + tq;
                                         const int r = carrier_at(sT[i], a, b);
                                         tr[carrier_slot(B, i, false)] = (int8_t)r;
-                                        if (B == 4 || i > 0) tr[carrier_slot(B, i, true)] = (int8_t)(-r);
+                                        if (i > 0) tr[carrier_slot(B, i, true)] = (int8_t)(-r);
                                     }
                                 };
                                 build_row(g, p_lo.y);
@@ -326,8 +333,8 @@ gemm_a8_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
                             static_for<MPG>([&](auto mc) {
                                 constexpr int MI = gi * MPG + decltype(mc)::value;
                                 uint2 lo, hi;
-                                a8_row_regs<B, 0, MI>(w, tab_lo, lo.x, lo.y);
-                                a8_row_regs<B, 1, MI>(w, tab_hi, hi.x, hi.y);
+                                a8_row_regs<B, 0, MI>(w, tab_lo, x16, lo.x, lo.y);
+                                a8_row_regs<B, 1, MI>(w, tab_hi, x16, hi.x, hi.y);
                                 *(uint2 *)(row_lo + place(MI)) = lo;
                                 *(uint2 *)(row_hi + place(MI)) = hi;
                             });

@@ -362,8 +362,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
         // Where the MMAs of a block are short the decoders set the pace, and a fence (some 200 cycles) is shared by a tile's
         // two blocks; a wide token tile wants its blocks as early as they are ready.
         constexpr bool ONE_FENCE = BNT <= 128 && STAGES >= 6;
-        float w4_t0 = 0.0f, w4_t1 = 0.0f;   // W4: positions of the two levels this lane evaluates for a table
-        if constexpr (B == 4) { w4_t0 = (float)(2 * t) / 7.0f; w4_t1 = (float)(2 * t + 1) / 7.0f; }
+        W4Lane w4{};
+        uint32_t x16 = 16u;
+        if constexpr (B == 4) { w4 = w4_lane(lane); x16 = c_w4_x16; }
 #pragma unroll 1
         while (walk.next(seg)) {
 #pragma unroll 1
@@ -386,11 +387,14 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
                     w[4 * NFQ + 0] = v.x; w[4 * NFQ + 1] = v.y;
                 }
             }
-            uint2 q_lo[GPT], q_hi[GPT];   // the parameter records of rows g and g + 8
+            uint2 q_lo[GPT], q_hi[GPT];   // the parameter records of rows g and g + 8; W4: of row lane / 2, whose tables the lane helps to build
             {
-                const uint8_t *prow = raw + d.code_bytes + ((rb * 16 + g) * GPT) * 8;
+                const uint8_t *prow = raw + d.code_bytes + ((rb * 16 + (B == 4 ? lane >> 1 : g)) * GPT) * 8;
 #pragma unroll
-                for (int i = 0; i < GPT; ++i) { q_lo[i] = *(const uint2 *)(prow + i * 8); q_hi[i] = *(const uint2 *)(prow + (8 * GPT + i) * 8); }
+                for (int i = 0; i < GPT; ++i) {
+                    q_lo[i] = *(const uint2 *)(prow + i * 8);
+                    if constexpr (B != 4) q_hi[i] = *(const uint2 *)(prow + (8 * GPT + i) * 8);
+                }
             }
             W3Table w3_lo{}, w3_hi{};   // W3: level tables of rows g and g + 8; one per tile when the group spans it
             if constexpr (B == 3 && G == 128) {
@@ -412,11 +416,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
                 __syncwarp();   // the tables before have been read
 #pragma unroll
                 for (int e = 0; e < n; ++e) {
-                    const uint2 p_lo = q_lo[gi0 + e], p_hi = q_hi[gi0 + e];
-                    const float s_lo = __uint_as_float(p_lo.x & 0x7FFFFFFFu), s_hi = __uint_as_float(p_hi.x & 0x7FFFFFFFu);
+                    const uint2 rec = q_lo[gi0 + e];
                     auto pack = [&](float a, float b) { return pack_act2(a, b, prm.f16); };
-                    w4_put(wtab + e * 256 + g * 16, p_lo, t, w4_t0, w4_t1, s_lo, pack);
-                    w4_put(wtab + e * 256 + (g + 8) * 16, p_hi, t, w4_t0, w4_t1, s_hi, pack);
+                    w4_put(wtab + e * 256, lane, w4, rec, __uint_as_float(rec.x & 0x7FFFFFFFu), pack);
                 }
                 __syncwarp();
             };
@@ -450,8 +452,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
                         }
                         const uint32_t x_lo = odd ? w[4 * H + 2 * (1 - e)] : w[4 * H + 2 * e], x_hi = odd ? w[4 * H + 2 * (1 - e) + 1] : w[4 * H + 2 * e + 1];
                         uint32_t o_lo[4], o_hi[4];
-                        w4_block(x_lo, w4_lo, o_lo);
-                        w4_block(x_hi, w4_hi, o_hi);
+                        w4_block(x_lo, w4_lo, x16, o_lo);
+                        w4_block(x_hi, w4_hi, x16, o_hi);
                         const int off = ((4 * u + t) ^ g) * 16;
                         *(uint4 *)(row_lo + off) = make_uint4(o_lo[0], o_lo[1], o_lo[2], o_lo[3]);
                         *(uint4 *)(row_hi + off) = make_uint4(o_hi[0], o_hi[1], o_hi[2], o_hi[3]);

@@ -3,8 +3,8 @@
 // path; Section 5.4 for Dynamic A8).
 //
 // Work decomposition: the NB x KT grid of 128 x 128 weight tiles is cut into P equal contiguous runs in row-block-major
-// order, one per CTA, one CTA per SM.  Eight warps, one per group of 16 rows, take a tile together; a CTA has two or three
-// such sets (gemv_sets), which take the tiles of the run in turn.  At the end of a row block the sets' sums meet in shared
+// order, one per CTA.  Eight warps, one per group of 16 rows, take a tile together; a CTA has up to three such sets
+// (gemv_sets), which take the tiles of the run in turn.  At the end of a row block the sets' sums meet in shared
 // memory, and the CTA either writes y (its run holds the whole K range) or a partial sum into one of its two slots; the CTA
 // that completes a row block adds the partials in K order (deterministic) and writes y.
 //
@@ -30,10 +30,17 @@ namespace cq {
 namespace {
 
 // MODE 0: model dtype.  MODE 1: Dynamic A8 (xq = INT8 carrier [M][x8_pitch], dxs = row scales).  NT: blocks of 8 tokens.
-// Sets of eight warps: three where 80 registers a thread suffice, two otherwise (two token blocks; INT8 carriers evaluated code
-// by code, which spilled).
+// Sets of eight warps in a CTA, and CTAs on an SM.  One large CTA reads the activations once per SM and hands over fewer
+// partial sums; it has three sets where 80 registers a thread suffice and two otherwise (two token blocks; INT8 carriers
+// evaluated code by code).  Dynamic A8 only copies its activations, and where runs are short it gains more from CTAs of
+// one set, which leave an SM one by one and let the next kernel's in earlier.  W4 G128, Dynamic A8, M = 16, large CTAs /
+// small ones: 4096 square (6.9 tiles an SM) 13.0 / 12.6 us (W6, M = 8: 18.0 / 16.5), 4096 x 14336 (24 tiles) 20.8 / 22.8,
+// 28672 x 4096 (48) 28.3 / 30.4.
 __host__ __device__ constexpr int gemv_sets(int B, int NT, int MODE) { return NT == 2 || (MODE == 1 && B >= 6) ? 2 : 3; }
+__host__ __device__ constexpr int gemv_occ(int B, int NT, int SETS) { return SETS > 1 ? 1 : NT == 2 || B >= 6 ? 2 : 3; }
+constexpr int A8_LONG_RUN = 12;   // tiles an SM
 // Routed products: one set to a CTA and two CTAs to an SM, so that the CTAs of many small matrices fill the SMs evenly.
+constexpr int GROUP_OCC = 2;
 __host__ __device__ constexpr int gemv_unit_bytes(int B, int G) { return 256 * B + 128 * (TILE / G); }
 __host__ __device__ constexpr int gemv_stages(int B, int G) { return gemv_unit_bytes(B, G) <= 1664 ? 4 : 3; }
 __host__ __device__ constexpr int gemv_ring_bytes(int B, int G, int SETS) { return SETS * 8 * gemv_stages(B, G) * gemv_unit_bytes(B, G); }
@@ -44,8 +51,8 @@ __host__ __device__ constexpr int gemv_table_bytes(int B, int MODE) { return MOD
 __host__ __device__ constexpr int gemv_fixed_bytes(int B, int G, int NT, int MODE, int SETS) {
     return gemv_ring_bytes(B, G, SETS) + gemv_comb_bytes(NT, SETS) + SETS * 8 * gemv_table_bytes(B, MODE);
 }
-// dynamic shared memory of a CTA: what an SM has for it less 1 KB for the system and 512 bytes that the kernel declares
-__host__ __device__ constexpr int gemv_smem(int SETS) { return (SETS == 1 ? 114 : 227) * 1024 - 1536; }
+// dynamic shared memory of a CTA: its share of the SM's 228 KB less 1 KB for the system and 512 bytes that the kernel declares
+__host__ __device__ constexpr int gemv_smem(int OCC) { return (228 / OCC) * 1024 - 1536; }
 // padding of a staged activation row, in elements: rows 64 bytes apart in the banks where a lane reads 16 bytes (W3, W4),
 // 32 where it reads 8
 __host__ __device__ constexpr int gemv_x_pad(int B, int MODE) { return MODE == 1 ? 32 : (B == 3 || B == 4 ? 32 : 16); }
@@ -53,8 +60,8 @@ __host__ __device__ constexpr int gemv_x_pad(int B, int MODE) { return MODE == 1
 __host__ __device__ constexpr int gemv_x_tile_bytes(int M, int MODE) { return MODE == 1 ? M * TILE : M * (TILE * 2 + 4); }
 __host__ __device__ constexpr int gemv_x_fixed_bytes(int M, int B, int MODE) { return M * gemv_x_pad(B, MODE) * (MODE == 1 ? 1 : 2) + 128; }
 // K tiles whose activations fit at a time
-__host__ __device__ constexpr int gemv_x_tiles(int B, int G, int NT, int MODE, int SETS, int M) {
-    return (gemv_smem(SETS) - gemv_fixed_bytes(B, G, NT, MODE, SETS) - gemv_x_fixed_bytes(M, B, MODE)) / gemv_x_tile_bytes(M, MODE);
+__host__ __device__ constexpr int gemv_x_tiles(int B, int G, int NT, int MODE, int SETS, int OCC, int M) {
+    return (gemv_smem(OCC) - gemv_fixed_bytes(B, G, NT, MODE, SETS) - gemv_x_fixed_bytes(M, B, MODE)) / gemv_x_tile_bytes(M, MODE);
 }
 
 // Tile v of the V = NB KT tiles belongs to run c, the largest with floor(V c / P) <= v.
@@ -114,8 +121,9 @@ gemv_body(const uint8_t *__restrict__ layout, const Dims &d, const uint16_t *__r
     for (int i = 0; i < NS - 1; ++i) ring_load(i);
     DecodeRegs dr = {};
     if constexpr (F16 && B != 3 && B != 4) dr = load_decode_regs();
-    float w4_t0 = 0.0f, w4_t1 = 0.0f;   // positions of the two levels this lane evaluates for a table
-    if constexpr (F16 && B == 4) { w4_t0 = (float)(2 * t) / 7.0f; w4_t1 = (float)(2 * t + 1) / 7.0f; }
+    W4Lane w4{};
+    uint32_t x16 = 16u;
+    if constexpr (B == 4) { w4 = w4_lane(lane); x16 = c_w4_x16; }
     if constexpr (MODE == 1 && carrier_by_table(B)) {
         if (threadIdx.x < L) s_t[threadIdx.x] = __fdiv_rn((float)threadIdx.x, (float)(L - 1));
     }
@@ -141,7 +149,8 @@ gemv_body(const uint8_t *__restrict__ layout, const Dims &d, const uint16_t *__r
         float *inv = reinterpret_cast<float *>(xs + (size_t)M * XS * ES);      // F16: [position][M]
         if (i0 > 0) __syncthreads();   // the tiles before are done with
         if constexpr (F16) {
-            // sixteen lanes take a token's 128 k of a tile, eight values each; four loads in flight
+            // sixteen lanes take a token's 128 k of a tile, eight values each; four loads in flight (eight, with the places
+            // counted again for the stores: 4096 square, W4, M = 8 10.4 -> 11.6 us)
             constexpr int STEP = THREADS / 16, BATCH = 4;
             int m = 0, p = (int)threadIdx.x >> 4;
             const int c = threadIdx.x & 15;
@@ -170,14 +179,19 @@ gemv_body(const uint8_t *__restrict__ layout, const Dims &d, const uint16_t *__r
                 }
             }
         } else {
-            const int cpr = n_st * (TILE / 16);   // 16-byte chunks of a row
-            for (int idx = threadIdx.x; idx < M * cpr; idx += THREADS) {
-                const int m = idx / cpr, c = idx - m * cpr;
+            // 16-byte chunks in the order the product reads (a8_row_regs; W4: natural); pitch a multiple of 128, zero beyond K
+            const int cpr = n_st * (TILE / 16);
+            int m = 0, c = threadIdx.x;
+            for (;;) {
+                while (c >= cpr) { c -= cpr; ++m; }
+                if (m >= M) break;
                 int kb = kbs + (c >> 3);
                 if (kb >= KT) kb -= KT;
-                // in the order the product reads (a8_row_regs; W4: natural); pitch a multiple of 128, zero beyond K
-                *reinterpret_cast<uint4 *>(xs + (size_t)m * XS + c * 16) = *reinterpret_cast<const uint4 *>(xq + (int64_t)m * x8_pitch + (int64_t)kb * TILE + (c & 7) * 16);
+                cp_async16((uint32_t)__cvta_generic_to_shared(xs + (size_t)m * XS + c * 16), xq + (int64_t)m * x8_pitch + (int64_t)kb * TILE + (c & 7) * 16);
+                c += THREADS;
             }
+            asm volatile("cp.async.commit_group;" ::: "memory");
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
         }
         __syncthreads();
         // this lane's B-fragment base per token block: row g of the block (token columns beyond M read the last real
@@ -199,7 +213,7 @@ gemv_body(const uint8_t *__restrict__ layout, const Dims &d, const uint16_t *__r
                 ring_load(fill);
                 const uint8_t *stage = ring + st * UB;
                 TileRegs<B, GPT> regs;
-                load_tile<B, GPT>(regs, stage + lane * 16, stage + 256 * B + g * GPT * 8, lane);
+                load_tile<B, GPT>(regs, stage + lane * 16, stage + 256 * B + record_offset<B, GPT>(lane), lane);
                 if (++st == NS) st = 0;
                 if (++fill == NS) fill = 0;
                 float acc[NT][4];
@@ -207,7 +221,7 @@ gemv_body(const uint8_t *__restrict__ layout, const Dims &d, const uint16_t *__r
                 for (int tb = 0; tb < NT; ++tb)
 #pragma unroll
                     for (int q = 0; q < 4; ++q) acc[tb][q] = 0.0f;
-                compute_tile<B, G, NT, MODE>(regs, dr, xs + (size_t)pos * TILE * ES, xo, ctab, s_t, w4_t0, w4_t1, g, t, acc);
+                compute_tile<B, G, NT, MODE>(regs, dr, xs + (size_t)pos * TILE * ES, xo, ctab, s_t, w4, x16, g, t, acc);
 #pragma unroll
                 for (int tb = 0; tb < NT; ++tb) {   // in true units: lane (g, t) holds rows g, g + 8 x tokens 2 t, 2 t + 1
                     float s0 = 1.0f, s1 = 1.0f;
@@ -306,18 +320,18 @@ gemv_body(const uint8_t *__restrict__ layout, const Dims &d, const uint16_t *__r
     }
 }
 
-template <int B, int G, int NT, int MODE>
-__global__ void __launch_bounds__(256 * gemv_sets(B, NT, MODE), 1)
+template <int B, int G, int NT, int MODE, int SETS>
+__global__ void __launch_bounds__(256 * SETS, gemv_occ(B, NT, SETS))
 gemv_kernel(const uint8_t *__restrict__ layout, Dims d, const uint16_t *__restrict__ x, const int8_t *__restrict__ xq,
             int64_t x8_pitch, const float *__restrict__ dxs, uint16_t *__restrict__ y, int M, float *__restrict__ partial,
             int *__restrict__ counters, int x_tiles, bool xf16) {
-    gemv_body<B, G, NT, MODE, gemv_sets(B, NT, MODE)>(layout, d, x, xq, x8_pitch, dxs, y, M, partial, counters, x_tiles, xf16);
+    gemv_body<B, G, NT, MODE, SETS>(layout, d, x, xq, x8_pitch, dxs, y, M, partial, counters, x_tiles, xf16);
 }
 
 // Routed products: blockIdx.y is a group, with its own matrix, rows and slice of the workspace.  (A kernel of its own:
 // the table among the parameters of every small product cost the sweep over formats at M = 1 four per cent.)
 template <int B, int G, int NT, int MODE>
-__global__ void __launch_bounds__(256, 2)
+__global__ void __launch_bounds__(256, GROUP_OCC)
 gemv_groups_kernel(Dims d, const uint16_t *__restrict__ x, const int8_t *__restrict__ xq, int64_t x8_pitch, const float *__restrict__ dxs,
                    uint16_t *__restrict__ y, float *__restrict__ partial, int *__restrict__ counters, int x_tiles, bool xf16,
                    const __grid_constant__ GroupTable groups) {
@@ -328,21 +342,21 @@ gemv_groups_kernel(Dims d, const uint16_t *__restrict__ x, const int8_t *__restr
                               x_tiles, xf16);
 }
 
-template <int B, int G, int NT, int MODE, bool GRP = false>
+template <int B, int G, int NT, int MODE, int SETS, bool GRP = false>
 cudaError_t launch_one(const void *layout, const Dims &d, const uint16_t *x, const int8_t *xq, int64_t x8_pitch,
                        const float *dxs, uint16_t *y, int M, int P, float *partial, int *counters,
                        bool act_f16, cudaStream_t st, const GroupTable *groups = nullptr) {
-    constexpr int SETS = GRP ? 1 : gemv_sets(B, NT, MODE);
-    static_assert(gemv_x_tiles(B, G, NT, MODE, SETS, 8 * NT) >= 2, "shared memory");
+    constexpr int OCC = GRP ? GROUP_OCC : gemv_occ(B, NT, SETS);
+    static_assert(gemv_x_tiles(B, G, NT, MODE, SETS, OCC, 8 * NT) >= 2, "shared memory");
     const int64_t V = (int64_t)d.NB * d.KT;
     int64_t run = (V + P - 1) / P;   // the longest run, or all of K, bounds the activations a CTA stages
     if (run > d.KT) run = d.KT;
-    const int fit = gemv_x_tiles(B, G, NT, MODE, SETS, M), x_tiles = (int)(run < fit ? run : fit);
+    const int fit = gemv_x_tiles(B, G, NT, MODE, SETS, OCC, M), x_tiles = (int)(run < fit ? run : fit);
     const size_t smem = (size_t)gemv_fixed_bytes(B, G, NT, MODE, SETS) + (size_t)gemv_x_fixed_bytes(M, B, MODE) + (size_t)x_tiles * gemv_x_tile_bytes(M, MODE);
     static std::atomic<uint64_t> attr_done{0};
     cudaError_t e;
-    if constexpr (GRP) e = ensure_func_attr(gemv_groups_kernel<B, G, NT, MODE>, attr_done, cudaFuncAttributeMaxDynamicSharedMemorySize, gemv_smem(SETS));
-    else e = ensure_func_attr(gemv_kernel<B, G, NT, MODE>, attr_done, cudaFuncAttributeMaxDynamicSharedMemorySize, gemv_smem(SETS));
+    if constexpr (GRP) e = ensure_func_attr(gemv_groups_kernel<B, G, NT, MODE>, attr_done, cudaFuncAttributeMaxDynamicSharedMemorySize, gemv_smem(OCC));
+    else e = ensure_func_attr(gemv_kernel<B, G, NT, MODE, SETS>, attr_done, cudaFuncAttributeMaxDynamicSharedMemorySize, gemv_smem(OCC));
     if (e != cudaSuccess) return e;
     // Programmatic overlap: this kernel may begin (and prefetch weights) while the previous kernel of the stream drains; it
     // waits for that kernel before touching anything but the weights.
@@ -352,28 +366,31 @@ cudaError_t launch_one(const void *layout, const Dims &d, const uint16_t *x, con
         return launch_overlapped(gemv_groups_kernel<B, G, NT, MODE>, grid, threads, smem, st, 1, d, x, xq, x8_pitch, dxs, y, partial, counters, x_tiles,
                                  act_f16, *groups);
     else
-        return launch_overlapped(gemv_kernel<B, G, NT, MODE>, grid, threads, smem, st, 1, (const uint8_t *)layout, d, x, xq, x8_pitch, dxs, y, M,
+        return launch_overlapped(gemv_kernel<B, G, NT, MODE, SETS>, grid, threads, smem, st, 1, (const uint8_t *)layout, d, x, xq, x8_pitch, dxs, y, M,
                                  partial, counters, x_tiles, act_f16);
 }
 
 template <int B, int G>
 cudaError_t dispatch_nt_mode(const void *layout, const Dims &d, const uint16_t *x, const int8_t *xq, int64_t x8_pitch,
-                             const float *dxs, uint16_t *y, int M, int mode, int P, float *partial, int *counters, bool act_f16, cudaStream_t st) {
-    if (mode == 0) {
-        if (M <= 8) return launch_one<B, G, 1, 0>(layout, d, x, xq, x8_pitch, dxs, y, M, P, partial, counters, act_f16, st);
-        return launch_one<B, G, 2, 0>(layout, d, x, xq, x8_pitch, dxs, y, M, P, partial, counters, act_f16, st);
-    }
-    if (M <= 8) return launch_one<B, G, 1, 1>(layout, d, x, xq, x8_pitch, dxs, y, M, P, partial, counters, act_f16, st);
-    return launch_one<B, G, 2, 1>(layout, d, x, xq, x8_pitch, dxs, y, M, P, partial, counters, act_f16, st);
+                             const float *dxs, uint16_t *y, int M, int mode, GemvPlan plan, float *partial, int *counters, bool act_f16, cudaStream_t st) {
+    auto launch = [&](auto nt, auto md, auto sets) {
+        return launch_one<B, G, decltype(nt)::value, decltype(md)::value, decltype(sets)::value>(layout, d, x, xq, x8_pitch, dxs, y, M, plan.ctas, partial, counters, act_f16, st);
+    };
+    constexpr std::integral_constant<int, 0> zero{};
+    constexpr std::integral_constant<int, 1> one{};
+    constexpr std::integral_constant<int, 2> two{};
+    if (mode == 0) return M <= 8 ? launch(one, zero, std::integral_constant<int, gemv_sets(B, 1, 0)>{}) : launch(two, zero, std::integral_constant<int, gemv_sets(B, 2, 0)>{});
+    if (plan.sets == 1) return M <= 8 ? launch(one, one, one) : launch(two, one, one);
+    return M <= 8 ? launch(one, one, std::integral_constant<int, gemv_sets(B, 1, 1)>{}) : launch(two, one, std::integral_constant<int, gemv_sets(B, 2, 1)>{});
 }
 
 template <int B>
 cudaError_t dispatch_g(const void *layout, const Dims &d, const uint16_t *x, const int8_t *xq, int64_t x8_pitch,
-                       const float *dxs, uint16_t *y, int M, int mode, int P, float *partial, int *counters, bool act_f16, cudaStream_t st) {
+                       const float *dxs, uint16_t *y, int M, int mode, GemvPlan plan, float *partial, int *counters, bool act_f16, cudaStream_t st) {
     switch (d.G) {
-        case 32: return dispatch_nt_mode<B, 32>(layout, d, x, xq, x8_pitch, dxs, y, M, mode, P, partial, counters, act_f16, st);
-        case 64: return dispatch_nt_mode<B, 64>(layout, d, x, xq, x8_pitch, dxs, y, M, mode, P, partial, counters, act_f16, st);
-        default: return dispatch_nt_mode<B, 128>(layout, d, x, xq, x8_pitch, dxs, y, M, mode, P, partial, counters, act_f16, st);
+        case 32: return dispatch_nt_mode<B, 32>(layout, d, x, xq, x8_pitch, dxs, y, M, mode, plan, partial, counters, act_f16, st);
+        case 64: return dispatch_nt_mode<B, 64>(layout, d, x, xq, x8_pitch, dxs, y, M, mode, plan, partial, counters, act_f16, st);
+        default: return dispatch_nt_mode<B, 128>(layout, d, x, xq, x8_pitch, dxs, y, M, mode, plan, partial, counters, act_f16, st);
     }
 }
 
@@ -382,8 +399,8 @@ template <int B, int G>
 cudaError_t launch_groups_g(const GroupTable &t, const Dims &d, const uint16_t *x, const int8_t *xq, const float *dxs, uint16_t *y, int mode,
                             bool act_f16, int P, int max_rows, float *partial, int *counters, cudaStream_t st) {
     const int64_t pitch = (int64_t)d.KT * TILE;
-    if (mode == 0) return launch_one<B, G, 2, 0, true>(nullptr, d, x, nullptr, pitch, nullptr, y, max_rows, P, partial, counters, act_f16, st, &t);
-    return launch_one<B, G, 2, 1, true>(nullptr, d, nullptr, xq, pitch, dxs, y, max_rows, P, partial, counters, act_f16, st, &t);
+    if (mode == 0) return launch_one<B, G, 2, 0, 1, true>(nullptr, d, x, nullptr, pitch, nullptr, y, max_rows, P, partial, counters, act_f16, st, &t);
+    return launch_one<B, G, 2, 1, 1, true>(nullptr, d, nullptr, xq, pitch, dxs, y, max_rows, P, partial, counters, act_f16, st, &t);
 }
 template <int B>
 cudaError_t launch_groups_b(const GroupTable &t, const Dims &d, const uint16_t *x, const int8_t *xq, const float *dxs, uint16_t *y, int mode,
@@ -426,10 +443,15 @@ int sm_count() {
     return n;
 }
 
-// Number of CTAs of the small-M path: one run of tiles each, one CTA per SM.
-GemvPlan gemv_plan(const Dims &d) {
+// CTAs of the small-M path: one run of tiles each, as many as are resident at once.
+GemvPlan gemv_plan(const Dims &d, int64_t M, int mode) {
     const int64_t T = (int64_t)d.NB * d.KT, sms = sm_count();
-    return {(int)(T < sms ? T : sms)};
+    const int NT = M <= 8 ? 1 : 2;
+    GemvPlan p;
+    p.sets = mode == 1 && T < A8_LONG_RUN * sms ? 1 : gemv_sets(d.B, NT, mode);
+    const int64_t places = sms * gemv_occ(d.B, NT, p.sets);
+    p.ctas = (int)(T < places ? T : places);
+    return p;
 }
 
 cudaError_t launch_gemv(const void *layout, const Dims &d, const uint16_t *x, uint16_t *y, int64_t M, int mode,
@@ -444,16 +466,17 @@ cudaError_t launch_gemv(const void *layout, const Dims &d, const uint16_t *x, ui
         cudaError_t e = launch_quantize_a8(x, M, d.K, xq, pitch, dxs, d.B != 4, act_f16, st);
         if (e != cudaSuccess) return e;
     }
-    const int Mi = (int)M, P = gemv_plan(d).ctas;
+    const int Mi = (int)M;
+    const GemvPlan gp = gemv_plan(d, M, mode);
     switch (d.B) {
-        case 1: return dispatch_g<1>(layout, d, x, xq, pitch, dxs, y, Mi, mode, P, partial, counters, act_f16, st);
-        case 2: return dispatch_g<2>(layout, d, x, xq, pitch, dxs, y, Mi, mode, P, partial, counters, act_f16, st);
-        case 3: return dispatch_g<3>(layout, d, x, xq, pitch, dxs, y, Mi, mode, P, partial, counters, act_f16, st);
-        case 4: return dispatch_g<4>(layout, d, x, xq, pitch, dxs, y, Mi, mode, P, partial, counters, act_f16, st);
-        case 5: return dispatch_g<5>(layout, d, x, xq, pitch, dxs, y, Mi, mode, P, partial, counters, act_f16, st);
-        case 6: return dispatch_g<6>(layout, d, x, xq, pitch, dxs, y, Mi, mode, P, partial, counters, act_f16, st);
-        case 7: return dispatch_g<7>(layout, d, x, xq, pitch, dxs, y, Mi, mode, P, partial, counters, act_f16, st);
-        default: return dispatch_g<8>(layout, d, x, xq, pitch, dxs, y, Mi, mode, P, partial, counters, act_f16, st);
+        case 1: return dispatch_g<1>(layout, d, x, xq, pitch, dxs, y, Mi, mode, gp, partial, counters, act_f16, st);
+        case 2: return dispatch_g<2>(layout, d, x, xq, pitch, dxs, y, Mi, mode, gp, partial, counters, act_f16, st);
+        case 3: return dispatch_g<3>(layout, d, x, xq, pitch, dxs, y, Mi, mode, gp, partial, counters, act_f16, st);
+        case 4: return dispatch_g<4>(layout, d, x, xq, pitch, dxs, y, Mi, mode, gp, partial, counters, act_f16, st);
+        case 5: return dispatch_g<5>(layout, d, x, xq, pitch, dxs, y, Mi, mode, gp, partial, counters, act_f16, st);
+        case 6: return dispatch_g<6>(layout, d, x, xq, pitch, dxs, y, Mi, mode, gp, partial, counters, act_f16, st);
+        case 7: return dispatch_g<7>(layout, d, x, xq, pitch, dxs, y, Mi, mode, gp, partial, counters, act_f16, st);
+        default: return dispatch_g<8>(layout, d, x, xq, pitch, dxs, y, Mi, mode, gp, partial, counters, act_f16, st);
     }
 }
 

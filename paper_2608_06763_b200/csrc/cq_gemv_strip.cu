@@ -9,9 +9,9 @@
 // Where a few units more per SM allow it, the CTAs take whole strips and exchange nothing at all (strip_plan).
 //
 // The activations are staged once per CTA for the whole of K, with a power-of-two scale per 128 k (a shuffle among the
-// sixteen lanes that hold them, no barrier), which the fp32 sum of each unit takes back.  Weights reach the registers as
-// in cq_gemv.cu: straight from global memory into a two- or three-deep prefetch, or through a ring in shared memory that
-// each warp fills for itself (cp.async: no barriers, nothing shared between warps).
+// sixteen lanes that hold them, no barrier), which the fp32 sum of each unit takes back.  Weights reach the registers
+// through a ring in shared memory that each warp fills for itself (cp.async: no barriers, nothing shared between warps),
+// or straight from global memory into a three-deep prefetch (strip_uses_ring).
 #include "cq_common.cuh"
 #include "cq_gemv_tile.cuh"
 #include "cq_internal.h"
@@ -26,10 +26,10 @@ constexpr int STRIP_THREADS = 32 * SW;
 constexpr int STRIP_SMEM = 227 * 1024 - 1024;
 
 __host__ __device__ constexpr int unit_bytes(int B, int G) { return 256 * B + 128 * (TILE / G); }
-// Prefetch in registers where it fits them, otherwise the ring (the rule of cq_gemv.cu, for the same reason).
-__host__ __device__ constexpr bool strip_uses_ring(int B, int G, int NT) {
-    return G == 32 || (B >= 5 && B <= 7) || NT == 2 || B == 4 || (B == 8 && G == 64);
-}
+// The ring, but for the narrow codes of one token: their records and codes fit three deep into the registers, and their
+// arithmetic is too short to pay for the way through shared memory (8192 square, G = 128: W1 9.2 us against 9.8, W3 13.5 against 14.0;
+// but W8 20.1 against 18.5, W4 15.4 against 14.4).
+__host__ __device__ constexpr bool strip_uses_ring(int B, int G, int NT) { return !(B <= 3 && G == 128 && NT == 1); }
 __host__ __device__ constexpr int strip_stages(int B, int G) { return unit_bytes(B, G) <= 1664 ? 4 : 3; }
 // shared memory behind the staged activations: unit scales, partial sums, W4 level tables, ring
 __host__ __device__ constexpr int strip_x_bytes(int KT, int NT) { return KT * TILE * NT * 2; }
@@ -65,7 +65,7 @@ gemv_strip_kernel(const __grid_constant__ StripParams p) {
     constexpr int UB = unit_bytes(B, G);
     constexpr bool RING = strip_uses_ring(B, G, NT);
     constexpr int NS = strip_stages(B, G);
-    constexpr int NBUF = RING ? 1 : (B <= 4 ? 3 : 2);
+    constexpr int NBUF = RING ? 1 : 3;
     extern __shared__ __align__(128) uint8_t smem[];
     const int KT = p.KT;
     float *s_inv = reinterpret_cast<float *>(smem + strip_x_bytes(KT, NT));                                      // [KT][NT]
@@ -96,7 +96,7 @@ gemv_strip_kernel(const __grid_constant__ StripParams p) {
     // ---- the load cursor: where the next unit's codes (of this lane) and records lie
     const uint8_t *tile0 = p.layout + ((size_t)(strip >> 3) * KT + kb) * (size_t)TB;
     const uint8_t *wl = tile0 + (strip & 7) * 256 * B + lane * 16;
-    const uint8_t *pl = tile0 + CB + (strip & 7) * 128 * GPT + (RING ? lane * 16 : g * GPT * 8);
+    const uint8_t *pl = tile0 + CB + (strip & 7) * 128 * GPT + (RING ? lane * 16 : record_offset<B, GPT>(lane));
     int l_strip = strip, l_kb = kb, to_load = left;
     auto advance = [&]() {
         wl += TB; pl += TB; --to_load;
@@ -138,10 +138,11 @@ gemv_strip_kernel(const __grid_constant__ StripParams p) {
     DecodeRegs dr = {};
     if constexpr (B != 3 && B != 4) dr = load_decode_regs();
     int8_t *ctab = nullptr;
-    float w4_t0 = 0.0f, w4_t1 = 0.0f;   // positions of the two levels this lane evaluates for a table
+    W4Lane w4{};
+    uint32_t x16 = 16u;
     if constexpr (B == 4) {
         ctab = reinterpret_cast<int8_t *>(s_tab) + warp * 256;
-        w4_t0 = (float)(2 * t) / 7.0f; w4_t1 = (float)(2 * t + 1) / 7.0f;
+        w4 = w4_lane(lane); x16 = c_w4_x16;
     }
     // The activations, the workspace and y may be produced or still used by the kernel launched before this one.
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -178,7 +179,7 @@ gemv_strip_kernel(const __grid_constant__ StripParams p) {
         for (int m = 0; m < NT; ++m)
 #pragma unroll
             for (int i = 0; i < 4; ++i) acc[m][i] = 0.0f;
-        compute_tile<B, G, NT, 2>(r, dr, reinterpret_cast<const uint8_t *>(xs + kb * TILE), xo, ctab, nullptr, w4_t0, w4_t1, g, t, acc);
+        compute_tile<B, G, NT, 2>(r, dr, reinterpret_cast<const uint8_t *>(xs + kb * TILE), xo, ctab, nullptr, w4, x16, g, t, acc);
 #pragma unroll
         for (int m = 0; m < NT; ++m) {
             const float inv = s_inv[kb * NT + m];
@@ -230,7 +231,7 @@ gemv_strip_kernel(const __grid_constant__ StripParams p) {
             ring_load(fill);
             const uint8_t *stage = ring + st * UB;
             TileRegs<B, GPT> regs;
-            load_tile<B, GPT>(regs, stage + lane * 16, stage + 256 * B + g * GPT * 8, lane);
+            load_tile<B, GPT>(regs, stage + lane * 16, stage + 256 * B + record_offset<B, GPT>(lane), lane);
             if (++st == NS) st = 0;
             if (++fill == NS) fill = 0;
             consume(regs);
@@ -287,15 +288,16 @@ gemv_strip_kernel(const __grid_constant__ StripParams p) {
     }
 }
 
-// How many CTAs, and whether they take whole strips.  Whole strips leave some SMs a strip more than others; shared ones
-// cost the exchange at the end of the kernel, some 1.3 us, which is what about 45 units of an SM take (a unit is 16 x 128
-// weights).
+// How many CTAs, and whether they take whole strips.  Whole strips leave some SMs up to a strip more than others; shared ones
+// cost the exchange at the end of the kernel, some 2.3 us, which is what about 50 units of an SM take at W4 (a unit is 16 x
+// 128 weights).  Whole / shared, one token, W4: 4096 square (64 units on the fullest SM, 55.4 on average) 6.1 / 7.4 us,
+// 8192 square (256, 221) 14.5 / 15.2, 28672 x 4096 (416, 387) 20.9 / 21.1, 4096 x 14336 (224, 194) 13.7 / 14.3.
 struct StripPlan { int ctas, whole; };
 StripPlan strip_plan(int64_t S, int64_t KT) {
     const int64_t P = sm_count(), T = S * KT;
     const int64_t whole_units = (S + P - 1) / P * KT;
     StripPlan r;
-    r.whole = whole_units - T / P <= 45;
+    r.whole = whole_units - T / P <= 50;
     const int64_t rounds = (S + P - 1) / P;
     r.ctas = (int)(r.whole ? (S + rounds - 1) / rounds : (T < P ? T : P));
     return r;

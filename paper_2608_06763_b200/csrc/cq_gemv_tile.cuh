@@ -77,8 +77,11 @@ __device__ __forceinline__ void store_half_chunk(__half *tile, int c, const uint
 template <int B, int GPT>
 struct TileRegs {
     uint32_t w[2 * B];
-    uint2 prm[2][GPT];  // {s bits, a | b << 16} of rows g and g + 8
+    uint2 prm[B == 4 ? 1 : 2][GPT];  // {s bits, a | b << 16} of rows g and g + 8; W4: of row lane / 2, whose tables the lane helps to build
 };
+// where a lane's records begin, behind those of the row block
+template <int B, int GPT>
+__device__ __forceinline__ int record_offset(int lane) { return (B == 4 ? lane >> 1 : lane >> 2) * GPT * 8; }
 
 __device__ __forceinline__ uint4 ld_stream16(const void *p) {
     uint4 v;
@@ -105,7 +108,7 @@ __device__ __forceinline__ void load_tile_g(T &r, const uint8_t *wl, const uint8
 #pragma unroll
     for (int gi = 0; gi < GPT; ++gi) {
         r.prm[0][gi] = ld_stream8(pl + gi * 8);
-        r.prm[1][gi] = ld_stream8(pl + (8 * GPT + gi) * 8);
+        if constexpr (B != 4) r.prm[1][gi] = ld_stream8(pl + (8 * GPT + gi) * 8);
     }
 }
 // A warp's slice of a ring stage -> registers.  wl = stage + row-block base + lane * 16 (codes);
@@ -125,7 +128,7 @@ __device__ __forceinline__ void load_tile(TileRegs<B, GPT> &r, const uint8_t *wl
 #pragma unroll
     for (int gi = 0; gi < GPT; ++gi) {
         r.prm[0][gi] = *reinterpret_cast<const uint2 *>(pl + gi * 8);
-        r.prm[1][gi] = *reinterpret_cast<const uint2 *>(pl + (8 * GPT + gi) * 8);
+        if constexpr (B != 4) r.prm[1][gi] = *reinterpret_cast<const uint2 *>(pl + (8 * GPT + gi) * 8);
     }
 }
 
@@ -199,11 +202,11 @@ __device__ __forceinline__ void group_model(const TileRegs<B, TILE / G> &r, cons
 // ctab = this warp's table space.
 template <int B, int G, int NT, int GI>
 __device__ __forceinline__ void group_a8(const TileRegs<B, TILE / G> &r, const int8_t *xs, const int (&xo)[NT], int8_t *ctab,
-                                         const float *tt, int g, int t, float (&acc)[NT][4]) {
+                                         const float *tt, const W4Lane &w4, uint32_t x16, int g, int t, float (&acc)[NT][4]) {
     constexpr int MPG = G / 32;                  // MMAs per group
     constexpr int L = B == 1 ? 1 : (1 << (B - 1));
     constexpr int NE = carrier_table_stride(B);   // bytes from one row's table to the next
-    const uint2 p_lo = r.prm[0][GI], p_hi = r.prm[1][GI];
+    const uint2 p_lo = r.prm[0][GI], p_hi = r.prm[B == 4 ? 0 : 1][GI];
     CarrierPoly poly_lo{}, poly_hi{};
     bool fix = false;
     if constexpr (B >= 6) {
@@ -212,7 +215,13 @@ __device__ __forceinline__ void group_a8(const TileRegs<B, TILE / G> &r, const i
     }
     CarrierTab tab_lo{}, tab_hi{};
     const int8_t *trow_lo = ctab + g * NE, *trow_hi = ctab + (g + 8) * NE;
-    if constexpr (carrier_by_table(B)) {  // lane (g, t) fills magnitudes i = t mod 4 of rows g and g + 8
+    if constexpr (B == 4) {
+        __syncwarp();
+        w4_put_carriers(ctab, 4 * g + t, w4, p_lo);
+        __syncwarp();
+        tab_lo = load_carrier_tab<B>(trow_lo);
+        tab_hi = load_carrier_tab<B>(trow_hi);
+    } else if constexpr (carrier_by_table(B)) {  // lane (g, t) fills magnitudes i = t mod 4 of rows g and g + 8
         __syncwarp();
         const __half2 ab_lo = as_h2(p_lo.y), ab_hi = as_h2(p_hi.y);
         const float a_lo = __low2float(ab_lo), b_lo = __high2float(ab_lo);
@@ -226,7 +235,7 @@ __device__ __forceinline__ void group_a8(const TileRegs<B, TILE / G> &r, const i
             ctab[(g + 8) * NE + up] = (int8_t)c_hi;
             ctab[(g + 8) * NE + dn] = (int8_t)(-c_hi);
         }
-        if (B != 4 && t == 0) { ctab[g * NE] = 0; ctab[(g + 8) * NE] = 0; }   // the reserved pattern (W4: magnitude 0)
+        if (t == 0) { ctab[g * NE] = 0; ctab[(g + 8) * NE] = 0; }   // the reserved pattern
         __syncwarp();
         tab_lo = load_carrier_tab<B>(trow_lo);
         tab_hi = load_carrier_tab<B>(trow_hi);
@@ -236,8 +245,8 @@ __device__ __forceinline__ void group_a8(const TileRegs<B, TILE / G> &r, const i
         constexpr int mi = decltype(mc)::value, MI = GI * MPG + mi;
         uint32_t A[4];
         if constexpr (B <= 5) {
-            a8_row_regs<B, 0, MI>(r.w, tab_lo, A[0], A[2]);
-            a8_row_regs<B, 1, MI>(r.w, tab_hi, A[1], A[3]);
+            a8_row_regs<B, 0, MI>(r.w, tab_lo, x16, A[0], A[2]);
+            a8_row_regs<B, 1, MI>(r.w, tab_hi, x16, A[1], A[3]);
         } else if (!fix) {
             a8_row_eval<B, 0, MI, false>(r.w, poly_lo, A[0], A[2]);
             a8_row_eval<B, 1, MI, false>(r.w, poly_hi, A[1], A[3]);
@@ -252,7 +261,8 @@ __device__ __forceinline__ void group_a8(const TileRegs<B, TILE / G> &r, const i
             else mma_s8(D[tb], A, bf.x, bf.y);
         }
     });
-    const float s_lo = __uint_as_float(p_lo.x & 0x7FFFFFFFu), s_hi = __uint_as_float(p_hi.x & 0x7FFFFFFFu);
+    float s_lo = __uint_as_float(p_lo.x & 0x7FFFFFFFu), s_hi = __uint_as_float(p_hi.x & 0x7FFFFFFFu);
+    if constexpr (B == 4) { const float s = s_lo; s_lo = __shfl_sync(0xffffffffu, s, 2 * g); s_hi = __shfl_sync(0xffffffffu, s, 2 * g + 16); }
 #pragma unroll
     for (int tb = 0; tb < NT; ++tb) {
         acc[tb][0] = fmaf(s_lo, (float)D[tb][0], acc[tb][0]);
@@ -423,24 +433,24 @@ __device__ __forceinline__ void group_dot_w3(const TileRegs<3, TILE / G> &r, con
 // ---- W4, model dtype: levels from the warp's tables (w4_block), unit scale; the group scale multiplies the fp32 group
 // sum.  The staged activations keep their natural order: lane t reads the eight of its word, k = 32 MI + 8 t + i.
 struct W4Rows { uint4 tab[2]; float s[2]; };   // rows g and g + 8
-__device__ __forceinline__ W4Rows w4_rows(uint2 p_lo, uint2 p_hi, uint8_t *wtab, float t0, float t1, int g, int t) {
+__device__ __forceinline__ W4Rows w4_rows(uint2 rec, uint8_t *wtab, const W4Lane &w4, int g, int t) {
     auto pack = [](float a, float b) { return as_u32(__floats2half2_rn(a, b)); };
     __syncwarp();   // the group before has been read
-    w4_put(wtab + g * 16, p_lo, t, t0, t1, 1.0f, pack);
-    w4_put(wtab + (g + 8) * 16, p_hi, t, t0, t1, 1.0f, pack);
+    w4_put(wtab, 4 * g + t, w4, rec, 1.0f, pack);
     __syncwarp();
     W4Rows r;
     r.tab[0] = *reinterpret_cast<const uint4 *>(wtab + g * 16);
     r.tab[1] = *reinterpret_cast<const uint4 *>(wtab + (g + 8) * 16);
-    r.s[0] = __uint_as_float(p_lo.x & 0x7FFFFFFFu);
-    r.s[1] = __uint_as_float(p_hi.x & 0x7FFFFFFFu);
+    const float s = __uint_as_float(rec.x & 0x7FFFFFFFu);
+    r.s[0] = __shfl_sync(0xffffffffu, s, 2 * g);
+    r.s[1] = __shfl_sync(0xffffffffu, s, 2 * g + 16);
     return r;
 }
 template <int G, int NT, int GI>
-__device__ __forceinline__ void group_dot_w4(const TileRegs<4, TILE / G> &r, const __half *xs, const int (&xo)[NT], uint8_t *wtab, float t0, float t1,
+__device__ __forceinline__ void group_dot_w4(const TileRegs<4, TILE / G> &r, const __half *xs, const int (&xo)[NT], uint8_t *wtab, const W4Lane &w4, uint32_t x16,
                                              int g, int t, float (&acc)[NT][4]) {
     constexpr int MPG = G / 32;
-    const W4Rows w = w4_rows(r.prm[0][GI], r.prm[1][GI], wtab, t0, t1, g, t);
+    const W4Rows w = w4_rows(r.prm[0][GI], wtab, w4, g, t);
     __half2 h[NT][2];
 #pragma unroll
     for (int tk = 0; tk < NT; ++tk) { h[tk][0] = __float2half2_rn(0.0f); h[tk][1] = h[tk][0]; }
@@ -452,7 +462,7 @@ __device__ __forceinline__ void group_dot_w4(const TileRegs<4, TILE / G> &r, con
 #pragma unroll
         for (int rr = 0; rr < 2; ++rr) {
             uint32_t lv[4];
-            w4_block(r.w[2 * MI + rr], w.tab[rr], lv);
+            w4_block(r.w[2 * MI + rr], w.tab[rr], x16, lv);
 #pragma unroll
             for (int tk = 0; tk < NT; ++tk) {
                 h[tk][rr] = __hfma2(as_h2(lv[0]), as_h2(xv[tk].x), h[tk][rr]);
@@ -469,16 +479,16 @@ __device__ __forceinline__ void group_dot_w4(const TileRegs<4, TILE / G> &r, con
     }
 }
 template <int G, int NT, int GI>
-__device__ __forceinline__ void group_model_w4(const TileRegs<4, TILE / G> &r, const __half *xs, const int (&xo)[NT], uint8_t *wtab, float t0, float t1,
+__device__ __forceinline__ void group_model_w4(const TileRegs<4, TILE / G> &r, const __half *xs, const int (&xo)[NT], uint8_t *wtab, const W4Lane &w4, uint32_t x16,
                                                int g, int t, float (&acc)[NT][4]) {
     constexpr int MPG = G / 32;
-    const W4Rows w = w4_rows(r.prm[0][GI], r.prm[1][GI], wtab, t0, t1, g, t);
+    const W4Rows w = w4_rows(r.prm[0][GI], wtab, w4, g, t);
     float D[2][NT][4];   // two accumulator sets so consecutive MMAs do not wait on each other
     static_for<MPG>([&](auto mc) {
         constexpr int mi = decltype(mc)::value, MI = GI * MPG + mi;
         uint32_t lo[4], hi[4];
-        w4_block(r.w[2 * MI], w.tab[0], lo);
-        w4_block(r.w[2 * MI + 1], w.tab[1], hi);
+        w4_block(r.w[2 * MI], w.tab[0], x16, lo);
+        w4_block(r.w[2 * MI + 1], w.tab[1], x16, hi);
         const uint32_t A0[4] = {lo[0], hi[0], lo[1], hi[1]}, A1[4] = {lo[2], hi[2], lo[3], hi[3]};   // k = 8 t + 0..3 | 4..7
 #pragma unroll
         for (int tb = 0; tb < NT; ++tb) {
@@ -498,14 +508,14 @@ __device__ __forceinline__ void group_model_w4(const TileRegs<4, TILE / G> &r, c
 
 template <int B, int G, int NT, int MODE>
 __device__ __forceinline__ void compute_tile(const TileRegs<B, TILE / G> &r, const DecodeRegs &dr, const uint8_t *xs, const int (&xo)[NT],
-                                             int8_t *ctab, const float *tt, float t0, float t1, int g, int t, float (&acc)[NT][4]) {
+                                             int8_t *ctab, const float *tt, const W4Lane &w4, uint32_t x16, int g, int t, float (&acc)[NT][4]) {
     constexpr int GPT = TILE / G;
     static_for<GPT>([&](auto gc) {
         constexpr int GI = decltype(gc)::value;
         if constexpr (MODE == 2 && B == 4) {
-            group_dot_w4<G, NT, GI>(r, reinterpret_cast<const __half *>(xs), xo, reinterpret_cast<uint8_t *>(ctab), t0, t1, g, t, acc);
+            group_dot_w4<G, NT, GI>(r, reinterpret_cast<const __half *>(xs), xo, reinterpret_cast<uint8_t *>(ctab), w4, x16, g, t, acc);
         } else if constexpr (MODE == 0 && B == 4) {
-            group_model_w4<G, NT, GI>(r, reinterpret_cast<const __half *>(xs), xo, reinterpret_cast<uint8_t *>(ctab), t0, t1, g, t, acc);
+            group_model_w4<G, NT, GI>(r, reinterpret_cast<const __half *>(xs), xo, reinterpret_cast<uint8_t *>(ctab), w4, x16, g, t, acc);
         } else if constexpr (MODE == 2 && B == 3) {
             group_dot_w3<G, NT, GI>(r, reinterpret_cast<const __half *>(xs), xo, acc);
         } else if constexpr (MODE == 2) {
@@ -519,7 +529,7 @@ __device__ __forceinline__ void compute_tile(const TileRegs<B, TILE / G> &r, con
             if (!fix) group_model<B, G, NT, GI, false>(r, dr, reinterpret_cast<const __half *>(xs), xo, acc);
             else group_model<B, G, NT, GI, true>(r, dr, reinterpret_cast<const __half *>(xs), xo, acc);
         } else {
-            group_a8<B, G, NT, GI>(r, reinterpret_cast<const int8_t *>(xs), xo, ctab, tt, g, t, acc);
+            group_a8<B, G, NT, GI>(r, reinterpret_cast<const int8_t *>(xs), xo, ctab, tt, w4, x16, g, t, acc);
         }
     });
 }

@@ -95,9 +95,9 @@ constexpr int MAX_GROUPS = 32;
 struct Group { const void *layout; int row0, rows, unit0; };
 struct GroupTable { int n; Group g[MAX_GROUPS]; };
 
-// Decomposition of the small-M path: number of CTAs (one contiguous run of tiles each).
-struct GemvPlan { int ctas; };
-GemvPlan gemv_plan(const Dims &d);
+// Decomposition of the small-M path: CTAs (one contiguous run of tiles each), sets of eight warps in each.
+struct GemvPlan { int ctas, sets; };
+GemvPlan gemv_plan(const Dims &d, int64_t M, int mode);
 
 // Small-M (M <= 16) split-K tensor-core GEMV, both activation modes.
 // prequantized (Dynamic A8 only): the workspace already holds the INT8 carrier and the row scales of x (x is not read)
