@@ -93,8 +93,12 @@ def _check(status: int, what: str):
         raise CubicQuantError(f"{what}: {L.cq_status_string(status).decode()} (cuda error {L.cq_last_cuda_error()})")
 
 
+# The current stream's handle without the Stream object around it: building one for each call took some 1.5 us of the host's time.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream() -> int:
-    return torch.cuda.current_stream().cuda_stream
+    return _raw_stream(torch.cuda.current_device()) if _raw_stream is not None else torch.cuda.current_stream().cuda_stream
 
 
 def _ptr(t: torch.Tensor) -> int:
@@ -177,9 +181,11 @@ def cq_gemm(pw: PackedWeights, x: torch.Tensor, mode: int = CQ_MODEL_DTYPE, work
         workspace = torch.zeros(cq_workspace_bytes(pw.B, pw.G, M, pw.N, pw.K, mode), dtype=torch.uint8, device=x.device)
     y = out if out is not None else torch.empty((M, pw.N), dtype=x.dtype, device=x.device)
     assert y.dtype == x.dtype
-    fn = lib().cq_gemm if x.dtype == torch.bfloat16 else lib().cq_gemm_f16
-    _check(fn(_ptr(pw.layout), pw.B, pw.G, _ptr(x), _ptr(y), M, pw.N, pw.K, mode, _ptr(workspace),
-                         workspace.numel(), _stream()), "cq_gemm")
+    L = _lib or lib()
+    fn = L.cq_gemm if x.dtype == torch.bfloat16 else L.cq_gemm_f16
+    status = fn(_ptr(pw.layout), pw.B, pw.G, _ptr(x), _ptr(y), M, pw.N, pw.K, mode, _ptr(workspace), workspace.numel(), _stream())
+    if status != 0:
+        _check(status, "cq_gemm")
     return y
 
 
