@@ -497,7 +497,7 @@ cudaError_t launch_a8(const GroupTable &groups, const Dims &d, const int8_t *x8,
     }
     if (plan.bn != BN) return cudaErrorInvalidConfiguration;
     p.t_full = (int)plan.t_full; p.slices = plan.slices;
-    return launch_overlapped(kern, dim3((unsigned)plan.ctas), A8_THREADS, smem, st, 1, xmap, p);
+    return launch_overlapped(kern, dim3((unsigned)plan.ctas), A8_THREADS, smem, st, 1, true, xmap, p);
 }
 
 // M: rows of x8; tile_m: the rows whose token tile is taken (of an ordinary product, M)

@@ -140,6 +140,11 @@ constexpr bool tc_rings_ok(int B, int G, int BN, int NACC, bool PAIR) {
         && tc_ring_bytes(B, G, BN, NACC, PAIR) + raw * tc_raw_stage_bytes(B, G) + tc_table_bytes(B) + 512 <= 227 * 1024;
 }
 
+// Whether a kernel starts while the one before it drains.  Not the 256-token tiles of one CTA: they leave SMs idle and share their
+// tiles along K, and the next kernel's CTAs and prefetches on those SMs cost more than the launch they hide (4096 square, W4,
+// 130 / 200 / 256 tokens 20.6 / 21.5 / 22.2 us one after another, 21.3 / 22.1 / 22.8 overlapped).
+constexpr bool tc_overlaps(int BN, int NACC, bool PAIR) { return PAIR || BN * NACC < 256; }
+
 __device__ __forceinline__ void named_barrier_sync(int id, int threads) {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
@@ -198,6 +203,11 @@ struct SegWalk {
     }
 };
 
+// Columns that the MMAs of an accumulator of BN tokens compute when `rows` tokens are left for it: a multiple of 16 (of a pair:
+// 32), none if there are none.  The shared-memory tile and the tensor memory keep their places for all BN; what lies beyond is
+// neither computed nor stored.  (200 tokens in a tile of 256: a layout tile takes 0.81 of the MMA time.)
+__device__ __forceinline__ int mma_columns(int64_t rows, int BN, bool pair) { return rows <= 0 ? 0 : rows >= BN ? BN : pair ? ((int)rows + 31) & ~31 : ((int)rows + 15) & ~15; }
+
 // One CTA computes tiles of 128 output channels x (NACC * BN) tokens: NACC accumulators of BN columns share
 // every decoded weight tile, which halves the decode work per flop at NACC = 2.
 template <int B, int G, int BN, int NACC, bool PAIR, bool SK>
@@ -234,7 +244,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
     // The kernel before this one may still be running (launch_overlapped): until its results are waited for, below, the barriers
     // and the tensor memory are set up and the first raw tiles are brought to L2 (not further: L2 sees every write to them).
     if (warp == 0 && lane == 0) prefetch_tensormap(&xmap);
-    if (warp == 2 + DEC_WARPS && lane == 0) {
+    if (tc_overlaps(BN, NACC, PAIR) && warp == 2 + DEC_WARPS && lane == 0) {
         SegWalk<SK, PAIR> first(prm, rank);
         Seg s0;
         if (first.next(s0))
@@ -286,7 +296,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
 #pragma unroll
                         for (int a = 0; a < NACC; ++a) {
                             uint8_t *dst = sB + s * B_STAGE_BYTES + a * B_TILE_BYTES;
-                            const int tok = group.row0 + seg.mt * BNT + a * BN + rank * BROWS;
+                            // of a pair, each CTA brings half of the columns that are computed
+                            const int half_n = PAIR ? mma_columns((int64_t)group.rows - (int64_t)seg.mt * BNT - a * BN, BN, PAIR) / 2 : 0;
+                            const int tok = group.row0 + seg.mt * BNT + a * BN + rank * half_n;
                             if constexpr (PAIR) tma_load_2d_pair(dst, &xmap, map_to_rank(&full[s], 0), (2 * t + half_k) * 64, tok);
                             else tma_load_2d(dst, &xmap, &full[s], (2 * t + half_k) * 64, tok);
                         }
@@ -315,7 +327,6 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
         // uniform; one elected lane issues.
         if (rank == 0) {
             constexpr int MM = PAIR ? 256 : 128;
-            const uint32_t idesc = prm.f16 ? idesc_f16(BN, MM) : idesc_bf16(BN, MM);
             auto commit = [&](uint64_t *bar) { if constexpr (PAIR) umma_commit_pair(bar); else umma_commit(bar); };
             const bool issuer = elect_one();
             int s = 0, segc = 0;
@@ -323,6 +334,14 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
             while (walk.next(seg)) {
                 if (SK && segc > 0) wait(acc_empty, (segc - 1) & 1, 8);   // every decoder has read the accumulators of the segment before
                 ++segc;
+                uint32_t idesc[NACC];
+                bool used[NACC];
+#pragma unroll
+                for (int a = 0; a < NACC; ++a) {
+                    const int n = mma_columns((int64_t)group.rows - (int64_t)seg.mt * BNT - a * BN, BN, PAIR);
+                    used[a] = n > 0;
+                    idesc[a] = prm.f16 ? idesc_f16(n, MM) : idesc_bf16(n, MM);
+                }
                 const int nkb = 2 * (seg.k1 - seg.k0);
                 for (int i = 0; i < nkb; ++i) {
                     wait(&full[s], phase, 3);
@@ -332,11 +351,12 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
                     if (issuer) {
 #pragma unroll
                         for (int a = 0; a < NACC; ++a) {
+                            if (NACC > 1 && !used[a]) continue;
                             const uint64_t bdesc = bdesc0 + (uint64_t)(a * (B_TILE_BYTES >> 4));
 #pragma unroll
                             for (int k = 0; k < 4; ++k) {  // four K = 16 steps, 32 bytes apart inside the swizzle atom
-                                if constexpr (PAIR) umma_bf16_pair(tmem_base + a * BN, adesc + 2 * k, bdesc + 2 * k, idesc, (i | k) != 0);
-                                else umma_bf16(tmem_base + a * BN, adesc + 2 * k, bdesc + 2 * k, idesc, (i | k) != 0);
+                                if constexpr (PAIR) umma_bf16_pair(tmem_base + a * BN, adesc + 2 * k, bdesc + 2 * k, idesc[a], (i | k) != 0);
+                                else umma_bf16(tmem_base + a * BN, adesc + 2 * k, bdesc + 2 * k, idesc[a], (i | k) != 0);
                             }
                         }
                         commit(&empty[s]);  // frees the stage when these MMAs have read it
@@ -364,7 +384,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
         constexpr bool ONE_FENCE = BNT <= 128 && STAGES >= 6;
         W4Lane w4{};
         uint32_t x16 = 16u;
-        if constexpr (B == 4) { w4 = w4_lane(lane); x16 = c_w4_x16; }
+        // wide token tiles have no register left for the sixteen, and the integer pipe is not what bounds them
+        if constexpr (B == 4) { w4 = w4_lane(lane); if (BNT <= 128) x16 = c_w4_x16; }
 #pragma unroll 1
         while (walk.next(seg)) {
 #pragma unroll 1
@@ -690,7 +711,7 @@ cudaError_t launch_bn(const GroupTable &groups, const Dims &d, const uint16_t *x
     cudaError_t ea = ensure_func_attr(kern, attr_done, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
     if (ea != cudaSuccess) return ea;
     p.partial = partial; p.counters = counters; p.f16 = act_f16;
-    return launch_overlapped(kern, dim3((unsigned)plan.ctas), TC_THREADS, smem, st, PAIR ? 2 : 1, xmap, p);
+    return launch_overlapped(kern, dim3((unsigned)plan.ctas), TC_THREADS, smem, st, PAIR ? 2 : 1, tc_overlaps(BN, NACC, PAIR), xmap, p);
 }
 
 // M: rows of x; plan: of the product, or (routed) the token tile of the class

@@ -363,10 +363,10 @@ cudaError_t launch_one(const void *layout, const Dims &d, const uint16_t *x, con
     const dim3 grid((unsigned)P, GRP ? (unsigned)groups->n : 1u);
     constexpr unsigned threads = 256 * SETS;
     if constexpr (GRP)
-        return launch_overlapped(gemv_groups_kernel<B, G, NT, MODE>, grid, threads, smem, st, 1, d, x, xq, x8_pitch, dxs, y, partial, counters, x_tiles,
+        return launch_overlapped(gemv_groups_kernel<B, G, NT, MODE>, grid, threads, smem, st, 1, true, d, x, xq, x8_pitch, dxs, y, partial, counters, x_tiles,
                                  act_f16, *groups);
     else
-        return launch_overlapped(gemv_kernel<B, G, NT, MODE, SETS>, grid, threads, smem, st, 1, (const uint8_t *)layout, d, x, xq, x8_pitch, dxs, y, M,
+        return launch_overlapped(gemv_kernel<B, G, NT, MODE, SETS>, grid, threads, smem, st, 1, true, (const uint8_t *)layout, d, x, xq, x8_pitch, dxs, y, M,
                                  partial, counters, x_tiles, act_f16);
 }
 

@@ -309,7 +309,7 @@ cudaError_t launch_strip_nt(const StripParams &p, int ctas, cudaStream_t st) {
     static std::atomic<uint64_t> attr_done{0};
     cudaError_t e = ensure_func_attr(gemv_strip_kernel<B, G, NT>, attr_done, cudaFuncAttributeMaxDynamicSharedMemorySize, STRIP_SMEM);
     if (e != cudaSuccess) return e;
-    return launch_overlapped(gemv_strip_kernel<B, G, NT>, dim3((unsigned)ctas), STRIP_THREADS, smem, st, 1, p);
+    return launch_overlapped(gemv_strip_kernel<B, G, NT>, dim3((unsigned)ctas), STRIP_THREADS, smem, st, 1, true, p);
 }
 template <int B>
 cudaError_t launch_strip_b(const StripParams &p, int G, int M, int ctas, cudaStream_t st) {

@@ -62,9 +62,10 @@ cudaError_t ensure_func_attr(Kern kern, std::atomic<uint64_t> &done, cudaFuncAtt
 }
 // Launch that may begin while the kernel before it in the stream drains (programmatic dependent launch): every kernel started
 // this way runs griddepcontrol.wait before it touches anything but weights and its own on-chip state.  What is hidden is
-// the launch itself and the set-up in front of the wait.  cluster: CTAs per cluster (1: none).
+// the launch itself and the set-up in front of the wait.  cluster: CTAs per cluster (1: none); overlap: false for the few kernels
+// that gain nothing by it.
 template <class... P, class... A>
-cudaError_t launch_overlapped(void (*kern)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t st, int cluster, A &&...args) {
+cudaError_t launch_overlapped(void (*kern)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t st, int cluster, bool overlap, A &&...args) {
     static const bool use_pdl = getenv("CQ_NO_PDL") == nullptr;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
@@ -73,7 +74,7 @@ cudaError_t launch_overlapped(void (*kern)(P...), dim3 grid, unsigned threads, s
     cfg.stream = st;
     cudaLaunchAttribute attr[2];
     int n = 0;
-    if (use_pdl) {
+    if (use_pdl && overlap) {
         attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         attr[n++].val.programmaticStreamSerializationAllowed = 1;
     }

@@ -480,7 +480,7 @@ cudaError_t launch_quantize_a8(const uint16_t *x, int64_t M, int64_t K, int8_t *
     int64_t threads = ((K >> 3) + 31) / 32 * 32;   // one 8-value chunk per thread when the row is short enough
     if (threads > 1024) threads = 1024;
     if (M > 64 && threads > 256) threads = 256;    // many rows: smaller CTAs fill the SMs better
-    return launch_overlapped(operand_order ? quantize_a8_kernel<true> : quantize_a8_kernel<false>, dim3((unsigned)M), (unsigned)threads, 0, st, 1, x, M, K,
+    return launch_overlapped(operand_order ? quantize_a8_kernel<true> : quantize_a8_kernel<false>, dim3((unsigned)M), (unsigned)threads, 0, st, 1, true, x, M, K,
                              x8, x8_pitch, dx, act_f16);
 }
 
@@ -490,7 +490,7 @@ cudaError_t launch_swiglu_quantize_a8(const uint16_t *h, int64_t M, int64_t I, i
     int64_t threads = ((I >> 3) + 31) / 32 * 32;
     if (threads > 1024) threads = 1024;
     if (M > 64 && threads > 256) threads = 256;
-    return launch_overlapped(operand_order ? swiglu_quantize_a8_kernel<true> : swiglu_quantize_a8_kernel<false>, dim3((unsigned)M), (unsigned)threads, 0, st, 1,
+    return launch_overlapped(operand_order ? swiglu_quantize_a8_kernel<true> : swiglu_quantize_a8_kernel<false>, dim3((unsigned)M), (unsigned)threads, 0, st, 1, true,
                              h, M, I, x8, x8_pitch, dx, act_f16);
 }
 

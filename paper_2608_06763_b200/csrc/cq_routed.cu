@@ -32,7 +32,7 @@ __global__ void __launch_bounds__(256) gather_rows_kernel(const uint16_t *__rest
 cudaError_t launch_gather_rows(const uint16_t *x, const int32_t *route_token, uint16_t *xg, int64_t R, int64_t T, int64_t K,
                                int *status, int *counters, int64_t n, cudaStream_t st) {
     const bool wide = K % 8 == 0 && ((reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(xg)) & 15u) == 0;
-    return launch_overlapped(gather_rows_kernel, dim3((unsigned)R), 256, 0, st, 1, x, route_token, xg, R, T, K, wide, status, counters, n);
+    return launch_overlapped(gather_rows_kernel, dim3((unsigned)R), 256, 0, st, 1, true, x, route_token, xg, R, T, K, wide, status, counters, n);
 }
 
 }  // namespace cq
