@@ -182,7 +182,7 @@ __global__ void __launch_bounds__(128) losses_kernel(const float *__restrict__ W
 // best is picked, so one LANE runs one candidate of one group and a block holds all candidates of a few groups:
 // forty-five of them at effort "fast", twice that under the joint objective.  Bound: the fp64 pipe and the issue slots
 // around it.  2048 x 4096, W4 G128, joint, with packing and layout: 222 ms with one thread per group (its levels and
-// indices in local memory, 14 warps per SM, M + 1 costs per weight), 23.8 ms so.  The sums over a group must be
+// indices in local memory, 14 warps per SM, M + 1 costs per weight), 16.7 ms so.  The sums over a group must be
 // taken in the order of its weights (they decide codes), so a lane walks its group alone; the weights sit in
 // shared memory and are the same address for the lanes of a group.  What a lane keeps per level (z, the carrier grid,
 // the guard) sits in its own column of shared memory, [level][thread], free of bank conflicts for any index.
@@ -328,14 +328,25 @@ __device__ __noinline__ int joint_level_exact(Columns<B> ln, double u, double s)
     }
     return best;
 }
-// the level of one weight
+// the level of one weight by the thresholds; sure: false if it has to be found by the definition
 template <int B, bool JOINT>
-__device__ __forceinline__ int level_of(const Lane<B> &ln, const Weight &w, double s) {
+__device__ __forceinline__ int threshold_level(const Lane<B> &ln, const Weight &w, bool &sure) {
     using S = SearchShape<B>;
     int i = 0;
     if constexpr (S::TAB) {
+        // the bisection of nearest_level, its thresholds picked by selects: M = 2^d - 1 of them take d comparisons and M - d
+        // selects, against M comparisons and M additions one by one
+        float c[S::M];
 #pragma unroll
-        for (int k = 0; k < S::M; ++k) i += (JOINT ? w.f > ln.reg[k] : !(w.f <= ln.reg[k])) ? 1 : 0;
+        for (int k = 0; k < S::M; ++k) c[k] = ln.reg[k];
+#pragma unroll
+        for (int n = S::M; n > 0; n >>= 1) {
+            const int h = n >> 1;
+            const bool up = JOINT ? w.f > c[h] : !(w.f <= c[h]);
+            i += up ? h + 1 : 0;
+#pragma unroll
+            for (int k = 0; k < h; ++k) c[k] = up ? c[h + 1 + k] : c[k];
+        }
     } else {
         int lo = 0, hi = S::M;
         while (lo < hi) {
@@ -345,22 +356,45 @@ __device__ __forceinline__ int level_of(const Lane<B> &ln, const Weight &w, doub
         }
         i = lo;
     }
+    sure = true;
     if constexpr (JOINT) {
         float lower;
         if constexpr (S::TAB) lower = ln.above[i * S::T];
         else lower = i > 0 ? ln.thr[(i - 1) * S::T] + ln.guard2 : -1.0f;
-        if (ln.exact_only || !(w.f > lower)) i = joint_level_exact<B>(ln, w.u, s);
+        sure = w.f > lower;
     }
     return i;
+}
+// f(weight, level) for the weights of a group in their order, STEP at a time: one branch for those that need the definition, and
+// their look-ups overlap.  (With the bisection above: 2048 x 4096, G = 128, joint, W4 23.5 -> 16.7 ms with four, 17.4 with two; W5
+// 41.3 -> 25 with two; four at W5 spill.)
+template <int B, bool JOINT, class F>
+__device__ __forceinline__ void for_levels(const Lane<B> &ln, const Weight *w, int G, double s, F &&f) {
+    constexpr int STEP = B == 3 || B == 5 ? 2 : 4;   // G is a multiple of 32
+#pragma unroll 1
+    for (int j = 0; j < G; j += STEP) {
+        Weight x[STEP];
+        int i[STEP];
+        bool sure[STEP], all = !JOINT || !ln.exact_only;
+#pragma unroll
+        for (int e = 0; e < STEP; ++e) {
+            x[e] = w[j + e];
+            i[e] = threshold_level<B, JOINT>(ln, x[e], sure[e]);
+            all = all && sure[e];
+        }
+        if (JOINT && !all) {
+#pragma unroll
+            for (int e = 0; e < STEP; ++e) if (ln.exact_only || !sure[e]) i[e] = joint_level_exact<B>(ln, x[e].u, s);
+        }
+#pragma unroll
+        for (int e = 0; e < STEP; ++e) f(x[e], i[e]);
+    }
 }
 // closed-form scale under the assignment that the thresholds in place give
 template <int B, bool JOINT>
 __device__ __forceinline__ double assigned_scale(const Lane<B> &ln, const Weight *w, int G, double s) {
     double num = 0.0, den = 0.0;
-#pragma unroll 2
-    for (int j = 0; j < G; ++j) {
-        const Weight x = w[j];
-        const int i = level_of<B, JOINT>(ln, x, s);
+    for_levels<B, JOINT>(ln, w, G, s, [&](const Weight &x, int i) {
         const double z = ln.z(i);
         if constexpr (JOINT) {
             const double zt = ln.zt(i);
@@ -368,7 +402,7 @@ __device__ __forceinline__ double assigned_scale(const Lane<B> &ln, const Weight
         } else {
             num += x.u * z; den += z * z;
         }
-    }
+    });
     return den > 0.0 ? num / den : s;
 }
 
@@ -397,14 +431,11 @@ __device__ __forceinline__ Fit score_serialised(Lane<B> &ln, const Weight *w, in
     const double sd = (double)s32;
     set_thresholds<B, JOINT>(ln, sd, umax);
     double loss = 0.0;
-#pragma unroll 2
-    for (int j = 0; j < G; ++j) {
-        const Weight x = w[j];
-        const int i = level_of<B, JOINT>(ln, x, sd);
+    for_levels<B, JOINT>(ln, w, G, sd, [&](const Weight &x, int i) {
         const double d = x.u - sd * ln.z(i);
         loss += d * d;
         if constexpr (JOINT) { const double d2 = x.u - sd * ln.zt(i); loss += d2 * d2; }
-    }
+    });
     f.s = s32;
     f.loss = loss < INFINITY ? loss : INFINITY;   // NaN never wins
     return f;
@@ -456,15 +487,12 @@ __device__ __noinline__ Fit try_candidate(Columns<B> columns, const Weight *w, i
         if (rf > 0) set_levels<B, JOINT>(ln, a, b);
         set_thresholds<B, JOINT>(ln, s, umax);
         double A00 = 0.0, A01 = 0.0, A02 = 0.0, A11 = 0.0, A12 = 0.0, A22 = 0.0, r0 = 0.0, r1 = 0.0, r2 = 0.0;
-#pragma unroll 2
-        for (int j = 0; j < G; ++j) {
-            const Weight x = w[j];
-            const int i = level_of<B, JOINT>(ln, x, s);
+        for_levels<B, JOINT>(ln, w, G, s, [&](const Weight &x, int i) {
             const double p0 = ln.phi[i], p1 = ln.phi[S::L + i], p2 = ln.phi[2 * S::L + i];
             r0 += p0 * x.u; r1 += p1 * x.u; r2 += p2 * x.u;
             A00 += p0 * p0; A01 += p0 * p1; A02 += p0 * p2;
             A11 += p1 * p1; A12 += p1 * p2; A22 += p2 * p2;
-        }
+        });
         double A[3][3] = {{A00, A01, A02}, {A01, A11, A12}, {A02, A12, A22}}, r[3] = {r0, r1, r2}, p[3];
         if (!solve_3x3(A, r, p)) break;
         if (!(p[0] > 0.0) || !isfinite(p[0])) break;
@@ -521,6 +549,7 @@ __global__ void __launch_bounds__(SearchShape<B>::T) search_kernel(const float *
     for (int i = tid; i < L; i += T) {
         const double t = (double)i / (double)M, t2 = t * t, t3 = t2 * t;
         s_td[i] = t; s_tf[i] = __fdiv_rn((float)i, (float)M);
+        
         s_phi[i] = t3; s_phi[L + i] = t - t3; s_phi[2 * L + i] = t2 - t3;
     }
     for (int i = tid; i < 128; i += T) s_r127[i] = (double)i / 127.0;
