@@ -249,16 +249,20 @@ __device__ __forceinline__ void w4_put(uint8_t *tables, int lane, const W4Lane &
     *reinterpret_cast<uint2 *>(tables + lane * 8) = make_uint2(prmt(v0, v1, 0x6420u), prmt(v0, v1, 0x7531u));
 }
 // Dynamic A8: carriers (carrier_at: clamping q to [0, 1] clamps them, adding 1.5 2^23 rounds to nearest even and leaves the
-// integer in the low bits), positive ones at 0 .. 7 of the row's table, negative ones at 8 .. 15
+// integer in the low bits), positive ones at 0 .. 7 of the row's table, negative ones at 8 .. 15.  That sum is a scalar one:
+// in packed form the compiler contracts it with the product by 127 although both name their rounding, and the carrier is off
+// by one wherever the fp32 product is a tie that the exact one is not.
 __device__ __forceinline__ void w4_put_carriers(int8_t *tables, int lane, const W4Lane &w, uint2 rec) {
     const __half2 ab = as_h2(rec.y);
     const float a = __low2float(ab), b = __high2float(ab);
     const uint64_t a2 = f2_dup(a), b2 = f2_dup(b), c2 = f2_dup(__fsub_rn(__fsub_rn(1.0f, a), b));
     auto pair = [&](uint64_t t, uint32_t &r0, uint32_t &r1) {
-        uint32_t t0, t1, h0, h1;
+        uint32_t t0, t1, h0, h1, v0, v1;
         f2_split(t, t0, t1);
         f2_split(f2_fma(t, f2_fma(t, c2, b2), a2), h0, h1);
-        f2_split(f2_add(f2_mul(f2_pack(mul_sat(t0, h0), mul_sat(t1, h1)), f2_dup(127.0f)), f2_dup(12582912.0f)), r0, r1);
+        f2_split(f2_mul(f2_pack(mul_sat(t0, h0), mul_sat(t1, h1)), f2_dup(127.0f)), v0, v1);
+        r0 = __float_as_uint(__fadd_rn(__uint_as_float(v0), 12582912.0f));
+        r1 = __float_as_uint(__fadd_rn(__uint_as_float(v1), 12582912.0f));
     };
     uint32_t r[4];
     pair(w.t01, r[0], r[1]);
