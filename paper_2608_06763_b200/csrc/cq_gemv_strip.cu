@@ -15,10 +15,13 @@
 #include "cq_common.cuh"
 #include "cq_gemv_tile.cuh"
 #include "cq_internal.h"
+#include "cq_tc_ptx.cuh"
 
 namespace cq {
 
 namespace {
+
+using namespace tc;
 
 constexpr int STRIP = 16;             // output channels of a strip
 constexpr int SW = 24;                // warps of a CTA: three to a scheduler and half the register file each
@@ -66,6 +69,7 @@ gemv_strip_kernel(const __grid_constant__ StripParams p) {
     constexpr bool RING = strip_uses_ring(B, G, NT);
     constexpr int NS = strip_stages(B, G);
     constexpr int NBUF = RING ? 1 : 3;
+    constexpr int PREFETCH = RING ? NS - 1 : NBUF;          // units on their way to L2 before the wait
     extern __shared__ __align__(128) uint8_t smem[];
     const int KT = p.KT;
     float *s_inv = reinterpret_cast<float *>(smem + strip_x_bytes(KT, NT));                                      // [KT][NT]
@@ -126,15 +130,6 @@ gemv_strip_kernel(const __grid_constant__ StripParams p) {
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
-    // weights do not depend on the kernel before this one
-    if constexpr (RING) {
-#pragma unroll
-        for (int i = 0; i < NS - 1; ++i) ring_load(i);
-    } else {
-        static_for<NBUF>([&](auto ic) {
-            if (to_load > 0) { load_tile_g<B, GPT>(buf_at(ic), wl, pl, lane); advance(); }
-        });
-    }
     DecodeRegs dr = {};
     if constexpr (B != 3 && B != 4) dr = load_decode_regs();
     int8_t *ctab = nullptr;
@@ -144,18 +139,40 @@ gemv_strip_kernel(const __grid_constant__ StripParams p) {
         ctab = reinterpret_cast<int8_t *>(s_tab) + warp * 256;
         w4 = w4_lane(lane); x16 = c_w4_x16;
     }
-    // The activations, the workspace and y may be produced or still used by the kernel launched before this one.
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    // Until here the kernel before this one may still be running, and it may be the one that writes the weights: their first
+    // units are brought to L2 and no further (L2 sees every write to them), and read after the wait.  It may also produce
+    // or still use the activations, the workspace and y.
+    if (lane < min(left, PREFETCH)) {
+        const int v = kb0 + v_begin + lane, s = strip0 + v / KT;
+        const uint8_t *tile = p.layout + ((size_t)(s >> 3) * KT + v % KT) * (size_t)TB;
+        prefetch_l2(tile + (s & 7) * 256 * B, 256 * B);
+        prefetch_l2(tile + CB + (s & 7) * 128 * GPT, 128 * GPT);
+    }
+    wait_for_previous_kernel();
 
-    // ---- activations: eight values per thread and step, sixteen lanes hold the 128 k of a tile
+    // ---- activations: eight values per thread and step, sixteen lanes hold the 128 k of a tile.  The first step's loads go out
+    // ahead of the weights', which fill the queue to L2.
     __half *xs = reinterpret_cast<__half *>(smem);
     const int chunks = KT * (TILE / 8);
+    auto x_chunk = [&](int m, int c) {   // K % 8 == 0 always
+        return (int64_t)c * 8 < p.K ? *reinterpret_cast<const uint4 *>(p.x + m * p.K + (int64_t)c * 8) : make_uint4(0u, 0u, 0u, 0u);
+    };
+    uint4 first[NT];
+#pragma unroll
+    for (int m = 0; m < NT; ++m) first[m] = x_chunk(m, threadIdx.x);
+    if constexpr (RING) {
+#pragma unroll
+        for (int i = 0; i < NS - 1; ++i) ring_load(i);
+    } else {
+        static_for<NBUF>([&](auto ic) {
+            if (to_load > 0) { load_tile_g<B, GPT>(buf_at(ic), wl, pl, lane); advance(); }
+        });
+    }
 #pragma unroll
     for (int m = 0; m < NT; ++m) {
+        uint4 v4 = first[m];
         for (int c = threadIdx.x; c < chunks; c += STRIP_THREADS) {
-            uint4 v4 = make_uint4(0u, 0u, 0u, 0u);
-            if ((int64_t)c * 8 < p.K) v4 = *reinterpret_cast<const uint4 *>(p.x + m * p.K + (int64_t)c * 8);   // K % 8 == 0 always
+            if (c >= STRIP_THREADS) v4 = x_chunk(m, c);
             uint32_t ws[4] = {v4.x, v4.y, v4.z, v4.w};
             // the largest in [2^10, 2^11): sixteen products of a normalised level stay in fp16
             const float back = scale_to_half(ws, p.xf16, 10, lane);   // chunks and threads are multiples of sixteen

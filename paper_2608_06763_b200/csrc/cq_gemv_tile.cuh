@@ -83,14 +83,16 @@ struct TileRegs {
 template <int B, int GPT>
 __device__ __forceinline__ int record_offset(int lane) { return (B == 4 ? lane >> 1 : lane >> 2) * GPT * 8; }
 
+// Streaming loads of weights.  Not through the non-coherent path: it asks that the memory is not written while the kernel
+// runs, and the kernel may have started before the one that writes it had ended (launch_overlapped).
 __device__ __forceinline__ uint4 ld_stream16(const void *p) {
     uint4 v;
-    asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    asm volatile("ld.global.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
     return v;
 }
 __device__ __forceinline__ uint2 ld_stream8(const void *p) {
     uint2 v;
-    asm volatile("ld.global.nc.L1::no_allocate.v2.u32 {%0,%1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p));
+    asm volatile("ld.global.L1::no_allocate.v2.u32 {%0,%1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p));
     return v;
 }
 template <int B, int GPT, class T>

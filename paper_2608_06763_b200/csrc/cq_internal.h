@@ -61,8 +61,8 @@ cudaError_t ensure_func_attr(Kern kern, std::atomic<uint64_t> &done, cudaFuncAtt
     return e;
 }
 // Launch that may begin while the kernel before it in the stream drains (programmatic dependent launch): every kernel started
-// this way runs griddepcontrol.wait before it touches anything but weights and its own on-chip state.  What is hidden is
-// the launch itself and the set-up in front of the wait.  cluster: CTAs per cluster (1: none); overlap: false for the few kernels
+// this way runs griddepcontrol.wait before it reads or writes any buffer; what comes before the wait is the set-up of its own
+// on-chip state and prefetches of weights to L2.  cluster: CTAs per cluster (1: none); overlap: false for the few kernels
 // that gain nothing by it.
 template <class... P, class... A>
 cudaError_t launch_overlapped(void (*kern)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t st, int cluster, bool overlap, A &&...args) {
