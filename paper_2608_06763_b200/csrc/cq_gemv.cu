@@ -74,10 +74,12 @@ __host__ __device__ inline int64_t run_of(int64_t v, int64_t V, int64_t P) { ret
 __device__ __forceinline__ void bar_sync(int id, int threads) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory"); }
 
 // ------------------------------------------------------------------------------------------
+// The inputs are not __restrict__ (the compiler could read them through the non-coherent path): the kernel may have started
+// before the one that writes them had ended.
 template <int B, int G, int NT, int MODE, int SETS>
 __device__ __forceinline__ void
-gemv_body(const uint8_t *__restrict__ layout, const Dims &d, const uint16_t *__restrict__ x, const int8_t *__restrict__ xq,
-          int64_t x8_pitch, const float *__restrict__ dxs, uint16_t *__restrict__ y, int M, float *__restrict__ partial,
+gemv_body(const uint8_t *layout, const Dims &d, const uint16_t *x, const int8_t *xq,
+          int64_t x8_pitch, const float *dxs, uint16_t *__restrict__ y, int M, float *__restrict__ partial,
           int *__restrict__ counters, int x_tiles, bool xf16) {
     constexpr int GPT = TILE / G;
     constexpr int L = B == 1 ? 1 : (1 << (B - 1));
@@ -343,8 +345,8 @@ gemv_body(const uint8_t *__restrict__ layout, const Dims &d, const uint16_t *__r
 
 template <int B, int G, int NT, int MODE, int SETS>
 __global__ void __launch_bounds__(256 * SETS, gemv_occ(B, NT, SETS))
-gemv_kernel(const uint8_t *__restrict__ layout, Dims d, const uint16_t *__restrict__ x, const int8_t *__restrict__ xq,
-            int64_t x8_pitch, const float *__restrict__ dxs, uint16_t *__restrict__ y, int M, float *__restrict__ partial,
+gemv_kernel(const uint8_t *layout, Dims d, const uint16_t *x, const int8_t *xq,
+            int64_t x8_pitch, const float *dxs, uint16_t *__restrict__ y, int M, float *__restrict__ partial,
             int *__restrict__ counters, int x_tiles, bool xf16) {
     gemv_body<B, G, NT, MODE, SETS>(layout, d, x, xq, x8_pitch, dxs, y, M, partial, counters, x_tiles, xf16);
 }
@@ -353,7 +355,7 @@ gemv_kernel(const uint8_t *__restrict__ layout, Dims d, const uint16_t *__restri
 // the table among the parameters of every small product cost the sweep over formats at M = 1 four per cent.)
 template <int B, int G, int NT, int MODE>
 __global__ void __launch_bounds__(256, GROUP_OCC)
-gemv_groups_kernel(Dims d, const uint16_t *__restrict__ x, const int8_t *__restrict__ xq, int64_t x8_pitch, const float *__restrict__ dxs,
+gemv_groups_kernel(Dims d, const uint16_t *x, const int8_t *xq, int64_t x8_pitch, const float *dxs,
                    uint16_t *__restrict__ y, float *__restrict__ partial, int *__restrict__ counters, int x_tiles, bool xf16,
                    const __grid_constant__ GroupTable groups) {
     const Group &gr = groups.g[blockIdx.y];

@@ -62,7 +62,8 @@ cudaError_t ensure_func_attr(Kern kern, std::atomic<uint64_t> &done, cudaFuncAtt
 }
 // Launch that may begin while the kernel before it in the stream drains (programmatic dependent launch): every kernel started
 // this way runs griddepcontrol.wait before it reads or writes any buffer; what comes before the wait is the set-up of its own
-// on-chip state and prefetches of weights to L2.  cluster: CTAs per cluster (1: none); overlap: false for the few kernels
+// on-chip state and prefetches of weights to L2.  Their inputs are not __restrict__: the non-coherent path, which that opens to
+// the compiler, wants memory that nobody writes from the kernel's start on.  cluster: CTAs per cluster (1: none); overlap: false for the few kernels
 // that gain nothing by it.
 template <class... P, class... A>
 cudaError_t launch_overlapped(void (*kern)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t st, int cluster, bool overlap, A &&...args) {

@@ -255,7 +255,7 @@ __global__ void __launch_bounds__(256) quantize_a8_scalar_kernel(const uint16_t 
 
 // 16-byte loads, 8-byte stores: K and the pitch multiples of 8, x 16-byte and x8 8-byte aligned
 template <bool OPERAND_ORDER>
-__global__ void __launch_bounds__(1024) quantize_a8_kernel(const uint16_t *__restrict__ x, int64_t M, int64_t K,
+__global__ void __launch_bounds__(1024) quantize_a8_kernel(const uint16_t *x, int64_t M, int64_t K,
                                                           int8_t *__restrict__ x8, int64_t x8_pitch,
                                                           float *__restrict__ dx, bool f16) {
     tc::wait_for_previous_kernel();   // x comes from it, and it may still read the carrier that this one replaces
@@ -342,7 +342,7 @@ __device__ __forceinline__ uint4 gated_act_chunk(const uint4 &g, const uint4 &u,
     return make_uint4(o[0], o[1], o[2], o[3]);
 }
 template <bool OPERAND_ORDER>
-__global__ void __launch_bounds__(1024) swiglu_quantize_a8_kernel(const uint16_t *__restrict__ h, int64_t M, int64_t I,
+__global__ void __launch_bounds__(1024) swiglu_quantize_a8_kernel(const uint16_t *h, int64_t M, int64_t I,
                                                                  int8_t *__restrict__ x8, int64_t x8_pitch,
                                                                  float *__restrict__ dx, bool f16) {
     tc::wait_for_previous_kernel();   // h comes from it

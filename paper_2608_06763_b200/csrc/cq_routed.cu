@@ -10,7 +10,7 @@ namespace cq {
 
 // xg[r][:] = x[route_token[r]][:] for r < R; 16-byte chunks when K is a multiple of 8, else element by element.
 // A route whose token index lies outside [0, T) gets a zero row (the caller owns the map; nothing is read out of range).
-__global__ void __launch_bounds__(256) gather_rows_kernel(const uint16_t *__restrict__ x, const int32_t *__restrict__ route_token,
+__global__ void __launch_bounds__(256) gather_rows_kernel(const uint16_t *x, const int32_t *route_token,
                                                          uint16_t *__restrict__ xg, int64_t R, int64_t T, int64_t K, bool wide,
                                                          int *__restrict__ status, int *__restrict__ counters, int64_t n) {
     tc::wait_for_previous_kernel();

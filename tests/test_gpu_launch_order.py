@@ -1,6 +1,7 @@
-"""Kernels that start while the one before them drains (programmatic dependent launch) read nothing that it writes: the
-weights are written by the kernel right before the product, into the buffer that the product before has just read.
-Output, workspace and inputs exist beforehand, so that no other kernel stands between the two."""
+"""Kernels that start while the one before them drains (programmatic dependent launch) read nothing that it writes: weights
+written by the kernel right before the product, into the buffer that the product before has just read, and activations
+that are the output of the product before.  Output, workspace and inputs exist beforehand, so that no other kernel
+stands between the two."""
 import pytest
 import torch
 
@@ -39,3 +40,44 @@ def test_weights_written_by_the_kernel_before(B, G, M, mode):
             cq.cq_gemm(pw, x, mode, ws, y)
         for *_, alone, y in versions:
             assert torch.equal(y.view(torch.int16), alone.view(torch.int16))
+
+
+@pytest.mark.parametrize("mode", [cq.CQ_MODEL_DTYPE, cq.CQ_DYN_A8])
+@pytest.mark.parametrize("M", [1, 2, 8, 16, 64, 300])
+@pytest.mark.parametrize("B,G", [(3, 128), (4, 64), (8, 32)])
+def test_activations_written_by_the_kernel_before(B, G, M, mode):
+    K, steps = 2048, 12
+    g = torch.Generator(device="cuda")
+    g.manual_seed(B + M)
+    top = (1 << (B - 1)) - 1
+
+    def matrix():
+        k = torch.randint(-top, top + 1, (K, K), generator=g, device="cuda").to(torch.int8)
+        s = 0.02 * (0.5 + torch.rand((K, K // G), generator=g, device="cuda"))
+        a, b = torch.full_like(s, 0.8).half(), torch.full_like(s, -0.1).half()
+        return cq.cq_repack(cq.cq_pack_codes(k, B), s, a, b, B, G, K, K)
+
+    chain = [matrix() for _ in range(3)]
+    x = torch.randn((M, K), generator=g, device="cuda").to(torch.bfloat16)
+    ws = [torch.zeros(cq.cq_workspace_bytes(B, G, M, K, K, mode), dtype=torch.uint8, device="cuda") for _ in chain]
+    ys = [torch.empty_like(x) for _ in range(steps)]
+    routes = torch.arange(M, device="cuda", dtype=torch.int32)
+    offset = [0, M // 2, M]
+
+    def run(wait):
+        h = x
+        for i in range(steps):
+            cq.cq_gemm(chain[i % 3], h, mode, ws[i % 3], ys[i])
+            h = ys[i]
+            if wait:
+                torch.cuda.synchronize()
+        r = cq.cq_gemm_routed(chain[:2], h, routes, offset, mode)   # the gather reads what the last product writes
+        torch.cuda.synchronize()
+        return [y.clone() for y in ys] + [r]
+
+    alone = run(True)
+    assert all(bool(torch.isfinite(y).all()) for y in alone)
+    for _ in range(10):
+        for y in ys:
+            y.zero_()
+        assert all(torch.equal(p, q) for p, q in zip(alone, run(False)))
