@@ -42,6 +42,11 @@ using namespace tc;
 __host__ __device__ constexpr int gemv_sets(int B, int NT, int MODE) { return NT == 2 || (MODE == 1 && B >= 6) ? 2 : 3; }
 __host__ __device__ constexpr int gemv_occ(int B, int NT, int SETS) { return SETS > 1 ? 1 : NT == 2 || B >= 6 ? 2 : 3; }
 constexpr int A8_LONG_RUN = 12;   // tiles an SM
+// In the model dtype CTAs of one set serve the calls with only a tile or two for an SM, where two or three sets of warps stage
+// activations and meet at barriers for one set's work: below one tile an SM (below two or three with one token block, by
+// the width).  One set / large CTAs: 1004 x 512, W1, 3 rows 5.0 / 7.8 us; 1536 x 640, W4, 4 rows 5.7 / 8.1; one token block, narrow codes, two
+// to three tiles an SM 9 % faster; sixteen rows, one to two tiles an SM 5 % slower.
+constexpr int model_long_run(int B, int NT) { return NT == 2 ? 1 : B >= 6 ? 2 : 3; }
 // Below this many tiles an SM the activation quantiser starts while the kernel before it drains (launch_quantize_a8): 1.9 % faster
 // over 153 such products one after another, against 0.3 % slower at 2 to 12 tiles and 3.9 % beyond.
 constexpr int A8_SHORT_CALL = 2;
@@ -70,9 +75,14 @@ __host__ __device__ constexpr int gemv_x_tiles(int B, int G, int NT, int MODE, i
     return (gemv_smem(OCC) - gemv_fixed_bytes(B, G, NT, MODE, SETS) - gemv_x_fixed_bytes(M, B, MODE)) / gemv_x_tile_bytes(M, MODE);
 }
 
-// Tile v of the V = NB KT tiles belongs to run c, the largest with floor(V c / P) <= v.
-__host__ __device__ inline int64_t run_start(int64_t c, int64_t V, int64_t P) { return V * c / P; }
-__host__ __device__ inline int64_t run_of(int64_t v, int64_t V, int64_t P) { return ((v + 1) * P - 1) / V; }
+// Tile v of the V = NB KT tiles belongs to run c, the largest with floor(V c / P) <= v.  V fits 32 bits (a tile has two
+// kilobytes and more) and P^2 does; 64-bit divisions, some hundred cycles each, would stand in the way of the first and the last
+// tile of a short run.
+__device__ __forceinline__ int run_start(unsigned c, unsigned V, unsigned P) { return (int)(c * (V / P) + c * (V % P) / P); }
+__device__ __forceinline__ int run_of(unsigned v, unsigned V, unsigned P) {
+    const uint64_t n = (uint64_t)(v + 1) * P - 1;
+    return (n >> 32) == 0 ? (int)((unsigned)n / V) : (int)(n / V);
+}
 
 __device__ __forceinline__ void bar_sync(int id, int threads) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory"); }
 
@@ -105,9 +115,9 @@ gemv_body(const uint8_t *layout, const Dims &d, const uint16_t *x, const int8_t 
 
     // This CTA's run: tiles [first, first + n) of the layout, which starts at kb0 of its first row block.
     const int KT = d.KT;
-    const int64_t V = (int64_t)d.NB * KT, first = run_start(blockIdx.x, V, gridDim.x);
-    const int n = (int)(run_start((int64_t)blockIdx.x + 1, V, gridDim.x) - first);
-    const int nb0 = (int)(first / KT), kb0 = (int)(first - (int64_t)nb0 * KT);
+    const int V = d.NB * KT, first = run_start(blockIdx.x, V, gridDim.x);
+    const int n = run_start(blockIdx.x + 1, V, gridDim.x) - first;
+    const int nb0 = first / KT, kb0 = first - nb0 * KT;
 
     // ---- this warp's slices of the tiles set, set + SETS, ... of the run, into its ring
     const uint8_t *wl = layout + (size_t)(first + set) * TB + rb * 256 * B + lane * 16;
@@ -151,7 +161,7 @@ gemv_body(const uint8_t *layout, const Dims &d, const uint16_t *x, const int8_t 
     for (int tb = 0; tb < NT; ++tb)
 #pragma unroll
         for (int i = 0; i < 4; ++i) total[tb][i] = 0.0f;
-    int st = 0, fill = NS - 1, seg = 0;
+    int st = 0, fill = NS - 1, seg = 0, nb = nb0;   // nb: the row block at hand
     bool primed = false;
     // The first copies of weights go out behind the loads of the first activations: they fill the queue to L2, and the activations
     // are what the CTA waits for (copies ahead of the loads: 0.8 % longer over 120 products of three to sixteen rows).
@@ -168,6 +178,7 @@ gemv_body(const uint8_t *layout, const Dims &d, const uint16_t *x, const int8_t 
         const int XS = n_st * TILE + XPAD;
         float *inv = reinterpret_cast<float *>(xs + (size_t)M * XS * ES);      // F16: [position][M]
         if (i0 > 0) __syncthreads();   // the tiles before are done with
+        if (F16 && SETS == 1 && !primed) prime();   // a short run: little enough to go first
         if constexpr (F16) {
             // sixteen lanes take a token's 128 k of a tile, eight values each; four loads in flight (eight, with the places
             // counted again for the stores: 4096 square, W4, M = 8 10.4 -> 11.6 us)
@@ -228,8 +239,7 @@ gemv_body(const uint8_t *layout, const Dims &d, const uint16_t *x, const int8_t 
 
         // ---- row block by row block
         for (int i = i0; i < i1;) {
-            const int nb = (int)((first + i) / KT);
-            const int e = (int)min((int64_t)i1, (int64_t)(nb + 1) * KT - first);   // end of the tiles of row block nb
+            const int block_end = (nb + 1) * KT - first, e = min(i1, block_end);   // end of the tiles of row block nb
             int it = i + (set - i % SETS + SETS) % SETS;                              // this set's first tile
             int pos = (it - i0) % n_st;   // n_st < KT: it - i0 < n_st anyway
 #pragma unroll 1
@@ -261,7 +271,7 @@ gemv_body(const uint8_t *layout, const Dims &d, const uint16_t *x, const int8_t 
                 while (pos >= n_st) pos -= n_st;
             }
             i = e;
-            if (i < n && (first + i) % KT != 0) continue;   // the row block goes on behind the next staging
+            if (i < n && i != block_end) continue;   // the row block goes on behind the next staging
 
             // ---- finish the row block (or this run's part of it)
             float *cb = comb + (seg & 1) * (SETS - 1) * 8 * NT * 4 * 32;
@@ -272,9 +282,9 @@ gemv_body(const uint8_t *layout, const Dims &d, const uint16_t *x, const int8_t 
                     for (int q = 0; q < 4; ++q) cb[((((set - 1) * 8 + rb) * NT + tb) * 4 + q) * 32 + lane] = total[tb][q];
             }
             ++seg;
-            __syncthreads();
+            if constexpr (SETS > 1) __syncthreads();
             if (set == 0) {
-                const int kb_begin = nb == nb0 ? kb0 : 0, kb_end = (int)(first + i - (int64_t)nb * KT);
+                const int kb_begin = nb == nb0 ? kb0 : 0, kb_end = first + i - nb * KT;
                 const bool whole = kb_begin == 0 && kb_end == KT;
                 // A run has at most two partial segments: one that starts inside a row block (its first) and one that
                 // starts a row block without finishing it (its last); each CTA owns two partial slots.
@@ -308,8 +318,8 @@ gemv_body(const uint8_t *layout, const Dims &d, const uint16_t *x, const int8_t 
                     }
                     bar_sync(1, 256);
                     if (s_last) {
-                        const int c_first = (int)run_of((int64_t)nb * KT, V, gridDim.x);   // its segment starts the row block: slot 0
-                        const int n_contrib = (int)run_of((int64_t)(nb + 1) * KT - 1, V, gridDim.x) - c_first + 1;
+                        const int c_first = run_of(nb * KT, V, gridDim.x);   // its segment starts the row block: slot 0
+                        const int n_contrib = run_of((nb + 1) * KT - 1, V, gridDim.x) - c_first + 1;
                         const float *pb = partial + ((size_t)c_first * 2 + 1) * (size_t)(M * TILE);   // slot 1 of CTA c_first + q
                         // four consecutive channels of one token per thread and step (128-bit loads), up to eight
                         // slots in flight, added in K order
@@ -341,6 +351,7 @@ gemv_body(const uint8_t *layout, const Dims &d, const uint16_t *x, const int8_t 
             for (int tb = 0; tb < NT; ++tb)
 #pragma unroll
                 for (int q = 0; q < 4; ++q) total[tb][q] = 0.0f;
+            ++nb;
         }
         i0 = i1;
     }
@@ -405,8 +416,11 @@ cudaError_t dispatch_nt_mode(const void *layout, const Dims &d, const uint16_t *
     constexpr std::integral_constant<int, 0> zero{};
     constexpr std::integral_constant<int, 1> one{};
     constexpr std::integral_constant<int, 2> two{};
+    if (plan.sets == 1) {
+        if (mode == 0) return M <= 8 ? launch(one, zero, one) : launch(two, zero, one);
+        return M <= 8 ? launch(one, one, one) : launch(two, one, one);
+    }
     if (mode == 0) return M <= 8 ? launch(one, zero, std::integral_constant<int, gemv_sets(B, 1, 0)>{}) : launch(two, zero, std::integral_constant<int, gemv_sets(B, 2, 0)>{});
-    if (plan.sets == 1) return M <= 8 ? launch(one, one, one) : launch(two, one, one);
     return M <= 8 ? launch(one, one, std::integral_constant<int, gemv_sets(B, 1, 1)>{}) : launch(two, one, std::integral_constant<int, gemv_sets(B, 2, 1)>{});
 }
 
@@ -474,7 +488,7 @@ GemvPlan gemv_plan(const Dims &d, int64_t M, int mode) {
     const int64_t T = (int64_t)d.NB * d.KT, sms = sm_count();
     const int NT = M <= 8 ? 1 : 2;
     GemvPlan p;
-    p.sets = mode == 1 && T < A8_LONG_RUN * sms ? 1 : gemv_sets(d.B, NT, mode);
+    p.sets = T < (mode == 1 ? A8_LONG_RUN : model_long_run(d.B, NT)) * sms ? 1 : gemv_sets(d.B, NT, mode);
     const int64_t places = sms * gemv_occ(d.B, NT, p.sets);
     p.ctas = (int)(T < places ? T : places);
     return p;
