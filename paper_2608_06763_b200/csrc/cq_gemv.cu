@@ -35,18 +35,12 @@ using namespace tc;
 // MODE 0: model dtype.  MODE 1: Dynamic A8 (xq = INT8 carrier [M][x8_pitch], dxs = row scales).  NT: blocks of 8 tokens.
 // Sets of eight warps in a CTA, and CTAs on an SM.  One large CTA reads the activations once per SM and hands over fewer
 // partial sums; it has three sets where 80 registers a thread suffice and two otherwise (two token blocks; INT8 carriers
-// evaluated code by code).  Dynamic A8 only copies its activations, and where runs are short it gains more from CTAs of
-// one set, which leave an SM one by one and let the next kernel's in earlier.  W4 G128, Dynamic A8, M = 16, large CTAs /
-// small ones: 4096 square (6.9 tiles an SM) 13.0 / 12.6 us (W6, M = 8: 18.0 / 16.5), 4096 x 14336 (24 tiles) 20.8 / 22.8,
-// 28672 x 4096 (48) 28.3 / 30.4.
+// evaluated code by code).  CTAs of one set serve the shortest calls, where most sets of a large CTA would have no tile.  Time of
+// one set / of large CTAs over 784 products, by tiles an SM: model dtype 0.94 below one tile, 1.04 at one to three, 1.07 beyond;
+// Dynamic A8 0.96 below one, 0.93 at one to two, 1.03 at two to three, 1.06 beyond.
 __host__ __device__ constexpr int gemv_sets(int B, int NT, int MODE) { return NT == 2 || (MODE == 1 && B >= 6) ? 2 : 3; }
 __host__ __device__ constexpr int gemv_occ(int B, int NT, int SETS) { return SETS > 1 ? 1 : NT == 2 || B >= 6 ? 2 : 3; }
-constexpr int A8_LONG_RUN = 12;   // tiles an SM
-// In the model dtype CTAs of one set serve the calls with only a tile or two for an SM, where two or three sets of warps stage
-// activations and meet at barriers for one set's work: below one tile an SM (below two or three with one token block, by
-// the width).  One set / large CTAs: 1004 x 512, W1, 3 rows 5.0 / 7.8 us; 1536 x 640, W4, 4 rows 5.7 / 8.1; one token block, narrow codes, two
-// to three tiles an SM 9 % faster; sixteen rows, one to two tiles an SM 5 % slower.
-constexpr int model_long_run(int B, int NT) { return NT == 2 ? 1 : B >= 6 ? 2 : 3; }
+constexpr int MODEL_LARGE_CTAS = 1, A8_LARGE_CTAS = 2;   // tiles an SM from which on CTAs are large
 // Below this many tiles an SM the activation quantiser starts while the kernel before it drains (launch_quantize_a8): 1.9 % faster
 // over 153 such products one after another, against 0.3 % slower at 2 to 12 tiles and 3.9 % beyond.
 constexpr int A8_SHORT_CALL = 2;
@@ -73,15 +67,6 @@ __host__ __device__ constexpr int gemv_x_fixed_bytes(int M, int B, int MODE) { r
 // K tiles whose activations fit at a time
 __host__ __device__ constexpr int gemv_x_tiles(int B, int G, int NT, int MODE, int SETS, int OCC, int M) {
     return (gemv_smem(OCC) - gemv_fixed_bytes(B, G, NT, MODE, SETS) - gemv_x_fixed_bytes(M, B, MODE)) / gemv_x_tile_bytes(M, MODE);
-}
-
-// Tile v of the V = NB KT tiles belongs to run c, the largest with floor(V c / P) <= v.  V fits 32 bits (a tile has two
-// kilobytes and more) and P^2 does; 64-bit divisions, some hundred cycles each, would stand in the way of the first and the last
-// tile of a short run.
-__device__ __forceinline__ int run_start(unsigned c, unsigned V, unsigned P) { return (int)(c * (V / P) + c * (V % P) / P); }
-__device__ __forceinline__ int run_of(unsigned v, unsigned V, unsigned P) {
-    const uint64_t n = (uint64_t)(v + 1) * P - 1;
-    return (n >> 32) == 0 ? (int)((unsigned)n / V) : (int)(n / V);
 }
 
 __device__ __forceinline__ void bar_sync(int id, int threads) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory"); }
@@ -183,9 +168,9 @@ gemv_body(const uint8_t *layout, const Dims &d, const uint16_t *x, const int8_t 
             // sixteen lanes take a token's 128 k of a tile, eight values each; four loads in flight (eight, with the places
             // counted again for the stores: 4096 square, W4, M = 8 10.4 -> 11.6 us)
             constexpr int STEP = THREADS / 16, BATCH = 4;
-            int m = 0, p = (int)threadIdx.x >> 4;
-            const int c = threadIdx.x & 15;
-            while (p >= n_st) { p -= n_st; ++m; }
+            const int dm = STEP / n_st, dp = STEP - dm * n_st, c = threadIdx.x & 15;
+            // (no loops that take n_st off one by one: with a tile or two staged, they run to a hundred steps)
+            int m = ((int)threadIdx.x >> 4) / n_st, p = ((int)threadIdx.x >> 4) - m * n_st;
             while (m < M) {
                 uint4 v[BATCH];
                 int mm[BATCH], pp[BATCH];
@@ -197,8 +182,8 @@ gemv_body(const uint8_t *layout, const Dims &d, const uint16_t *x, const int8_t 
                     if (kb >= KT) kb -= KT;
                     const int64_t k = (int64_t)kb * TILE + c * 8;
                     if (m < M && k < d.K) v[u] = *reinterpret_cast<const uint4 *>(x + (int64_t)m * d.K + k);   // K % 8 == 0 always
-                    p += STEP;
-                    while (p >= n_st) { p -= n_st; ++m; }
+                    m += dm; p += dp;
+                    if (p >= n_st) { p -= n_st; ++m; }
                 }
 #pragma unroll
                 for (int u = 0; u < BATCH; ++u) {
@@ -212,15 +197,14 @@ gemv_body(const uint8_t *layout, const Dims &d, const uint16_t *x, const int8_t 
             if (!primed) prime();
         } else {
             // 16-byte chunks in the order the product reads (a8_row_regs; W4: natural); pitch a multiple of 128, zero beyond K
-            const int cpr = n_st * (TILE / 16);
-            int m = 0, c = threadIdx.x;
-            for (;;) {
-                while (c >= cpr) { c -= cpr; ++m; }
-                if (m >= M) break;
+            const int cpr = n_st * (TILE / 16), dm = THREADS / cpr, dc = THREADS - dm * cpr;
+            int m = (int)threadIdx.x / cpr, c = (int)threadIdx.x - m * cpr;
+            while (m < M) {
                 int kb = kbs + (c >> 3);
                 if (kb >= KT) kb -= KT;
                 cp_async16((uint32_t)__cvta_generic_to_shared(xs + (size_t)m * XS + c * 16), xq + (int64_t)m * x8_pitch + (int64_t)kb * TILE + (c & 7) * 16);
-                c += THREADS;
+                m += dm; c += dc;
+                if (c >= cpr) { c -= cpr; ++m; }
             }
             asm volatile("cp.async.commit_group;" ::: "memory");
             if (!primed) {
@@ -488,7 +472,7 @@ GemvPlan gemv_plan(const Dims &d, int64_t M, int mode) {
     const int64_t T = (int64_t)d.NB * d.KT, sms = sm_count();
     const int NT = M <= 8 ? 1 : 2;
     GemvPlan p;
-    p.sets = T < (mode == 1 ? A8_LONG_RUN : model_long_run(d.B, NT)) * sms ? 1 : gemv_sets(d.B, NT, mode);
+    p.sets = T < (mode == 1 ? A8_LARGE_CTAS : MODEL_LARGE_CTAS) * sms ? 1 : gemv_sets(d.B, NT, mode);
     const int64_t places = sms * gemv_occ(d.B, NT, p.sets);
     p.ctas = (int)(T < places ? T : places);
     return p;

@@ -44,10 +44,6 @@ __host__ __device__ constexpr int64_t strip_smem_bytes(int B, int G, int NT, int
     return KT * TILE * NT * 2 + (KT * NT * 4 + 15) / 16 * 16 + strip_slot_bytes(NT) + strip_table_bytes(B) + strip_ring_bytes(B, G, NT);
 }
 
-// u in [0, U) dealt out as P contiguous runs, run c = [floor(U c / P), floor(U (c + 1) / P)); none is empty if P <= U
-__host__ __device__ inline int64_t run_start(int64_t c, int64_t U, int64_t P) { return U * c / P; }
-__host__ __device__ inline int64_t run_of(int64_t u, int64_t U, int64_t P) { return ((u + 1) * P - 1) / U; }
-
 struct StripParams {
     const uint8_t *layout;
     const uint16_t *x;
@@ -79,18 +75,17 @@ gemv_strip_kernel(const __grid_constant__ StripParams p) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
 
     // This CTA's units [u0, u0 + U), and this warp's [v, v_end) of them, counted from u0.
-    const int64_t total_units = (int64_t)p.S * KT;
-    int64_t u0;
-    int U;
+    const int total_units = p.S * KT;
+    int u0, U;
     if (p.whole) {
-        const int s0 = (int)run_start(blockIdx.x, p.S, gridDim.x), s1 = (int)run_start((int64_t)blockIdx.x + 1, p.S, gridDim.x);
-        u0 = (int64_t)s0 * KT;
+        const int s0 = run_start(blockIdx.x, p.S, gridDim.x), s1 = run_start(blockIdx.x + 1, p.S, gridDim.x);
+        u0 = s0 * KT;
         U = (s1 - s0) * KT;
     } else {
         u0 = run_start(blockIdx.x, total_units, gridDim.x);
-        U = (int)(run_start((int64_t)blockIdx.x + 1, total_units, gridDim.x) - u0);
+        U = run_start(blockIdx.x + 1, total_units, gridDim.x) - u0;
     }
-    const int strip0 = (int)(u0 / KT), kb0 = (int)(u0 - (int64_t)strip0 * KT);   // the CTA's first unit
+    const int strip0 = u0 / KT, kb0 = u0 - strip0 * KT;   // the CTA's first unit
     const int NW = min(SW, U);                                                    // warps with work
     const int v_begin = warp < NW ? (int)((uint32_t)U * (uint32_t)warp / (uint32_t)NW) : 0;
     const int v_end = warp < NW ? (int)((uint32_t)U * (uint32_t)(warp + 1) / (uint32_t)NW) : 0;
@@ -257,12 +252,12 @@ gemv_strip_kernel(const __grid_constant__ StripParams p) {
     __syncthreads();
 
     // ---- strips that several warps (or CTAs) share: a warp per strip adds the sums in K order, a lane per row and token
-    const int last_strip = (int)((u0 + U - 1) / KT);
+    const int last_strip = (u0 + U - 1) / KT;
     const int row = lane & 15, tok = lane >> 4;
     for (int s = strip0 + warp; s <= last_strip; s += SW) {
         const int a = max(0, (s - strip0) * KT - kb0), b = min(U, (s + 1 - strip0) * KT - kb0);   // this CTA's units of the strip
         const bool begins = s > strip0 || kb0 == 0, ends = (s + 1 - strip0) * KT - kb0 <= U;
-        const int wf = (int)run_of(a, U, NW), wl_ = (int)run_of(b - 1, U, NW);
+        const int wf = run_of(a, U, NW), wl_ = run_of(b - 1, U, NW);
         if (begins && ends && wf == wl_) continue;   // one warp had all of it and wrote y
         const bool mine = tok < NT;
         float sum = 0.0f;
@@ -275,8 +270,8 @@ gemv_strip_kernel(const __grid_constant__ StripParams p) {
             // The CTA that delivers the last of the strip's partial sums adds them in K order.  The lanes' stores are
             // ordered before lane 0's release by the warp barrier; its acquire and the second one make the others' visible.
             if (mine) __stcg(p.partial + (((size_t)blockIdx.x * 2 + (begins ? 1 : 0)) * NT + tok) * STRIP + row, sum);
-            const int c_first = (int)run_of((int64_t)s * KT, total_units, gridDim.x);
-            const int n = (int)run_of((int64_t)(s + 1) * KT - 1, total_units, gridDim.x) - c_first + 1;
+            const int c_first = run_of(s * KT, total_units, gridDim.x);
+            const int n = run_of((s + 1) * KT - 1, total_units, gridDim.x) - c_first + 1;
             const int sh = 8 * (c_first & 3);
             __syncwarp();
             int last = 0;

@@ -7,6 +7,15 @@
 namespace cq {
 namespace {
 
+// V tiles (or units) dealt out as P contiguous runs, run c = [floor(V c / P), floor(V (c + 1) / P)), and the run that holds v; none
+// is empty if P <= V.  V fits 32 bits (a unit has some four hundred bytes and more) and P^2 does; 64-bit divisions, some hundred
+// cycles each, would stand in the way of the first and the last tile of a short run.
+__device__ __forceinline__ int run_start(unsigned c, unsigned V, unsigned P) { return (int)(c * (V / P) + c * (V % P) / P); }
+__device__ __forceinline__ int run_of(unsigned v, unsigned V, unsigned P) {
+    const uint64_t n = (uint64_t)(v + 1) * P - 1;
+    return (n >> 32) == 0 ? (int)((unsigned)n / V) : (int)(n / V);
+}
+
 __device__ __forceinline__ void mma_f16(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
     asm(
         "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};\n"
