@@ -301,15 +301,20 @@ gemv_strip_kernel(const __grid_constant__ StripParams p) {
 }
 
 // How many CTAs, and whether they take whole strips.  Whole strips leave some SMs up to a strip more than others; shared ones
-// cost the exchange at the end of the kernel, some 2.3 us, which is what about 50 units of an SM take at W4 (a unit is 16 x
-// 128 weights).  Whole / shared, one token, W4: 4096 square (64 units on the fullest SM, 55.4 on average) 6.1 / 7.4 us,
-// 8192 square (256, 221) 14.5 / 15.2, 28672 x 4096 (416, 387) 20.9 / 21.1, 4096 x 14336 (224, 194) 13.7 / 14.3.
+// cost the exchange at the end of the kernel, some 1.5 us.  Whole strips win up to a surplus of some 55 units (16 x 128 weights) on the
+// fullest SM with three bits and fewer, 45 with four and five, 28 with more; at two tokens 45, 32 and 22: 50 kB of
+// weights, less a fifth at two tokens, and at most 60 units, where the narrow codes take as long as their bytes do not.  Over 219
+// products of one and two tokens this is 0.2 % off the better of the two each time; the same 50 units for all formats 0.7 %, and
+// 5504 x 6656, W7 G32, two tokens 19.5 us shared, 22.7 whole.
 struct StripPlan { int ctas, whole; };
-StripPlan strip_plan(int64_t S, int64_t KT) {
-    const int64_t P = sm_count(), T = S * KT;
+StripPlan strip_plan(const Dims &d, int64_t M) {
+    const int64_t S = (d.N + STRIP - 1) / STRIP, KT = d.KT, P = sm_count(), T = S * KT;
     const int64_t whole_units = (S + P - 1) / P * KT;
+    int64_t surplus = 50000 / unit_bytes(d.B, d.G > TILE ? TILE : d.G);
+    if (surplus > 60) surplus = 60;
+    if (M == 2) surplus = surplus * 4 / 5;
     StripPlan r;
-    r.whole = whole_units - T / P <= 50;
+    r.whole = whole_units - T / P <= surplus;
     const int64_t rounds = (S + P - 1) / P;
     r.ctas = (int)(r.whole ? (S + rounds - 1) / rounds : (T < P ? T : P));
     return r;
@@ -340,7 +345,7 @@ bool gemv_strip_ok(const Dims &d, int64_t M, const Workspace &plan) {
     if (M < 1 || M > 2) return false;
     const int G = d.G > TILE ? TILE : d.G;   // wide groups run the G = 128 code
     if (strip_smem_bytes(d.B, G, (int)M, d.KT) > STRIP_SMEM) return false;
-    const StripPlan sp = strip_plan((d.N + STRIP - 1) / STRIP, d.KT);
+    const StripPlan sp = strip_plan(d, M);
     return sp.whole || (sp.ctas <= 255 && (size_t)sp.ctas <= plan.counters_bytes && (size_t)sp.ctas * 2 * STRIP * (size_t)M * 4 <= plan.partial_bytes);
 }
 
@@ -349,7 +354,7 @@ cudaError_t launch_gemv_strip(const void *layout, const Dims &d, const uint16_t 
     StripParams p;
     p.layout = (const uint8_t *)layout; p.x = x; p.y = y; p.partial = partial; p.counters = counters;
     p.N = d.N; p.K = d.K; p.KT = d.KT; p.S = (int)((d.N + STRIP - 1) / STRIP); p.xf16 = act_f16;
-    const StripPlan sp = strip_plan(p.S, p.KT);
+    const StripPlan sp = strip_plan(d, M);
     p.whole = sp.whole;
     switch (d.B) {
         case 1: return launch_strip_b<1>(p, d.G, (int)M, sp.ctas, st);
