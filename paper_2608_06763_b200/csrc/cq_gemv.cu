@@ -41,9 +41,6 @@ using namespace tc;
 __host__ __device__ constexpr int gemv_sets(int B, int NT, int MODE) { return NT == 2 || (MODE == 1 && B >= 6) ? 2 : 3; }
 __host__ __device__ constexpr int gemv_occ(int B, int NT, int SETS) { return SETS > 1 ? 1 : NT == 2 || B >= 6 ? 2 : 3; }
 constexpr int MODEL_LARGE_CTAS = 1, A8_LARGE_CTAS = 2;   // tiles an SM from which on CTAs are large
-// Below this many tiles an SM the activation quantiser starts while the kernel before it drains (launch_quantize_a8): 1.9 % faster
-// over 153 such products one after another, against 0.3 % slower at 2 to 12 tiles and 3.9 % beyond.
-constexpr int A8_SHORT_CALL = 2;
 // Routed products: one set to a CTA and two CTAs to an SM, so that the CTAs of many small matrices fill the SMs evenly.
 constexpr int GROUP_OCC = 2;
 __host__ __device__ constexpr int gemv_unit_bytes(int B, int G) { return 256 * B + 128 * (TILE / G); }
@@ -487,7 +484,7 @@ cudaError_t launch_gemv(const void *layout, const Dims &d, const uint16_t *x, ui
     float *dxs = reinterpret_cast<float *>(ws + plan.dx_off);
     const int64_t pitch = (int64_t)d.KT * TILE;
     if (mode == 1 && !prequantized) {
-        cudaError_t e = launch_quantize_a8(x, M, d.K, xq, pitch, dxs, d.B != 4, act_f16, st, (int64_t)d.NB * d.KT < A8_SHORT_CALL * sm_count());
+        cudaError_t e = launch_quantize_a8(x, M, d.K, xq, pitch, dxs, d.B != 4, act_f16, st);
         if (e != cudaSuccess) return e;
     }
     const int Mi = (int)M;

@@ -22,7 +22,7 @@ cudaError_t launch_a8_partials(const void *layout, const Dims &d, const int8_t *
 // act_f16 (here and below): the 16-bit activation / output patterns are binary16 instead of bfloat16
 // operand_order: x8 in the order of cq_decode.cuh that the INT8 products of every width but four bits read; natural order otherwise
 cudaError_t launch_quantize_a8(const uint16_t *x, int64_t M, int64_t K, int8_t *x8, int64_t x8_pitch, float *dx,
-                               bool operand_order, bool act_f16, cudaStream_t st, bool overlap = false);
+                               bool operand_order, bool act_f16, cudaStream_t st);
 // h[M][2 I] (gate | up, model dtype) -> INT8 carrier of silu(gate) * up, and its row scales
 cudaError_t launch_swiglu_quantize_a8(const uint16_t *h, int64_t M, int64_t I, int8_t *x8, int64_t x8_pitch, float *dx,
                                       bool operand_order, bool act_f16, cudaStream_t st);

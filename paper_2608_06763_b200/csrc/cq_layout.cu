@@ -468,12 +468,14 @@ cudaError_t launch_a8_partials(const void *layout, const Dims &d, const int8_t *
     a8_partials_kernel<<<blocks_for(M * d.N * (d.K / d.G), 128), 128, 0, st>>>(layout, d, x8, M, P);
     return cudaGetLastError();
 }
-// The quantisers are launched when the kernel before them has ended (overlap: not so, for the shortest products, cq_gemv.cu).  Started
-// early, their CTAs settle beside those of the running product and wait there, and the product runs the slower for it: MLP of
-// an 8B model, W4 G128, 100 rows: 95 us, 118 with the gated one started early; 4096 x 14336, W3 G128, Dynamic A8, 200 rows: 46.9
-// and 59.4.
+// Whether a quantiser of M rows starts while the kernel before it drains.  Beyond 64 rows its many small CTAs settle beside those
+// of the running product and wait there, and the product runs the slower for it: MLP of an 8B model, W4 G128, 100 rows 94 us,
+// 118 with the gated quantiser started early; 4096 x 14336, W3 G128, Dynamic A8, 200 rows 46.8 and 59.4.  Up to 64 rows the launch
+// that is hidden counts for more in a stream (22 products of 4 to 64 rows 3 % faster early, 18 MLPs of 4 to 40 rows 4 %; in a
+// captured graph, whose launches are shorter, the products are 3 % slower early and the MLPs the same).
+static bool quantiser_overlaps(int64_t M) { return M <= 64; }
 cudaError_t launch_quantize_a8(const uint16_t *x, int64_t M, int64_t K, int8_t *x8, int64_t x8_pitch, float *dx,
-                               bool operand_order, bool act_f16, cudaStream_t st, bool overlap) {
+                               bool operand_order, bool act_f16, cudaStream_t st) {
     const bool wide = K % 8 == 0 && x8_pitch % 8 == 0 && (reinterpret_cast<uintptr_t>(x) & 15u) == 0 &&
                       (reinterpret_cast<uintptr_t>(x8) & 7u) == 0;
     if (operand_order && !(wide && x8_pitch % 32 == 0)) return cudaErrorInvalidValue;   // internal callers pad the pitch to 128
@@ -484,7 +486,7 @@ cudaError_t launch_quantize_a8(const uint16_t *x, int64_t M, int64_t K, int8_t *
     int64_t threads = ((K >> 3) + 31) / 32 * 32;   // one 8-value chunk per thread when the row is short enough
     if (threads > 1024) threads = 1024;
     if (M > 64 && threads > 256) threads = 256;    // many rows: smaller CTAs fill the SMs better
-    return launch_overlapped(operand_order ? quantize_a8_kernel<true> : quantize_a8_kernel<false>, dim3((unsigned)M), (unsigned)threads, 0, st, 1, overlap, x, M, K,
+    return launch_overlapped(operand_order ? quantize_a8_kernel<true> : quantize_a8_kernel<false>, dim3((unsigned)M), (unsigned)threads, 0, st, 1, quantiser_overlaps(M), x, M, K,
                              x8, x8_pitch, dx, act_f16);
 }
 
@@ -494,9 +496,8 @@ cudaError_t launch_swiglu_quantize_a8(const uint16_t *h, int64_t M, int64_t I, i
     int64_t threads = ((I >> 3) + 31) / 32 * 32;
     if (threads > 1024) threads = 1024;
     if (M > 64 && threads > 256) threads = 256;
-    const auto kern = operand_order ? swiglu_quantize_a8_kernel<true> : swiglu_quantize_a8_kernel<false>;
-    kern<<<(unsigned)M, (unsigned)threads, 0, st>>>(h, M, I, x8, x8_pitch, dx, act_f16);
-    return cudaGetLastError();
+    return launch_overlapped(operand_order ? swiglu_quantize_a8_kernel<true> : swiglu_quantize_a8_kernel<false>, dim3((unsigned)M), (unsigned)threads, 0, st, 1,
+                             quantiser_overlaps(M), h, M, I, x8, x8_pitch, dx, act_f16);
 }
 
 // ---------------------------------------------------------------- cq_debug_wait_timeout
