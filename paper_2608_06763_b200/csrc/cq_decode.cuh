@@ -207,7 +207,7 @@ __device__ __forceinline__ uint32_t mul_sat(uint32_t a, uint32_t b) {
 // ---- W4: eight magnitudes of a (row, group) by table.  In the model dtype the levels are 16-bit values, kept as
 // {low bytes of magnitudes 0-3, high bytes of 0-3, low bytes of 4-7, high bytes of 4-7}.  A half-word of the layout is the selector
 // of four neighbouring weights; two byte permutes fetch their low and high bytes, two more put the bytes together, and the
-// sign bits go into the high bytes by one exclusive or.  Thirteen integer instructions for eight weights, against some forty for
+// sign bits go into the high bytes by one exclusive or.  Twelve integer instructions and a product for eight weights, against some forty for
 // the half2 polynomial, its scale in fp32 and the rounding to the operand's type; the levels themselves are evaluated in fp32
 // and rounded once.  Measured on the linears of an 8B layer, G = 128: M = 1 66.6 -> 56.8 us, M = 13 109.7 -> 105.5,
 // M = 200 (binary16) 194.8 -> 167.7, M = 1024 509.5 -> 491.6 (what is left there is not the decode).  The integer pipe takes one

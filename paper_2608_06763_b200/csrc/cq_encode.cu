@@ -208,8 +208,8 @@ struct __align__(16) Weight { double u; float f; int pad; };   // |w| as fp64 an
 template <int B>
 struct SearchShape {
     static constexpr int M = (1 << (B - 1)) - 1, L = M + 1, T = 128;
-    // Up to sixteen levels: levels and carrier grid in tables, thresholds in registers, compared one by one.  More: a
-    // lane's column would be kilobytes, so it holds the thresholds (bisected) and the carriers as bytes, and a level is
+    // Up to sixteen levels: levels and carrier grid in tables, thresholds in registers, bisected by selects.  More: a lane's
+    // column would be kilobytes, so it holds the thresholds (bisected where they lie) and the carriers as bytes, and a level is
     // computed again when it is read.
     static constexpr bool TAB = B <= 5;
     static constexpr int COL = TAB ? L * (8 + 8 + 4) : L * (4 + 1);      // bytes of a lane's column
@@ -549,7 +549,6 @@ __global__ void __launch_bounds__(SearchShape<B>::T) search_kernel(const float *
     for (int i = tid; i < L; i += T) {
         const double t = (double)i / (double)M, t2 = t * t, t3 = t2 * t;
         s_td[i] = t; s_tf[i] = __fdiv_rn((float)i, (float)M);
-        
         s_phi[i] = t3; s_phi[L + i] = t - t3; s_phi[2 * L + i] = t2 - t3;
     }
     for (int i = tid; i < 128; i += T) s_r127[i] = (double)i / 127.0;

@@ -123,7 +123,7 @@ gemm_a8_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
     uint8_t *sRaw = sB + A8_STAGES * B_STAGE_BYTES;
     int8_t *sTab = reinterpret_cast<int8_t *>(sRaw + A8_RAW_STAGES * prm.raw_stage_bytes);   // [work warp][16 rows][NCODE]
     float *sScale = reinterpret_cast<float *>(sTab + (B >= 3 ? A8_WORK_WARPS * 16 * NCODE : 0));                      // [SRING][128][GPT]
-    float *sT = sScale + A8_SRING * 128 * GPT;                                                 // t_i = i / M, i = 0..127
+    float *sT = sScale + A8_SRING * 128 * GPT;                                                 // W3, W5: t_i = i / M
     uint64_t *bars = reinterpret_cast<uint64_t *>(sT + 128);
     uint64_t *st_full = bars, *st_empty = st_full + A8_STAGES;
     uint64_t *raw_full = st_empty + A8_STAGES, *raw_empty = raw_full + A8_RAW_STAGES;
@@ -168,7 +168,7 @@ gemm_a8_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__
         tmem_slot[3] = prm.f16 ? 1u : 0u;   // the output dtype, parked in shared memory: a register held across the main loop is one too many
         // tmem_slot[4 .. 9]: slice count, slice, tile, row block, token tile and group of this CTA (written above)
     }
-    if (threadIdx.x < 128) sT[threadIdx.x] = __fdiv_rn((float)threadIdx.x, (float)Mx);  // the pinned t = i / M
+    if ((B == 3 || B == 5) && threadIdx.x <= Mx) sT[threadIdx.x] = __fdiv_rn((float)threadIdx.x, (float)Mx);  // the pinned t = i / M of the tables
     if (warp == 1) {
         tmem_alloc(tmem_slot, TMEM_COLS);
         tmem_relinquish();

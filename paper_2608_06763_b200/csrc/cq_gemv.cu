@@ -87,7 +87,8 @@ gemv_body(const uint8_t *layout, const Dims &d, const uint16_t *x, const int8_t 
     extern __shared__ __align__(128) uint8_t smem[];
     __shared__ int s_last;
     __shared__ float s_dx[16];                                         // Dynamic A8: d_x / 127
-    __shared__ float s_t[MODE == 1 && carrier_by_table(B) ? 16 : 1];   // Dynamic A8: t_i = i / M of the carrier tables
+    constexpr bool T_TABLE = MODE == 1 && (B == 3 || B == 5);          // W4 lanes keep their positions in registers
+    __shared__ float s_t[T_TABLE ? 16 : 1];                            // Dynamic A8: t_i = i / M of the carrier tables
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
     const int set = warp >> 3, rb = warp & 7;
     uint8_t *ring = smem + warp * NS * UB;
@@ -122,7 +123,7 @@ gemv_body(const uint8_t *layout, const Dims &d, const uint16_t *x, const int8_t 
     W4Lane w4{};
     uint32_t x16 = 16u;
     if constexpr (B == 4) { w4 = w4_lane(lane); x16 = c_w4_x16; }
-    if constexpr (MODE == 1 && carrier_by_table(B)) {
+    if constexpr (T_TABLE) {
         if (threadIdx.x < L) s_t[threadIdx.x] = __fdiv_rn((float)threadIdx.x, (float)(L - 1));
     }
     // Until here the kernel before this one may still be running, and it may be the one that writes the weights: the first of
