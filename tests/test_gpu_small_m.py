@@ -82,3 +82,47 @@ def test_strips(N, K, B, G, M):
 ])
 def test_row_blocks(N, K, B, G, M, mode):
     check(N, K, B, G, M, mode, torch.float16 if N == 2816 else torch.bfloat16)
+
+
+def every_part_counts(N, K, B, G, M, mode, dtype, lift):
+    """As check, but with sums to which every group contributes alike: plain activations, or (lift) the first half of K scaled
+    down by a power of two that its group scales take back.  One power of two for a whole row of activations would leave nothing
+    of that half in binary16."""
+    k, s, pw = matrix(N, K, B, G, seed=N + K + B)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(M)
+    x = torch.randn((M, K), generator=g, device="cuda")
+    if lift:
+        down, groups = 2.0 ** -34 if dtype == torch.bfloat16 else 2.0 ** -12, K // G // 2
+        x[:, : groups * G] *= down
+        s = s.clone()
+        s[:, :groups] /= down
+        codes, _, a, b = cq.cq_unpack(pw)
+        pw = cq.cq_repack(codes, s, a, b, B, G, N, K)
+    x = x.to(dtype)
+    ws = torch.zeros(cq.cq_workspace_bytes(B, G, M, N, K, mode), dtype=torch.uint8, device="cuda")
+    y = cq.cq_gemm(pw, x, mode, ws)
+    check_y(y.double().cpu().numpy(), reference(k, s, pw, x, mode).cpu().numpy(), f"{N}x{K} W{B} G{G} M={M} mode={mode} lift={lift}")
+
+
+@pytest.mark.parametrize("lift", [False, True])
+@pytest.mark.parametrize("M", [1, 2])
+@pytest.mark.parametrize("N,K,B,G", [
+    (2000, 512, 3, 64), (2377, 1056, 6, 32),
+    (300, 28672, 1, 128), (300, 28672, 3, 128), (300, 28672, 2, 64),            # shared strips, at one token without the ring and with it
+    (3200, 12288, 1, 128), (3200, 12288, 2, 128), (3200, 12288, 3, 128), (3200, 12288, 4, 128), (3200, 12288, 8, 32),
+    (5248, 1280, 7, 64),                                                         # whole strips, three on some SMs
+])
+def test_strips_every_part_counts(N, K, B, G, M, lift):
+    every_part_counts(N, K, B, G, M, cq.CQ_MODEL_DTYPE, torch.float16 if N == 2000 else torch.bfloat16, lift)
+
+
+@pytest.mark.parametrize("mode,lift", [(cq.CQ_MODEL_DTYPE, False), (cq.CQ_MODEL_DTYPE, True), (cq.CQ_DYN_A8, False)])
+@pytest.mark.parametrize("M", [3, 8, 16])
+@pytest.mark.parametrize("N,K,B,G", [
+    (100, 384, 4, 128),                                                          # a tile each to CTAs of one set
+    (2048, 1024, 5, 128), (2304, 1024, 4, 64), (4736, 1024, 3, 128),             # just below one and two tiles an SM, and at two
+    (2816, 2048, 4, 64), (8192, 8192, 8, 128), (24576, 1056, 6, 32),
+])
+def test_row_blocks_every_part_counts(N, K, B, G, M, mode, lift):
+    every_part_counts(N, K, B, G, M, mode, torch.float16 if N == 2816 else torch.bfloat16, lift)
