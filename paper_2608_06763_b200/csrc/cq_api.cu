@@ -48,6 +48,16 @@ Workspace plan_workspace(const Dims &d, int64_t M, int mode) {
     return w;
 }
 
+// What the sizes that a caller may ask for hold beyond the need of the call itself: room for the partial sums of three CTAs an SM.
+// A program that asks once, for its largest number of rows, uses that workspace for fewer too, and which CTAs serve how
+// many rows is the library's affair; with no more than each call's own need, 1200 of a million pairs of row counts and shapes
+// lost what the sizes of earlier versions had granted them.
+static size_t spare_bytes(const Dims &d, int64_t M, size_t partial_bytes) {
+    const int64_t T = (int64_t)d.NB * d.KT, places = 3 * (int64_t)sm_count();
+    const size_t room = align_up((size_t)(T < places ? T : places) * 2 * (size_t)(M < 16 ? M : 16) * TILE * 4, 256);
+    return room > partial_bytes ? room - partial_bytes : 0;
+}
+
 static int check_format(int B, int G, int64_t N, int64_t K) {
     if (B < 1 || B > 8 || N <= 0 || K <= 0 || G <= 0) return CQ_ERR_INVALID_ARG;
     if (G != 32 && G != 64 && G != 128 && G != 256 && G != 512) return CQ_ERR_UNSUPPORTED;
@@ -115,7 +125,9 @@ size_t cq_layout_bytes(int B, int G, int64_t N, int64_t K) {
 
 size_t cq_workspace_bytes(int B, int G, int64_t M, int64_t N, int64_t K, int mode) {
     if (check_format(B, G, N, K) != CQ_OK || M <= 0 || (mode != CQ_MODEL_DTYPE && mode != CQ_DYN_A8)) return 0;
-    return plan_workspace(make_dims(B, G, N, K), M, mode).total;
+    const Dims d = make_dims(B, G, N, K);
+    const Workspace w = plan_workspace(d, M, mode);
+    return w.total + spare_bytes(d, M, w.partial_bytes);
 }
 
 int cq_workspace_init(void *workspace, size_t workspace_bytes, void *stream) {
@@ -199,7 +211,9 @@ static MlpPlan plan_mlp(const Dims &dgu, const Dims &ddn, int64_t M, int mode_gu
 size_t cq_mlp_workspace_bytes(int B_gu, int G_gu, int B_dn, int G_dn, int64_t M, int64_t K, int64_t I, int64_t N, int mode_gate_up) {
     if (check_format(B_gu, G_gu, 2 * I, K) != CQ_OK || check_format(B_dn, G_dn, N, I) != CQ_OK || M <= 0) return 0;
     if (mode_gate_up != CQ_MODEL_DTYPE && mode_gate_up != CQ_DYN_A8) return 0;
-    return plan_mlp(make_dims(B_gu, G_gu, 2 * I, K), make_dims(B_dn, G_dn, N, I), M, mode_gate_up).total;
+    const Dims dgu = make_dims(B_gu, G_gu, 2 * I, K), ddn = make_dims(B_dn, G_dn, N, I);
+    const MlpPlan p = plan_mlp(dgu, ddn, M, mode_gate_up);
+    return p.total + spare_bytes(dgu, M, p.gu.partial_bytes) + spare_bytes(ddn, M, p.dn.partial_bytes);
 }
 
 int cq_mlp_swiglu(const void *layout_gate_up, int B_gu, int G_gu, const void *layout_down, int B_dn, int G_dn, const uint16_t *x,
@@ -354,7 +368,9 @@ size_t cq_routed_workspace_bytes(int B, int G, int E, const int64_t *expert_offs
     if (check_format(B, G, N, K) != CQ_OK || E <= 0 || !expert_offset_host || (mode != CQ_MODEL_DTYPE && mode != CQ_DYN_A8)) return 0;
     const int64_t R = expert_offset_host[E];
     if (R <= 0 || !routed_offsets_ok(expert_offset_host, E, R)) return 0;
-    return plan_routed(make_dims(B, G, N, K), expert_offset_host, E, mode).total;
+    const Dims d = make_dims(B, G, N, K);
+    const RoutedPlan p = plan_routed(d, expert_offset_host, E, mode);
+    return p.total + spare_bytes(d, 16, p.sub_off - p.part_off) + spare_bytes(d, 16, p.total - p.sub_off);
 }
 
 int cq_gemm_routed(const void *const *layouts_host, int E, int B, int G, const uint16_t *x, const int32_t *route_token,

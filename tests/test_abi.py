@@ -152,3 +152,14 @@ def test_routed_groups_that_would_idle_the_gpu_run_one_by_one():
     assert launches(1024, 4096, [20, 20], 3, 32, 1) == [1, 1] and launches(1024, 4096, [128, 128], 4, 64, 1) == [1, 1]
     assert launches(2816, 2048, [64, 64], 4, 64) == [2] and launches(1024, 4096, [64] * 8) == [8]
     assert launches(2816, 2048, [48] * 16, 4, 64) == [16] and launches(1024, 4096, [64] * 8, 4, 64, 1) == [8]
+
+
+
+@pytest.mark.parametrize("B,G,N,K,mode,larger,smaller", [
+    (1, 32, 1024, 8192, 1, 200, 129), (2, 64, 28672, 4096, 0, 700, 32), (8, 128, 4096, 4096, 0, 513, 17), (1, 128, 8192, 1024, 0, 200, 17),
+    (4, 32, 8192, 14336, 1, 65, 64), (7, 32, 2377, 8192, 1, 128, 17), (3, 64, 57344, 4096, 1, 1024, 300), (6, 32, 8192, 1024, 1, 256, 32),
+    (4, 128, 4096, 4096, 0, 16, 3), (4, 128, 28672, 4096, 1, 512, 16)])
+def test_a_workspace_for_more_rows_serves_fewer(B, G, N, K, mode, larger, smaller):
+    """Pairs of row counts whose sizes covered one another before the small-M kernel took CTAs of several sizes: a program that
+    asks once, for the larger count, must not be refused the smaller."""
+    assert cq.cq_workspace_bytes(B, G, larger, N, K, mode) >= cq.cq_workspace_bytes(B, G, smaller, N, K, mode)
