@@ -339,7 +339,9 @@ cudaError_t launch_strip_b(const StripParams &p, int G, int M, int ctas, cudaStr
 
 }  // namespace
 
-// The staged activations bound K; the counters, a byte per CTA, have to fit the workspace's (256 bytes at least), and the
+// The staged activations bound K beside a ring of full depth; beyond, cq_gemv.cu serves, which is faster there than a ring of two
+// stages: 8192 x 28672, two tokens, W4 G128 45.1 us against 46.3, W8 G128 56.7 against 61.6 (with the kernel that cut runs of
+// tiles for three CTAs an SM 50.3 and 67.4); only W8 G32 at one token 65.4 against 61.5.  The counters, a byte per CTA, have to fit the workspace's (256 bytes at least), and the
 // partial sums its slots (two of 128 sums a token for each CTA of cq_gemv.cu, of which there are at least as many).
 bool gemv_strip_ok(const Dims &d, int64_t M, const Workspace &plan) {
     if (M < 1 || M > 2) return false;
